@@ -19,7 +19,7 @@
 #include <tuple>
 #include <vector>
 
-#include "kernels.h"
+#include "team.cuh"
 
 using namespace upr;
 
@@ -106,8 +106,7 @@ __global__ void k_fill_i64(int64_t *a, int64_t n, int64_t v) {
 namespace {
 // Slots of the device counters (upr_ctx::counts).
 enum {
-    CNT_CAND = 0, CNT_M, CNT_P, CNT_S, CNT_A, CNT_I, CNT_HUB, CNT_BADPART, CNT_L1, CNT_X, CNT_EVM, CNT_EVI,
-    CNT_I1, CNT_OVER0, CNT_INFEAS, CNT_HIST, CNT_EXACT, CNT_SORTP, CNT_SLOTS = 32
+    CNT_CAND = 0, CNT_M, CNT_P, CNT_S, CNT_A, CNT_I, CNT_HUB, CNT_BADPART, CNT_L1, CNT_X, CNT_OVER0, CNT_INFEAS, CNT_HIST, CNT_EXACT, CNT_SORTP, CNT_SLOTS = 32
 };
 
 // Per-call sums of the step graph's rounds (upr_ctx::dstats): candidates,
@@ -256,24 +255,23 @@ struct upr_ctx {
     int32_t *part0, *part; int64_t *C0, *C, *cut; int32_t *W;
     int64_t *BW, *PW, *F; int8_t *first_slot;
     // node-indexed
-    int32_t *cand_tgt, *cand_gain, *flags, *flags2, *excl_i, *m_pos, *r_to, *r_at, *pos, *dest, *prop_tgt, *prop_gain;
+    int32_t *cand_tgt, *cand_gain, *flags, *flags2, *m_pos, *r_to, *r_at, *prop_tgt, *prop_gain;
     int64_t *cand_s0;
     // lists
-    int32_t *idxA, *idxB, *idxC, *idxD, *L1, *Pq;
-    int64_t *score;
+    int32_t *idxA, *idxB, *idxC, *L1, *Pq;
+    int32_t *score;
     int32_t *M_node, *M_from, *M_to; int64_t *M_score;
     int32_t *R_node, *R_from, *R_to, *R_sub;
-    int32_t *X_node, *X_from, *X_to, *final_to; int8_t *X_isr;
+    int32_t *X_node, *X_from, *X_to;
     int32_t *I_node, *I_from, *I_to; int64_t *I_gain, *Gsum;
     SortBuf sb[3];
-    int64_t *c_sorted, *c_excl, *delta, *d_excl;
-    uint64_t *packed, *qmax;
+    int64_t *c_sorted, *c_excl, *seg_base;
+    uint64_t *packed;
     uint64_t *prio_rep;                 // [2 * kPrioBins] rebalancing: a key per prefilter bin
-    int32_t *emit, *qbefore, *em_excl, *pos_m;
+    int32_t *emit, *qbefore, *pos_m;
     int32_t *diff, *diff_excl;
-    int32_t *hub_flag, *hub_excl, *hubs;
-    int32_t *seg_first, *rbeg, *rend, *ebeg, *eend, *qfin, *left, *left_excl;
-    long long *best_parts, *best;
+    int32_t *seg_first, *rbeg, *rend, *ebeg, *eend, *qfin, *left_excl;
+    long long *best;
     int8_t *over_d, *excl_d, *reject_d;
     long long *Cd;                   // [K] block-weight changes of a fused rebalancing sub-round
     unsigned long long *prio_hist;   // [K][kPrioBins] proposal prefilter (null: K too large, no prefilter)
@@ -284,6 +282,8 @@ struct upr_ctx {
     uint64_t *vacc; int32_t *vflags; int64_t *scal, *cut_parts;
     int2 *pk;                 // exact gains: position in I and blocks before/after, per node
     Scratch tmp;              // scan / sort temporaries
+    Team team;                // the team launches of this binding
+    int beside = 1;           // contexts that refine at the same time as this one, with it
     // pinned host mirrors
     int64_t *h = nullptr;     // pinned scratch
     int8_t *h8 = nullptr;
@@ -336,18 +336,17 @@ void layout(upr_ctx *c, Arena &A) {
     c->PW = A.take<int64_t>(k * kSlots);
     c->F = A.take<int64_t>(kSlots);
     c->first_slot = A.take<int8_t>(k);
-    for (int32_t **p : {&c->cand_tgt, &c->cand_gain, &c->flags, &c->m_pos, &c->r_to, &c->pos, &c->dest, &c->prop_tgt,
+    for (int32_t **p : {&c->cand_tgt, &c->cand_gain, &c->flags, &c->m_pos, &c->r_to, &c->prop_tgt,
                         &c->prop_gain, &c->idxA, &c->idxB, &c->idxC, &c->M_node, &c->M_from, &c->M_to, &c->R_node,
                         &c->R_from, &c->R_to, &c->R_sub, &c->I_node, &c->I_from, &c->I_to, &c->emit, &c->qbefore,
-                        &c->em_excl, &c->pos_m, &c->hub_flag, &c->hub_excl, &c->hubs, &c->L1, &c->r_at, &c->Pq})
+                        &c->pos_m, &c->L1, &c->r_at, &c->Pq})
         *p = A.take<int32_t>(n);
-    for (int32_t **p : {&c->flags2, &c->excl_i, &c->idxD, &c->X_node, &c->X_from, &c->X_to, &c->final_to})
+    for (int32_t **p : {&c->flags2, &c->X_node, &c->X_from, &c->X_to})
         *p = A.take<int32_t>(n2 + 1);
     c->diff = A.take<int32_t>(n + 2);
     c->diff_excl = A.take<int32_t>(n + 2);
-    c->X_isr = A.take<int8_t>(n2);
     c->cand_s0 = A.take<int64_t>(n);
-    c->score = A.take<int64_t>(n);
+    c->score = A.take<int32_t>(n);
     c->M_score = A.take<int64_t>(n);
     c->I_gain = A.take<int64_t>(n);
     c->Gsum = A.take<int64_t>(n);
@@ -359,14 +358,11 @@ void layout(upr_ctx *c, Arena &A) {
     }
     c->c_sorted = A.take<int64_t>(n2);
     c->c_excl = A.take<int64_t>(n2);
-    c->delta = A.take<int64_t>(n2);
-    c->d_excl = A.take<int64_t>(n2);
     c->packed = A.take<uint64_t>(n2);
-    c->qmax = A.take<uint64_t>(n2);
+    c->seg_base = A.take<int64_t>(k);
     c->prio_rep = A.take<uint64_t>(2 * (size_t)kPrioBins);
-    for (int32_t **p : {&c->seg_first, &c->rbeg, &c->rend, &c->ebeg, &c->eend, &c->qfin, &c->left, &c->left_excl})
+    for (int32_t **p : {&c->seg_first, &c->rbeg, &c->rend, &c->ebeg, &c->eend, &c->qfin, &c->left_excl})
         *p = A.take<int32_t>(k);
-    c->best_parts = A.take<long long>(2048);
     c->best = A.take<long long>(2);
     c->over_d = A.take<int8_t>(k);
     c->excl_d = A.take<int8_t>(k);
@@ -391,6 +387,11 @@ void layout(upr_ctx *c, Arena &A) {
     c->tmp.ticket = A.take<unsigned int>(64);
     c->tmp.err = A.take<int32_t>(1);
     c->tmp.epoch = A.take<uint32_t>(1);
+    c->team.size = team_size((int64_t)n, c->beside);
+    c->team.hist = A.take<int32_t>((size_t)c->team.size * team::kSortBins);
+    c->team.tot = A.take<long long>((size_t)team::kTotSlots * team::kTeamMax);
+    c->team.bar = reinterpret_cast<unsigned long long *>(c->tmp.ticket + 16);     // (cleared at every binding)
+    c->team.err = c->tmp.err;
 }
 
 enum MemKind { kHost = 0, kDevice = 1 };
@@ -944,16 +945,15 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     const int64_t n = c->n;
     const int32_t K = G.K();
     const bool batch = c->ng > 1;
-    const int kbits = std::max(1, bit_length((uint64_t)(K - 1)));
     upr_trace *T = tr ? tr->t : nullptr;
     int32_t *cnt = c->counts;
     RebalCtl *ctl = c->ctl;
-    const Count cN{nullptr, n};
-    uint64_t *ko; uint32_t *vo;
 
     UPR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * CNT_SLOTS, s));
-    UPR_CUDA(cudaMemcpyAsync(c->part, c->part0, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-    UPR_CUDA(cudaMemcpyAsync(c->C, c->C0, sizeof(int64_t) * K, cudaMemcpyDeviceToDevice, s));
+    if (rebalance_only || n == 0) {     // (else the selection's ordering does it)
+        UPR_CUDA(cudaMemcpyAsync(c->part, c->part0, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+        UPR_CUDA(cudaMemcpyAsync(c->C, c->C0, sizeof(int64_t) * K, cudaMemcpyDeviceToDevice, s));
+    }
     // ---- (a) gain table of the round-start partition (kept from the previous
     // round of this call when it is valid)
     // (in the step graph the table is always carried: round 1's build runs before it)
@@ -998,22 +998,19 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         });
         if (c->prm.lock_rebalanced)        // the oscillation guard (Sec. 2)
             guard_filter(c->locked, n, c->flags, c->cand_tgt, c->cand_s0, c->cand_gain, s);
-        select_flags(c->flags, c->idxA, cnt + CNT_CAND, cN, c->tmp, s);
-        const Count cC{cnt + CNT_CAND, n};
-        // ---- (b3) inflow penalties: order by (target, s0 desc, id)
-        cand_keys(c->idxA, cnt + CNT_CAND, c->cand_tgt, c->cand_s0, c->gbits, c->sb[0].k, c->sb[0].v, n, s);
-        c->sb[0].run(cC, c->gbits + kbits, c->tmp, s, &ko, &vo);
-        cand_gather(G, c->idxA, vo, cnt + CNT_CAND, c->cand_tgt, c->c_sorted, c->seg_first, n, s);
-        exclusive_sum_i64(c->c_sorted, c->c_excl, cC, c->tmp, s);
-        inflow_filter(G, c->idxA, vo, cnt + CNT_CAND, c->cand_tgt, c->cand_gain, c->c_excl, c->seg_first, pen,
-                      c->flags2, c->score, n, s);
-        select_flags(c->flags2, c->idxB, cnt + CNT_M, cC, c->tmp, s);
-        // ---- M ordered by (score desc, id), applied
-        uint64_t *k2; uint32_t *v2;
-        move_keys(c->idxB, cnt + CNT_M, c->score, c->gbits, c->sb[1].k, c->sb[1].v, n, s);
-        c->sb[1].run(Count{cnt + CNT_M, n}, c->gbits, c->tmp, s, &k2, &v2);
-        apply_moves(G, c->idxA, c->idxB, v2, cnt + CNT_M, c->cand_tgt, c->score, c->part0, c->part, c->C, c->M_node,
-                    c->M_from, c->M_to, c->M_score, c->m_pos, c->scal + 1, n, s);
+        // ---- (b3) inflow penalties, M ordered by (score desc, id), applied
+        SelOrder so{};
+        so.team = c->team;
+        so.cand_tgt = c->cand_tgt; so.cand_gain = c->cand_gain; so.cand_s0 = c->cand_s0;
+        so.pen = pen;
+        so.part0 = c->part0; so.C0 = c->C0; so.part = c->part; so.C = c->C;
+        so.score = c->score;
+        so.c_excl = c->c_excl; so.seg_base = c->seg_base;
+        so.bufA = c->sb[0].k; so.bufB = c->sb[1].k;
+        so.M_node = c->M_node; so.M_from = c->M_from; so.M_to = c->M_to; so.M_score = c->M_score; so.m_pos = c->m_pos;
+        so.deg_sum = c->scal + 1;
+        so.d_cand = cnt + CNT_CAND; so.d_moves = cnt + CNT_M;
+        select_order(G, so, c->gbits, s);
         // W' for P o M: the delta update costs two atomics per adjacency entry of a
         // moved node, a rebuild streams the graph and the table once; each kernel
         // checks on the device which of the two applies
@@ -1030,80 +1027,31 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
 
     // ---- (c1) interleave M and R_1..R_k (or append R after M: a variant of Sec. 7.2)
     const int32_t *dM = cnt + CNT_M, *dR = &ctl->nR;
-    count_affine(dM, 2, nullptr, 0, cnt + CNT_EVM, s);
-    count_affine(dM, 1, dR, 0, cnt + CNT_X, s);
-    if (c->prm.append) {
-        seq_append(c->M_node, c->M_from, c->M_to, dM, c->R_node, c->R_from, c->R_to, dR, 2 * n, c->X_node, c->X_from,
-                   c->X_to, c->X_isr, s);
-    } else {
-    UPR_CUDA(cudaMemsetAsync(c->rbeg, 0, sizeof(int32_t) * K, s));
-    UPR_CUDA(cudaMemsetAsync(c->rend, 0, sizeof(int32_t) * K, s));
-    UPR_CUDA(cudaMemsetAsync(c->ebeg, 0, sizeof(int32_t) * K, s));
-    UPR_CUDA(cudaMemsetAsync(c->eend, 0, sizeof(int32_t) * K, s));
-    uint64_t *kRB; uint32_t *RB;
-    seq_rb_keys(c->R_from, dR, n, c->sb[0].k, c->sb[0].v, s);
-    c->sb[0].run(Count{dR, n}, kbits, c->tmp, s, &kRB, &RB);
-    seq_rb_bounds(c->R_node, c->R_from, RB, dR, n, G.vwgt, c->c_sorted, c->rbeg, c->rend, s);
-    exclusive_sum_i64(c->c_sorted, c->c_excl, Count{dR, n}, c->tmp, s);
-    uint64_t *kEV; uint32_t *EV;
-    const Count cEVM{cnt + CNT_EVM, 2 * n};
-    seq_ev_keys(c->M_from, c->M_to, dM, n, c->sb[1].k, c->sb[1].v, s);
-    c->sb[1].run(cEVM, kbits, c->tmp, s, &kEV, &EV);
-    seq_ev_delta(c->M_node, EV, kEV, dM, n, G.vwgt, c->delta, c->ebeg, c->eend, s);
-    exclusive_sum_i64(c->delta, c->d_excl, cEVM, c->tmp, s);
-    seq_ev_need(EV, kEV, dM, n, c->delta, c->d_excl, c->ebeg, c->C0, c->Lb, c->rbeg, c->rend, c->c_excl,
-                c->c_sorted, c->packed, s);
-    inclusive_max_u64(c->packed, c->qmax, cEVM, c->tmp, s);
-    seq_ev_emit(EV, kEV, dM, n, c->qmax, c->ebeg, c->emit, c->qbefore, s);
-    exclusive_sum_i32(c->emit, c->em_excl, Count{dM, n}, c->tmp, s);
-    seq_block_final(K, c->ebeg, c->eend, c->qmax, c->rbeg, c->rend, c->qfin, c->left, s);
-    exclusive_sum_i32(c->left, c->left_excl, fixed(K), c->tmp, s);
-    seq_place_m(c->M_node, c->M_from, c->M_to, dM, n, c->em_excl, c->pos_m, c->X_node, c->X_from, c->X_to, c->X_isr,
-                s);
-    seq_place_r(c->R_node, c->R_from, c->R_to, RB, dR, n, c->rbeg, EV, c->ebeg, c->eend, c->qmax, c->pos_m, c->qfin,
-                c->left_excl, c->em_excl, c->emit, dM, c->X_node, c->X_from, c->X_to, c->X_isr, s);
-    }
-
-    // ---- (c1) merge double moves
-    const Count cX{cnt + CNT_X, 2 * n};
-    seq_merge_flags(c->X_node, c->X_to, c->X_isr, cnt + CNT_X, 2 * n, c->m_pos, c->r_to, c->part0, c->flags2,
-                    c->final_to, s);
-    select_flags(c->flags2, c->idxD, cnt + CNT_I, cX, c->tmp, s);
     const int32_t *dI = cnt + CNT_I;
-    seq_build_I(c->idxD, dI, n, c->X_node, c->final_to, c->part0, c->I_node, c->I_from, c->I_to, c->pos, c->dest, s);
-    // a batch: each graph's moves are a subsequence of I in its own order;
-    // a stable sort by graph makes them contiguous (X_* are free by now)
+    // (a batch: I sorted by graph, into X_*, free once I is built)
+    SeqBuild sq{};
+    sq.team = c->team;
+    sq.M_node = c->M_node; sq.M_from = c->M_from; sq.M_to = c->M_to; sq.dM = dM;
+    sq.R_node = c->R_node; sq.R_from = c->R_from; sq.R_to = c->R_to; sq.dR = dR;
+    sq.part0 = c->part0; sq.m_pos = c->m_pos; sq.r_to = c->r_to; sq.C0 = c->C0;
+    sq.append = c->prm.append;
+    // (24 n bytes each: two neighbouring 16 n arrays)
+    sq.bufA = c->sb[0].k; sq.bufB = c->sb[1].k; sq.ex = c->c_sorted;
+    sq.qmax = reinterpret_cast<uint32_t *>(c->packed);
+    sq.rbeg = c->rbeg; sq.rend = c->rend; sq.ebeg = c->ebeg; sq.eend = c->eend; sq.qfin = c->qfin;
+    sq.left_excl = c->left_excl;
+    sq.emit = c->emit; sq.pos_m = c->pos_m;
+    sq.X_node = c->X_node; sq.X_from = c->X_from; sq.X_to = c->X_to; sq.fin = c->flags2;
+    sq.I_node = c->I_node; sq.I_from = c->I_from; sq.I_to = c->I_to;
+    sq.pk = c->pk; sq.diff = c->diff; sq.deg_sum = c->scal + 3;
+    sq.dX = cnt + CNT_X; sq.dI = cnt + CNT_I;
+    sq.O_node = c->X_node; sq.O_from = c->X_from; sq.O_to = c->X_to; sq.seg_beg = c->seg_beg; sq.seg_end = c->seg_end;
+    seq_build(G, sq, s);
     const int32_t *Iv = c->I_node, *If = c->I_from, *It = c->I_to;
-    if (batch) {
-        seq_sort_by_graph(G, c->I_node, c->I_from, c->I_to, dI, n, c->sb[0].k, c->sb[0].v, c->sb[0].ka, c->sb[0].va,
-                          c->tmp, c->X_node, c->X_from, c->X_to, c->pos, c->dest, c->seg_beg, c->seg_end, s);
-        Iv = c->X_node; If = c->X_from; It = c->X_to;
-    }
+    if (batch) { Iv = c->X_node; If = c->X_from; It = c->X_to; }
 
     // ---- (c2) exact gains, balanced prefixes, best prefix
-    seq_gains(G, Iv, If, It, dI, n, c->part0, c->pk, c->I_gain, c->hub_chunks, c->n_chunks, c->scal + 3, s);
-    inclusive_sum_i64(c->I_gain, c->Gsum, Count{dI, n}, c->tmp, s);
-    count_affine(dI, 2, nullptr, 0, cnt + CNT_EVI, s);
-    count_affine(dI, 1, nullptr, 1, cnt + CNT_I1, s);
-    uint64_t *kE; uint32_t *E;
-    const Count cEVI{cnt + CNT_EVI, 2 * n};
-    seq_iev_keys(If, It, dI, n, c->sb[2].k, c->sb[2].v, s);
-    c->sb[2].run(cEVI, kbits, c->tmp, s, &kE, &E);
-    UPR_CUDA(cudaMemsetAsync(c->ebeg, 0, sizeof(int32_t) * K, s));
-    seq_iev_delta(Iv, E, kE, dI, n, G.vwgt, c->delta, c->ebeg, s);
-    exclusive_sum_i64(c->delta, c->d_excl, cEVI, c->tmp, s);
-    clear_count(c->diff, dI, 1, n, s);
-    seq_iev_transitions(E, kE, dI, n, c->delta, c->d_excl, c->ebeg, c->C0, c->Lb, c->diff, s);
-    exclusive_sum_i32(c->diff, c->diff_excl, Count{cnt + CNT_I1, n + 1}, c->tmp, s);
-    if (!cap) UPR_CUDA(cudaMemcpyAsync(c->hcut, c->cut, sizeof(int64_t), cudaMemcpyDeviceToHost, s));   // cut before the round
-    if (!batch) {
-        count_over(G, c->C0, cnt + CNT_OVER0, s);
-        seq_best(c->Gsum, c->diff, c->diff_excl, dI, n, cnt + CNT_OVER0, c->best_parts, c->best, cnt + CNT_INFEAS, s);
-    } else {
-        count_over(G, c->C0, c->over0_g, s);
-        seq_best_seg(G, Iv, dI, n, c->seg_beg, c->Gsum, c->diff, c->diff_excl, c->over0_g, c->best_g, c->best_j, c->cut,
-                     c->infeas_g, c->tot, s);
-    }
+    seq_gains(G, Iv, If, It, dI, n, c->pk, c->I_gain, c->hub_chunks, c->n_chunks, s);
     if (G.sp.on() && !cap) {
         // a sparse row without room for a new block: nothing of the round is
         // applied yet; the caller runs it again on rows built afresh (which
@@ -1112,7 +1060,6 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         UPR_CUDA(cudaMemcpyAsync(c->hcnt + 41, c->sp_over, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         UPR_CUDA(cudaStreamSynchronize(s));
         if (c->hcnt[41] != 0) {
-            reset_nodes(c->I_node, dI, n, c->pos, INT32_MAX, s);
             reset_nodes(c->M_node, dM, n, c->m_pos, -1, s);
             reset_nodes(c->R_node, dR, n, c->r_to, -1, s);
             UPR_CUDA(cudaMemsetAsync(c->sp_over, 0, sizeof(int32_t), s));
@@ -1120,20 +1067,38 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
             return build ? kRedoDense : kRedoFresh;
         }
     }
-    if (!batch) seq_apply_prefix(G, c->I_node, c->I_from, c->I_to, n, c->best, c->part0, c->C0, c->cut, s);
-    else seq_apply_prefix_seg(G, Iv, If, It, dI, n, c->seg_beg, c->best_j, c->part0, c->C0, s);
+    if (tr) UPR_CUDA(cudaMemcpyAsync(c->hcut, c->cut, sizeof(int64_t), cudaMemcpyDeviceToHost, s));   // cut before the round
+    const bool guard = c->prm.lock_rebalanced && !rebalance_only;
+    SeqBest sb{};
+    sb.team = c->team;
+    sb.I_node = Iv; sb.I_from = If; sb.I_to = It; sb.dI = dI;
+    sb.gain = c->I_gain; sb.Gsum = c->Gsum;
+    sb.bufA = c->sb[0].k; sb.bufB = c->sb[1].k;
+    sb.diff = c->diff; sb.diff_excl = c->diff_excl;
+    sb.part0 = c->part0; sb.C0 = c->C0; sb.cut = c->cut;
+    sb.best = c->best; sb.undone = c->scal + 2;
+    sb.d_over0 = cnt + CNT_OVER0; sb.d_infeasible = cnt + CNT_INFEAS;
+    sb.reset = guard ? 0 : 1;
+    sb.M_node = c->M_node; sb.dM = dM; sb.R_node = c->R_node; sb.dR = dR; sb.m_pos = c->m_pos; sb.r_to = c->r_to;
+    seq_best(G, sb, s);
+    if (batch) {
+        count_over(G, c->C0, c->over0_g, s);
+        seq_best_seg(G, Iv, dI, n, c->seg_beg, c->Gsum, c->diff, c->diff_excl, c->over0_g, c->best_g, c->best_j, c->cut,
+                     c->infeas_g, c->tot, s);
+        seq_apply_prefix_seg(G, Iv, If, It, dI, n, c->seg_beg, c->best_j, c->part0, c->C0, s);
+    }
     // the table goes from W(P o I) to W(P o I^{j*}) for the next round
     {
         const Rollback rb{Iv, If, It, dI, c->best, batch ? G.gid : nullptr, c->seg_beg, c->best_j};
-        if (c->prm.lock_rebalanced && !rebalance_only) guard_locks(rb, n, n, c->m_pos, c->r_to, c->locked, s);
-        table_rollback(G, rb, n, c->pos, c->W, c->hub_chunks, c->n_chunks, c->scal + 2, s);
+        if (guard) {
+            guard_locks(rb, n, n, c->m_pos, c->r_to, c->locked, s);
+            reset_nodes(c->M_node, dM, n, c->m_pos, -1, s);
+            reset_nodes(c->R_node, dR, n, c->r_to, -1, s);
+        }
+        table_rollback(G, rb, n, c->pk, c->W, c->hub_chunks, c->n_chunks, c->scal + 2, s);
         gain_table(G, c->part0, c->W, c->hub_chunks, c->n_chunks, c->n_tiles ? c->tiles : nullptr, c->n_tiles,
                    c->tile_nodes, c->scal + 2, s);
     }
-    // reset node-indexed markers for the next round
-    reset_nodes(c->I_node, dI, n, c->pos, INT32_MAX, s);
-    reset_nodes(c->M_node, dM, n, c->m_pos, -1, s);
-    reset_nodes(c->R_node, dR, n, c->r_to, -1, s);
     if (cap) {                  // the step graph: the round's counts go to the device sums
         k_round_stats<<<1, 32, 0, s>>>(cnt, ctl, c->best, c->tot, batch ? 1 : 0, c->tmp.err, c->dstats);
         UPR_LAUNCH_CHECK();
@@ -1921,7 +1886,7 @@ void parallel_segments(int64_t n, int parts, F fn) {
 // a binding rewrites in full.
 std::vector<int64_t> bind_key(const upr_ctx *c) {
     static_assert(sizeof(upr_params) % sizeof(int64_t) == 0, "parameters as whole words");
-    std::vector<int64_t> key = {c->n, c->m, c->k, c->ng, c->G.kmask, c->G.adjw != nullptr, c->G.vwgt != nullptr,
+    std::vector<int64_t> key = {c->n, c->m, c->k, c->ng, c->team.size, c->G.kmask, c->G.adjw != nullptr, c->G.vwgt != nullptr,
                                 c->sp_slots, c->sp_buf_cap, c->sparse_on, c->n_chunks, c->n_tiles, c->tile_nodes,
                                 c->gbits, c->cbits, c->wmax, c->Lmax, c->total_w, c->eps_ppm,
                                 (int64_t)(uintptr_t)c->mem, (int64_t)c->mem_bytes, (int64_t)(uintptr_t)c->W};
@@ -2034,7 +1999,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     } up_guard{c};
     if (ng == 1 && m > 0 && c->mem) {
         upr_ctx dry;
-        dry.n = n; dry.m = m; dry.k = k; dry.ng = ng;
+        dry.n = n; dry.m = m; dry.k = k; dry.ng = ng; dry.beside = c->beside;
         Arena D;
         D.base = reinterpret_cast<char *>((uintptr_t)1 << 20);
         layout(&dry, D);
@@ -2227,7 +2192,6 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     UPR_CUDA(cudaMemsetAsync(c->ctl, 0, sizeof(RebalCtl), s));
     UPR_CUDA(cudaMemsetAsync(c->counts, 0, 64 * sizeof(int32_t), s));
     UPR_CUDA(cudaMemsetAsync(c->Cd, 0, sizeof(long long) * (size_t)c->G.K(), s));
-    fill_i32(c->pos, n, INT32_MAX, s);
     fill_i32(c->m_pos, n, -1, s);
     fill_i32(c->r_to, n, -1, s);
     UPR_CUDA(cudaStreamSynchronize(s));
@@ -2277,11 +2241,23 @@ upr_status ctx_rebind(upr_ctx *c, const upr_graph *g, int32_t k, double eps, con
 size_t ctx_arena_bytes(const upr_ctx *c) { return c ? c->mem_bytes + sizeof(int64_t) * (size_t)c->xs_cap : 0; }
 
 upr_status ctx_rebind_batch(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, const double *eps,
-                            const upr_params *params) {
+                            const upr_params *params, int beside) {
     upr_params prm;
     upr_params_default(&prm);
     if (params) prm = *params;
+    c->beside = std::max(1, beside);
     return guarded(c, [&] { return bind_graphs(c, gs, ng, k, eps, prm); });
+}
+
+upr_status ctx_create_batch(const upr_graph *graphs, int32_t n_graphs, int32_t k, const double *eps,
+                            const upr_params *params, int beside, upr_ctx **out) {
+    if (!out || !graphs || !eps || n_graphs < 1) return UPR_ERR_INVALID;
+    upr_ctx *c = new (std::nothrow) upr_ctx();
+    if (!c) return UPR_ERR_OOM;
+    const upr_status st = ctx_rebind_batch(c, graphs, n_graphs, k, eps, params, beside);
+    if (st != UPR_OK) { free_ctx(c); return st; }
+    *out = c;
+    return UPR_OK;
 }
 
 }  // namespace upr
@@ -2327,13 +2303,7 @@ upr_status upr_refine(upr_ctx *c, int32_t *part, int32_t rounds, uint64_t seed, 
 
 upr_status upr_batch_create(const upr_graph *graphs, int32_t n_graphs, int32_t k, const double *eps,
                             const upr_params *params, upr_ctx **out) {
-    if (!out || !graphs || !eps || n_graphs < 1) return UPR_ERR_INVALID;
-    upr_ctx *c = new (std::nothrow) upr_ctx();
-    if (!c) return UPR_ERR_OOM;
-    const upr_status st = upr::ctx_rebind_batch(c, graphs, n_graphs, k, eps, params);
-    if (st != UPR_OK) { free_ctx(c); return st; }
-    *out = c;
-    return UPR_OK;
+    return upr::ctx_create_batch(graphs, n_graphs, k, eps, params, 1, out);
 }
 
 upr_status upr_batch_create_mixed(const upr_graph *graphs, int32_t n_graphs, const int32_t *k, const double *eps,

@@ -135,6 +135,17 @@ struct Scratch {
     int32_t *err;
 };
 
+// What a team launch needs (team.cuh): the grid barrier's arrival counter, the
+// error word, per-CTA digit totals [size][256] and per-CTA scan totals, and
+// the number of CTAs (one per binding, since the counter counts by it).
+struct Team {
+    unsigned long long *bar = nullptr;
+    int32_t *err = nullptr;
+    int32_t *hist = nullptr;
+    long long *tot = nullptr;
+    int size = 1;
+};
+
 // Grid-stride loop over a device-held count (all threads of the grid).
 #define UPR_FOR(i, cnt) \
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (cnt); i += (int64_t)gridDim.x * blockDim.x)
@@ -150,10 +161,6 @@ size_t scan_temp_bytes(int64_t n);
 size_t radix_temp_bytes(int64_t n);
 void exclusive_sum_i32(const int32_t *in, int32_t *out, Count n, Scratch tmp, cudaStream_t s);
 void exclusive_sum_i64(const int64_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s);
-void inclusive_sum_i64(const int64_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s);
-void exclusive_sum_i32_to_i64(const int32_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s);
-void inclusive_max_u64(const uint64_t *in, uint64_t *out, Count n, Scratch tmp, cudaStream_t s);
-void iota_u32(uint32_t *v, int64_t n, cudaStream_t s);
 // Stable LSD sort on key bits [0, bits); returns true if the result is in the *_alt buffers
 // (a property of `bits` alone, known when the launches are enqueued).
 bool radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, Count n, int bits,
@@ -276,19 +283,32 @@ struct LaneCfg { int32_t G, CH; };
 int lane_candidates(int32_t k, LaneCfg *out);
 void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Penalty pen, int32_t *cand_tgt,
                   int64_t *cand_s0, int32_t *cand_gain, int32_t *flags, LaneCfg cfg, cudaStream_t s);
-void cand_keys(const int32_t *cand_idx, const int32_t *d_count, const int32_t *cand_tgt, const int64_t *cand_s0,
-               int gbits, uint64_t *keys, uint32_t *vals, int64_t max_count, cudaStream_t s);
-void cand_gather(const GraphDev &g, const int32_t *cand_idx, const uint32_t *order, const int32_t *d_count,
-                 const int32_t *cand_tgt, int64_t *c_sorted, int32_t *seg_first, int64_t max_count, cudaStream_t s);
-void inflow_filter(const GraphDev &g, const int32_t *cand_idx, const uint32_t *order, const int32_t *d_count,
-                   const int32_t *cand_tgt, const int32_t *cand_gain, const int64_t *c_excl, const int32_t *seg_first,
-                   Penalty pen, int32_t *keep_flag, int64_t *score, int64_t max_count, cudaStream_t s);
-void move_keys(const int32_t *m_idx, const int32_t *d_count, const int64_t *score, int gbits, uint64_t *keys,
-               uint32_t *vals, int64_t max_count, cudaStream_t s);
-void apply_moves(const GraphDev &g, const int32_t *cand_idx, const int32_t *m_idx, const uint32_t *order,
-                 const int32_t *d_count, const int32_t *cand_tgt, const int64_t *score, const int32_t *part0,
-                 int32_t *part, int64_t *C, int32_t *M_node, int32_t *M_from, int32_t *M_to, int64_t *M_score,
-                 int32_t *m_pos, int64_t *deg_sum, int64_t max_count, cudaStream_t s);
+// Step (b3): the candidates' inflow penalties, M in its order and applied
+// (team.cuh).  bufA / bufB: 16 n bytes each.
+struct SelOrder {
+    Team team;
+    const int32_t *cand_tgt, *cand_gain;      // [n] best target (-1: no candidate) and its gain
+    const int64_t *cand_s0;                   // [n] score without inflow
+    Penalty pen;
+    const int32_t *part0;
+    const int64_t *C0;
+    int32_t *part;                            // [n] becomes part0 with M applied
+    int64_t *C;                               // [K] becomes C0 with M applied
+    int32_t *score;                           // [n] kept score of a candidate, else 0
+    int64_t *c_excl, *seg_base;               // [n], [K] scratch
+    void *bufA, *bufB;
+    int32_t *M_node, *M_from, *M_to;
+    int64_t *M_score;
+    int32_t *m_pos;
+    int64_t *deg_sum;                         // degree sum of M
+    int32_t *d_cand, *d_moves;                // candidates, |M|
+    // set by select_order
+    int64_t n = 0;
+    int K = 0, kbits = 0;
+    const int32_t *vwgt = nullptr;
+    const int64_t *xadj = nullptr;
+};
+void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s);
 
 // ---- rebalance.cu: step (d)
 // Device-resident control block of the rebalancing loop.
@@ -353,8 +373,11 @@ upr_status mixed_rebind(MixedBatch *mb, const upr_graph *graphs, int32_t n_graph
 void mixed_destroy(MixedBatch *mb);
 // engine.cu: a context bound to other graphs (its arena reused when large enough)
 upr_status ctx_rebind(upr_ctx *c, const upr_graph *g, int32_t k, double eps, const upr_params *params);
+// (beside: how many contexts, this one included, refine at the same time)
 upr_status ctx_rebind_batch(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, const double *eps,
-                            const upr_params *params);
+                            const upr_params *params, int beside = 1);
+upr_status ctx_create_batch(const upr_graph *graphs, int32_t n_graphs, int32_t k, const double *eps,
+                            const upr_params *params, int beside, upr_ctx **out);
 int64_t mixed_nodes(const MixedBatch *mb);
 upr_status mixed_refine(MixedBatch *mb, int32_t *part, int32_t rounds, uint64_t seed, upr_status *status,
                         int64_t *cut_in, int64_t *cut_out, upr_stats *stats);
@@ -484,62 +507,70 @@ void rebalance_end(const GraphDev &g, const int64_t *C, int8_t *excl, const int8
                    RebalCtl *ctl, cudaStream_t s);
 
 // ---- sequence.cu: step (c); every count lives in device memory, `max` bounds it
-void count_affine(const int32_t *a, int32_t a_mul, const int32_t *b, int32_t add, int32_t *out, cudaStream_t s);
 void fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t s);
-void clear_count(int32_t *a, const int32_t *d_n, int32_t extra, int64_t max, cudaStream_t s);
 void reset_nodes(const int32_t *nodes, const int32_t *d_cnt, int64_t max, int32_t *arr, int32_t val, cudaStream_t s);
 // out[g] = number of blocks of graph g above L_max
 void count_over(const GraphDev &g, const int64_t *C, int32_t *out, cudaStream_t s);
-void seq_rb_keys(const int32_t *R_from, const int32_t *d_nR, int64_t max, uint64_t *keys, uint32_t *vals,
-                 cudaStream_t s);
-void seq_rb_bounds(const int32_t *R_node, const int32_t *R_from, const uint32_t *RB, const int32_t *d_nR, int64_t max,
-                   const int32_t *vwgt, int64_t *rc, int32_t *rbeg, int32_t *rend, cudaStream_t s);
-void seq_ev_keys(const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM, int64_t max, uint64_t *keys,
-                 uint32_t *vals, cudaStream_t s);
-void seq_ev_delta(const int32_t *M_node, const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max,
-                  const int32_t *vwgt, int64_t *delta, int32_t *ebeg, int32_t *eend, cudaStream_t s);
-void seq_ev_need(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max, const int64_t *delta,
-                 const int64_t *d_excl, const int32_t *ebeg, const int64_t *C0, const int64_t *Lb,
-                 const int32_t *rbeg, const int32_t *rend, const int64_t *rc_excl, const int64_t *rc, uint64_t *packed,
-                 cudaStream_t s);
-void seq_ev_emit(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max, const uint64_t *qmax,
-                 const int32_t *ebeg, int32_t *emit, int32_t *qbefore_m, cudaStream_t s);
-void seq_block_final(int32_t K, const int32_t *ebeg, const int32_t *eend, const uint64_t *qmax, const int32_t *rbeg,
-                     const int32_t *rend, int32_t *qfin, int32_t *left, cudaStream_t s);
-void seq_place_m(const int32_t *M_node, const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM, int64_t max,
-                 const int32_t *em_excl, int32_t *pos_m, int32_t *X_node, int32_t *X_from, int32_t *X_to,
-                 int8_t *X_isr, cudaStream_t s);
-// X = M followed by R (the appended sequence, a variant of Sec. 7.2); max
-// bounds |M| + |R|
-void seq_append(const int32_t *M_node, const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM,
-                const int32_t *R_node, const int32_t *R_from, const int32_t *R_to, const int32_t *d_nR, int64_t max,
-                int32_t *X_node, int32_t *X_from, int32_t *X_to, int8_t *X_isr, cudaStream_t s);
-void seq_place_r(const int32_t *R_node, const int32_t *R_from, const int32_t *R_to, const uint32_t *RB,
-                 const int32_t *d_nR, int64_t max, const int32_t *rbeg, const uint32_t *EV, const int32_t *ebeg,
-                 const int32_t *eend, const uint64_t *qmax, const int32_t *pos_m, const int32_t *qfin,
-                 const int32_t *left_excl, const int32_t *em_excl, const int32_t *emit, const int32_t *d_nM,
-                 int32_t *X_node, int32_t *X_from, int32_t *X_to, int8_t *X_isr, cudaStream_t s);
-void seq_merge_flags(const int32_t *X_node, const int32_t *X_to, const int8_t *X_isr, const int32_t *d_nX, int64_t max,
-                     const int32_t *m_pos, const int32_t *r_to, const int32_t *part0, int32_t *keep, int32_t *final_to,
-                     cudaStream_t s);
-void seq_build_I(const int32_t *Ix, const int32_t *d_nI, int64_t max, const int32_t *X_node, const int32_t *final_to,
-                 const int32_t *part0, int32_t *I_node, int32_t *I_from, int32_t *I_to, int32_t *pos, int32_t *dest,
-                 cudaStream_t s);
-// pk: n words of scratch (each node's position in I and blocks before/after)
+// X = the interleaving of M and R (append: M, then R), merged into I (d_nI
+// moves; a batch's also sorted by graph into O_*, graph g's moves in
+// [seg_beg[g], seg_end[g])), and every node's packed state for seq_gains.
+// bufA, bufB: 24 n bytes each; ex: 24 n bytes; qmax: 12 n bytes.
+struct SeqBuild {
+    Team team;
+    const int32_t *M_node, *M_from, *M_to, *dM;
+    const int32_t *R_node, *R_from, *R_to, *dR;
+    const int32_t *part0, *m_pos, *r_to;
+    const int64_t *C0;
+    int32_t append;
+    void *bufA, *bufB;
+    int64_t *ex;                                             // prefix sums over the sorted entries and events
+    uint32_t *qmax;                                          // emitted part of R_b after each event
+    int32_t *rbeg, *rend, *ebeg, *eend, *qfin, *left_excl;   // [K]
+    int32_t *emit, *pos_m;                                   // [n]
+    int32_t *X_node, *X_from, *X_to, *fin;                   // [2n]
+    int32_t *I_node, *I_from, *I_to;
+    int2 *pk;
+    int32_t *diff;                                           // cleared up to d_nI
+    int64_t *deg_sum;                                        // degrees of I's nodes, added
+    int32_t *dX, *dI;
+    int32_t *O_node, *O_from, *O_to, *seg_beg, *seg_end;     // batches
+    // set by seq_build
+    int64_t n = 0;
+    int32_t k = 0, kmask = 0, K = 0, ng = 0;
+    int kbits = 0, ngbits = 0;
+    const int32_t *vwgt = nullptr, *gid = nullptr;
+    const int64_t *xadj = nullptr, *Lb = nullptr;
+};
+void seq_build(const GraphDev &g, SeqBuild a, cudaStream_t s);
 void seq_gains(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-               const int32_t *d_nI, int64_t max, const int32_t *part0, int2 *pk, int64_t *gain,
-               const HubChunk *hub_chunks, int64_t n_chunks, int64_t *deg_sum, cudaStream_t s);
-void seq_iev_keys(const int32_t *I_from, const int32_t *I_to, const int32_t *d_nI, int64_t max, uint64_t *keys,
-                  uint32_t *vals, cudaStream_t s);
-void seq_iev_delta(const int32_t *I_node, const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nI, int64_t max,
-                   const int32_t *vwgt, int64_t *delta, int32_t *ebeg, cudaStream_t s);
-void seq_iev_transitions(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nI, int64_t max,
-                         const int64_t *delta, const int64_t *d_excl, const int32_t *ebeg, const int64_t *C0,
-                         const int64_t *Lb, int32_t *diff, cudaStream_t s);
-void seq_best(const int64_t *Gsum, const int32_t *diff, const int32_t *diff_excl, const int32_t *d_nI, int64_t max,
-              const int32_t *d_over0, long long *parts, long long *out, int32_t *infeasible, cudaStream_t s);
-void seq_apply_prefix(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-                      int64_t max, const long long *best, int32_t *part0, int64_t *C0, int64_t *cut, cudaStream_t s);
+               const int32_t *d_nI, int64_t max, const int2 *pk, int64_t *gain, const HubChunk *hub_chunks,
+               int64_t n_chunks, cudaStream_t s);
+// Prefix gains Gsum and the overloaded blocks after every prefix (diff,
+// diff_excl); one graph: the best balanced prefix (best = gain, length; -1:
+// none, *d_infeasible set) applied to part0, C0 and *cut, and *undone = the
+// degree sum of the moves after it.  reset: m_pos and r_to of M and R go back to -1.
+struct SeqBest {
+    Team team;
+    const int32_t *I_node, *I_from, *I_to, *dI;
+    const int64_t *gain;
+    int64_t *Gsum;
+    void *bufA, *bufB;
+    int32_t *diff, *diff_excl;
+    int32_t *part0;
+    int64_t *C0, *cut;
+    long long *best;
+    int64_t *undone;
+    int32_t *d_over0, *d_infeasible;
+    int reset;
+    const int32_t *M_node, *dM, *R_node, *dR;
+    int32_t *m_pos, *r_to;
+    // set by seq_best
+    int32_t K = 0;
+    int kbits = 0;
+    const int32_t *vwgt = nullptr, *gid = nullptr;
+    const int64_t *xadj = nullptr, *Lb = nullptr;
+};
+void seq_best(const GraphDev &g, SeqBest a, cudaStream_t s);
 // The moves of I undone after the best prefix: positions i >= j* (one graph,
 // best[1] = j*, -1 = none kept) or i - seg_beg[g] >= best_j[g] (a batch, gid set).
 struct Rollback {
@@ -556,18 +587,12 @@ void guard_locks(const struct Rollback &rb, int64_t max, int64_t n, const int32_
                  int8_t *locked, cudaStream_t s);
 void guard_filter(const int8_t *locked, int64_t n, int32_t *flags, int32_t *cand_tgt, int64_t *cand_s0,
                   int32_t *cand_gain, cudaStream_t s);
-// W(P o I) -> W(P o I^{j*}): delta updates of the undone moves (pos = positions
-// in I), or nothing when 4 * (their degree sum, left in *deg_sum) >= m, in which
-// case the caller rebuilds with gain_table(..., deg_sum).
-void table_rollback(const GraphDev &g, const Rollback &rb, int64_t max, const int32_t *pos, int32_t *W,
+// W(P o I) -> W(P o I^{j*}): delta updates of the undone moves (pk: positions
+// in I), or nothing when 4 * (their degree sum *deg_sum; a batch's is summed
+// here, onto the 0 that seq_best left) >= m, in which case the caller rebuilds
+// with gain_table(..., deg_sum).
+void table_rollback(const GraphDev &g, const Rollback &rb, int64_t max, const int2 *pk, int32_t *W,
                     const HubChunk *hub_chunks, int64_t n_chunks, int64_t *deg_sum, cudaStream_t s);
-// Batches: I (length *d_nI) stably sorted by graph into O_*; pos/dest of the
-// moved nodes set from the sorted order; seg_beg/seg_end[g] bound graph g's
-// moves (both 0 for a graph without moves).
-void seq_sort_by_graph(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-                       const int32_t *d_nI, int64_t max, uint64_t *keys, uint32_t *vals, uint64_t *keys_alt,
-                       uint32_t *vals_alt, Scratch tmp, int32_t *O_node, int32_t *O_from, int32_t *O_to, int32_t *pos,
-                       int32_t *dest, int32_t *seg_beg, int32_t *seg_end, cudaStream_t s);
 // Per graph: the best eligible prefix j* (ties: shortest; none: infeasible,
 // j* = 0), cut[g] -= G_g(j*); tot = (sum j*, sum G(j*), infeasible graphs).
 void seq_best_seg(const GraphDev &g, const int32_t *I_node, const int32_t *d_nI, int64_t max, const int32_t *seg_beg,

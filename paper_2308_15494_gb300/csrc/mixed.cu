@@ -192,9 +192,9 @@ upr_status mixed_bind(MixedBatch *mb, const upr_graph *graphs, int32_t n_graphs,
             upr_params p = prm;
             p.stream = mb->streams[g];
             grc[g] = mb->sub[g] ? ctx_rebind_batch(mb->sub[g], gs[g].data(), (int32_t)gs[g].size(), ks[g],
-                                                   es[g].data(), &p)
-                                : upr_batch_create(gs[g].data(), (int32_t)gs[g].size(), ks[g], es[g].data(), &p,
-                                                   &mb->sub[g]);
+                                                   es[g].data(), &p, (int)G)
+                                : ctx_create_batch(gs[g].data(), (int32_t)gs[g].size(), ks[g], es[g].data(), &p,
+                                                   (int)G, &mb->sub[g]);
         });
     for (auto &t : th) t.join();
     for (size_t g = 0; g < G; g++)

@@ -1,4 +1,4 @@
-// Device-wide primitives written for this library: scans (sum / max),
+// Device-wide primitives written for this library: scans (sums),
 // stable LSD radix sort of (64-bit key, 32-bit value) pairs and stable
 // compaction by flags (of the indices, or of values, in place if wanted).  Every ordered list the refinement produces comes out of these,
 // never out of the order of atomic operations, so results are deterministic.
@@ -39,7 +39,7 @@ constexpr int kPTile = kThreads * kPI;
 __device__ __forceinline__ int64_t ptiles_of(int64_t n) { return (n + kPTile - 1) / kPTile; }
 
 template <typename Op, typename T, typename TIn>
-__device__ __forceinline__ void scan_tile(const TIn *in, T *out, int64_t n, int inclusive, int vec,
+__device__ __forceinline__ void scan_tile(const TIn *in, T *out, int64_t n, int vec,
                                           const ScanState<T> &st, uint32_t epoch, int64_t tile, bool alone,
                                           T *s_warp, T *s_excl) {
     TIn x[kPI];
@@ -60,9 +60,8 @@ __device__ __forceinline__ void scan_tile(const TIn *in, T *out, int64_t n, int 
     T y[kPI];
 #pragma unroll
     for (int j = 0; j < kPI; j++) {
-        const T nxt = Op::template apply<T>(run, (T)x[j]);
-        y[j] = inclusive ? nxt : run;
-        run = nxt;
+        y[j] = run;
+        run = Op::template apply<T>(run, (T)x[j]);
     }
     store_items(out, tile * kPTile, n, (vec & 2) != 0, y);
     __syncthreads();
@@ -70,7 +69,7 @@ __device__ __forceinline__ void scan_tile(const TIn *in, T *out, int64_t n, int 
 
 template <typename Op, typename T, typename TIn>
 __global__ void __launch_bounds__(kThreads) k_scan(const TIn *in, T *out, const int32_t *__restrict__ d_n,
-                                                   int64_t n_max, int inclusive, int vec, ScanState<T> st) {
+                                                   int64_t n_max, int vec, ScanState<T> st) {
     __shared__ T s_warp[kWarps];
     __shared__ T s_excl;
     __shared__ uint32_t s_tile;
@@ -79,14 +78,14 @@ __global__ void __launch_bounds__(kThreads) k_scan(const TIn *in, T *out, const 
     const unsigned parts = participants(tiles);
     if (blockIdx.x >= parts) return;
     if (tiles == 1) {
-        scan_tile<Op>(in, out, n, inclusive, vec, st, 0u, 0, true, s_warp, &s_excl);
+        scan_tile<Op>(in, out, n, vec, st, 0u, 0, true, s_warp, &s_excl);
         return;
     }
     const uint32_t epoch = call_epoch(st);
     for (;;) {
         const int64_t tile = next_tile(st.ctr, &s_tile);
         if (tile >= tiles) break;
-        scan_tile<Op>(in, out, n, inclusive, vec, st, epoch, tile, false, s_warp, &s_excl);
+        scan_tile<Op>(in, out, n, vec, st, epoch, tile, false, s_warp, &s_excl);
     }
     finish_tiles(st, parts, epoch);
 }
@@ -95,12 +94,12 @@ __global__ void __launch_bounds__(kThreads) k_scan(const TIn *in, T *out, const 
 
 
 template <typename Op, typename T, typename TIn>
-void scan_impl(const TIn *in, T *out, Count n, bool inclusive, Scratch tmp, cudaStream_t s) {
+void scan_impl(const TIn *in, T *out, Count n, Scratch tmp, cudaStream_t s) {
     if (n.max <= 0) return;
     const int vin = aligned16(in) ? 1 : 0;
     const int vio = vin | (aligned16(out) ? 2 : 0);
     const int64_t tiles_max = ceil_div(n.max, kPTile);
-    k_scan<Op, T, TIn><<<tile_grid((const void *)k_scan<Op, T, TIn>, tiles_max), kThreads, 0, s>>>(in, out, n.d, n.max, inclusive ? 1 : 0, vio,
+    k_scan<Op, T, TIn><<<tile_grid((const void *)k_scan<Op, T, TIn>, tiles_max), kThreads, 0, s>>>(in, out, n.d, n.max, vio,
                                                                   scan_state<T>(tmp, tiles_max));
     UPR_LAUNCH_CHECK();
 }
@@ -329,11 +328,6 @@ __global__ void __launch_bounds__(kThreads) k_radix_small(const uint64_t *__rest
     for (int i = threadIdx.x; i < n; i += kThreads) { okeys[i] = s_k[i]; ovals[i] = s_v[i]; }
 }
 
-__global__ void k_iota_u32(uint32_t *v, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) v[i] = (uint32_t)i;
-}
-
 }  // namespace
 
 size_t scan_temp_bytes(int64_t n) {
@@ -347,25 +341,10 @@ size_t radix_temp_bytes(int64_t n) {
 }
 
 void exclusive_sum_i32(const int32_t *in, int32_t *out, Count n, Scratch tmp, cudaStream_t s) {
-    scan_impl<OpSum, int32_t, int32_t>(in, out, n, false, tmp, s);
+    scan_impl<OpSum, int32_t, int32_t>(in, out, n, tmp, s);
 }
 void exclusive_sum_i64(const int64_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s) {
-    scan_impl<OpSum, int64_t, int64_t>(in, out, n, false, tmp, s);
-}
-void inclusive_sum_i64(const int64_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s) {
-    scan_impl<OpSum, int64_t, int64_t>(in, out, n, true, tmp, s);
-}
-void exclusive_sum_i32_to_i64(const int32_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s) {
-    scan_impl<OpSum, int64_t, int32_t>(in, out, n, false, tmp, s);
-}
-void inclusive_max_u64(const uint64_t *in, uint64_t *out, Count n, Scratch tmp, cudaStream_t s) {
-    scan_impl<OpMax, uint64_t, uint64_t>(in, out, n, true, tmp, s);
-}
-
-void iota_u32(uint32_t *v, int64_t n, cudaStream_t s) {
-    if (n <= 0) return;
-    k_iota_u32<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(v, n);
-    UPR_LAUNCH_CHECK();
+    scan_impl<OpSum, int64_t, int64_t>(in, out, n, tmp, s);
 }
 
 bool radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, Count n, int bits,
@@ -390,7 +369,7 @@ bool radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32
     for (int p = 0; p < passes; p++) {
         k_radix_hist<<<grid_h, kThreads, 0, s>>>(ka, n.d, n.max, 8 * p, hist, d_hist_n);
         UPR_LAUNCH_CHECK();
-        scan_impl<OpSum, int32_t, int32_t>(hist, hist, Count{d_hist_n, (int64_t)kBins * tiles_max}, false, tmp, s);
+        scan_impl<OpSum, int32_t, int32_t>(hist, hist, Count{d_hist_n, (int64_t)kBins * tiles_max}, tmp, s);
         k_radix_scatter<<<grid_s, kThreads, 0, s>>>(ka, va, kb, vb, n.d, n.max, 8 * p, hist);
         UPR_LAUNCH_CHECK();
         uint64_t *tk = ka; ka = kb; kb = tk;

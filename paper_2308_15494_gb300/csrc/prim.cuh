@@ -23,10 +23,6 @@ struct OpSum {
     template <typename T> __device__ __forceinline__ static T apply(T a, T b) { return a + b; }
     template <typename T> __device__ __forceinline__ static T identity() { return T(0); }
 };
-struct OpMax {
-    template <typename T> __device__ __forceinline__ static T apply(T a, T b) { return a > b ? a : b; }
-    template <typename T> __device__ __forceinline__ static T identity() { return T(0); }   // unsigned only
-};
 
 // Block-wide exclusive scan of one value per thread; returns the exclusive
 // prefix, *total receives the block aggregate.
@@ -183,6 +179,26 @@ __device__ __forceinline__ void finish_tiles(const ScanState<T> &st, unsigned pa
         *st.epoch = epoch >= kEpochLimit ? 0u : epoch;
         __threadfence();
     }
+}
+
+// Grid barrier on a 64-bit arrival counter that only grows: the barrier that
+// a CTA reaches with arrival number `old` ends when the count reaches the
+// next multiple of the grid size.
+__device__ __forceinline__ void grid_sync(unsigned long long *count, int32_t *err) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned long long old = atomicAdd(count, 1ull);
+        const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
+        for (int it = 0;; it++) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+            if (v >= target) break;
+            if (it >= kMaxSpin || ((it & 1023) == 1023 && gave_up(err))) { atomicOr(err, 2); break; }
+            if (it >= 16) __nanosleep(32);
+        }
+    }
+    __syncthreads();
 }
 
 // Exclusive prefix (over the preceding tiles) of `total` for tile t, computed

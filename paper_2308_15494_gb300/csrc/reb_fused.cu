@@ -751,26 +751,6 @@ __global__ void k_fr_end(int64_t *__restrict__ C, long long *__restrict__ Cd, co
 // barrier (no early return), and every wait is bounded: a wait that gives up
 // sets the error word and the launch runs to its end.
 
-// Grid barrier on a 64-bit arrival counter that only grows: the barrier that
-// a CTA reaches with arrival number `old` ends when the count reaches the
-// next multiple of the grid size.
-__device__ __forceinline__ void grid_sync(unsigned long long *count, int32_t *err) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned long long old = atomicAdd(count, 1ull);
-        const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
-        for (int it = 0;; it++) {
-            unsigned long long v;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
-            if (v >= target) break;
-            if (it >= kMaxSpin || ((it & 1023) == 1023 && gave_up(err))) { atomicOr(err, 2); break; }
-            if (it >= 16) __nanosleep(32);
-        }
-    }
-    __syncthreads();
-}
-
 // Sum of tc[0..t) (all threads get it).
 __device__ __forceinline__ int32_t tiles_before(const int32_t *tc, int64_t t, int32_t *s_warp) {
     int32_t v = 0;

@@ -2,7 +2,7 @@
 // Sec. 4.3), each boundary node's best move by gain minus penalty
 // (Alg. 1), penalties with the inflow of better-ranked candidates,
 // the global move order M (Sec. 4.4), and the application of M.
-#include "kernels.h"
+#include "team.cuh"
 
 namespace upr {
 namespace {
@@ -492,102 +492,156 @@ __global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, const i
     }
 }
 
-__global__ void k_cand_keys(const int32_t *__restrict__ cand_idx, const int32_t *__restrict__ d_count,
-                            const int32_t *__restrict__ cand_tgt, const int64_t *__restrict__ cand_s0, int gbits,
-                            uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_count;
-    const uint64_t top = (1ull << gbits) - 1ull;
-    UPR_FOR(i, cnt) {
-        const int32_t v = cand_idx[i];
-        keys[i] = ((uint64_t)cand_tgt[v] << gbits) | (top - (uint64_t)cand_s0[v]);
-        vals[i] = (uint32_t)i;
+// ---- (b3) in one team launch: the candidates ordered by (target, score
+// desc, id), the penalties with the inflow of better-ranked candidates, M
+// ordered by (score desc, id) and applied.  One launch replaces about thirty
+// (keys, radix passes of three launches each, scans, compactions), each 3 to
+// 10 us for lists of 10^4 to 10^6 nodes, nearly all of it latency.
+// Keys hold (largest - score), so their width follows the largest score that
+// occurs, not the largest omega(I(v)): power-law graphs sort in two 8-bit
+// passes where the bound asks for three.  The node itself is the sort's value
+// and the kept scores go to a node-indexed array, so nothing is compacted.
+template <class Item>
+__global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
+    __shared__ team::Smem s;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    const int64_t n = a.n;
+    // the working partition and block weights start from the round's; the
+    // candidates' largest score
+    uint32_t mx = 0;
+    UPR_TEAM_FOR(v, n) {
+        a.part[v] = a.part0[v];
+        a.score[v] = 0;
+        if (a.cand_tgt[v] >= 0) mx = max(mx, (uint32_t)a.cand_s0[v]);
     }
-}
+    UPR_TEAM_FOR(b, a.K) a.C[b] = a.C0[b];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.deg_sum = 0;
+    team::publish<team::Max>(t, s, 0, team::warp_all<team::Max>(mx));
+    team::sync(t);
+    long long top;
+    team::collect<team::Max>(t, 0, &top);
+    const int sbits = top > 0 ? team::bits_of((uint32_t)top - 1) : 0;
+    using Key = typename Item::Key;
+    int64_t cand;
+    Item *bufA = reinterpret_cast<Item *>(a.bufA), *bufB = reinterpret_cast<Item *>(a.bufB);
+    const Item *S = team::sort(
+        t, s, n,
+        [&](int64_t v, Item &it) {
+            const int32_t tgt = a.cand_tgt[v];
+            if (tgt < 0) return false;
+            it.key = ((Key)tgt << sbits) | (Key)((uint32_t)top - (uint32_t)a.cand_s0[v]);
+            it.val = (uint32_t)v;
+            return true;
+        },
+        sbits + a.kbits, bufA, bufB, &cand);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_cand = (int32_t)cand;
 
-__global__ void k_cand_gather(const int32_t *__restrict__ cand_idx, const uint32_t *__restrict__ order,
-                              const int32_t *__restrict__ d_count, const int32_t *__restrict__ cand_tgt,
-                              const int32_t *__restrict__ vwgt, int64_t *__restrict__ c_sorted,
-                              int32_t *__restrict__ seg_first) {
-    const int64_t cnt = *d_count;
-    UPR_FOR(j, cnt) {
-        const int32_t v = cand_idx[order[j]];
-        c_sorted[j] = vwgt ? vwgt[v] : 1;
-        const int32_t t = cand_tgt[v];
-        if (j == 0 || cand_tgt[cand_idx[order[j - 1]]] != t) seg_first[t] = (int32_t)j;
+    // weight of the better-ranked candidates of the same target: the position
+    // in the target's run with unit weights, a difference of prefix sums else
+    const team::Seg g = team::warp_seg(cand);
+    long long base = 0;
+    if (a.vwgt) {
+        long long x = 0;
+        for (int64_t j = g.b + lane; j < g.e; j += 32) x += a.vwgt[S[j].val];
+        const long long mine = team::publish<team::Sum>(t, s, 1, team::warp_all<team::Sum>(x));
+        team::sync(t);
+        long long all;
+        base = team::collect<team::Sum>(t, 1, &all) + mine;
     }
-}
-
-__global__ void k_inflow(const int32_t *__restrict__ cand_idx, const uint32_t *__restrict__ order,
-                         const int32_t *__restrict__ d_count, const int32_t *__restrict__ cand_tgt,
-                         const int32_t *__restrict__ cand_gain, const int32_t *__restrict__ vwgt,
-                         const int64_t *__restrict__ c_excl, const int32_t *__restrict__ seg_first, Penalty pen,
-                         int32_t *__restrict__ keep, int64_t *__restrict__ score) {
-    const int64_t cnt = *d_count;
-    UPR_FOR(j, cnt) {
-        const uint32_t i = order[j];
-        const int32_t v = cand_idx[i];
-        const int32_t t = cand_tgt[v];
-        const int64_t c = vwgt ? vwgt[v] : 1;
-        const int64_t inflow = c_excl[j] - c_excl[seg_first[t]];
-        const int64_t p = penalty(pen, t, pen.C[t] + inflow + c - pen.Lb[t], c);
-        const int64_t s = (int64_t)cand_gain[v] - p;
-        const bool kp = p >= 0 && s > 0;
-        keep[i] = kp ? 1 : 0;
-        score[i] = kp ? s : 0;
-    }
-}
-
-__global__ void k_move_keys(const int32_t *__restrict__ m_idx, const int32_t *__restrict__ d_count,
-                            const int64_t *__restrict__ score, int gbits, uint64_t *__restrict__ keys,
-                            uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_count;
-    UPR_FOR(j, cnt) {
-        keys[j] = ((1ull << gbits) - 1ull) - (uint64_t)score[m_idx[j]];
-        vals[j] = (uint32_t)j;
-    }
-}
-
-__global__ void k_apply_moves(const int32_t *__restrict__ cand_idx, const int32_t *__restrict__ m_idx,
-                              const uint32_t *__restrict__ order, const int32_t *__restrict__ d_count,
-                              const int32_t *__restrict__ cand_tgt, const int64_t *__restrict__ score,
-                              const int32_t *__restrict__ vwgt, const int64_t *__restrict__ xadj,
-                              const int32_t *__restrict__ part0, int32_t *__restrict__ part,
-                              unsigned long long *__restrict__ C, int32_t K, int32_t *__restrict__ M_node,
-                              int32_t *__restrict__ M_from, int32_t *__restrict__ M_to,
-                              int64_t *__restrict__ M_score, int32_t *__restrict__ m_pos,
-                              unsigned long long *__restrict__ deg_sum) {
-    extern __shared__ unsigned long long s_delta[];
-    BlockDelta bd = make_block_delta(s_delta, K, C);
-    bd.init();
-    const int64_t cnt = *d_count;
-    long long degs = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < cnt; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = base + threadIdx.x;
-        int32_t a = -1, b = -1;
-        long long c = 0;
-        if (p < cnt) {
-            const int32_t i = m_idx[order[p]];
-            const int32_t v = cand_idx[i];
-            a = part0[v];
-            b = cand_tgt[v];
-            c = vwgt ? vwgt[v] : 1;
-            M_node[p] = v;
-            M_from[p] = a;
-            M_to[p] = b;
-            M_score[p] = score[i];
-            m_pos[v] = (int32_t)p;
-            part[v] = b;
-            degs += xadj[v + 1] - xadj[v];
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        long long pre = j;
+        if (a.vwgt) {
+            const long long c = j < g.e ? a.vwgt[S[j].val] : 0;
+            const long long inc = team::warp_incl<team::Sum>(c);
+            pre = base + inc - c;
+            base += __shfl_sync(0xffffffffu, inc, 31);
+            if (j < g.e) a.c_excl[j] = pre;
         }
-        bd.add(a, -c);
-        bd.add(b, c);
+        if (j < g.e) {
+            const Key tg = S[j].key >> sbits;
+            if (j == 0 || (S[j - 1].key >> sbits) != tg) a.seg_base[tg] = pre;
+        }
     }
-    bd.flush(C);
+    team::sync(t);
+    uint32_t kept_top = 0;
+    for (int64_t j = g.b + lane; j < g.e; j += 32) {
+        const Item it = S[j];
+        const int32_t tg = (int32_t)(it.key >> sbits);
+        const int32_t v = (int32_t)it.val;
+        const int64_t c = a.vwgt ? a.vwgt[v] : 1;
+        const int64_t inflow = (a.vwgt ? a.c_excl[j] : j) - a.seg_base[tg];
+        const int64_t p = penalty(a.pen, tg, a.pen.C[tg] + inflow + c - a.pen.Lb[tg], c);
+        const int64_t sc = (int64_t)a.cand_gain[v] - p;
+        if (p >= 0 && sc > 0) {
+            a.score[v] = (int32_t)sc;
+            kept_top = max(kept_top, (uint32_t)sc);
+        }
+    }
+    team::publish<team::Max>(t, s, 2, team::warp_all<team::Max>(kept_top));
+    team::sync(t);
+    long long ktop;
+    team::collect<team::Max>(t, 2, &ktop);
+
+    // M by (score desc, node id), applied
+    int64_t cnt;
+    using team::Item32;
+    const Item32 *M = team::sort(
+        t, s, n,
+        [&](int64_t v, Item32 &it) {
+            const int32_t sc = a.score[v];
+            it.key = (uint32_t)ktop - (uint32_t)sc;
+            it.val = (uint32_t)v;
+            return sc > 0;
+        },
+        ktop > 0 ? team::bits_of((uint32_t)ktop - 1) : 0, reinterpret_cast<Item32 *>(a.bufA),
+        reinterpret_cast<Item32 *>(a.bufB), &cnt);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_moves = (int32_t)cnt;
+    BlockDelta bd = make_block_delta(s.cnt64, a.K, reinterpret_cast<unsigned long long *>(a.C));
+    bd.init();
+    long long degs = 0;
+    const team::Seg gm = team::warp_seg(cnt);
+    for (int64_t p0 = gm.b; p0 < gm.e; p0 += 32) {
+        const int64_t p = p0 + lane;
+        int32_t from = -1, to = -1;
+        long long c = 0;
+        if (p < gm.e) {
+            const Item32 it = M[p];
+            const int32_t v = (int32_t)it.val;
+            from = a.part0[v];
+            to = a.cand_tgt[v];
+            c = a.vwgt ? a.vwgt[v] : 1;
+            a.M_node[p] = v;
+            a.M_from[p] = from;
+            a.M_to[p] = to;
+            a.M_score[p] = (int64_t)((uint32_t)ktop - it.key);
+            a.m_pos[v] = (int32_t)p;
+            a.part[v] = to;
+            degs += a.xadj[v + 1] - a.xadj[v];
+        }
+        bd.add(from, -c);
+        bd.add(to, c);
+    }
+    bd.flush(reinterpret_cast<unsigned long long *>(a.C));
     degs = warp_sum(degs);
-    if ((threadIdx.x & 31) == 0 && degs) atomicAdd(deg_sum, (unsigned long long)degs);
+    if (lane == 0 && degs) atomicAdd(reinterpret_cast<unsigned long long *>(a.deg_sum), (unsigned long long)degs);
 }
 
 }  // namespace
+
+void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s) {
+    if (g.n <= 0) return;
+    a.n = g.n;
+    a.K = g.K();
+    a.vwgt = g.vwgt;
+    a.xadj = g.xadj;
+    a.kbits = 1;
+    while ((1ll << a.kbits) < a.K) a.kbits++;
+    // (scores are at most omega(I(v)), so they have at most gbits bits)
+    if (gbits + a.kbits <= 32) launch_team(k_sel_order<team::Item32>, a, a.team.size, s);
+    else launch_team(k_sel_order<team::Item64>, a, a.team.size, s);
+}
 
 void buckets(const GraphDev &g, const int32_t *part, const int32_t *W, int32_t t_num, int32_t t_den, int64_t *BW,
              int64_t *PW, int8_t *first, int8_t *avail_out, int32_t *slot_out, cudaStream_t s, int64_t *cut2,
@@ -717,51 +771,6 @@ void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Pena
         default: UPR_SEL(32); break;
     }
 #undef UPR_SEL
-    UPR_LAUNCH_CHECK();
-}
-
-void cand_keys(const int32_t *cand_idx, const int32_t *d_count, const int32_t *cand_tgt, const int64_t *cand_s0,
-               int gbits, uint64_t *keys, uint32_t *vals, int64_t max_count, cudaStream_t s) {
-    if (max_count <= 0) return;
-    k_cand_keys<<<grid_for(max_count), 256, 0, s>>>(cand_idx, d_count, cand_tgt, cand_s0, gbits, keys,
-                                                                   vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void cand_gather(const GraphDev &g, const int32_t *cand_idx, const uint32_t *order, const int32_t *d_count,
-                 const int32_t *cand_tgt, int64_t *c_sorted, int32_t *seg_first, int64_t max_count, cudaStream_t s) {
-    if (max_count <= 0) return;
-    k_cand_gather<<<grid_for(max_count), 256, 0, s>>>(cand_idx, order, d_count, cand_tgt, g.vwgt,
-                                                                     c_sorted, seg_first);
-    UPR_LAUNCH_CHECK();
-}
-
-void inflow_filter(const GraphDev &g, const int32_t *cand_idx, const uint32_t *order, const int32_t *d_count,
-                   const int32_t *cand_tgt, const int32_t *cand_gain, const int64_t *c_excl, const int32_t *seg_first,
-                   Penalty pen, int32_t *keep_flag, int64_t *score, int64_t max_count, cudaStream_t s) {
-    if (max_count <= 0) return;
-    k_inflow<<<grid_for(max_count), 256, 0, s>>>(cand_idx, order, d_count, cand_tgt, cand_gain, g.vwgt,
-                                                                c_excl, seg_first, pen, keep_flag, score);
-    UPR_LAUNCH_CHECK();
-}
-
-void move_keys(const int32_t *m_idx, const int32_t *d_count, const int64_t *score, int gbits, uint64_t *keys,
-               uint32_t *vals, int64_t max_count, cudaStream_t s) {
-    if (max_count <= 0) return;
-    k_move_keys<<<grid_for(max_count), 256, 0, s>>>(m_idx, d_count, score, gbits, keys, vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void apply_moves(const GraphDev &g, const int32_t *cand_idx, const int32_t *m_idx, const uint32_t *order,
-                 const int32_t *d_count, const int32_t *cand_tgt, const int64_t *score, const int32_t *part0,
-                 int32_t *part, int64_t *C, int32_t *M_node, int32_t *M_from, int32_t *M_to, int64_t *M_score,
-                 int32_t *m_pos, int64_t *deg_sum, int64_t max_count, cudaStream_t s) {
-    UPR_CUDA(cudaMemsetAsync(deg_sum, 0, sizeof(int64_t), s));
-    if (max_count <= 0) return;
-    const int64_t blocks = std::min<int64_t>(ceil_div(max_count, 256), (int64_t)device_sm_count() * 4);
-    k_apply_moves<<<(unsigned)blocks, 256, block_delta_smem(g.K()), s>>>(
-        cand_idx, m_idx, order, d_count, cand_tgt, score, g.vwgt, g.xadj, part0, part, (unsigned long long *)C, g.K(),
-        M_node, M_from, M_to, M_score, m_pos, (unsigned long long *)deg_sum);
     UPR_LAUNCH_CHECK();
 }
 

@@ -17,258 +17,20 @@
 // All list lengths (|M|, |R|, |I|) are read from device memory.
 #include <climits>
 
-#include "kernels.h"
+#include "team.cuh"
 
 namespace upr {
 namespace {
 
 __device__ __forceinline__ int64_t cw(const int32_t *vwgt, int32_t v) { return vwgt ? (int64_t)vwgt[v] : 1; }
 
-// out = a_mul * (*a) + (b ? *b : 0) + add
-__global__ void k_count_affine(const int32_t *__restrict__ a, int32_t a_mul, const int32_t *__restrict__ b,
-                               int32_t add, int32_t *__restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *out = a_mul * (*a) + (b ? *b : 0) + add;
-}
-
-// keys/vals for R grouped by source block
-__global__ void k_rb_keys(const int32_t *__restrict__ R_from, const int32_t *__restrict__ d_nR,
-                          uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t nR = *d_nR;
-    UPR_FOR(i, nR) {
-        keys[i] = (uint64_t)R_from[i];
-        vals[i] = (uint32_t)i;
-    }
-}
-
-// per R_b position: node weight; block bounds [rbeg[b], rend[b])
-__global__ void k_rb_bounds(const int32_t *__restrict__ R_node, const int32_t *__restrict__ R_from,
-                            const uint32_t *__restrict__ RB, const int32_t *__restrict__ d_nR,
-                            const int32_t *__restrict__ vwgt, int64_t *__restrict__ rc, int32_t *__restrict__ rbeg,
-                            int32_t *__restrict__ rend) {
-    const int64_t nR = *d_nR;
-    UPR_FOR(q, nR) {
-        const uint32_t i = RB[q];
-        rc[q] = cw(vwgt, R_node[i]);
-        const int32_t b = R_from[i];
-        if (q == 0 || R_from[RB[q - 1]] != b) rbeg[b] = (int32_t)q;
-        if (q == nR - 1 || R_from[RB[q + 1]] != b) rend[b] = (int32_t)(q + 1);
-    }
-}
-
-// events of M: 2i = leave M_from[i], 2i+1 = enter M_to[i]
-__global__ void k_ev_keys(const int32_t *__restrict__ M_from, const int32_t *__restrict__ M_to,
-                          const int32_t *__restrict__ d_nM, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t nev = 2 * (int64_t)*d_nM;
-    UPR_FOR(e, nev) {
-        const int64_t i = e >> 1;
-        keys[e] = (uint64_t)((e & 1) ? M_to[i] : M_from[i]);
-        vals[e] = (uint32_t)e;
-    }
-}
-
-__global__ void k_ev_delta(const int32_t *__restrict__ M_node, const uint32_t *__restrict__ EV,
-                           const uint64_t *__restrict__ ekeys, const int32_t *__restrict__ d_nM,
-                           const int32_t *__restrict__ vwgt, int64_t *__restrict__ delta, int32_t *__restrict__ ebeg,
-                           int32_t *__restrict__ eend) {
-    const int64_t nev = 2 * (int64_t)*d_nM;
-    UPR_FOR(q, nev) {
-        const uint32_t e = EV[q];
-        const int64_t c = cw(vwgt, M_node[e >> 1]);
-        delta[q] = (e & 1) ? c : -c;
-        const int32_t b = (int32_t)ekeys[q];
-        if (q == 0 || (int32_t)ekeys[q - 1] != b) ebeg[b] = (int32_t)q;
-        if (q == nev - 1 || (int32_t)ekeys[q + 1] != b) eend[b] = (int32_t)(q + 1);
-    }
-}
-
-// need(q) for inflow events into blocks with R_b non-empty; packed with the block for the max-scan
-__global__ void k_ev_need(const uint32_t *__restrict__ EV, const uint64_t *__restrict__ ekeys,
-                          const int32_t *__restrict__ d_nM, const int64_t *__restrict__ delta,
-                          const int64_t *__restrict__ d_excl, const int32_t *__restrict__ ebeg,
-                          const int64_t *__restrict__ C0, const int64_t *__restrict__ Lb,
-                          const int32_t *__restrict__ rbeg, const int32_t *__restrict__ rend,
-                          const int64_t *__restrict__ rc_excl, const int64_t *__restrict__ rc,
-                          uint64_t *__restrict__ packed) {
-    const int64_t nev = 2 * (int64_t)*d_nM;
-    UPR_FOR(q, nev) {
-        const uint32_t e = EV[q];
-        const int32_t b = (int32_t)ekeys[q];
-        uint32_t need = 0;
-        const int32_t r0 = rbeg[b], r1 = rend[b];
-        if ((e & 1) && r1 > r0) {
-            const int64_t D = C0[b] + (d_excl[q] + delta[q]) - d_excl[ebeg[b]];
-            const int64_t Lmax = Lb[b];
-            if (D > Lmax) {
-                // smallest x in [1, |R_b|] with D - (weight of R_b[0..x)) <= L_max, else |R_b|
-                const int64_t base = rc_excl[r0];
-                int lo = 1, hi = r1 - r0;
-                while (lo < hi) {
-                    const int mid = lo + ((hi - lo) >> 1);
-                    const int64_t w = rc_excl[r0 + mid - 1] + rc[r0 + mid - 1] - base;
-                    if (D - w <= Lmax) hi = mid; else lo = mid + 1;
-                }
-                need = (uint32_t)lo;
-            }
-        }
-        packed[q] = ((uint64_t)(uint32_t)b << 32) | need;
-    }
-}
-
-// per M move: emissions after it (e_i) and the R_b count before them
-__global__ void k_ev_emit(const uint32_t *__restrict__ EV, const uint64_t *__restrict__ ekeys,
-                          const int32_t *__restrict__ d_nM, const uint64_t *__restrict__ qmax,
-                          const int32_t *__restrict__ ebeg, int32_t *__restrict__ emit,
-                          int32_t *__restrict__ qbefore_m) {
-    const int64_t nev = 2 * (int64_t)*d_nM;
-    UPR_FOR(q, nev) {
-        const uint32_t e = EV[q];
-        if (!(e & 1)) continue;
-        const int32_t b = (int32_t)ekeys[q];
-        const uint32_t after = (uint32_t)qmax[q];
-        const uint32_t before = q == ebeg[b] ? 0u : (uint32_t)qmax[q - 1];
-        emit[e >> 1] = (int32_t)(after - before);
-        qbefore_m[e >> 1] = (int32_t)before;
-    }
-}
-
-// per block: final emitted count and leftover count
-__global__ void k_block_final(int32_t K, const int32_t *__restrict__ ebeg, const int32_t *__restrict__ eend,
-                              const uint64_t *__restrict__ qmax, const int32_t *__restrict__ rbeg,
-                              const int32_t *__restrict__ rend, int32_t *__restrict__ qfin,
-                              int32_t *__restrict__ left) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= K) return;
-    const int32_t f = eend[b] > ebeg[b] ? (int32_t)(uint32_t)qmax[eend[b] - 1] : 0;
-    qfin[b] = f;
-    left[b] = (rend[b] - rbeg[b]) - f;
-}
-
-// positions of M moves in X
-__global__ void k_place_m(const int32_t *__restrict__ M_node, const int32_t *__restrict__ M_from,
-                          const int32_t *__restrict__ M_to, const int32_t *__restrict__ d_nM,
-                          const int32_t *__restrict__ em_excl, int32_t *__restrict__ pos_m,
-                          int32_t *__restrict__ X_node, int32_t *__restrict__ X_from, int32_t *__restrict__ X_to,
-                          int8_t *__restrict__ X_isr) {
-    const int64_t nM = *d_nM;
-    UPR_FOR(i, nM) {
-        const int32_t p = (int32_t)i + em_excl[i];
-        pos_m[i] = p;
-        X_node[p] = M_node[i];
-        X_from[p] = M_from[i];
-        X_to[p] = M_to[i];
-        X_isr[p] = 0;
-    }
-}
-
-// positions of R moves in X
-__global__ void k_place_r(const int32_t *__restrict__ R_node, const int32_t *__restrict__ R_from,
-                          const int32_t *__restrict__ R_to, const uint32_t *__restrict__ RB,
-                          const int32_t *__restrict__ d_nR, const int32_t *__restrict__ rbeg,
-                          const uint32_t *__restrict__ EV, const int32_t *__restrict__ ebeg,
-                          const int32_t *__restrict__ eend, const uint64_t *__restrict__ qmax,
-                          const int32_t *__restrict__ pos_m, const int32_t *__restrict__ qfin,
-                          const int32_t *__restrict__ left_excl, const int32_t *__restrict__ em_excl,
-                          const int32_t *__restrict__ emit, const int32_t *__restrict__ d_nM,
-                          int32_t *__restrict__ X_node, int32_t *__restrict__ X_from, int32_t *__restrict__ X_to,
-                          int8_t *__restrict__ X_isr) {
-    const int64_t nR = *d_nR, nM = *d_nM;
-    const int64_t tail0 = nM + (nM > 0 ? (int64_t)em_excl[nM - 1] + emit[nM - 1] : 0);
-    UPR_FOR(q, nR) {
-        const uint32_t i = RB[q];
-        const int32_t b = R_from[i];
-        const uint32_t r = (uint32_t)(q - rbeg[b]);
-        int64_t p;
-        if ((int32_t)r < qfin[b]) {
-            // first event of b with running max > r (an inflow event)
-            int lo = ebeg[b], hi = eend[b] - 1;
-            while (lo < hi) {
-                const int mid = lo + ((hi - lo) >> 1);
-                if ((uint32_t)qmax[mid] > r) hi = mid; else lo = mid + 1;
-            }
-            const uint32_t before = lo == ebeg[b] ? 0u : (uint32_t)qmax[lo - 1];
-            p = (int64_t)pos_m[EV[lo] >> 1] + 1 + (r - before);
-        } else {
-            p = tail0 + left_excl[b] + (r - (uint32_t)qfin[b]);
-        }
-        X_node[p] = R_node[i];
-        X_from[p] = R_from[i];
-        X_to[p] = R_to[i];
-        X_isr[p] = 1;
-    }
-}
-
-// merging: an R move of a node that also has an M move folds into the M move
-__global__ void k_merge_flags(const int32_t *__restrict__ X_node, const int32_t *__restrict__ X_to,
-                              const int8_t *__restrict__ X_isr, const int32_t *__restrict__ d_nX,
-                              const int32_t *__restrict__ m_pos, const int32_t *__restrict__ r_to,
-                              const int32_t *__restrict__ part0, int32_t *__restrict__ keep,
-                              int32_t *__restrict__ final_to) {
-    const int64_t nX = *d_nX;
-    UPR_FOR(x, nX) {
-        const int32_t v = X_node[x];
-        int32_t to = X_to[x];
-        bool k = true;
-        if (X_isr[x]) {
-            if (m_pos[v] >= 0) k = false;
-        } else if (r_to[v] >= 0) {
-            to = r_to[v];
-        }
-        if (k && to == part0[v]) k = false;
-        keep[x] = k ? 1 : 0;
-        final_to[x] = to;
-    }
-}
-
-__global__ void k_build_I(const int32_t *__restrict__ Ix, const int32_t *__restrict__ d_nI,
-                          const int32_t *__restrict__ X_node, const int32_t *__restrict__ final_to,
-                          const int32_t *__restrict__ part0, int32_t *__restrict__ I_node,
-                          int32_t *__restrict__ I_from, int32_t *__restrict__ I_to, int32_t *__restrict__ pos,
-                          int32_t *__restrict__ dest) {
-    const int64_t nI = *d_nI;
-    UPR_FOR(i, nI) {
-        const int32_t x = Ix[i];
-        const int32_t v = X_node[x];
-        I_node[i] = v;
-        I_from[i] = part0[v];
-        I_to[i] = final_to[x];
-        pos[v] = (int32_t)i;
-        dest[v] = final_to[x];
-    }
-}
-
 // Exact gain of the i-th move of I: neighbours moved earlier in I count in
 // their new block, all others in their round-start block.  Warp per move;
-// hub moves (degree > kHubDegree) are left to k_gains_hub.
+// hub moves (degree > kHubDegree) are left to k_gains_hub_chunks.
 // Block of each node at every step of I, packed for one 8-byte gather per
 // adjacency entry: x = the node's position in I (INT32_MAX when it does not
 // move), y = (local block before its move) | (local block after it) << 16.
-// Before step i a neighbour u is in its later block iff x < i.
-__global__ void k_pk_fill(const int32_t *__restrict__ part0, int64_t n, int32_t k, int32_t kmask,
-                          int2 *__restrict__ pk) {
-    UPR_FOR(u, n) {
-        const uint32_t l = (uint32_t)blk_local(part0[u], k, kmask);
-        pk[u] = make_int2(INT32_MAX, (int32_t)(l | (l << 16)));
-    }
-}
-
-// Also adds the degrees of the moved nodes to *deg_sum (the adjacency the
-// exact gains read: the step's algorithmic bytes).
-__global__ void k_pk_moves(const int32_t *__restrict__ I_node, const int32_t *__restrict__ I_from,
-                           const int32_t *__restrict__ I_to, const int32_t *__restrict__ d_nI, int32_t k,
-                           int32_t kmask, const int64_t *__restrict__ xadj, int2 *__restrict__ pk,
-                           unsigned long long *__restrict__ deg_sum) {
-    const int64_t nI = *d_nI;
-    unsigned long long deg = 0;
-    UPR_FOR(i, nI) {
-        const int32_t v = I_node[i];
-        const uint32_t a = (uint32_t)blk_local(I_from[i], k, kmask), b = (uint32_t)blk_local(I_to[i], k, kmask);
-        pk[v] = make_int2((int32_t)i, (int32_t)(a | (b << 16)));
-        deg += (unsigned long long)(xadj[v + 1] - xadj[v]);
-    }
-    deg = warp_sum(deg);
-    if ((threadIdx.x & 31) == 0 && deg) atomicAdd(deg_sum, deg);
-}
-
+// Before step i a neighbour u is in its later block iff x < i (k_seq_build fills it).
 __device__ __forceinline__ uint32_t block_before(int2 p, int64_t i) {
     const uint32_t code = (uint32_t)p.y;
     return p.x < i ? (code >> 16) : (code & 0xffffu);
@@ -333,49 +95,6 @@ __global__ void __launch_bounds__(512) k_gains_hub_chunks(const HubChunk *__rest
     }
 }
 
-// block events of I for the weight trajectory: 2i = leave I_from[i], 2i+1 = enter I_to[i]
-__global__ void k_iev_keys(const int32_t *__restrict__ I_from, const int32_t *__restrict__ I_to,
-                           const int32_t *__restrict__ d_nI, uint64_t *__restrict__ keys,
-                           uint32_t *__restrict__ vals) {
-    const int64_t nev = 2 * (int64_t)*d_nI;
-    UPR_FOR(e, nev) {
-        const int64_t i = e >> 1;
-        keys[e] = (uint64_t)((e & 1) ? I_to[i] : I_from[i]);
-        vals[e] = (uint32_t)e;
-    }
-}
-
-__global__ void k_iev_delta(const int32_t *__restrict__ I_node, const uint32_t *__restrict__ EV,
-                            const uint64_t *__restrict__ ekeys, const int32_t *__restrict__ d_nI,
-                            const int32_t *__restrict__ vwgt, int64_t *__restrict__ delta,
-                            int32_t *__restrict__ ebeg) {
-    const int64_t nev = 2 * (int64_t)*d_nI;
-    UPR_FOR(q, nev) {
-        const uint32_t e = EV[q];
-        const int64_t c = cw(vwgt, I_node[e >> 1]);
-        delta[q] = (e & 1) ? c : -c;
-        const int32_t b = (int32_t)ekeys[q];
-        if (q == 0 || (int32_t)ekeys[q - 1] != b) ebeg[b] = (int32_t)q;
-    }
-}
-
-// Changes of the number of overloaded blocks, at prefix length j = i + 1.
-__global__ void k_iev_transitions(const uint32_t *__restrict__ EV, const uint64_t *__restrict__ ekeys,
-                                  const int32_t *__restrict__ d_nI, const int64_t *__restrict__ delta,
-                                  const int64_t *__restrict__ d_excl, const int32_t *__restrict__ ebeg,
-                                  const int64_t *__restrict__ C0, const int64_t *__restrict__ Lb,
-                                  int32_t *__restrict__ diff) {
-    const int64_t nev = 2 * (int64_t)*d_nI;
-    UPR_FOR(q, nev) {
-        const int32_t b = (int32_t)ekeys[q];
-        const int64_t Lmax = Lb[b];
-        const int64_t before = C0[b] + d_excl[q] - d_excl[ebeg[b]];
-        const int64_t after = before + delta[q];
-        const int t = (after > Lmax ? 1 : 0) - (before > Lmax ? 1 : 0);
-        if (t) atomicAdd(&diff[(EV[q] >> 1) + 1], t);
-    }
-}
-
 // number of blocks above L_max, per graph (out[0..ng) zeroed by the caller)
 __global__ void k_count_over(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb, int32_t K, int32_t k,
                              int32_t *__restrict__ out) {
@@ -393,115 +112,462 @@ __device__ __forceinline__ Best better(Best x, Best y) {
     return x;
 }
 
-__global__ void k_best_partial(const int64_t *__restrict__ Gsum, const int32_t *__restrict__ diff,
-                               const int32_t *__restrict__ diff_excl, const int32_t *__restrict__ d_nI,
-                               const int32_t *__restrict__ d_over0, long long *__restrict__ part_g,
-                               long long *__restrict__ part_j) {
-    __shared__ long long s_g[8], s_j[8];
-    const int64_t nI = *d_nI;
-    const int32_t over0 = *d_over0;
-    Best b{0, -1};
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= nI; j += (int64_t)gridDim.x * blockDim.x) {
-        const bool elig = over0 + diff_excl[j] + diff[j] == 0;
-        if (elig) b = better(b, Best{j == 0 ? 0 : Gsum[j - 1], j});
+// ---- (c1) in one team launch (team.cuh): X = the interleaving of M and the
+// R_b (or M then R), the merged sequence I, and the packed state of every node
+// for the exact gains; a batch's I also sorted by graph.  One launch replaces
+// about thirty.  R's entries and M's events are sorted by block together: R
+// comes first in the input, so in every block's run its R_b precedes its
+// events, and one sort, one scan and one walk serve both.
+constexpr uint32_t kIsR = 1u << 31;       // in a sort key: an entry of R (blocks have at most 30 bits)
+
+__device__ __forceinline__ uint32_t blk_of(uint32_t key) { return key & ~kIsR; }
+
+// Move (v, to) of M or R at position x of X: its fate after merging (an R move
+// of a node with an M move folds into the M move; a move back to the
+// round-start block is dropped).
+__device__ __forceinline__ void put_x(const SeqBuild &a, int64_t x, int32_t v, int32_t from, int32_t to, bool isr) {
+    a.X_node[x] = v;
+    a.X_from[x] = from;
+    a.X_to[x] = to;
+    int32_t fin = to;
+    if (isr) {
+        if (a.m_pos[v] >= 0) fin = -1;
+    } else {
+        const int32_t r = a.r_to[v];
+        if (r >= 0) fin = r;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        Best y{__shfl_xor_sync(0xffffffffu, b.g, o), __shfl_xor_sync(0xffffffffu, b.j, o)};
-        b = better(b, y);
-    }
-    if ((threadIdx.x & 31) == 0) { s_g[threadIdx.x >> 5] = b.g; s_j[threadIdx.x >> 5] = b.j; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        Best t{0, -1};
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t = better(t, Best{s_g[w], s_j[w]});
-        part_g[blockIdx.x] = t.g;
-        part_j[blockIdx.x] = t.j;
-    }
+    a.fin[x] = fin == a.part0[v] ? -1 : fin;
 }
 
-__global__ void __launch_bounds__(1024) k_best_final(const long long *__restrict__ part_g,
-                                                    const long long *__restrict__ part_j, int parts,
-                                                    long long *__restrict__ out, int32_t *__restrict__ infeasible) {
-    __shared__ long long s_g[32], s_j[32];
-    Best b{0, -1};
-    for (int p = threadIdx.x; p < parts; p += blockDim.x) b = better(b, Best{part_g[p], part_j[p]});
-    for (int o = 16; o > 0; o >>= 1) {
-        Best y{__shfl_xor_sync(0xffffffffu, b.g, o), __shfl_xor_sync(0xffffffffu, b.j, o)};
-        b = better(b, y);
+__global__ void __launch_bounds__(team::kTT, 1) k_seq_build(const SeqBuild a) {
+    __shared__ team::Smem s;
+    using team::Item32;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const int64_t n = a.n, nM = *a.dM, nR = *a.dR, K = a.K;
+    const int64_t nX = nM + nR;
+    Item32 *A = reinterpret_cast<Item32 *>(a.bufA), *B = reinterpret_cast<Item32 *>(a.bufB);
+    UPR_TEAM_FOR(u, n) {
+        const uint32_t l = (uint32_t)blk_local(a.part0[u], a.k, a.kmask);
+        a.pk[u] = make_int2(INT32_MAX, (int32_t)(l | (l << 16)));
     }
-    if ((threadIdx.x & 31) == 0) { s_g[threadIdx.x >> 5] = b.g; s_j[threadIdx.x >> 5] = b.j; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        Best t{0, -1};
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t = better(t, Best{s_g[w], s_j[w]});
-        out[0] = t.g;
-        out[1] = t.j;
-        if (t.j < 0) *infeasible = 1;
-    }
-}
-
-__global__ void k_apply_prefix(const int32_t *__restrict__ I_node, const int32_t *__restrict__ I_from,
-                               const int32_t *__restrict__ I_to, const long long *__restrict__ best,
-                               const int32_t *__restrict__ vwgt, int32_t *__restrict__ part0,
-                               unsigned long long *__restrict__ C0, int32_t K, long long *__restrict__ cut) {
-    extern __shared__ unsigned long long s_delta[];
-    BlockDelta bd = make_block_delta(s_delta, K, C0);
-    bd.init();
-    const long long len = best[1];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && len >= 0) atomicAdd((unsigned long long *)cut, (unsigned long long)(-best[0]));
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < len; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = base + threadIdx.x;
-        int32_t a = -1, b = -1;
-        long long c = 0;
-        if (j < len) {
-            const int32_t v = I_node[j];
-            a = I_from[j];
-            b = I_to[j];
-            c = vwgt ? vwgt[v] : 1;
-            part0[v] = b;
+    if (a.append || nR == 0) {
+        UPR_TEAM_FOR(i, nX) {
+            const bool r = i >= nM;
+            const int64_t j = r ? i - nM : i;
+            put_x(a, i, r ? a.R_node[j] : a.M_node[j], r ? a.R_from[j] : a.M_from[j], r ? a.R_to[j] : a.M_to[j], r);
         }
-        bd.add(a, -c);
-        bd.add(b, c);
+    } else {
+        UPR_TEAM_FOR(b, K) a.rbeg[b] = a.rend[b] = a.ebeg[b] = a.eend[b] = 0;
+        // entries of R and events of M (2i = leave M_from[i], 2i + 1 = enter M_to[i]) by block
+        int64_t L;
+        const Item32 *S = team::sort(
+            t, s, nR + 2 * nM,
+            [&](int64_t i, Item32 &it) {
+                if (i < nR) {
+                    it.key = (uint32_t)a.R_from[i] | kIsR;
+                    it.val = (uint32_t)i;
+                } else {
+                    const int64_t e = i - nR;
+                    it.key = (uint32_t)((e & 1) ? a.M_to[e >> 1] : a.M_from[e >> 1]);
+                    it.val = (uint32_t)e;
+                }
+                return true;
+            },
+            a.kbits, A, B, &L);
+        const team::Seg g = team::warp_seg(L);
+        // runs of every block, and the two prefix sums: weights of R's
+        // entries, weight changes of M's events (each over its own kind)
+        long long sr = 0, sd = 0;
+        for (int64_t j = g.b + lane; j < g.e; j += 32) {
+            const Item32 it = S[j];
+            const uint32_t b = blk_of(it.key);
+            const uint32_t kp = j > 0 ? S[j - 1].key : ~0u, kn = j + 1 < L ? S[j + 1].key : ~0u;
+            if (it.key & kIsR) {
+                if (kp != it.key) a.rbeg[b] = (int32_t)j;
+                if (kn != it.key) a.rend[b] = (int32_t)(j + 1);
+                const long long c = cw(a.vwgt, a.R_node[it.val]);
+                a.ex[j] = c;
+                sr += c;
+            } else {
+                if (kp != it.key) a.ebeg[b] = (int32_t)j;
+                if (kn != it.key) a.eend[b] = (int32_t)(j + 1);
+                const long long c = cw(a.vwgt, a.M_node[it.val >> 1]);
+                const long long d = (it.val & 1) ? c : -c;
+                a.ex[j] = d;
+                sd += d;
+            }
+        }
+        long long all;
+        const long long mr = team::publish<team::Sum>(t, s, 0, team::warp_all<team::Sum>(sr));
+        const long long md = team::publish<team::Sum>(t, s, 1, team::warp_all<team::Sum>(sd));
+        team::sync(t);
+        sr = team::collect<team::Sum>(t, 0, &all) + mr;
+        sd = team::collect<team::Sum>(t, 1, &all) + md;
+        for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+            const int64_t j = j0 + lane;
+            const bool ok = j < g.e;
+            const bool isr = ok && (S[j].key & kIsR);
+            const long long x = ok ? a.ex[j] : 0;
+            const long long ir = team::warp_incl<team::Sum>(isr ? x : 0), id = team::warp_incl<team::Sum>(isr ? 0 : x);
+            if (ok) a.ex[j] = isr ? sr + ir - x : sd + id - x;
+            sr += __shfl_sync(full, ir, 31);
+            sd += __shfl_sync(full, id, 31);
+        }
+        team::sync(t);
+        // need of every event that enters a block with R_b non-empty; packed
+        // with the block, so that the running maximum restarts at each block
+        long long mx = 0;
+        for (int64_t j = g.b + lane; j < g.e; j += 32) {
+            const Item32 it = S[j];
+            const uint32_t b = blk_of(it.key);
+            uint32_t need = 0;
+            if (!(it.key & kIsR) && (it.val & 1)) {
+                const int32_t r0 = a.rbeg[b], r1 = a.rend[b];
+                if (r1 > r0) {
+                    const int64_t Lmax = a.Lb[b];
+                    const int64_t D = a.C0[b] + a.ex[j] + cw(a.vwgt, a.M_node[it.val >> 1]) - a.ex[a.ebeg[b]];
+                    if (D > Lmax) {
+                        // smallest x in [1, |R_b|] with D - (weight of R_b[0..x)) <= L_max, else |R_b|
+                        const int64_t base = a.ex[r0];
+                        int lo = 1, hi = r1 - r0;
+                        while (lo < hi) {
+                            const int mid = lo + ((hi - lo) >> 1);
+                            if (D - (a.ex[r0 + mid] - base) <= Lmax) hi = mid; else lo = mid + 1;
+                        }
+                        need = (uint32_t)lo;
+                    }
+                }
+            }
+            a.qmax[j] = need;
+            mx = max(mx, (long long)(((uint64_t)b << 32) | need));
+        }
+        const long long mq = team::publish<team::Max>(t, s, 2, team::warp_all<team::Max>(mx));
+        team::sync(t);
+        mx = max(team::collect<team::Max>(t, 2, &all), mq);
+        for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+            const int64_t j = j0 + lane;
+            const bool ok = j < g.e;
+            Item32 it{0, 0};
+            if (ok) it = S[j];
+            const uint32_t b = blk_of(it.key);
+            const long long p = ok ? (long long)(((uint64_t)b << 32) | a.qmax[j]) : 0;
+            const long long inc = max(mx, team::warp_incl<team::Max>(p));
+            long long prev = __shfl_up_sync(full, inc, 1);
+            if (lane == 0) prev = mx;
+            mx = __shfl_sync(full, inc, 31);
+            if (!ok) continue;
+            const uint32_t after = (uint32_t)inc;
+            a.qmax[j] = after;
+            if (!(it.key & kIsR) && (it.val & 1)) {
+                const uint32_t before = (uint32_t)(prev >> 32) == b ? (uint32_t)prev : 0u;
+                a.emit[it.val >> 1] = (int32_t)(after - before);
+            }
+        }
+        team::sync(t);
+        // emissions before every M move; per block, what is left of R_b after M
+        const team::Seg gm = team::warp_seg(nM), gk = team::warp_seg(K);
+        long long se = 0, sl = 0;
+        for (int64_t i = gm.b + lane; i < gm.e; i += 32) se += a.emit[i];
+        for (int64_t b = gk.b + lane; b < gk.e; b += 32) {
+            const int32_t f = a.eend[b] > a.ebeg[b] ? (int32_t)a.qmax[a.eend[b] - 1] : 0;
+            a.qfin[b] = f;
+            sl += (a.rend[b] - a.rbeg[b]) - f;
+        }
+        const long long me = team::publish<team::Sum>(t, s, 3, team::warp_all<team::Sum>(se));
+        const long long ml = team::publish<team::Sum>(t, s, 4, team::warp_all<team::Sum>(sl));
+        team::sync(t);
+        long long emitted;
+        se = team::collect<team::Sum>(t, 3, &emitted) + me;
+        sl = team::collect<team::Sum>(t, 4, &all) + ml;
+        for (int64_t i0 = gm.b; i0 < gm.e; i0 += 32) {
+            const int64_t i = i0 + lane;
+            const long long x = i < gm.e ? a.emit[i] : 0;
+            const long long inc = team::warp_incl<team::Sum>(x);
+            if (i < gm.e) {
+                const int64_t p = i + se + inc - x;
+                a.pos_m[i] = (int32_t)p;
+                put_x(a, p, a.M_node[i], a.M_from[i], a.M_to[i], false);
+            }
+            se += __shfl_sync(full, inc, 31);
+        }
+        for (int64_t b0 = gk.b; b0 < gk.e; b0 += 32) {
+            const int64_t b = b0 + lane;
+            const long long x = b < gk.e ? (a.rend[b] - a.rbeg[b]) - a.qfin[b] : 0;
+            const long long inc = team::warp_incl<team::Sum>(x);
+            if (b < gk.e) a.left_excl[b] = (int32_t)(sl + inc - x);
+            sl += __shfl_sync(full, inc, 31);
+        }
+        team::sync(t);
+        // R's entries: after the event that emits them, or behind M in block order
+        for (int64_t j = g.b + lane; j < g.e; j += 32) {
+            const Item32 it = S[j];
+            if (!(it.key & kIsR)) continue;
+            const uint32_t b = blk_of(it.key), i = it.val;
+            const uint32_t r = (uint32_t)(j - a.rbeg[b]);
+            int64_t p;
+            if ((int32_t)r < a.qfin[b]) {
+                // first event of b with running max > r (an inflow event)
+                const int first = a.ebeg[b];
+                int lo = first, hi = a.eend[b] - 1;
+                while (lo < hi) {
+                    const int mid = lo + ((hi - lo) >> 1);
+                    if (a.qmax[mid] > r) hi = mid; else lo = mid + 1;
+                }
+                const uint32_t before = lo == first ? 0u : a.qmax[lo - 1];
+                p = (int64_t)a.pos_m[S[lo].val >> 1] + 1 + (r - before);
+            } else {
+                p = nM + emitted + a.left_excl[b] + (r - (uint32_t)a.qfin[b]);
+            }
+            put_x(a, p, a.R_node[i], a.R_from[i], a.R_to[i], true);
+        }
     }
-    bd.flush(C0);
+    team::sync(t);
+    // the moves left after merging, in order: I
+    const team::Seg gx = team::warp_seg(nX);
+    long long keep = 0;
+    for (int64_t x = gx.b + lane; x < gx.e; x += 32) keep += a.fin[x] >= 0;
+    const long long mk = team::publish<team::Sum>(t, s, 5, team::warp_all<team::Sum>(keep));
+    team::sync(t);
+    long long nI;
+    keep = team::collect<team::Sum>(t, 5, &nI) + mk;
+    long long deg = 0;
+    for (int64_t x0 = gx.b; x0 < gx.e; x0 += 32) {
+        const int64_t x = x0 + lane;
+        const int32_t to = x < gx.e ? a.fin[x] : -1;
+        const unsigned kept = __ballot_sync(full, to >= 0);
+        if (to >= 0) {
+            const int64_t i = keep + __popc(kept & ((1u << lane) - 1u));
+            const int32_t v = a.X_node[x], from = a.part0[v];
+            a.I_node[i] = v;
+            a.I_from[i] = from;
+            a.I_to[i] = to;
+            if (!a.gid) {
+                const uint32_t lf = (uint32_t)blk_local(from, a.k, a.kmask), lo = (uint32_t)blk_local(to, a.k, a.kmask);
+                a.pk[v] = make_int2((int32_t)i, (int32_t)(lf | (lo << 16)));
+            }
+            deg += a.xadj[v + 1] - a.xadj[v];
+        }
+        keep += __popc(kept);
+    }
+    deg = warp_sum(deg);
+    if (lane == 0 && deg) atomicAdd(reinterpret_cast<unsigned long long *>(a.deg_sum), (unsigned long long)deg);
+    UPR_TEAM_FOR(j, nI + 1) a.diff[j] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *a.dX = (int32_t)nX;
+        *a.dI = (int32_t)nI;
+    }
+    if (!a.gid) return;
+    // a batch: each graph's moves contiguous, in their own order
+    UPR_TEAM_FOR(g, a.ng) a.seg_beg[g] = a.seg_end[g] = 0;
+    team::sync(t);
+    int64_t cnt;
+    const Item32 *S = team::sort(
+        t, s, nI,
+        [&](int64_t i, Item32 &it) {
+            it.key = (uint32_t)a.gid[a.I_node[i]];
+            it.val = (uint32_t)i;
+            return true;
+        },
+        a.ngbits, A, B, &cnt);
+    UPR_TEAM_FOR(q, nI) {
+        const Item32 it = S[q];
+        const int32_t i = (int32_t)it.val, v = a.I_node[i], from = a.I_from[i], to = a.I_to[i];
+        a.O_node[q] = v;
+        a.O_from[q] = from;
+        a.O_to[q] = to;
+        const uint32_t lf = (uint32_t)blk_local(from, a.k, a.kmask), lo = (uint32_t)blk_local(to, a.k, a.kmask);
+        a.pk[v] = make_int2((int32_t)q, (int32_t)(lf | (lo << 16)));
+        if (q == 0 || S[q - 1].key != it.key) a.seg_beg[it.key] = (int32_t)q;
+        if (q == nI - 1 || S[q + 1].key != it.key) a.seg_end[it.key] = (int32_t)(q + 1);
+    }
+}
+
+// ---- (c2) after the exact gains, in one team launch: prefix gains, the
+// number of overloaded blocks after every move (the moves' block events sorted
+// by block, a segmented sum of their weights), and for one graph the best
+// balanced prefix, applied, with the degree sum of the undone moves; the
+// markers of M and R go back to "none" (unless the oscillation guard still
+// needs them).  Replaces about twenty launches.
+struct Segd { int head; long long sum; };         // a run boundary inside, the sum since the last one
+__device__ __forceinline__ Segd seg_op(Segd x, Segd y) { return Segd{x.head | y.head, y.head ? y.sum : x.sum + y.sum}; }
+__device__ __forceinline__ Segd seg_incl(Segd v) {
+    for (int o = 1; o < 32; o <<= 1) {
+        const Segd u{__shfl_up_sync(0xffffffffu, v.head, o), __shfl_up_sync(0xffffffffu, v.sum, o)};
+        if ((threadIdx.x & 31) >= o) v = seg_op(u, v);
+    }
+    return v;
+}
+__device__ __forceinline__ Segd seg_at(Segd v, int lane) {
+    return Segd{__shfl_sync(0xffffffffu, v.head, lane), __shfl_sync(0xffffffffu, v.sum, lane)};
+}
+
+__global__ void __launch_bounds__(team::kTT, 1) k_seq_best(const SeqBest a) {
+    __shared__ team::Smem s;
+    using team::Item32;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const int64_t nI = *a.dI;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.undone = 0;
+    if (a.reset) {
+        const int64_t nM = *a.dM, nR = *a.dR;
+        UPR_TEAM_FOR(i, nM) a.m_pos[a.M_node[i]] = -1;
+        UPR_TEAM_FOR(i, nR) a.r_to[a.R_node[i]] = -1;
+    }
+    const team::Seg gi = team::warp_seg(nI);
+    long long sg = 0;
+    for (int64_t i = gi.b + lane; i < gi.e; i += 32) sg += a.gain[i];
+    const long long mg = team::publish<team::Sum>(t, s, 0, team::warp_all<team::Sum>(sg));
+    int64_t nev;
+    const Item32 *S = team::sort(
+        t, s, 2 * nI,
+        [&](int64_t e, Item32 &it) {
+            it.key = (uint32_t)((e & 1) ? a.I_to[e >> 1] : a.I_from[e >> 1]);
+            it.val = (uint32_t)e;
+            return true;
+        },
+        a.kbits, reinterpret_cast<Item32 *>(a.bufA), reinterpret_cast<Item32 *>(a.bufB), &nev);
+    long long all;
+    sg = team::collect<team::Sum>(t, 0, &all) + mg;
+    for (int64_t i0 = gi.b; i0 < gi.e; i0 += 32) {
+        const int64_t i = i0 + lane;
+        const long long inc = team::warp_incl<team::Sum>(i < gi.e ? a.gain[i] : 0);
+        if (i < gi.e) a.Gsum[i] = sg + inc;
+        sg += __shfl_sync(full, inc, 31);
+    }
+    // the weight of every event's block before it: a segmented sum over the
+    // sorted events (per warp, per CTA, then over the CTAs)
+    const team::Seg g = team::warp_seg(nev);
+    auto event = [&](int64_t j) {
+        const Item32 it = S[j];
+        const long long c = cw(a.vwgt, a.I_node[it.val >> 1]);
+        return Segd{j == 0 || S[j - 1].key != it.key, (it.val & 1) ? c : -c};
+    };
+    Segd acc{0, 0};
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        acc = seg_op(acc, seg_at(seg_incl(j < g.e ? event(j) : Segd{0, 0}), 31));
+    }
+    __shared__ int s_head[team::kTW];
+    if (lane == 0) { s.w[warp] = acc.sum; s_head[warp] = acc.head; }
+    __syncthreads();
+    const Segd winc = seg_incl(Segd{s_head[lane], s.w[lane]});
+    Segd mine = seg_at(winc, warp > 0 ? warp - 1 : 0);
+    if (warp == 0) mine = Segd{0, 0};
+    if (threadIdx.x == team::kTT - 1) {
+        t.tot[1 * team::kTeamMax + blockIdx.x] = winc.sum;
+        t.tot[2 * team::kTeamMax + blockIdx.x] = winc.head;
+    }
+    team::sync(t);
+    Segd carry{0, 0};
+    for (int c0 = 0; c0 < (int)blockIdx.x; c0 += 32) {
+        const int c = c0 + lane;
+        Segd x{0, 0};
+        if (c < (int)blockIdx.x)
+            x = Segd{(int)t.tot[2 * team::kTeamMax + c], t.tot[1 * team::kTeamMax + c]};
+        carry = seg_op(carry, seg_at(seg_incl(x), 31));
+    }
+    carry = seg_op(carry, mine);
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const bool ok = j < g.e;
+        const Segd x = ok ? event(j) : Segd{0, 0};
+        const Segd inc = seg_incl(x);
+        const long long after_d = inc.head ? inc.sum : carry.sum + inc.sum;
+        if (ok) {
+            const Item32 it = S[j];
+            const int64_t Lmax = a.Lb[it.key], after = a.C0[it.key] + after_d, before = after - x.sum;
+            const int d = (after > Lmax ? 1 : 0) - (before > Lmax ? 1 : 0);
+            if (d) atomicAdd(&a.diff[(it.val >> 1) + 1], d);
+        }
+        carry = seg_op(carry, seg_at(inc, 31));
+    }
+    team::sync(t);
+    // overloaded blocks after every prefix
+    const team::Seg gj = team::warp_seg(nI + 1);
+    long long so = 0;
+    for (int64_t j = gj.b + lane; j < gj.e; j += 32) so += a.diff[j];
+    int over0 = 0;
+    if (!a.gid) {
+        if (threadIdx.x == 0) s.tot[0] = 0;
+        __syncthreads();
+        for (int b = threadIdx.x; b < a.K; b += team::kTT)
+            if (a.C0[b] > a.Lb[b]) atomicAdd(&s.tot[0], 1);
+    }
+    const long long mo = team::publish<team::Sum>(t, s, 3, team::warp_all<team::Sum>(so));   // (a CTA barrier)
+    over0 = s.tot[0];
+    team::sync(t);
+    so = team::collect<team::Sum>(t, 3, &all) + mo;
+    Best best{0, -1};
+    for (int64_t j0 = gj.b; j0 < gj.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const long long x = j < gj.e ? a.diff[j] : 0;
+        const long long inc = team::warp_incl<team::Sum>(x);
+        if (j < gj.e) {
+            a.diff_excl[j] = (int32_t)(so + inc - x);
+            if (!a.gid && over0 + so + inc == 0) best = better(best, Best{j == 0 ? 0 : a.Gsum[j - 1], j});
+        }
+        so += __shfl_sync(full, inc, 31);
+    }
+    if (a.gid) return;          // (a batch: per graph, in kernels of their own)
+    auto warp_best = [&](Best b) {
+        for (int o = 16; o > 0; o >>= 1)
+            b = better(b, Best{__shfl_xor_sync(full, b.g, o), __shfl_xor_sync(full, b.j, o)});
+        return b;
+    };
+    best = warp_best(best);
+    __shared__ long long s_j[team::kTW];
+    if (lane == 0) { s.w[warp] = best.g; s_j[warp] = best.j; }
+    __syncthreads();
+    best = warp_best(Best{s.w[lane], s_j[lane]});
+    if (threadIdx.x == 0) {
+        t.tot[4 * team::kTeamMax + blockIdx.x] = best.g;
+        t.tot[5 * team::kTeamMax + blockIdx.x] = best.j;
+    }
+    team::sync(t);
+    best = Best{0, -1};
+    for (int c = lane; c < (int)gridDim.x; c += 32)
+        best = better(best, Best{t.tot[4 * team::kTeamMax + c], t.tot[5 * team::kTeamMax + c]});
+    best = warp_best(best);
+    // the prefix applied; the degrees of the moves after it
+    BlockDelta bd = make_block_delta(s.cnt64, a.K, reinterpret_cast<unsigned long long *>(a.C0));
+    bd.init();
+    long long degs = 0;
+    for (int64_t i0 = gi.b; i0 < gi.e; i0 += 32) {
+        const int64_t i = i0 + lane;
+        int32_t from = -1, to = -1;
+        long long c = 0;
+        if (i < gi.e) {
+            const int32_t v = a.I_node[i];
+            if (i < best.j) {
+                from = a.I_from[i];
+                to = a.I_to[i];
+                c = cw(a.vwgt, v);
+                a.part0[v] = to;
+            } else {
+                degs += a.xadj[v + 1] - a.xadj[v];
+            }
+        }
+        bd.add(from, -c);
+        bd.add(to, c);
+    }
+    bd.flush(reinterpret_cast<unsigned long long *>(a.C0));
+    degs = warp_sum(degs);
+    if (lane == 0 && degs) atomicAdd(reinterpret_cast<unsigned long long *>(a.undone), (unsigned long long)degs);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.best[0] = best.g;
+        a.best[1] = best.j;
+        *a.d_over0 = over0;
+        if (best.j < 0) *a.d_infeasible = 1;
+        else *a.cut -= best.g;
+    }
 }
 
 // ---- batches: I sorted by graph (stable), then per-graph segments
 // [seg_beg[g], seg_end[g]) of I; G_g(j) and eligibility are differences of
 // the global prefix sums taken at the segment start.
-
-// keys: graph of each move of I
-__global__ void k_i_graph_keys(const int32_t *__restrict__ I_node, const int32_t *__restrict__ d_nI,
-                               const int32_t *__restrict__ gid, uint64_t *__restrict__ keys,
-                               uint32_t *__restrict__ vals) {
-    const int64_t nI = *d_nI;
-    UPR_FOR(i, nI) {
-        keys[i] = (uint64_t)gid[I_node[i]];
-        vals[i] = (uint32_t)i;
-    }
-}
-
-// I in graph order (out arrays), pos/dest of the moved nodes, segment bounds
-__global__ void k_i_permute(const uint32_t *__restrict__ order, const uint64_t *__restrict__ gkeys,
-                            const int32_t *__restrict__ d_nI, const int32_t *__restrict__ I_node,
-                            const int32_t *__restrict__ I_from, const int32_t *__restrict__ I_to,
-                            int32_t *__restrict__ O_node, int32_t *__restrict__ O_from, int32_t *__restrict__ O_to,
-                            int32_t *__restrict__ pos, int32_t *__restrict__ dest, int32_t *__restrict__ seg_beg,
-                            int32_t *__restrict__ seg_end) {
-    const int64_t nI = *d_nI;
-    UPR_FOR(q, nI) {
-        const uint32_t i = order[q];
-        const int32_t v = I_node[i];
-        O_node[q] = v;
-        O_from[q] = I_from[i];
-        O_to[q] = I_to[i];
-        pos[v] = (int32_t)q;
-        dest[v] = I_to[i];
-        const int32_t g = (int32_t)gkeys[q];
-        if (q == 0 || (int32_t)gkeys[q - 1] != g) seg_beg[g] = (int32_t)q;
-        if (q == nI - 1 || (int32_t)gkeys[q + 1] != g) seg_end[g] = (int32_t)(q + 1);
-    }
-}
 
 // per graph: best gain so far = 0 if the empty prefix is eligible, else "none"
 __global__ void k_best_seg_init(const int32_t *__restrict__ over0, int32_t ng, long long *__restrict__ best_g,
@@ -685,7 +751,7 @@ __global__ void k_table_rollback(Rollback rb, const int64_t *__restrict__ xadj, 
 }
 
 __global__ void __launch_bounds__(512) k_table_rollback_hubs(Rollback rb, const HubChunk *__restrict__ chunks,
-                                                             const int32_t *__restrict__ pos,
+                                                             const int2 *__restrict__ pk,
                                                              const int32_t *__restrict__ adj,
                                                              const int32_t *__restrict__ adjw, int32_t k,
                                                              int32_t kmask, int32_t *__restrict__ W,
@@ -693,7 +759,7 @@ __global__ void __launch_bounds__(512) k_table_rollback_hubs(Rollback rb, const 
                                                              SparseRows sp) {
     if (*deg_sum * 4 >= m) return;
     const HubChunk ch = chunks[blockIdx.x];
-    const int32_t i = pos[ch.v];
+    const int32_t i = pk[ch.v].x;
     if (i == INT32_MAX || !rolled_back(rb, i)) return;
     const int32_t a = blk_local(rb.I_to[i], k, kmask), b = blk_local(rb.I_from[i], k, kmask);
     for (int64_t e = ch.begin + threadIdx.x; e < ch.end; e += blockDim.x) {
@@ -706,24 +772,6 @@ __global__ void __launch_bounds__(512) k_table_rollback_hubs(Rollback rb, const 
         int32_t *row = W + (int64_t)adj[e] * k;
         atomicSub(&row[a], w);
         atomicAdd(&row[b], w);
-    }
-}
-
-// The variant of Sec. 7.2 without interleaving: X = M, then R in its order.
-__global__ void k_seq_append(const int32_t *__restrict__ M_node, const int32_t *__restrict__ M_from,
-                             const int32_t *__restrict__ M_to, const int32_t *__restrict__ d_nM,
-                             const int32_t *__restrict__ R_node, const int32_t *__restrict__ R_from,
-                             const int32_t *__restrict__ R_to, const int32_t *__restrict__ d_nR,
-                             int32_t *__restrict__ X_node, int32_t *__restrict__ X_from, int32_t *__restrict__ X_to,
-                             int8_t *__restrict__ X_isr) {
-    const int64_t nM = *d_nM, nR = *d_nR;
-    UPR_FOR(i, nM + nR) {
-        const bool r = i >= nM;
-        const int64_t j = r ? i - nM : i;
-        X_node[i] = r ? R_node[j] : M_node[j];
-        X_from[i] = r ? R_from[j] : M_from[j];
-        X_to[i] = r ? R_to[j] : M_to[j];
-        X_isr[i] = r ? 1 : 0;
     }
 }
 
@@ -762,28 +810,12 @@ __global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) {
     UPR_FOR(i, n) a[i] = v;
 }
 
-// a[0 .. *d_n + extra) = 0
-__global__ void k_clear_count(int32_t *a, const int32_t *__restrict__ d_n, int32_t extra) {
-    const int64_t n = (int64_t)*d_n + extra;
-    UPR_FOR(i, n) a[i] = 0;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------- wrappers
-void count_affine(const int32_t *a, int32_t a_mul, const int32_t *b, int32_t add, int32_t *out, cudaStream_t s) {
-    k_count_affine<<<1, 32, 0, s>>>(a, a_mul, b, add, out);
-    UPR_LAUNCH_CHECK();
-}
-
 void fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t s) {
     if (n <= 0) return;
     k_fill_i32<<<grid_for(n), 256, 0, s>>>(a, n, v);
-    UPR_LAUNCH_CHECK();
-}
-
-void clear_count(int32_t *a, const int32_t *d_n, int32_t extra, int64_t max, cudaStream_t s) {
-    k_clear_count<<<grid_for(max + extra), 256, 0, s>>>(a, d_n, extra);
     UPR_LAUNCH_CHECK();
 }
 
@@ -799,90 +831,25 @@ void count_over(const GraphDev &g, const int64_t *C, int32_t *out, cudaStream_t 
     UPR_LAUNCH_CHECK();
 }
 
-void seq_rb_keys(const int32_t *R_from, const int32_t *d_nR, int64_t max, uint64_t *keys, uint32_t *vals,
-                 cudaStream_t s) {
-    k_rb_keys<<<grid_for(max), 256, 0, s>>>(R_from, d_nR, keys, vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_rb_bounds(const int32_t *R_node, const int32_t *R_from, const uint32_t *RB, const int32_t *d_nR, int64_t max,
-                   const int32_t *vwgt, int64_t *rc, int32_t *rbeg, int32_t *rend, cudaStream_t s) {
-    k_rb_bounds<<<grid_for(max), 256, 0, s>>>(R_node, R_from, RB, d_nR, vwgt, rc, rbeg, rend);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_ev_keys(const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM, int64_t max, uint64_t *keys,
-                 uint32_t *vals, cudaStream_t s) {
-    k_ev_keys<<<grid_for(2 * max), 256, 0, s>>>(M_from, M_to, d_nM, keys, vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_ev_delta(const int32_t *M_node, const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max,
-                  const int32_t *vwgt, int64_t *delta, int32_t *ebeg, int32_t *eend, cudaStream_t s) {
-    k_ev_delta<<<grid_for(2 * max), 256, 0, s>>>(M_node, EV, ekeys, d_nM, vwgt, delta, ebeg, eend);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_ev_need(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max, const int64_t *delta,
-                 const int64_t *d_excl, const int32_t *ebeg, const int64_t *C0, const int64_t *Lb,
-                 const int32_t *rbeg, const int32_t *rend, const int64_t *rc_excl, const int64_t *rc, uint64_t *packed,
-                 cudaStream_t s) {
-    k_ev_need<<<grid_for(2 * max), 256, 0, s>>>(EV, ekeys, d_nM, delta, d_excl, ebeg, C0, Lb, rbeg, rend, rc_excl, rc,
-                                                packed);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_ev_emit(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nM, int64_t max, const uint64_t *qmax,
-                 const int32_t *ebeg, int32_t *emit, int32_t *qbefore_m, cudaStream_t s) {
-    k_ev_emit<<<grid_for(2 * max), 256, 0, s>>>(EV, ekeys, d_nM, qmax, ebeg, emit, qbefore_m);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_block_final(int32_t K, const int32_t *ebeg, const int32_t *eend, const uint64_t *qmax, const int32_t *rbeg,
-                     const int32_t *rend, int32_t *qfin, int32_t *left, cudaStream_t s) {
-    k_block_final<<<(unsigned)ceil_div(K, 256), 256, 0, s>>>(K, ebeg, eend, qmax, rbeg, rend, qfin, left);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_place_m(const int32_t *M_node, const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM, int64_t max,
-                 const int32_t *em_excl, int32_t *pos_m, int32_t *X_node, int32_t *X_from, int32_t *X_to,
-                 int8_t *X_isr, cudaStream_t s) {
-    k_place_m<<<grid_for(max), 256, 0, s>>>(M_node, M_from, M_to, d_nM, em_excl, pos_m, X_node, X_from, X_to, X_isr);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_place_r(const int32_t *R_node, const int32_t *R_from, const int32_t *R_to, const uint32_t *RB,
-                 const int32_t *d_nR, int64_t max, const int32_t *rbeg, const uint32_t *EV, const int32_t *ebeg,
-                 const int32_t *eend, const uint64_t *qmax, const int32_t *pos_m, const int32_t *qfin,
-                 const int32_t *left_excl, const int32_t *em_excl, const int32_t *emit, const int32_t *d_nM,
-                 int32_t *X_node, int32_t *X_from, int32_t *X_to, int8_t *X_isr, cudaStream_t s) {
-    k_place_r<<<grid_for(max), 256, 0, s>>>(R_node, R_from, R_to, RB, d_nR, rbeg, EV, ebeg, eend, qmax, pos_m, qfin,
-                                            left_excl, em_excl, emit, d_nM, X_node, X_from, X_to, X_isr);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_merge_flags(const int32_t *X_node, const int32_t *X_to, const int8_t *X_isr, const int32_t *d_nX, int64_t max,
-                     const int32_t *m_pos, const int32_t *r_to, const int32_t *part0, int32_t *keep, int32_t *final_to,
-                     cudaStream_t s) {
-    k_merge_flags<<<grid_for(max), 256, 0, s>>>(X_node, X_to, X_isr, d_nX, m_pos, r_to, part0, keep, final_to);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_build_I(const int32_t *Ix, const int32_t *d_nI, int64_t max, const int32_t *X_node, const int32_t *final_to,
-                 const int32_t *part0, int32_t *I_node, int32_t *I_from, int32_t *I_to, int32_t *pos, int32_t *dest,
-                 cudaStream_t s) {
-    k_build_I<<<grid_for(max), 256, 0, s>>>(Ix, d_nI, X_node, final_to, part0, I_node, I_from, I_to, pos, dest);
-    UPR_LAUNCH_CHECK();
+void seq_build(const GraphDev &g, SeqBuild a, cudaStream_t s) {
+    a.n = g.n;
+    a.k = g.k;
+    a.kmask = g.kmask;
+    a.K = g.K();
+    a.ng = g.ng;
+    a.vwgt = g.vwgt;
+    a.gid = g.gid;
+    a.xadj = g.xadj;
+    a.Lb = g.Lb;
+    a.kbits = a.ngbits = 1;
+    while ((1ll << a.kbits) < a.K) a.kbits++;
+    while ((1ll << a.ngbits) < a.ng) a.ngbits++;
+    launch_team(k_seq_build, a, a.team.size, s);
 }
 
 void seq_gains(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-               const int32_t *d_nI, int64_t max, const int32_t *part0, int2 *pk, int64_t *gain,
-               const HubChunk *hub_chunks, int64_t n_chunks, int64_t *deg_sum, cudaStream_t s) {
-    k_pk_fill<<<grid_for(g.n), 256, 0, s>>>(part0, g.n, g.k, g.kmask, pk);
-    UPR_LAUNCH_CHECK();
-    k_pk_moves<<<grid_for(max), 256, 0, s>>>(I_node, I_from, I_to, d_nI, g.k, g.kmask, g.xadj, pk,
-                                             reinterpret_cast<unsigned long long *>(deg_sum));
-    UPR_LAUNCH_CHECK();
+               const int32_t *d_nI, int64_t max, const int2 *pk, int64_t *gain, const HubChunk *hub_chunks,
+               int64_t n_chunks, cudaStream_t s) {
     // two waves of CTAs (moved nodes differ widely in degree)
     const unsigned blocks = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>(ceil_div(max * 32, 256), (int64_t)device_sm_count() * 16));
@@ -894,66 +861,33 @@ void seq_gains(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, 
     }
 }
 
-void seq_iev_keys(const int32_t *I_from, const int32_t *I_to, const int32_t *d_nI, int64_t max, uint64_t *keys,
-                  uint32_t *vals, cudaStream_t s) {
-    k_iev_keys<<<grid_for(2 * max), 256, 0, s>>>(I_from, I_to, d_nI, keys, vals);
-    UPR_LAUNCH_CHECK();
+void seq_best(const GraphDev &g, SeqBest a, cudaStream_t s) {
+    a.K = g.K();
+    a.vwgt = g.vwgt;
+    a.gid = g.gid;
+    a.xadj = g.xadj;
+    a.Lb = g.Lb;
+    a.kbits = 1;
+    while ((1ll << a.kbits) < a.K) a.kbits++;
+    launch_team(k_seq_best, a, a.team.size, s);
 }
 
-void seq_iev_delta(const int32_t *I_node, const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nI, int64_t max,
-                   const int32_t *vwgt, int64_t *delta, int32_t *ebeg, cudaStream_t s) {
-    k_iev_delta<<<grid_for(2 * max), 256, 0, s>>>(I_node, EV, ekeys, d_nI, vwgt, delta, ebeg);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_iev_transitions(const uint32_t *EV, const uint64_t *ekeys, const int32_t *d_nI, int64_t max,
-                         const int64_t *delta, const int64_t *d_excl, const int32_t *ebeg, const int64_t *C0,
-                         const int64_t *Lb, int32_t *diff, cudaStream_t s) {
-    k_iev_transitions<<<grid_for(2 * max), 256, 0, s>>>(EV, ekeys, d_nI, delta, d_excl, ebeg, C0, Lb, diff);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_best(const int64_t *Gsum, const int32_t *diff, const int32_t *diff_excl, const int32_t *d_nI, int64_t max,
-              const int32_t *d_over0, long long *parts, long long *out, int32_t *infeasible, cudaStream_t s) {
-    const int nparts = (int)std::min<int64_t>(ceil_div(max + 1, 256), 1024);
-    k_best_partial<<<nparts, 256, 0, s>>>(Gsum, diff, diff_excl, d_nI, d_over0, parts, parts + 1024);
-    UPR_LAUNCH_CHECK();
-    k_best_final<<<1, 1024, 0, s>>>(parts, parts + 1024, nparts, out, infeasible);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_apply_prefix(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-                      int64_t max, const long long *best, int32_t *part0, int64_t *C0, int64_t *cut, cudaStream_t s) {
-    const int64_t blocks = std::min<int64_t>(ceil_div(max > 0 ? max : 1, 256), (int64_t)device_sm_count() * 4);
-    k_apply_prefix<<<(unsigned)blocks, 256, block_delta_smem(g.K()), s>>>(
-        I_node, I_from, I_to, best, g.vwgt, part0, (unsigned long long *)C0, g.K(), (long long *)cut);
-    UPR_LAUNCH_CHECK();
-}
-
-void table_rollback(const GraphDev &g, const Rollback &rb, int64_t max, const int32_t *pos, int32_t *W,
+void table_rollback(const GraphDev &g, const Rollback &rb, int64_t max, const int2 *pk, int32_t *W,
                     const HubChunk *hub_chunks, int64_t n_chunks, int64_t *deg_sum, cudaStream_t s) {
-    UPR_CUDA(cudaMemsetAsync(deg_sum, 0, sizeof(int64_t), s));
     if (max <= 0) return;
-    k_rollback_degsum<<<grid_for(max), 256, 0, s>>>(rb, g.xadj, (unsigned long long *)deg_sum);
-    UPR_LAUNCH_CHECK();
+    if (rb.gid) {           // (one graph: summed by k_seq_best)
+        k_rollback_degsum<<<grid_for(max), 256, 0, s>>>(rb, g.xadj, (unsigned long long *)deg_sum);
+        UPR_LAUNCH_CHECK();
+    }
     const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(max * 32, 256), (int64_t)device_sm_count() * 16);
     k_table_rollback<<<blocks, 256, 0, s>>>(rb, g.xadj, g.adj, g.adjw, g.k, g.kmask, W, deg_sum, g.m,
                                                       g.sp);
     UPR_LAUNCH_CHECK();
     if (n_chunks > 0) {
-        k_table_rollback_hubs<<<(unsigned)n_chunks, 512, 0, s>>>(rb, hub_chunks, pos, g.adj, g.adjw, g.k, g.kmask, W,
+        k_table_rollback_hubs<<<(unsigned)n_chunks, 512, 0, s>>>(rb, hub_chunks, pk, g.adj, g.adjw, g.k, g.kmask, W,
                                                                  deg_sum, g.m, g.sp);
         UPR_LAUNCH_CHECK();
     }
-}
-
-void seq_append(const int32_t *M_node, const int32_t *M_from, const int32_t *M_to, const int32_t *d_nM,
-                const int32_t *R_node, const int32_t *R_from, const int32_t *R_to, const int32_t *d_nR, int64_t max,
-                int32_t *X_node, int32_t *X_from, int32_t *X_to, int8_t *X_isr, cudaStream_t s) {
-    if (max <= 0) return;
-    k_seq_append<<<grid_for(max), 256, 0, s>>>(M_node, M_from, M_to, d_nM, R_node, R_from, R_to, d_nR, X_node, X_from,
-                                              X_to, X_isr);
-    UPR_LAUNCH_CHECK();
 }
 
 void guard_locks(const Rollback &rb, int64_t max, int64_t n, const int32_t *m_pos, const int32_t *r_to,
@@ -968,23 +902,6 @@ void guard_filter(const int8_t *locked, int64_t n, int32_t *flags, int32_t *cand
                   int32_t *cand_gain, cudaStream_t s) {
     if (n <= 0) return;
     k_guard_filter<<<grid_for(n), 256, 0, s>>>(locked, n, flags, cand_tgt, cand_s0, cand_gain);
-    UPR_LAUNCH_CHECK();
-}
-
-void seq_sort_by_graph(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
-                       const int32_t *d_nI, int64_t max, uint64_t *keys, uint32_t *vals, uint64_t *keys_alt,
-                       uint32_t *vals_alt, Scratch tmp, int32_t *O_node, int32_t *O_from, int32_t *O_to, int32_t *pos,
-                       int32_t *dest, int32_t *seg_beg, int32_t *seg_end, cudaStream_t s) {
-    UPR_CUDA(cudaMemsetAsync(seg_beg, 0, sizeof(int32_t) * g.ng, s));
-    UPR_CUDA(cudaMemsetAsync(seg_end, 0, sizeof(int32_t) * g.ng, s));
-    if (max <= 0) return;
-    k_i_graph_keys<<<grid_for(max), 256, 0, s>>>(I_node, d_nI, g.gid, keys, vals);
-    UPR_LAUNCH_CHECK();
-    int gbits = 1;
-    while ((1ll << gbits) < g.ng) gbits++;
-    const bool alt = radix_sort_pairs(keys, vals, keys_alt, vals_alt, Count{d_nI, max}, gbits, tmp, s);
-    k_i_permute<<<grid_for(max), 256, 0, s>>>(alt ? vals_alt : vals, alt ? keys_alt : keys, d_nI, I_node, I_from, I_to,
-                                              O_node, O_from, O_to, pos, dest, seg_beg, seg_end);
     UPR_LAUNCH_CHECK();
 }
 

@@ -55,9 +55,6 @@ using JobPtr = std::shared_ptr<Job>;
 size_t upr_ctx_footprint(int64_t n, int64_t m, int32_t k, int32_t ng);
 
 namespace upr {
-upr_status ctx_rebind(upr_ctx *c, const upr_graph *g, int32_t k, double eps, const upr_params *params);
-upr_status ctx_rebind_batch(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, const double *eps,
-                            const upr_params *params);
 size_t ctx_arena_bytes(const upr_ctx *c);
 }
 
