@@ -51,16 +51,7 @@ struct Arena {
     }
 };
 
-struct SortBuf {
-    uint64_t *k, *ka;
-    uint32_t *v, *va;
-    // sorts (k, v) on `bits` bits; returns the buffers holding the result
-    void run(Count n, int bits, Scratch tmp, cudaStream_t s, uint64_t **ko, uint32_t **vo) {
-        bool alt = radix_sort_pairs(k, v, ka, va, n, bits, tmp, s);
-        *ko = alt ? ka : k;
-        *vo = alt ? va : v;
-    }
-};
+struct SortBuf { uint64_t *k, *ka; uint32_t *v, *va; };
 
 // Host-side F_r[l] = floor(tau_r * (3/2)^l * 2^Q), tau_r = tau_1 + (1 - tau_1)(r-1)/max(R-1,1)
 // F[l] = floor(tau * (3/2)^l * 2^Q) for tau = num / den
@@ -106,13 +97,12 @@ __global__ void k_fill_i64(int64_t *a, int64_t n, int64_t v) {
 namespace {
 // Slots of the device counters (upr_ctx::counts).
 enum {
-    CNT_CAND = 0, CNT_M, CNT_P, CNT_S, CNT_A, CNT_I, CNT_HUB, CNT_BADPART, CNT_L1, CNT_X, CNT_OVER0, CNT_INFEAS, CNT_HIST, CNT_EXACT, CNT_SORTP, CNT_SLOTS = 32
+    CNT_CAND = 0, CNT_M, CNT_P, CNT_A, CNT_I, CNT_BADPART = 7, CNT_L1, CNT_X, CNT_OVER0, CNT_INFEAS, CNT_EXACT, CNT_SLOTS = 32
 };
 
 // Per-call sums of the step graph's rounds (upr_ctx::dstats): candidates,
 // moves, rebalancing moves, sub-rounds, sequence length, applied moves, the
-// primitives' error word, infeasible rounds, interleaved length, runs of the
-// sub-rounds' conditional sort passes.
+// barriers' error word, infeasible rounds, interleaved length.
 __global__ void k_round_stats(const int32_t *__restrict__ cnt, const RebalCtl *__restrict__ ctl,
                               const long long *__restrict__ best, const int64_t *__restrict__ tot, int batch,
                               const int32_t *__restrict__ err, long long *__restrict__ d) {
@@ -127,7 +117,6 @@ __global__ void k_round_stats(const int32_t *__restrict__ cnt, const RebalCtl *_
     d[6] |= *err;
     d[7] += infeasible ? 1 : 0;
     d[8] += cnt[CNT_X];
-    d[9] += cnt[CNT_SORTP];
 }
 }  // namespace
 
@@ -198,15 +187,13 @@ struct upr_ctx {
     cudaGraphExec_t reb_exec = nullptr;
     uint64_t gen = 0, reb_gen = ~0ull;  // binding generation; the one reb_exec belongs to
     LaneCfg reb_cfg{};
-    int reb_body_kernels = 0;
+    int reb_body_kernels = 0, reb_head_kernels = 0;
     cudaStream_t s_up = nullptr;      // binding: the early upload of the adjacency
     cudaEvent_t ev_up = nullptr, ev_prev = nullptr;
     int64_t *xs = nullptr;            // binding: the packed offsets and the schedule counts (bind.cu), kept
     int64_t xs_cap = 0;
     HostSeg *segs_d = nullptr;        // binding a batch: the segments of a gather of host arrays, kept
     int64_t segs_cap = 0;
-    int reb_if_kernels = 0;           // kernels of the conditional sort passes in the sub-round body
-    cudaStream_t s_if = nullptr;      // capture stream of that conditional body
     int64_t rounds_bound = 0;         // rounds run since the binding
     bool cut_pending = false;         // the next build also computes the cut of part0 (load_part skipped it)
     int32_t lp_attempts = 0;          // label propagation rounds run by the current call (kept or not)
@@ -258,7 +245,7 @@ struct upr_ctx {
     int32_t *cand_tgt, *cand_gain, *flags, *flags2, *m_pos, *r_to, *r_at, *prop_tgt, *prop_gain;
     int64_t *cand_s0;
     // lists
-    int32_t *idxA, *idxB, *idxC, *L1, *Pq;
+    int32_t *idxA, *L1;
     int32_t *score;
     int32_t *M_node, *M_from, *M_to; int64_t *M_score;
     int32_t *R_node, *R_from, *R_to, *R_sub;
@@ -267,13 +254,12 @@ struct upr_ctx {
     SortBuf sb[3];
     int64_t *c_sorted, *c_excl, *seg_base;
     uint64_t *packed;
-    uint64_t *prio_rep;                 // [2 * kPrioBins] rebalancing: a key per prefilter bin
+    unsigned long long *prio_rep;       // [kPrioBins] rebalancing: a key per prefilter bin
     int32_t *emit, *qbefore, *pos_m;
     int32_t *diff, *diff_excl;
-    int32_t *seg_first, *rbeg, *rend, *ebeg, *eend, *qfin, *left_excl;
+    int32_t *rbeg, *rend, *ebeg, *eend, *qfin, *left_excl;
     long long *best;
     int8_t *over_d, *excl_d, *reject_d;
-    long long *Cd;                   // [K] block-weight changes of a fused rebalancing sub-round
     unsigned long long *prio_hist;   // [K][kPrioBins] proposal prefilter (null: K too large, no prefilter)
     int32_t *prio_cut;               // [K]
     int32_t *counts;          // device counters (CNT_* slots)
@@ -281,7 +267,6 @@ struct upr_ctx {
     long long *dstats;        // [16] per-call sums of the step graph's rounds
     uint64_t *vacc; int32_t *vflags; int64_t *scal, *cut_parts;
     int2 *pk;                 // exact gains: position in I and blocks before/after, per node
-    Scratch tmp;              // scan / sort temporaries
     Team team;                // the team launches of this binding
     int beside = 1;           // contexts that refine at the same time as this one, with it
     // pinned host mirrors
@@ -337,9 +322,9 @@ void layout(upr_ctx *c, Arena &A) {
     c->F = A.take<int64_t>(kSlots);
     c->first_slot = A.take<int8_t>(k);
     for (int32_t **p : {&c->cand_tgt, &c->cand_gain, &c->flags, &c->m_pos, &c->r_to, &c->prop_tgt,
-                        &c->prop_gain, &c->idxA, &c->idxB, &c->idxC, &c->M_node, &c->M_from, &c->M_to, &c->R_node,
+                        &c->prop_gain, &c->idxA, &c->M_node, &c->M_from, &c->M_to, &c->R_node,
                         &c->R_from, &c->R_to, &c->R_sub, &c->I_node, &c->I_from, &c->I_to, &c->emit, &c->qbefore,
-                        &c->pos_m, &c->L1, &c->r_at, &c->Pq})
+                        &c->pos_m, &c->L1, &c->r_at})
         *p = A.take<int32_t>(n);
     for (int32_t **p : {&c->flags2, &c->X_node, &c->X_from, &c->X_to})
         *p = A.take<int32_t>(n2 + 1);
@@ -360,14 +345,13 @@ void layout(upr_ctx *c, Arena &A) {
     c->c_excl = A.take<int64_t>(n2);
     c->packed = A.take<uint64_t>(n2);
     c->seg_base = A.take<int64_t>(k);
-    c->prio_rep = A.take<uint64_t>(2 * (size_t)kPrioBins);
-    for (int32_t **p : {&c->seg_first, &c->rbeg, &c->rend, &c->ebeg, &c->eend, &c->qfin, &c->left_excl})
+    c->prio_rep = A.take<unsigned long long>((size_t)kPrioBins);
+    for (int32_t **p : {&c->rbeg, &c->rend, &c->ebeg, &c->eend, &c->qfin, &c->left_excl})
         *p = A.take<int32_t>(k);
     c->best = A.take<long long>(2);
     c->over_d = A.take<int8_t>(k);
     c->excl_d = A.take<int8_t>(k);
     c->reject_d = A.take<int8_t>(k);
-    c->Cd = A.take<long long>(k);
     const bool prefilter = k * (size_t)kPrioBins <= ((size_t)1 << 22);
     c->prio_hist = prefilter ? A.take<unsigned long long>(k * kPrioBins) : nullptr;
     c->prio_cut = prefilter ? A.take<int32_t>(k) : nullptr;
@@ -379,19 +363,12 @@ void layout(upr_ctx *c, Arena &A) {
     c->scal = A.take<int64_t>(4);    // [0] wmax, [1] degree sum of M, [2] degree sum of undone moves
     c->cut_parts = A.take<int64_t>(kCutParts + 1);   // twice the input cut: partial sums, total
     c->pk = A.take<int2>(n);
-    c->tmp.tiles_cap = ceil_div(std::max<int64_t>((int64_t)n2 + 2, (int64_t)k + 2), 2048);   // lists of nodes, events, blocks
-    c->tmp.mem_bytes = radix_temp_bytes(c->tmp.tiles_cap * 2048);
-    c->tmp.scan_bytes = scan_temp_bytes(c->tmp.tiles_cap * 2048);
-    c->tmp.mem = A.take<char>(c->tmp.mem_bytes);
-    c->tmp.scan = A.take<char>(c->tmp.scan_bytes);
-    c->tmp.ticket = A.take<unsigned int>(64);
-    c->tmp.err = A.take<int32_t>(1);
-    c->tmp.epoch = A.take<uint32_t>(1);
     c->team.size = team_size((int64_t)n, c->beside);
     c->team.hist = A.take<int32_t>((size_t)c->team.size * team::kSortBins);
+    c->team.hist64 = A.take<unsigned long long>(2 * (size_t)c->team.size * team::kSortBins);
     c->team.tot = A.take<long long>((size_t)team::kTotSlots * team::kTeamMax);
-    c->team.bar = reinterpret_cast<unsigned long long *>(c->tmp.ticket + 16);     // (cleared at every binding)
-    c->team.err = c->tmp.err;
+    c->team.bar = A.take<unsigned long long>(1);
+    c->team.err = A.take<int32_t>(1);
 }
 
 enum MemKind { kHost = 0, kDevice = 1 };
@@ -574,32 +551,6 @@ void set_pack(const upr_ctx *c, Penalty &pen) {
     }
 }
 
-// The fused form of a rebalancing sub-round applies: one graph, K <= 256, a
-// one-word key, the prefilter, and per-(block, tile) sums that fit the
-// 2n-entry buffers they use (UPR_FUSED=0 in the environment turns it off:
-// the general form computes the same sub-round).
-bool fused_rebalance(const upr_ctx *c, int key_bits) {
-    static int env = -1;
-    if (env < 0) { const char *v = getenv("UPR_FUSED"); env = (v && *v == '0') ? 0 : 1; }
-    const int64_t n = std::max<int64_t>(c->n, 1);
-    return env == 1 && rebalance_fused_ok(c->G, key_bits, c->prio_hist != nullptr) &&
-           (int64_t)c->G.K() * ceil_div(n, (int64_t)2048) <= 2 * n;
-}
-
-// The fused sub-round's steps after the proposals in one cooperative launch
-// (UPR_MEGA=0 in the environment: one launch per step, the same results).
-bool mega_rebalance() {
-    static int env = -1;
-    if (env < 0) {
-        const char *v = getenv("UPR_MEGA");
-        int coop = 0, dev = 0;
-        UPR_CUDA(cudaGetDevice(&dev));
-        UPR_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        env = (v && *v == '0') || !coop ? 0 : 1;
-    }
-    return env == 1;
-}
-
 // One rebalancing sub-round (Sec. 6), enqueued on s.  Every argument is fixed
 // for the binding (the sub-round number and every list length live in device
 // memory), so the same launches can be captured once and replayed.  first:
@@ -611,16 +562,12 @@ bool enqueue_subround(upr_ctx *c, const RebalState &st, int32_t *light, bool fir
                       cudaGraphConditionalHandle cond = 0) {
     const GraphDev &G = c->G;
     const int64_t n = c->n;
-    const int kbits = std::max(1, bit_length((uint64_t)(G.K() - 1)));
     int32_t *cnt = c->counts;
     RebalCtl *ctl = c->ctl;
-    const Count cS{cnt + CNT_S, n};
-    // a graph-resident loop in the fused form begins each sub-round at the
-    // end of the one before (and the first before the loop, merged_loop_head)
-    const bool merged = cond && fused_rebalance(c, 1 + c->gbits + 2 * c->cbits);
-    if (!merged)
-        rebalance_begin(G, c->C, c->excl_d, c->over_d, c->reject_d, cnt + CNT_L1, c->prm.max_subrounds, ctl, light,
-                        s);
+    // (one graph: begun by the end of the one before, the first by rebalance_start)
+    if (c->ng > 1)
+        rebalance_begin_batch(G, c->C, c->excl_d, c->over_d, c->reject_d, cnt + CNT_L1, c->prm.max_subrounds, ctl,
+                              light, s);
     if (first)
         run_tuned(c, c->prop_tuned, c->prop_cfg, c->prop_cands, &c->prop_pending, c->ev_tune + 6,
                   [&](LaneCfg cfg) {
@@ -634,142 +581,65 @@ bool enqueue_subround(upr_ctx *c, const RebalState &st, int32_t *light, bool fir
     // node without a proposal has no block with room for it (the lightest
     // allowed block has the most room, and rooms only shrink), so it never
     // proposes again
-    const int key_bits = 1 + c->gbits + 2 * c->cbits;
-    if (fused_rebalance(c, key_bits)) {
-        // the same sub-round in fused passes (reb_fused.cu): the proposers
-        // with the prefilter histogram, the cut bins, the kept proposals as
-        // (key, node), one sort by key, selection and admission from
-        // per-tile block sums, R appended and the moves applied
-        uint64_t *rep = c->prio_rep;
-        int32_t *exact = cnt + CNT_EXACT;
-        if (mega_rebalance()) {
-            // steps 1 and 3-7 in one cooperative launch (the sort buffers of
-            // sb[1] and sb[2] hold the compacted proposers: free here)
-            RebalMega m{};
-            m.flags = c->flags;
-            m.list = c->L1;
-            m.lsrc = st.lsrc;
-            m.lgain = st.lgain;
-            m.d_n1 = &ctl->n1_active;
-            m.list2 = reinterpret_cast<int32_t *>(c->sb[1].v);
-            m.lsrc2 = reinterpret_cast<int32_t *>(c->sb[1].va);
-            m.lgain2 = reinterpret_cast<int32_t *>(c->sb[2].v);
-            m.gbits = c->gbits;
-            m.cbits = c->cbits;
-            m.gain_only = c->prm.gain_priority;
-            m.hist = c->prio_hist;
-            m.rep = rep;
-            m.cut = c->prio_cut;
-            m.over = c->over_d;
-            m.C = c->C;
-            m.keys = c->sb[0].k;
-            m.keys_alt = c->sb[0].ka;
-            m.vals = c->sb[0].v;
-            m.vals_alt = c->sb[0].va;
-            m.part = c->part;
-            m.prop_tgt = c->prop_tgt;
-            m.sel = reinterpret_cast<int8_t *>(c->flags2);
-            m.h0 = reinterpret_cast<long long *>(c->c_sorted);
-            m.h1 = reinterpret_cast<long long *>(c->c_excl);
-            m.reject = c->reject_d;
-            m.ctl = ctl;
-            m.R_node = c->R_node; m.R_from = c->R_from; m.R_to = c->R_to; m.R_sub = c->R_sub;
-            m.r_to = c->r_to; m.r_at = c->r_at;
-            m.Cd = c->Cd;
-            m.d_np = cnt + CNT_L1;
-            m.d_nk = cnt + CNT_P;
-            m.d_na = cnt + CNT_A;
-            m.exact = exact;
-            rebalance_fused_mega(G, m, key_bits, n, c->tmp, s);
-            table_move(G, c->W, c->R_node, c->R_from, c->R_to, cnt + CNT_A, &ctl->nR, nullptr, n, c->hub_chunks,
-                       c->n_chunks, HubMoves{nullptr, c->r_to, c->r_at, &ctl->nR, cnt + CNT_A, c->R_from, c->R_to}, s);
-            rebalance_fused_end(G, c->C, c->Cd, c->excl_d, c->reject_d, cnt + CNT_A, ctl, s, cond,
-                                c->prm.max_subrounds, merged ? c->over_d : nullptr, c->reject_d, cnt + CNT_L1);
-            return cond != 0;
-        }
-        rebalance_fused_compact_hist(G, c->flags, c->L1, &ctl->n1_active, n, cnt + CNT_L1, st.lgain, st.lsrc,
-                                     c->gbits, c->cbits, c->prm.gain_priority, c->prio_hist, rep, exact, c->tmp, s);
-        rebalance_prio_cut(G, c->over_d, c->C, c->prio_hist, c->prio_cut, s);
-        rebalance_fused_keep_keys(G, c->L1, cnt + CNT_L1, n, st.lgain, st.lsrc, c->prio_cut, c->gbits, c->cbits,
-                                  c->prm.gain_priority, c->sb[0].k, c->sb[0].v, cnt + CNT_P, rep, exact, c->tmp, s);
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        static int if_env = -1;
-        if (if_env < 0) { const char *v = getenv("UPR_SORT_IF"); if_env = (v && *v == '0') ? 0 : 1; }
-        if (if_env) UPR_CUDA(cudaStreamIsCapturing(s, &cs));
-        if (cs == cudaStreamCaptureStatusActive && !c->s_if)
-            UPR_CUDA(cudaStreamCreateWithFlags(&c->s_if, cudaStreamNonBlocking));
-        int if_kernels = 0;
-        rebalance_fused_sort(c->sb[0].k, c->sb[0].v, c->sb[0].ka, c->sb[0].va, cnt + CNT_P, n, key_bits, c->gbits,
-                             c->cbits, exact, c->tmp, s, c->s_if, cnt + CNT_SORTP, &if_kernels);
-        if (cs == cudaStreamCaptureStatusActive) c->reb_if_kernels = if_kernels;
-        const uint32_t *U = c->sb[0].va;
-        rebalance_fused_select_admit(G, U, cnt + CNT_P, n, c->part, c->prop_tgt, c->C,
-                                     reinterpret_cast<int8_t *>(c->flags2), reinterpret_cast<long long *>(c->c_sorted),
-                                     reinterpret_cast<long long *>(c->c_excl), cnt + CNT_HIST, c->reject_d, ctl,
-                                     c->R_node, c->R_from, c->R_to, c->R_sub, c->r_to, c->r_at, c->Cd, cnt + CNT_A,
-                                     c->tmp, s);
-        table_move(G, c->W, c->R_node, c->R_from, c->R_to, cnt + CNT_A, &ctl->nR, nullptr, n, c->hub_chunks,
-                   c->n_chunks, HubMoves{nullptr, c->r_to, c->r_at, &ctl->nR, cnt + CNT_A, c->R_from, c->R_to}, s);
-        rebalance_fused_end(G, c->C, c->Cd, c->excl_d, c->reject_d, cnt + CNT_A, ctl, s, cond, c->prm.max_subrounds,
-                            merged ? c->over_d : nullptr, c->reject_d, cnt + CNT_L1);
-        return cond != 0;
-    }
-    select_values(c->flags, c->L1, c->L1, cnt + CNT_L1, Count{&ctl->n1_active, n}, c->tmp, s);
-    // proposals that cannot be in their source's minimal prefix are dropped
-    // before the ordering; P lists the others in node order
-    const int32_t *Pn = c->L1;
-    int32_t *dP = cnt + CNT_L1;
-    if (c->prio_hist) {
-        rebalance_prefilter(G, c->L1, cnt + CNT_L1, n, nullptr, c->prop_gain, c->part, c->over_d, c->C, c->gbits,
-                            c->cbits, c->prm.gain_priority, c->prio_hist, c->prio_cut, c->flags2, s);
-        select_values(c->flags2, c->L1, c->Pq, cnt + CNT_P, Count{cnt + CNT_L1, n}, c->tmp, s);
-        Pn = c->Pq;
-        dP = cnt + CNT_P;
-    }
-    const Count cP{dP, n};
-    uint64_t *kA; uint32_t *A;
-    if (key_bits <= 63) {
-        rebalance_prio_keys(G, Pn, dP, c->prop_gain, c->gbits, c->cbits, c->prm.gain_priority, c->sb[0].k,
-                            c->sb[0].v, n, s);
-        c->sb[0].run(cP, key_bits, c->tmp, s, &kA, &A);
-    } else {                // a 128-bit key: two stable sorts in sb[0]'s buffers
-        rebalance_prio_sort_wide(G, Pn, dP, c->prop_gain, c->gbits, c->cbits, c->prm.gain_priority,
-                                 SortPairs{c->sb[0].k, c->sb[0].ka, c->sb[0].v, c->sb[0].va}, n, c->tmp, s, &A);
-    }
-    // per source: the minimal prefix covering the excess
-    uint64_t *kB; uint32_t *B;
-    rebalance_block_keys(Pn, A, nullptr, dP, c->part, c->sb[1].k, c->sb[1].v, n, s);
-    c->sb[1].run(cP, kbits, c->tmp, s, &kB, &B);
-    rebalance_seg_weights(G, Pn, A, nullptr, B, kB, dP, c->c_sorted, c->seg_first, n, s);
-    exclusive_sum_i64(c->c_sorted, c->c_excl, cP, c->tmp, s);
-    rebalance_mark_selected(B, kB, dP, c->c_excl, c->seg_first, st, c->flags2, n, s);
-    select_flags(c->flags2, c->idxB, cnt + CNT_S, cP, c->tmp, s);
-    // per target: the longest prefix that fits
-    uint64_t *kT; uint32_t *Tq;
-    rebalance_block_keys(Pn, A, c->idxB, cnt + CNT_S, c->prop_tgt, c->sb[2].k, c->sb[2].v, n, s);
-    c->sb[2].run(cS, kbits, c->tmp, s, &kT, &Tq);
-    rebalance_seg_weights(G, Pn, A, c->idxB, Tq, kT, cnt + CNT_S, c->c_sorted, c->seg_first, n, s);
-    exclusive_sum_i64(c->c_sorted, c->c_excl, cS, c->tmp, s);
-    rebalance_mark_admitted(Tq, kT, cnt + CNT_S, c->c_sorted, c->c_excl, c->seg_first, st, c->flags2, c->reject_d,
-                            n, s);
-    select_flags(c->flags2, c->idxC, cnt + CNT_A, cS, c->tmp, s);
-    rebalance_apply(G, Pn, A, c->idxB, c->idxC, cnt + CNT_A, c->prop_tgt, c->part, c->C, ctl, c->R_node,
-                    c->R_from, c->R_to, c->R_sub, c->r_to, c->r_at, n, s);
-    table_move(G, c->W, c->R_node, c->R_from, c->R_to, cnt + CNT_A, &ctl->nR, nullptr, n, c->hub_chunks,
-               c->n_chunks, HubMoves{nullptr, c->r_to, c->r_at, &ctl->nR, cnt + CNT_A, c->R_from, c->R_to}, s);
-    rebalance_end(G, c->C, c->excl_d, c->reject_d, cnt + CNT_A, ctl, s);
-    return false;
+    RebalTeam m{};
+    m.team = c->team;
+    m.flags = c->flags;
+    m.list = c->L1;
+    m.lsrc = st.lsrc;
+    m.lgain = st.lgain;
+    m.d_n1 = &ctl->n1_active;
+    m.list2 = reinterpret_cast<int32_t *>(c->sb[2].k);
+    m.lsrc2 = m.list2 + n;
+    m.lgain2 = m.lsrc2 + n;
+    m.gbits = c->gbits;
+    m.cbits = c->cbits;
+    m.gain_only = c->prm.gain_priority;
+    m.hist = c->prio_hist;
+    m.rep = c->prio_rep;
+    m.cut = c->prio_cut;
+    m.exact = cnt + CNT_EXACT;
+    m.over = c->over_d;
+    m.C = c->C;
+    m.bufA = c->sb[0].k;            // (two neighbouring 16 n arrays each)
+    m.bufB = c->sb[1].k;
+    m.U = c->sb[2].v;
+    m.at = reinterpret_cast<int32_t *>(c->sb[2].va);
+    m.c_excl = c->c_excl;
+    m.seg_base = c->seg_base;
+    m.part = c->part;
+    m.prop_tgt = c->prop_tgt;
+    m.reject = c->reject_d;
+    m.ctl = ctl;
+    m.R_node = c->R_node; m.R_from = c->R_from; m.R_to = c->R_to; m.R_sub = c->R_sub;
+    m.r_to = c->r_to; m.r_at = c->r_at;
+    m.d_np = cnt + CNT_L1;
+    m.d_nk = cnt + CNT_P;
+    m.d_na = cnt + CNT_A;
+    rebalance_order(G, m, s);
+    table_move(G, c->W, c->R_node, c->R_from, c->R_to, cnt + CNT_A, &ctl->nR, nullptr, n, c->hub_chunks, c->n_chunks,
+               HubMoves{nullptr, c->r_to, c->r_at, &ctl->nR, cnt + CNT_A, c->R_from, c->R_to}, s);
+    rebalance_end(G, c->C, c->excl_d, c->reject_d, c->over_d, cnt + CNT_A, cnt + CNT_L1, c->prm.max_subrounds, ctl, s,
+                  cond);
+    return cond != 0 && c->ng == 1;
 }
 
-// The kernel before a graph-resident loop: the fused form begins the first
-// sub-round there (setting the condition), the general form only sets the
-// condition (its body begins each sub-round itself).
-void loop_head(upr_ctx *c, int32_t *light, cudaGraphConditionalHandle cond, cudaStream_t s) {
-    if (fused_rebalance(c, 1 + c->gbits + 2 * c->cbits))
-        rebalance_begin(c->G, c->C, c->excl_d, c->over_d, c->reject_d, c->counts + CNT_L1, c->prm.max_subrounds,
-                        c->ctl, light, s, cond);
-    else
-        rebalance_continue(c->ctl, c->prm.max_subrounds, cond, s);
+// The kernel before the loop: a batch's first list (and, graph-resident, the
+// loop's condition, since its body begins each sub-round itself); one graph's
+// first list and the first sub-round's begin, with the condition.
+void loop_head(upr_ctx *c, cudaGraphConditionalHandle cond, cudaStream_t s) {
+    RebalStart a{};
+    a.team = c->team;
+    a.part = c->part;
+    a.C = c->C;
+    a.list = c->L1;
+    a.d_list = c->counts + CNT_L1;
+    a.excl = c->excl_d; a.over = c->over_d; a.reject = c->reject_d;
+    a.max_subrounds = c->prm.max_subrounds;
+    a.ctl = c->ctl;
+    a.cond = cond;
+    if (c->ng > 1) rebalance_init_batch(c->G, c->C, c->excl_d, c->ctl, s);
+    rebalance_start(c->G, a, s);
+    if (c->ng > 1 && cond) rebalance_continue(c->ctl, c->prm.max_subrounds, cond, s);
 }
 
 // The rebalancing loop as a graph: a kernel sets the condition of a while
@@ -791,13 +661,15 @@ bool rebalance_graph(upr_ctx *c, const RebalState &st, int32_t *light) {
         UPR_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 0, 0));
         UPR_CUDA(cudaStreamBeginCaptureToGraph(c->s_cap, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
         capturing = true;
-        loop_head(c, light, cond, c->s_cap);
-        captured++;
+        const long long h0 = g_upr_launches;
+        loop_head(c, cond, c->s_cap);
+        c->reb_head_kernels = (int)(g_upr_launches - h0);
+        captured += c->reb_head_kernels;
         cudaGraph_t out = nullptr;
         capturing = false;
         UPR_CUDA(cudaStreamEndCapture(c->s_cap, &out));
-        cudaGraphNode_t head[1];
-        size_t n_head = 1;
+        cudaGraphNode_t head[8];       // (a batch: clear, init, list, condition)
+        size_t n_head = 8;
         UPR_CUDA(cudaGraphGetNodes(g, head, &n_head));
         cudaGraphNodeParams cp = {};
         cp.type = cudaGraphNodeTypeConditional;
@@ -846,22 +718,14 @@ void rebalance_phase(upr_ctx *c, int32_t r, RoundInfo &ri, TraceSink *tr) {
     const bool batch = c->ng > 1;
     int32_t *cnt = c->counts;
     RebalCtl *ctl = c->ctl;
-    const Count cN{nullptr, n};
-    if (c->prio_hist)
-        UPR_CUDA(cudaMemsetAsync(c->prio_hist, 0, sizeof(unsigned long long) * K * kPrioBins, s));
-    rebalance_init(G, c->C, c->excl_d, ctl, s);
-    rebalance_flag_in_blocks(c->part, n, c->excl_d, c->flags, s);
-    select_flags(c->flags, c->L1, cnt + CNT_L1, cN, c->tmp, s);
     int32_t *light = batch ? c->light_g : &ctl->light;
     RebalState st{c->C, c->over_d, c->excl_d, light, c->Lb};
     {
         const int kb = std::max(1, bit_length((uint64_t)(G.k - 1)));
         if (!batch && !G.vwgt && c->gbits + kb <= 31) st.pack_bits = kb;
     }
-    if (fused_rebalance(c, 1 + c->gbits + 2 * c->cbits)) {
-        st.lsrc = c->emit;          // list-indexed proposal blocks and gains (sequence-phase arrays, free here)
-        st.lgain = c->qbefore;
-    }
+    st.lsrc = c->emit;          // list-indexed proposal blocks and gains (sequence-phase arrays, free here)
+    st.lgain = c->qbefore;
     if (c->capturing) {
         // inside the step graph: the loop as a while node whose body is one
         // sub-round followed by the condition kernel (captured on a side
@@ -873,7 +737,7 @@ void rebalance_phase(upr_ctx *c, int32_t r, RoundInfo &ri, TraceSink *tr) {
         UPR_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, nullptr, nullptr, nullptr));
         cudaGraphConditionalHandle cond;
         UPR_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 0, 0));
-        loop_head(c, light, cond, s);
+        loop_head(c, cond, s);
         UPR_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
         cudaGraphNodeParams cp = {};
         cp.type = cudaGraphNodeTypeConditional;
@@ -905,7 +769,10 @@ void rebalance_phase(upr_ctx *c, int32_t r, RoundInfo &ri, TraceSink *tr) {
     if (c->prm.graphs && pays && !tuning && !tr && !log_enabled() && rebalance_graph(c, st, light)) {
         UPR_CUDA(cudaGraphLaunch(c->reb_exec, s));
         ri.graph = true;
-    } else for (int32_t h = 1; h <= c->prm.max_subrounds; h++) {
+        return;
+    }
+    loop_head(c, 0, s);
+    for (int32_t h = 1; h <= c->prm.max_subrounds; h++) {
         enqueue_subround(c, st, light, h == 1, s);
         UPR_CUDA(cudaMemcpyAsync(c->hctl, ctl, sizeof(RebalCtl), cudaMemcpyDeviceToHost, s));
         UPR_CUDA(cudaStreamSynchronize(s));
@@ -917,10 +784,8 @@ void rebalance_phase(upr_ctx *c, int32_t r, RoundInfo &ri, TraceSink *tr) {
             int32_t hc[CNT_SLOTS];
             UPR_CUDA(cudaMemcpy(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost));
             const auto t1 = std::chrono::steady_clock::now();
-            fprintf(stderr, "upr round %d sub-round %d: listed %d proposals %d kept %d selected %d "
-                            "admitted %d (%.3f ms)\n",
-                    r, h, c->hctl->n1_active, hc[CNT_L1], c->prio_hist ? hc[CNT_P] : hc[CNT_L1], hc[CNT_S],
-                    hc[CNT_A],
+            fprintf(stderr, "upr round %d sub-round %d: proposals %d kept %d admitted %d (%.3f ms)\n",
+                    r, h, hc[CNT_L1], hc[CNT_P], hc[CNT_A],
                     std::chrono::duration<double, std::milli>(t1 - t_sub).count());
             t_sub = std::chrono::steady_clock::now();
         }
@@ -1100,7 +965,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
                    c->tile_nodes, c->scal + 2, s);
     }
     if (cap) {                  // the step graph: the round's counts go to the device sums
-        k_round_stats<<<1, 32, 0, s>>>(cnt, ctl, c->best, c->tot, batch ? 1 : 0, c->tmp.err, c->dstats);
+        k_round_stats<<<1, 32, 0, s>>>(cnt, ctl, c->best, c->tot, batch ? 1 : 0, c->team.err, c->dstats);
         UPR_LAUNCH_CHECK();
         c->table_valid = true;
         return UPR_OK;
@@ -1110,14 +975,14 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     UPR_CUDA(cudaMemcpyAsync(c->hctl, ctl, sizeof(RebalCtl), cudaMemcpyDeviceToHost, s));
     if (!batch) UPR_CUDA(cudaMemcpyAsync(c->hbest, c->best, sizeof(long long) * 2, cudaMemcpyDeviceToHost, s));
     else UPR_CUDA(cudaMemcpyAsync(c->hbest, c->tot, sizeof(long long) * 3, cudaMemcpyDeviceToHost, s));
-    UPR_CUDA(cudaMemcpyAsync(c->hcnt + 40, c->tmp.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    UPR_CUDA(cudaMemcpyAsync(c->hcnt + 40, c->team.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     UPR_CUDA(cudaStreamSynchronize(s));
     if (c->sel_pending) {
         settle_tuning(&c->sel_cfg, &c->sel_tuned, &c->sel_pending, c->sel_cands, c->ev_tune, 0.05f);
         if (c->sel_tuned) remember_tuning(c, 0, c->sel_cfg);
     }
-    // a bounded wait of a primitive gave up: the round's lists are not trustworthy
-    if (c->hcnt[40] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "primitive wait"}; }
+    // a bounded wait of a barrier gave up: the round's lists are not trustworthy
+    if (c->hcnt[40] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "barrier wait"}; }
     {
         float a = 0, b = 0, d = 0, t = 0;
         UPR_CUDA(cudaEventElapsedTime(&t, c->ev[0], c->ev[1]));
@@ -1133,8 +998,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     ri.n_rebal = c->hctl->nR;
     ri.subrounds = c->hctl->subrounds;
     if (ri.graph)
-        g_upr_launches += (1 + (long long)c->reb_body_kernels * ri.subrounds +
-                           (long long)c->reb_if_kernels * hc[CNT_SORTP]);
+        g_upr_launches += (c->reb_head_kernels + (long long)c->reb_body_kernels * ri.subrounds);
     ri.n_inter = hc[CNT_X];
     ri.n_seq = hc[CNT_I];
     // one graph: an infeasible round applies nothing and is an error; a
@@ -1239,7 +1103,6 @@ void free_ctx(upr_ctx *c) {
     if (c->step_exec) cudaGraphExecDestroy(c->step_exec);
     if (c->s_cap) cudaStreamDestroy(c->s_cap);
     if (c->s_body) cudaStreamDestroy(c->s_body);
-    if (c->s_if) cudaStreamDestroy(c->s_if);
     if (c->xs) cudaFree(c->xs);
     if (c->segs_d) cudaFree(c->segs_d);
     if (c->s_up) cudaStreamDestroy(c->s_up);
@@ -1350,7 +1213,6 @@ int lp_round_once(upr_ctx *c, int64_t *cut, int64_t *active_next, RoundInfo &ri)
     const int32_t K = G.K();
     int32_t *cnt = c->counts;
     RebalCtl *ctl = c->ctl;
-    const Count cN{nullptr, n};
     UPR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * CNT_SLOTS, s));
     UPR_CUDA(cudaMemcpyAsync(c->part, c->part0, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
     UPR_CUDA(cudaMemcpyAsync(c->C, c->C0, sizeof(int64_t) * K, cudaMemcpyDeviceToDevice, s));
@@ -1369,8 +1231,7 @@ int lp_round_once(upr_ctx *c, int64_t *cut, int64_t *active_next, RoundInfo &ri)
     Penalty pen{c->PW, c->F, c->C0, c->Lsel, c->first_slot};
     set_pack(c, pen);
     select_moves(G, c->part0, c->W, pen, c->cand_tgt, c->cand_s0, c->cand_gain, c->flags, c->sel_cfg, s);
-    lp_filter(c->flags, c->lp_active, n, s);
-    select_flags(c->flags, c->idxA, cnt + CNT_M, cN, c->tmp, s);
+    lp_list(LpList{c->team, c->flags, c->lp_active, n, c->idxA, cnt + CNT_M}, s);
     lp_apply(G, c->idxA, cnt + CNT_M, c->cand_tgt, c->cand_gain, c->part0, c->part, c->C, c->M_node, c->M_from,
              c->M_to, c->M_score, c->m_pos, c->scal + 1, n, s);
     table_move(G, c->W, c->M_node, c->M_from, c->M_to, cnt + CNT_M, nullptr, c->scal + 1, n, c->hub_chunks,
@@ -1423,10 +1284,10 @@ int lp_round_once(upr_ctx *c, int64_t *cut, int64_t *active_next, RoundInfo &ri)
     }
     reset_nodes(c->M_node, dM, n, c->m_pos, -1, s);
     reset_nodes(c->R_node, dR, n, c->r_to, -1, s);
-    UPR_CUDA(cudaMemcpyAsync(c->hcnt + 40, c->tmp.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    UPR_CUDA(cudaMemcpyAsync(c->hcnt + 40, c->team.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     UPR_CUDA(cudaMemcpyAsync(c->hcnt + CNT_L1, cnt + CNT_L1, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     UPR_CUDA(cudaStreamSynchronize(s));
-    if (c->hcnt[40] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "primitive wait"}; }
+    if (c->hcnt[40] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "barrier wait"}; }
     *active_next = kept ? c->hcnt[CNT_L1] : 0;
     return kept ? 1 : 0;
 }
@@ -1592,7 +1453,7 @@ bool run_step_graph(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
     long long d[16];
     UPR_CUDA(cudaMemcpyAsync(d, c->dstats, sizeof(d), cudaMemcpyDeviceToHost, s));
     UPR_CUDA(cudaStreamSynchronize(s));
-    if (d[6] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "primitive wait"}; }
+    if (d[6] != 0) { c->table_valid = false; throw CudaError{cudaErrorLaunchTimeout, "barrier wait"}; }
     if (d[7] != 0) { c->table_valid = false; throw CudaError{cudaErrorInvalidValue, "step graph: infeasible round"}; }
     st.rounds_run += rounds;
     st.n_candidates += d[0];
@@ -1602,7 +1463,7 @@ bool run_step_graph(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
     st.n_sequence += d[4];
     st.n_applied += d[5];
     st.rebalance_graphs += rounds;
-    g_upr_launches += (c->step_kernels + (long long)c->reb_body_kernels * d[3] + (long long)c->reb_if_kernels * d[9]);
+    g_upr_launches += (c->step_kernels + (long long)c->reb_body_kernels * d[3]);
     return true;
 }
 
@@ -2184,14 +2045,12 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     c->gbits = std::max(1, bit_length((uint64_t)c->wmax));
     // the arena may hold another binding's data: clear every word a kernel
     // reads before writing it
-    UPR_CUDA(cudaMemsetAsync(c->tmp.ticket, 0, 64 * sizeof(unsigned int), s));
-    UPR_CUDA(cudaMemsetAsync(c->tmp.mem, 0, c->tmp.mem_bytes, s));
-    UPR_CUDA(cudaMemsetAsync(c->tmp.scan, 0, c->tmp.scan_bytes, s));
-    UPR_CUDA(cudaMemsetAsync(c->tmp.err, 0, sizeof(int32_t), s));
-    UPR_CUDA(cudaMemsetAsync(c->tmp.epoch, 0, sizeof(uint32_t), s));
+    UPR_CUDA(cudaMemsetAsync(c->team.bar, 0, sizeof(unsigned long long), s));
+    UPR_CUDA(cudaMemsetAsync(c->team.err, 0, sizeof(int32_t), s));
+    if (c->prio_hist)
+        UPR_CUDA(cudaMemsetAsync(c->prio_hist, 0, sizeof(unsigned long long) * (size_t)c->G.K() * kPrioBins, s));
     UPR_CUDA(cudaMemsetAsync(c->ctl, 0, sizeof(RebalCtl), s));
     UPR_CUDA(cudaMemsetAsync(c->counts, 0, 64 * sizeof(int32_t), s));
-    UPR_CUDA(cudaMemsetAsync(c->Cd, 0, sizeof(long long) * (size_t)c->G.K(), s));
     fill_i32(c->m_pos, n, -1, s);
     fill_i32(c->r_to, n, -1, s);
     UPR_CUDA(cudaStreamSynchronize(s));

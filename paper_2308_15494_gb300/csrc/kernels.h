@@ -112,36 +112,15 @@ __device__ __forceinline__ int32_t blk_graph(const GraphDev &g, int32_t p) { ret
 __device__ __forceinline__ int64_t node_c(const GraphDev &g, int64_t v) { return g.vwgt ? (int64_t)g.vwgt[v] : 1; }
 __device__ __forceinline__ int32_t edge_w(const GraphDev &g, int64_t e) { return g.adjw ? g.adjw[e] : 1; }
 
-// An element count that may live in device memory: d (nullable) holds the
-// actual count, max is a static upper bound used to size grids and buffers.
-struct Count {
-    const int32_t *d;
-    int64_t max;
-};
-inline Count fixed(int64_t n) { return Count{nullptr, n}; }
-
-// Scratch memory of the primitives: status words and partial results, tile
-// and ticket counters (zero between calls: the last CTA of a call resets
-// them), the call counter whose value tags status words (host memory,
-// advanced at every call; calls on one scratch are serialised by their
-// stream) and an error word set when a bounded wait gives up.
-struct Scratch {
-    char *mem;              // radix status and digit counts (radix_temp_bytes(tiles_cap * 2048))
-    char *scan;             // scan / compaction status (scan_temp_bytes(tiles_cap * 2048)); never overlaps mem
-    size_t mem_bytes, scan_bytes;
-    int64_t tiles_cap;      // tiles of the longest list; fixes the layout of both regions
-    unsigned int *ticket;   // [0] next tile, [1] finished CTAs, [2] radix count ticket
-    uint32_t *epoch;        // device word: the primitives' last call tag
-    int32_t *err;
-};
-
 // What a team launch needs (team.cuh): the grid barrier's arrival counter, the
-// error word, per-CTA digit totals [size][256] and per-CTA scan totals, and
-// the number of CTAs (one per binding, since the counter counts by it).
+// error word (set when a bounded wait gives up), per-CTA digit totals
+// [size][256], block-weight totals [2][size][256] and scan totals, and the
+// number of CTAs (one per binding, since the counter counts by it).
 struct Team {
     unsigned long long *bar = nullptr;
     int32_t *err = nullptr;
     int32_t *hist = nullptr;
+    unsigned long long *hist64 = nullptr;
     long long *tot = nullptr;
     int size = 1;
 };
@@ -155,21 +134,6 @@ inline unsigned grid_for(int64_t max) {
     const int64_t b = ceil_div(max > 0 ? max : 1, 256);
     return (unsigned)std::min<int64_t>(b, (int64_t)device_sm_count() * 8);
 }
-
-// ---- prim.cu
-size_t scan_temp_bytes(int64_t n);
-size_t radix_temp_bytes(int64_t n);
-void exclusive_sum_i32(const int32_t *in, int32_t *out, Count n, Scratch tmp, cudaStream_t s);
-void exclusive_sum_i64(const int64_t *in, int64_t *out, Count n, Scratch tmp, cudaStream_t s);
-// Stable LSD sort on key bits [0, bits); returns true if the result is in the *_alt buffers
-// (a property of `bits` alone, known when the launches are enqueued).
-bool radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, Count n, int bits,
-                      Scratch tmp, cudaStream_t s);
-// out_idx[0..*d_count) = indices i < n with flags[i] != 0, ascending.
-void select_flags(const int32_t *flags, int32_t *out_idx, int32_t *d_count, Count n, Scratch tmp, cudaStream_t s);
-// out[j] = vals[i] for the j-th i with flags[i] != 0 (index order); out may be vals.
-void select_values(const int32_t *flags, const int32_t *vals, int32_t *out, int32_t *d_count, Count n, Scratch tmp,
-                   cudaStream_t s);
 
 // ---- graph.cu: step (e), step (a), create-time work
 struct HubChunk { int32_t v; int32_t pad; int64_t begin, end; };
@@ -328,17 +292,14 @@ struct RebalState {
     const int8_t *excl;   // [K] not a target: overloaded at the first sub-round, or rejected a move
     const int32_t *light; // [ng] lightest non-excluded block of each graph, or -1
     const int64_t *Lb;    // [K] L_max of each block's graph
-    // optional (null: not written): per listed node i with a proposal, its
-    // block and gain by list index, so that later passes over the list read
-    // them in order instead of gathering them by node
+    // per listed node i with a proposal, its block and gain by list index, so
+    // that later passes over the list read them in order
     int32_t *lsrc = nullptr, *lgain = nullptr;
     // > 0 (unit node weights, one graph, 1 + gb + pack_bits <= 32): the dense
     // proposal kernel scores a column as one integer, (omega << pack_bits) +
     // (2^pack_bits - 1 - b), pack_bits = the bits of a column index
     int pack_bits = 0;
 };
-// flags[v] = 1 for the nodes of the marked blocks
-void rebalance_flag_in_blocks(const int32_t *part, int64_t n, const int8_t *mark, int32_t *flags, cudaStream_t s);
 // Proposals of the listed nodes in overloaded blocks: prop_tgt/prop_gain by node, flags by list position.
 void rebalance_propose_scalar_list(const GraphDev &g, const int32_t *list, const int32_t *d_n1, int64_t n1_max,
                                    const int32_t *part, const int32_t *W, RebalState st, int32_t *prop_tgt,
@@ -346,24 +307,74 @@ void rebalance_propose_scalar_list(const GraphDev &g, const int32_t *list, const
 void rebalance_propose_list(const GraphDev &g, const int32_t *list, const int32_t *d_n1, int64_t n1_max,
                             const int32_t *part, const int32_t *W, RebalState st, int32_t *prop_tgt,
                             int32_t *prop_gain, int32_t *flags, LaneCfg cfg, cudaStream_t s);
-// Proposal prefilter (exact): a source's proposals in the priority bins after
-// the one where its cumulative weight reaches the excess can never be in its
-// minimal prefix.  keep[i] = 1 for listed node i (list/d_n1; flags from the
-// proposal kernel, or null when every listed node proposes) when it proposes
-// and is not in such a bin.  hist (K * kPrioBins, zero on entry) is left zero.
 constexpr int kPrioBins = 256;
-void rebalance_prefilter(const GraphDev &g, const int32_t *list, const int32_t *d_n1, int64_t n1_max,
-                         const int32_t *flags, const int32_t *prop_gain, const int32_t *part, const int8_t *over,
-                         const int64_t *C, int gbits, int cbits, int gain_only, unsigned long long *hist,
-                         int32_t *cut, int32_t *keep, cudaStream_t s);
-// The four buffers of a two-array radix sort (keys and values, and their alternates).
-struct SortPairs { uint64_t *k, *ka; uint32_t *v, *va; };
-// A priority key wider than 63 bits (1 + gbits + 2 cbits > 63): the proposals
-// P[0..*d_np) ordered by their 128-bit keys, two stable sorts (low word, then
-// high word); *order receives the buffer holding the order (indices into P).
-void rebalance_prio_sort_wide(const GraphDev &g, const int32_t *P, const int32_t *d_np, const int32_t *prop_gain,
-                              int gbits, int cbits, int gain_only, SortPairs sp, int64_t np_max, Scratch tmp,
-                              cudaStream_t s, uint32_t **order);
+// The first list: the nodes of the overloaded blocks, in node order.  One
+// graph: also the excluded set, the control block and the first sub-round's
+// begin (cond: the condition of a graph-resident loop).
+struct RebalStart {
+    Team team;
+    const int32_t *part;
+    const int64_t *C;
+    int32_t *list, *d_list;
+    int8_t *excl, *over, *reject;
+    int32_t max_subrounds;
+    RebalCtl *ctl;
+    cudaGraphConditionalHandle cond;
+    // set by rebalance_start
+    int64_t n = 0;
+    int K = 0, batch = 0;
+    const int64_t *Lb = nullptr;
+};
+void rebalance_start(const GraphDev &g, RebalStart a, cudaStream_t s);
+// A sub-round after its proposals: the proposers (flags by list index, their
+// blocks and gains in lsrc / lgain) become the list, the minimal prefix per
+// source and the longest fitting prefix per target in priority order are
+// appended to R at ctl->nR (*d_na of them) and applied to part and C.
+// Proposal prefilter (exact; hist null: none): a source's proposals in the
+// priority bins after the one where its cumulative weight reaches the excess
+// can never be in its minimal prefix.  hist (K * kPrioBins, zero) is left zero.
+// bufA, bufB: 32 n bytes each.
+struct RebalTeam {
+    Team team;
+    const int32_t *flags;
+    int32_t *list;
+    const int32_t *lsrc, *lgain, *d_n1;
+    int32_t *list2, *lsrc2, *lgain2;         // [n] scratch
+    int gbits, cbits, gain_only;             // gain_only: the priority is the gain alone (Sec. 7.2), else Sec. 6.1's
+    unsigned long long *hist, *rep;          // prefilter weights; [kPrioBins] a key per bin
+    int32_t *cut, *exact;                    // [K] cut bin per source; every bin holds one key value
+    const int8_t *over;
+    int64_t *C;
+    void *bufA, *bufB;
+    uint32_t *U;                             // [n] the kept proposals in priority order
+    int32_t *at;                             // [n] their targets while selected, then while admitted
+    int64_t *c_excl, *seg_base;              // [n], [K] scratch (K > 256)
+    int32_t *part;
+    const int32_t *prop_tgt;
+    int8_t *reject;
+    const RebalCtl *ctl;
+    int32_t *R_node, *R_from, *R_to, *R_sub, *r_to, *r_at;
+    int32_t *d_np, *d_nk, *d_na;             // proposers, kept, admitted
+    // set by rebalance_order
+    int K = 0, kbits = 0;
+    const int32_t *vwgt = nullptr;
+    const int64_t *Lb = nullptr;
+};
+void rebalance_order(const GraphDev &g, RebalTeam a, cudaStream_t s);
+// Loop control of a batch: the excluded set and the control block; a
+// sub-round's begin (light: each graph's lightest non-excluded block).
+void rebalance_init_batch(const GraphDev &g, const int64_t *C, int8_t *excl, RebalCtl *ctl, cudaStream_t s);
+void rebalance_begin_batch(const GraphDev &g, const int64_t *C, const int8_t *excl, int8_t *over, int8_t *reject,
+                           const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, int32_t *light, cudaStream_t s);
+// Sets the condition of a graph's while node: another sub-round is due.
+void rebalance_continue(const RebalCtl *ctl, int32_t max_subrounds, cudaGraphConditionalHandle handle,
+                        cudaStream_t s);
+// A sub-round's end; one graph: the next one begins in the same kernel (over,
+// d_n1, and cond as rebalance_start's).
+void rebalance_end(const GraphDev &g, const int64_t *C, int8_t *excl, int8_t *reject, int8_t *over,
+                   const int32_t *d_na, const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, cudaStream_t s,
+                   cudaGraphConditionalHandle cond = 0);
+
 // ---- mixed.cu: one context over batches of different k (one batch per k)
 struct MixedBatch;
 upr_status mixed_create(const upr_graph *graphs, int32_t n_graphs, const int32_t *k, const double *eps,
@@ -383,128 +394,6 @@ upr_status mixed_refine(MixedBatch *mb, int32_t *part, int32_t rounds, uint64_t 
                         int64_t *cut_in, int64_t *cut_out, upr_stats *stats);
 upr_status mixed_cut(MixedBatch *mb, const int32_t *part, int64_t *cut, int64_t *block_weights);
 upr_status mixed_info(const MixedBatch *mb, int32_t *n_graphs, int64_t *node_offsets, int64_t *lmax);
-
-// ---- reb_fused.cu: one rebalancing sub-round in fused passes (one graph,
-// K <= 256, a key of at most 63 bits, the prefilter on); same results as the
-// general form.  K * ceil(n / 2048) must not exceed the histogram buffers.
-bool rebalance_fused_ok(const GraphDev &g, int key_bits, bool prefilter);
-// list[0..*d_out) = the listed nodes with flags set (in place, in order), and
-// the prefilter's (source, bin) weights added to hist
-// (rep: [kPrioBins] one key per bin; *exact set to 1 for k_fr_keep_keys to clear)
-// (lgain, lsrc: the proposals' gains and blocks by list index, compacted with the list)
-void rebalance_fused_compact_hist(const GraphDev &g, const int32_t *flags, int32_t *list, const int32_t *d_n,
-                                  int64_t n_max, int32_t *d_out, int32_t *lgain, int32_t *lsrc, int gbits, int cbits,
-                                  int gain_only, unsigned long long *hist, uint64_t *rep, int32_t *exact, Scratch tmp,
-                                  cudaStream_t s);
-// (keys, vals)[0..*d_out) = (priority key, node) of the proposals whose bin is
-// not after their source's cut; *exact cleared when a kept key differs from its bin's rep
-void rebalance_fused_keep_keys(const GraphDev &g, const int32_t *list, const int32_t *d_n, int64_t n_max,
-                               const int32_t *lgain, const int32_t *lsrc, const int32_t *cut, int gbits, int cbits,
-                               int gain_only, uint64_t *keys, uint32_t *vals, int32_t *d_out, const uint64_t *rep,
-                               int32_t *exact, Scratch tmp, cudaStream_t s);
-// Steps 1 and 3-7 of the fused sub-round (compaction with the prefilter
-// histogram, cut bins, kept keys, the sort, selection, admission and the
-// moves) in one cooperative launch with grid barriers: the same results as
-// the separate fused kernels.  The wrapper sets the fields after `exact`.
-struct RebalMega {
-    const int32_t *flags;                    // [n1] proposer flags by list index
-    int32_t *list, *lsrc, *lgain;            // [n1] the list (becomes the proposers), their blocks and gains
-    const int32_t *d_n1;                     // n1
-    int32_t *list2, *lsrc2, *lgain2;         // [n] the compacted proposers, their blocks and gains
-    int gbits, cbits, gain_only;
-    unsigned long long *hist;                // [K * kPrioBins] prefilter weights (rows of overloaded sources cleared)
-    uint64_t *rep;                           // [kPrioBins] some proposal's key per bin
-    int32_t *cut;                            // [K] cut bin per source
-    const int8_t *over;
-    const int64_t *C;
-    uint64_t *keys, *keys_alt;               // [n] kept keys; the sorted keys
-    uint32_t *vals, *vals_alt;               // [n] kept nodes; the sorted nodes
-    int32_t *part;
-    const int32_t *prop_tgt;
-    int8_t *sel;                             // [n] per sorted proposal: 1 selected, 2 admitted
-    long long *h0, *h1;                      // [K * tiles] per-(block, tile) weights and their row prefixes
-    int8_t *reject;
-    const RebalCtl *ctl;
-    int32_t *R_node, *R_from, *R_to, *R_sub, *r_to, *r_at;
-    long long *Cd;
-    int32_t *d_np, *d_nk, *d_na;             // proposers, kept, admitted
-    int32_t *exact;
-    // set by rebalance_fused_mega
-    const int32_t *vwgt = nullptr;
-    const int64_t *Lb = nullptr;
-    int K = 0, passes = 0, vec = 0;
-    int32_t *tab = nullptr;                  // tile counts 3 x [tcap], digit totals [256], digit counts [256 * tcap]
-    int64_t tcap = 0;
-    unsigned long long *bar = nullptr;       // the grid barrier's arrival counter
-    int32_t *err = nullptr;
-};
-void rebalance_fused_mega(const GraphDev &g, RebalMega m, int key_bits, int64_t n_max, Scratch tmp, cudaStream_t s);
-// Stable sort of (keys, vals)[0..*d_n) by key (key_bits, an odd number of
-// 8-bit passes), or by the key's prefilter bin alone when *exact; the result
-// is in the alternate buffers (returns true).  While s is being captured and
-// s_aux and later_runs are given, the passes after the first are captured on
-// s_aux as the body of a conditional node that runs only when they sort
-// anything; each run adds 1 to *later_runs, and *later_kernels = the body's
-// kernels (0 when no such node was made).
-bool rebalance_fused_sort(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, const int32_t *d_n,
-                          int64_t n_max, int key_bits, int gbits, int cbits, const int32_t *exact, Scratch tmp,
-                          cudaStream_t s, cudaStream_t s_aux = nullptr, int32_t *later_runs = nullptr,
-                          int *later_kernels = nullptr);
-// U[0..*d_np): proposals (nodes) in priority order.  Minimal prefix per
-// source, longest fitting prefix per target, the admitted appended to R at
-// ctl->nR (count *d_na), part / r_to / r_at updated, block-weight changes
-// added to Cd; sel (np int8) and the two histograms (K * ceil(np / 2048)
-// int64 each) are scratch.
-void rebalance_fused_select_admit(const GraphDev &g, const uint32_t *U, const int32_t *d_np, int64_t np_max,
-                                  int32_t *part, const int32_t *prop_tgt, const int64_t *C, int8_t *sel,
-                                  long long *h0, long long *h1, int32_t *d_hist_n, int8_t *reject,
-                                  const RebalCtl *ctl, int32_t *R_node, int32_t *R_from, int32_t *R_to,
-                                  int32_t *R_sub, int32_t *r_to, int32_t *r_at, long long *Cd, int32_t *d_na,
-                                  Scratch tmp, cudaStream_t s);
-// C += Cd, Cd = 0; then k_reb_end's update of the excluded set and the stop
-// flag; with cond (a graph-resident loop) also the loop's condition, as
-// rebalance_continue sets it.  With begin_next (over, reject and d_n1
-// given) the next sub-round's begin follows in the same kernel (as
-// rebalance_begin) and the condition is "that sub-round runs".
-void rebalance_fused_end(const GraphDev &g, int64_t *C, long long *Cd, int8_t *excl, const int8_t *reject,
-                         const int32_t *d_na, RebalCtl *ctl, cudaStream_t s, cudaGraphConditionalHandle cond = 0,
-                         int32_t max_subrounds = 0, int8_t *over = nullptr, int8_t *reject_next = nullptr,
-                         const int32_t *d_n1 = nullptr);
-// The prefilter's cut bin of every overloaded source (hist rows read are cleared).
-void rebalance_prio_cut(const GraphDev &g, const int8_t *over, const int64_t *C, unsigned long long *hist, int32_t *cut,
-                        cudaStream_t s);
-// gain_only: the priority is the gain alone (a variant of Sec. 7.2), else g/c
-// for g < 0 and g*c for g >= 0 (Sec. 6.1)
-void rebalance_prio_keys(const GraphDev &g, const int32_t *P, const int32_t *d_np, const int32_t *prop_gain,
-                         int gbits, int cbits, int gain_only, uint64_t *keys, uint32_t *vals, int64_t np_max,
-                         cudaStream_t s);
-void rebalance_block_keys(const int32_t *P, const uint32_t *A, const int32_t *S, const int32_t *d_cnt,
-                          const int32_t *blk_of_node, uint64_t *keys, uint32_t *vals, int64_t cnt_max, cudaStream_t s);
-void rebalance_seg_weights(const GraphDev &g, const int32_t *P, const uint32_t *A, const int32_t *S,
-                           const uint32_t *B, const uint64_t *bkeys, const int32_t *d_cnt, int64_t *c_sorted,
-                           int32_t *seg_first, int64_t cnt_max, cudaStream_t s);
-void rebalance_mark_selected(const uint32_t *B, const uint64_t *bkeys, const int32_t *d_cnt, const int64_t *c_excl,
-                             const int32_t *seg_first, RebalState st, int32_t *sel, int64_t cnt_max, cudaStream_t s);
-void rebalance_mark_admitted(const uint32_t *T, const uint64_t *bkeys, const int32_t *d_cnt, const int64_t *c_sorted,
-                             const int64_t *c_excl, const int32_t *seg_first, RebalState st, int32_t *adm,
-                             int8_t *reject, int64_t cnt_max, cudaStream_t s);
-void rebalance_apply(const GraphDev &g, const int32_t *P, const uint32_t *A, const int32_t *S, const int32_t *Adm,
-                     const int32_t *d_na, const int32_t *prop_tgt, int32_t *part, int64_t *C, const RebalCtl *ctl,
-                     int32_t *R_node, int32_t *R_from, int32_t *R_to, int32_t *R_sub, int32_t *r_to, int32_t *r_at,
-                     int64_t na_max, cudaStream_t s);
-// Loop control over the K blocks of g (C = current block weights).  light
-// receives each graph's lightest non-excluded block (&ctl->light for one graph).
-void rebalance_init(const GraphDev &g, const int64_t *C, int8_t *excl, RebalCtl *ctl, cudaStream_t s);
-// cond (one graph, a graph-resident loop whose body does not begin with this
-// kernel): also sets the loop's condition to "this sub-round runs"
-void rebalance_begin(const GraphDev &g, const int64_t *C, const int8_t *excl, int8_t *over, int8_t *reject,
-                     const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, int32_t *light, cudaStream_t s,
-                     cudaGraphConditionalHandle cond = 0);
-// Sets the condition of a graph's while node: another sub-round is due.
-void rebalance_continue(const RebalCtl *ctl, int32_t max_subrounds, cudaGraphConditionalHandle handle,
-                        cudaStream_t s);
-void rebalance_end(const GraphDev &g, const int64_t *C, int8_t *excl, const int8_t *reject, const int32_t *d_na,
-                   RebalCtl *ctl, cudaStream_t s);
 
 // ---- sequence.cu: step (c); every count lives in device memory, `max` bounds it
 void fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t s);
@@ -606,8 +495,15 @@ void seq_apply_prefix_seg(const GraphDev &g, const int32_t *I_node, const int32_
 // ---- lp.cu: unconstrained label propagation (Sec. 5)
 // active[v] = 1 for the boundary nodes of part (table W of part)
 void lp_boundary(const GraphDev &g, const int32_t *part, const int32_t *W, int8_t *active, cudaStream_t s);
-// flags[v] = 0 where active[v] = 0
-void lp_filter(int32_t *flags, const int8_t *active, int64_t n, cudaStream_t s);
+// list[0..*d_cnt) = the active nodes with a set flag, in node order
+struct LpList {
+    Team team;
+    const int32_t *flags;
+    const int8_t *active;
+    int64_t n;
+    int32_t *list, *d_cnt;
+};
+void lp_list(const LpList &a, cudaStream_t s);
 // the listed movers (d_cnt of them, node order) to cand_tgt: part (a copy of
 // part0), C, the move list, m_pos markers and the movers' degree sum
 void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, const int32_t *cand_tgt,

@@ -1,7 +1,7 @@
 // Unconstrained label propagation (Sec. 5): the kernels of one round that the
 // FM round does not already have.  The round itself (selection without a
 // penalty, rebalancing, the net-improvement check) is driven from engine.cu.
-#include "kernels.h"
+#include "team.cuh"
 
 namespace upr {
 namespace {
@@ -17,9 +17,25 @@ __global__ void k_lp_boundary(const GraphDev g, const int32_t *__restrict__ part
     }
 }
 
-// a node outside V_a does not move
-__global__ void k_lp_filter(int32_t *__restrict__ flags, const int8_t *__restrict__ active, int64_t n) {
-    UPR_FOR(v, n) if (flags[v] && !active[v]) flags[v] = 0;
+// The movers, in node order: candidates in V_a.
+__global__ void __launch_bounds__(team::kTT, 1) k_lp_list(const LpList a) {
+    __shared__ team::Smem s;
+    const int lane = threadIdx.x & 31;
+    const team::Seg g = team::warp_seg(a.n);
+    long long cnt = 0;
+    for (int64_t v = g.b + lane; v < g.e; v += 32) cnt += a.flags[v] && a.active[v];
+    const long long mine = team::publish<team::Sum>(a.team, s, 0, team::warp_all<team::Sum>(cnt));
+    team::sync(a.team);
+    long long all;
+    int64_t pos = team::collect<team::Sum>(a.team, 0, &all) + mine;
+    for (int64_t v0 = g.b; v0 < g.e; v0 += 32) {
+        const int64_t v = v0 + lane;
+        const bool f = v < g.e && a.flags[v] && a.active[v];
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (f) a.list[pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
+        pos += __popc(m);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_cnt = (int32_t)all;
 }
 
 // All moves at once: the listed nodes (node order) to their targets; the move
@@ -197,11 +213,7 @@ void lp_boundary(const GraphDev &g, const int32_t *part, const int32_t *W, int8_
     UPR_LAUNCH_CHECK();
 }
 
-void lp_filter(int32_t *flags, const int8_t *active, int64_t n, cudaStream_t s) {
-    if (n == 0) return;
-    k_lp_filter<<<grid_for(n), 256, 0, s>>>(flags, active, n);
-    UPR_LAUNCH_CHECK();
-}
+void lp_list(const LpList &a, cudaStream_t s) { launch_team(k_lp_list, a, a.team.size, s); }
 
 void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, const int32_t *cand_tgt,
               const int32_t *cand_gain, const int32_t *part0, int32_t *part, int64_t *C, int32_t *M_node,

@@ -8,7 +8,9 @@
 // the host or as one CUDA graph whose condition k_reb_continue sets.
 #include <cstddef>
 
-#include "kernels.h"
+#include <type_traits>
+
+#include "team.cuh"
 
 namespace upr {
 namespace {
@@ -260,40 +262,9 @@ __global__ void __launch_bounds__(256) k_propose_sparse(const GraphDev g, const 
     }
 }
 
-// list[i] = nodes of the blocks marked in `mark`
-__global__ void k_flag_in_blocks(const int32_t *__restrict__ part, int64_t n, const int8_t *__restrict__ mark,
-                                 int32_t *__restrict__ flags) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) flags[v] = mark[part[v]] ? 1 : 0;
-}
-
 // ---- loop control.  One graph: one CTA each (K = k <= 4096).  A batch: a
 // grid over the graphs, warp per graph; the last CTA to finish (ticket)
 // updates the control block.
-// Start of rebalancing: the blocks overloaded now are never targets.
-__global__ void k_reb_init(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb, int32_t K,
-                           int8_t *__restrict__ excl, RebalCtl *__restrict__ ctl) {
-    __shared__ int s_any;
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    for (int b = threadIdx.x; b < K; b += blockDim.x) {
-        const bool o = C[b] > Lb[b];
-        excl[b] = o ? 1 : 0;
-        if (o) s_any = 1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ctl->active = 0;
-        ctl->stopped = s_any ? 0 : 1;
-        ctl->light = -1;
-        ctl->subrounds = 0;
-        ctl->nR = 0;
-        ctl->n1_active = 0;
-        ctl->flag = 0;
-        ctl->ticket = 0;
-    }
-}
-
 // The last CTA of a batch controller grid: true in thread 0 of that CTA.
 __device__ __forceinline__ bool last_cta(RebalCtl *ctl) {
     __shared__ bool s_last;
@@ -332,50 +303,43 @@ __global__ void k_reb_init_batch(const int64_t *__restrict__ C, const int64_t *_
     }
 }
 
-// Start of the next sub-round (h = the number run so far + 1): overloaded
-// set, lightest allowed block, activity.
-__global__ void k_reb_begin(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb, int32_t k,
-                            const int8_t *__restrict__ excl, int8_t *__restrict__ over, int8_t *__restrict__ reject,
-                            const int32_t *__restrict__ d_n1, int32_t max_subrounds, RebalCtl *__restrict__ ctl,
-                            cudaGraphConditionalHandle cond) {
-    __shared__ int s_any;
-    __shared__ long long s_w[256];
-    __shared__ int s_b[256];
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    long long bw = 0;
-    int bb = -1;
-    for (int b = threadIdx.x; b < k; b += blockDim.x) {
-        const bool o = C[b] > Lb[b];
+// Start of the next sub-round of one graph (h = the number run so far + 1), by
+// one CTA of any size: overloaded set, lightest allowed block, activity; with
+// cond also the condition of a graph-resident loop, "this sub-round runs".
+__device__ __forceinline__ void begin_subround(const int64_t *C, const int64_t *Lb, int32_t K, const int8_t *excl,
+                                               int8_t *over, int8_t *reject, int32_t n1, int32_t max_subrounds,
+                                               RebalCtl *ctl, cudaGraphConditionalHandle cond) {
+    __shared__ long long s_bw[32];
+    __shared__ int32_t s_bb[32];
+    int64_t bw = 0;
+    int32_t bb = -1;
+    int any = 0;
+    for (int b = threadIdx.x; b < K; b += blockDim.x) {
+        const int64_t c = C[b];
+        const bool o = c > Lb[b];
         over[b] = o ? 1 : 0;
         reject[b] = 0;
-        if (o) s_any = 1;
-        if (!excl[b] && (bb < 0 || C[b] < bw)) { bw = C[b]; bb = b; }
+        any |= o;
+        // lightest: smallest weight, ties to the smaller block
+        if (!excl[b] && (bb < 0 || -c > bw)) { bw = -c; bb = b; }
     }
-    s_w[threadIdx.x] = bw;
-    s_b[threadIdx.x] = bb;
+    any = __syncthreads_or(any);
+    group_argmax<32>(bw, bb);
+    if ((threadIdx.x & 31) == 0) { s_bw[threadIdx.x >> 5] = bw; s_bb[threadIdx.x >> 5] = bb; }
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            const int b2 = s_b[threadIdx.x + o];
-            const long long w2 = s_w[threadIdx.x + o];
-            const int b1 = s_b[threadIdx.x];
-            if (b2 >= 0 && (b1 < 0 || w2 < s_w[threadIdx.x] || (w2 == s_w[threadIdx.x] && b2 < b1))) {
-                s_b[threadIdx.x] = b2;
-                s_w[threadIdx.x] = w2;
-            }
-        }
-        __syncthreads();
-    }
+    if (threadIdx.x >= 32) return;
+    const bool in = threadIdx.x < blockDim.x >> 5;
+    bw = in ? s_bw[threadIdx.x] : 0;
+    bb = in ? s_bb[threadIdx.x] : -1;
+    group_argmax<32>(bw, bb);
     if (threadIdx.x == 0) {
         const int32_t h = ctl->subrounds + 1;
-        const bool run = !ctl->stopped && s_any && h <= max_subrounds;
+        const bool run = !ctl->stopped && any && h <= max_subrounds;
         ctl->active = run ? 1 : 0;
         if (!run) ctl->stopped = 1;
         if (run) ctl->subrounds = h;
-        ctl->light = s_b[0];
-        ctl->n1_active = run ? *d_n1 : 0;
-        // a graph-resident loop whose body starts without this kernel: its condition
+        ctl->light = bb;
+        ctl->n1_active = run ? n1 : 0;
         if (cond) cudaGraphSetConditional(cond, run ? 1u : 0u);
     }
 }
@@ -422,23 +386,28 @@ __global__ void k_reb_begin_batch(const int64_t *__restrict__ C, const int64_t *
 // End of a sub-round: targets that rejected a move are excluded from now on;
 // stop when nothing was admitted and no target was newly excluded, or when no
 // block is overloaded any more (the next sub-round would find nothing to do).
-__global__ void k_reb_end(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb, int32_t K,
-                          int8_t *__restrict__ excl, const int8_t *__restrict__ reject,
-                          const int32_t *__restrict__ d_na, RebalCtl *__restrict__ ctl) {
-    __shared__ int s_grew, s_over;
-    if (threadIdx.x == 0) s_grew = 0, s_over = 0;
-    __syncthreads();
-    if (!ctl->active) return;
-    for (int b = threadIdx.x; b < K; b += blockDim.x) {
-        if (reject[b] && !excl[b]) { excl[b] = 1; s_grew = 1; }
-        if (C[b] > Lb[b]) s_over = 1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+// One graph: the next sub-round begins in the same kernel.
+__global__ void __launch_bounds__(256) k_reb_end(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb,
+                                                 int32_t K, int8_t *excl, int8_t *reject, int8_t *over,
+                                                 const int32_t *__restrict__ d_na, const int32_t *__restrict__ d_n1,
+                                                 int32_t max_subrounds, RebalCtl *ctl,
+                                                 cudaGraphConditionalHandle cond) {
+    const bool active = ctl->active != 0;
+    int grew = 0, any = 0;
+    if (active)
+        for (int b = threadIdx.x; b < K; b += blockDim.x) {
+            if (reject[b] && !excl[b]) { excl[b] = 1; grew = 1; }
+            if (C[b] > Lb[b]) any = 1;
+        }
+    grew = __syncthreads_or(grew);
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0 && active) {
         const int32_t na = *d_na;
         ctl->nR += na;
-        if ((na == 0 && !s_grew) || !s_over) ctl->stopped = 1;
+        if ((na == 0 && !grew) || !any) ctl->stopped = 1;
     }
+    __syncthreads();
+    begin_subround(C, Lb, K, excl, over, reject, *d_n1, max_subrounds, ctl, cond);
 }
 
 __global__ void k_reb_end_batch(const int64_t *__restrict__ C, const int64_t *__restrict__ Lb, int32_t K,
@@ -484,44 +453,6 @@ __device__ __forceinline__ unsigned __int128 prio_key_wide(int64_t g, uint64_t c
 
 // gain_only (the variant of Sec. 7.2): the priority is the gain alone, the
 // key of weight 1 (g >= 0 first by g, then g < 0 by |g|: g descending).
-__global__ void k_prio_keys(const int32_t *__restrict__ P, const int32_t *__restrict__ d_np,
-                            const int32_t *__restrict__ prop_gain, const int32_t *__restrict__ vwgt, int gbits,
-                            int cbits, int gain_only, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_np;
-    UPR_FOR(i, cnt) {
-        const int32_t u = P[i];
-        keys[i] = prio_key(prop_gain[u], (vwgt && !gain_only) ? (uint64_t)vwgt[u] : 1ull, gbits, cbits);
-        vals[i] = (uint32_t)i;
-    }
-}
-
-// The two words of a wide key: the low words of the proposals in list order
-// (sorted first), then the high words in the order of that sort (A0), whose
-// stable sort completes the order.
-__global__ void k_prio_keys_lo(const int32_t *__restrict__ P, const int32_t *__restrict__ d_np,
-                               const int32_t *__restrict__ prop_gain, const int32_t *__restrict__ vwgt, int gbits,
-                               int cbits, int gain_only, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_np;
-    UPR_FOR(i, cnt) {
-        const int32_t u = P[i];
-        keys[i] = (uint64_t)prio_key_wide(prop_gain[u], (vwgt && !gain_only) ? (uint64_t)vwgt[u] : 1ull, gbits, cbits);
-        vals[i] = (uint32_t)i;
-    }
-}
-
-__global__ void k_prio_keys_hi(const int32_t *__restrict__ P, const uint32_t *__restrict__ A0,
-                               const int32_t *__restrict__ d_np, const int32_t *__restrict__ prop_gain,
-                               const int32_t *__restrict__ vwgt, int gbits, int cbits, int gain_only,
-                               uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_np;
-    UPR_FOR(j, cnt) {
-        const uint32_t i = A0[j];
-        const int32_t u = P[i];
-        keys[j] = (uint64_t)(prio_key_wide(prop_gain[u], (vwgt && !gain_only) ? (uint64_t)vwgt[u] : 1ull, gbits,
-                                           cbits) >> 64);
-        vals[j] = i;
-    }
-}
 
 // ---- prefilter of the proposals.  A source keeps the minimal prefix of its
 // proposals (priority order) that covers its excess; that prefix is usually a
@@ -545,198 +476,475 @@ __device__ __forceinline__ int prio_bin(int64_t g, uint64_t c, int cbits) {
     return 128 + (int)(r < 127ull ? r : 127ull);
 }
 
-// Per source block, the weight of its proposals by bin.  The proposals are
-// the listed nodes with a set flag.  Each CTA sums into a small shared hash
-// table keyed by (block, bin) first (the weight piles up on a few bins of each
-// block), then adds its entries to the global histogram.
+// ---- the ordered part of a sub-round in one team launch (team.cuh): the
+// proposers compacted (they are the next sub-round's list), the prefilter, the
+// kept proposals in priority order, the minimal prefix per source, the longest
+// fitting prefix per target, R appended and the moves applied.
+//
+// The weight before a proposal in its source's (then its target's) order needs
+// no sort by block when the blocks' counts fit a CTA's shared memory (RANK,
+// K <= 256): every warp sums the weights per block of its segment of the
+// priority order, and one barrier later walks the segment again from the sums
+// of the segments before, exactly as a sort pass ranks its digits.  With more
+// blocks (batches) the proposals are sorted by block, stably, instead.
+// When every prefilter bin holds one key value among the kept proposals (with
+// unit weights and gains of moderate size it does), sorting by the bin gives
+// the key order in one pass; else the keys are sorted, less their smallest.
+// Eight barriers in the common form; what bounds a sub-round is their latency
+// and, in the first sub-rounds, the lists.  Per sub-round, against a kernel
+// with thirteen barriers of 304 CTAs that scanned tile sums: R-MAT scale 18,
+// k = 8 37 us (56 before), scale 22, k = 64 81 us (110 before).  It also stands
+// for the forty launches a sub-round took with several graphs, more than 256
+// blocks or some key widths (Chung-Lu n = 10^6, weights, k = 23: 6.6 -> 5.3 ms
+// a refinement; 1024 graphs in one context 19.0 -> 16.4 ms).
 constexpr int kHistSlots = 2048;
 constexpr uint32_t kHistEmpty = 0xffffffffu;
+constexpr unsigned long long kNoKey = ~0ull;
+constexpr int kRankK = 256;
 
-__global__ void __launch_bounds__(256) k_prio_hist(const int32_t *__restrict__ list, const int32_t *__restrict__ d_n1,
-                                                   const int32_t *__restrict__ flags,
-                                                   const int32_t *__restrict__ prop_gain,
-                                                   const int32_t *__restrict__ vwgt, const int32_t *__restrict__ part,
-                                                   int gbits, int cbits, int gain_only,
-                                                   unsigned long long *__restrict__ hist) {
-    __shared__ uint32_t s_key[kHistSlots];
-    __shared__ unsigned long long s_val[kHistSlots];
-    for (int i = threadIdx.x; i < kHistSlots; i += blockDim.x) { s_key[i] = kHistEmpty; s_val[i] = 0; }
-    __syncthreads();
-    const int64_t n1 = *d_n1;
-    UPR_FOR(i, n1) {
-        if (flags && !flags[i]) continue;
-        const int32_t u = list[i];
-        const uint64_t c = vwgt ? (uint64_t)vwgt[u] : 1ull;
-        const uint32_t key = (uint32_t)part[u] * kPrioBins + prio_bin(prop_gain[u], gain_only ? 1ull : c, cbits);
-        uint32_t h = (key * 0x9E3779B1u) >> 21;          // 11 bits: kHistSlots
-        bool done = false;
-        for (int probe = 0; probe < 32 && !done; probe++) {
-            uint32_t cur = s_key[h];
-            if (cur == kHistEmpty) {
-                cur = atomicCAS(&s_key[h], kHistEmpty, key);
-                if (cur == kHistEmpty) cur = key;
-            }
-            if (cur == key) {
-                atomicAdd(&s_val[h], (unsigned long long)c);
-                done = true;
-            }
-            h = (h + 1) & (kHistSlots - 1);
-        }
-        if (!done) atomicAdd(&hist[key], (unsigned long long)c);   // crowded table: straight to the histogram
+struct __align__(32) Item128 {
+    using Key = unsigned __int128;
+    unsigned __int128 key;
+    uint32_t val, pad[3];
+};
+
+// The weight of this lane's group (equal digits) and of its earlier lanes.
+template <bool UNIT>
+__device__ __forceinline__ long long group_before(unsigned peers, long long c, long long *tot) {
+    const int lane = threadIdx.x & 31;
+    if (UNIT) {
+        *tot = __popc(peers);
+        return __popc(peers & ((1u << lane) - 1u));
+    }
+    long long before = 0, all = 0;
+    for (unsigned m = peers; m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        const long long x = __shfl_sync(peers, c, l);
+        all += x;
+        if (l < lane) before += x;
+    }
+    *tot = all;
+    return before;
+}
+
+// One RANK step over the items [g.b, g.e) of this warp: visit(j, digit, before)
+// for every item with digit(j) >= 0, before = the weight of the items of the
+// same digit before it in the whole list.  hist: [P * K].  One barrier inside.
+template <bool UNIT, class Digit, class Weight, class Visit>
+__device__ __forceinline__ void rank_walk(const Team &t, team::Smem &s, void *dyn, const team::Seg &g, int K,
+                                          unsigned long long *hist, Digit digit, Weight weight, Visit visit) {
+    using Row = typename std::conditional<UNIT, int, unsigned long long>::type;
+    Row *rows = UNIT ? reinterpret_cast<Row *>(s.cnt()) : reinterpret_cast<Row *>(dyn);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    Row *row = rows + warp * K;
+    for (int i = lane; i < K; i += 32) row[i] = 0;
+    __syncwarp();
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const int d = j < g.e ? digit(j) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        long long tot;
+        group_before<UNIT>(peers, UNIT || d < 0 ? 1 : weight(j), &tot);
+        if (d >= 0 && (peers & lt) == 0) row[d] += (Row)tot;
+        __syncwarp();
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kHistSlots; i += blockDim.x)
-        if (s_key[i] != kHistEmpty) atomicAdd(&hist[s_key[i]], s_val[i]);
-}
-
-// Per overloaded source: the first bin where the cumulative weight reaches the
-// excess C - L_max (the last bin when it never does); the histogram row is
-// cleared for the next sub-round.  One CTA of kPrioBins threads per block.
-__global__ void __launch_bounds__(kPrioBins) k_prio_cut(int32_t K, const int8_t *__restrict__ over,
-                                                       const int64_t *__restrict__ C, const int64_t *__restrict__ Lb,
-                                                       unsigned long long *__restrict__ hist,
-                                                       int32_t *__restrict__ cut) {
-    __shared__ unsigned long long s_warp[kPrioBins / 32];
-    __shared__ int s_cut;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    for (int32_t a = blockIdx.x; a < K; a += gridDim.x) {
-        if (!over[a]) continue;                       // uniform over the CTA
-        unsigned long long *row = hist + (int64_t)a * kPrioBins;
-        const unsigned long long v = row[t];
-        unsigned long long inc = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
+    for (int d = threadIdx.x; d < K; d += team::kTT) {
+        unsigned long long run = 0;
+#pragma unroll 8
+        for (int w = 0; w < team::kTW; w++) {
+            const Row c = rows[w * K + d];
+            rows[w * K + d] = (Row)run;
+            run += c;
         }
-        if (lane == 31) s_warp[warp] = inc;
-        if (t == 0) s_cut = kPrioBins - 1;
-        __syncthreads();
-        for (int w = 0; w < warp; w++) inc += s_warp[w];
-        const unsigned long long excess = (unsigned long long)(C[a] - Lb[a]);
-        if (inc >= excess) atomicMin(&s_cut, t);
-        row[t] = 0;
-        __syncthreads();
-        if (t == 0) cut[a] = s_cut;
-        __syncthreads();
+        hist[(int64_t)blockIdx.x * K + d] = run;
+        s.rep[d] = 0;
     }
-}
-
-// keep[i]: listed node i proposes and its bin is not after its source's cut
-__global__ void k_prio_keep(const int32_t *__restrict__ list, const int32_t *__restrict__ d_n1,
-                            const int32_t *__restrict__ flags, const int32_t *__restrict__ prop_gain,
-                            const int32_t *__restrict__ vwgt, const int32_t *__restrict__ part,
-                            const int32_t *__restrict__ cut, int gbits, int cbits, int gain_only,
-                            int32_t *__restrict__ keep) {
-    const int64_t n1 = *d_n1;
-    UPR_FOR(i, n1) {
-        int32_t k = 0;
-        if (!flags || flags[i]) {
-            const int32_t u = list[i];
-            const uint64_t c = vwgt ? (uint64_t)vwgt[u] : 1ull;
-            k = prio_bin(prop_gain[u], gain_only ? 1ull : c, cbits) <= cut[part[u]] ? 1 : 0;
+    team::sync(t);
+    {
+        const int d = threadIdx.x & (kRankK - 1);
+        unsigned long long v = 0;
+        if (d < K)
+            for (int c = threadIdx.x / kRankK; c < (int)blockIdx.x; c += team::kTT / kRankK)
+                v += hist[(int64_t)c * K + d];
+        if (v) atomicAdd(&s.rep[d], v);
+    }
+    __syncthreads();
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const int d = j < g.e ? digit(j) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        long long tot;
+        const long long in = group_before<UNIT>(peers, UNIT || d < 0 ? 1 : weight(j), &tot);
+        Row at = 0;
+        if (d >= 0) at = row[d];
+        __syncwarp();
+        if (d >= 0) {
+            if ((peers & lt) == 0) row[d] = at + (Row)tot;
+            visit(j, d, (int64_t)(s.rep[d] + (unsigned long long)at) + in);
         }
-        keep[i] = k;
+        __syncwarp();
     }
 }
 
-// Block-id key (source or target) of the entries listed through idx/order.
-__global__ void k_block_keys(const int32_t *__restrict__ P, const uint32_t *__restrict__ A,
-                             const int32_t *__restrict__ S, const int32_t *__restrict__ d_cnt,
-                             const int32_t *__restrict__ blk_of_node, uint64_t *__restrict__ keys,
-                             uint32_t *__restrict__ vals) {
-    const int64_t cnt = *d_cnt;
-    UPR_FOR(i, cnt) {
-        const int64_t j = S ? S[i] : i;
-        const int32_t u = P[A[j]];
-        keys[i] = (uint64_t)blk_of_node[u];
-        vals[i] = (uint32_t)i;
+// The same by a sort (any K): the items with digit(j) >= 0 sorted by digit,
+// visited in that order.
+template <class Digit, class Weight, class Visit>
+__device__ __forceinline__ void sort_walk(const RebalTeam &a, team::Smem &s, int slot, int64_t n, Digit digit,
+                                          Weight weight, Visit visit) {
+    using team::Item32;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    int64_t cnt;
+    const Item32 *S = team::sort(
+        t, s, n,
+        [&](int64_t j, Item32 &it) {
+            const int d = digit(j);
+            it.key = (uint32_t)d;
+            it.val = (uint32_t)j;
+            return d >= 0;
+        },
+        a.kbits, reinterpret_cast<Item32 *>(a.bufA), reinterpret_cast<Item32 *>(a.bufB), &cnt);
+    const team::Seg g = team::warp_seg(cnt);
+    long long base = 0;
+    if (a.vwgt) {
+        long long x = 0, all;
+        for (int64_t q = g.b + lane; q < g.e; q += 32) x += weight(S[q].val);
+        const long long mine = team::publish<team::Sum>(t, s, slot, team::warp_all<team::Sum>(x));
+        team::sync(t);
+        base = team::collect<team::Sum>(t, slot, &all) + mine;
+    }
+    for (int64_t q0 = g.b; q0 < g.e; q0 += 32) {
+        const int64_t q = q0 + lane;
+        long long pre = q;
+        if (a.vwgt) {
+            const long long c = q < g.e ? weight(S[q].val) : 0;
+            const long long inc = team::warp_incl<team::Sum>(c);
+            pre = base + inc - c;
+            base += __shfl_sync(0xffffffffu, inc, 31);
+            if (q < g.e) a.c_excl[q] = pre;
+        }
+        if (q < g.e && (q == 0 || S[q - 1].key != S[q].key)) a.seg_base[S[q].key] = pre;
+    }
+    team::sync(t);
+    for (int64_t q = g.b + lane; q < g.e; q += 32) {
+        const Item32 it = S[q];
+        visit((int64_t)it.val, (int)it.key, (a.vwgt ? a.c_excl[q] : q) - a.seg_base[it.key]);
     }
 }
 
-// For entries in block-sorted order: weights, and the first position of each block.
-__global__ void k_seg_weights(const int32_t *__restrict__ P, const uint32_t *__restrict__ A,
-                              const int32_t *__restrict__ S, const uint32_t *__restrict__ B,
-                              const uint64_t *__restrict__ bkeys, const int32_t *__restrict__ d_cnt,
-                              const int32_t *__restrict__ vwgt, int64_t *__restrict__ c_sorted,
-                              int32_t *__restrict__ seg_first) {
-    const int64_t cnt = *d_cnt;
-    UPR_FOR(q, cnt) {
-        const int64_t i = B[q];
-        const int64_t j = S ? S[i] : i;
-        const int32_t u = P[A[j]];
-        c_sorted[q] = vwgt ? vwgt[u] : 1;
-        const int32_t b = (int32_t)bkeys[q];
-        if (q == 0 || (int32_t)bkeys[q - 1] != b) seg_first[b] = (int32_t)q;
+template <bool UNIT, bool RANK, bool WIDE>
+__global__ void __launch_bounds__(team::kTT, 1) k_reb_team(const RebalTeam a) {
+    __shared__ team::Smem s;
+    extern __shared__ unsigned long long s_dyn[];
+    using team::Item32;
+    using KeyItem = typename std::conditional<WIDE, Item128, team::Item64>::type;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+    const int K = a.K;
+    const int64_t n1 = *a.d_n1;
+    if (n1 == 0) {                           // (no sub-round runs, or nothing is listed)
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_np = *a.d_nk = *a.d_na = 0;
+        return;
     }
-}
+    auto weight_of = [&](int32_t v) -> uint64_t { return UNIT ? 1ull : (uint64_t)a.vwgt[v]; };
+    auto bin_of = [&](int64_t gain, int32_t v) { return prio_bin(gain, a.gain_only ? 1ull : weight_of(v), a.cbits); };
 
-// Minimal prefix per source: entry selected iff the weight before it in its
-// source's priority order is below the source's excess.
-__global__ void k_mark_selected(const uint32_t *__restrict__ B, const uint64_t *__restrict__ bkeys,
-                                const int32_t *__restrict__ d_cnt, const int64_t *__restrict__ c_excl,
-                                const int32_t *__restrict__ seg_first, RebalState st, int32_t *__restrict__ sel) {
-    const int64_t cnt = *d_cnt;
-    UPR_FOR(q, cnt) {
-        const int32_t b = (int32_t)bkeys[q];
-        const int64_t before = c_excl[q] - c_excl[seg_first[b]];
-        sel[B[q]] = before < st.C[b] - st.Lb[b] ? 1 : 0;
+    // ---- the proposers counted; their weight per (source, bin), summed in a
+    // shared hash table first (it piles up on a few bins of each source)
+    const team::Seg g1 = team::warp_seg(n1);
+    {
+        uint32_t *s_key = reinterpret_cast<uint32_t *>(s.cnt64);
+        unsigned long long *s_val = s.cnt64 + kHistSlots / 2;
+        if (a.hist) {
+            for (int i = threadIdx.x; i < kHistSlots; i += team::kTT) { s_key[i] = kHistEmpty; s_val[i] = 0; }
+            __syncthreads();
+        }
+        long long cnt = 0;
+        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 32) {
+            const int64_t i = i0 + lane;
+            const bool f = i < g1.e && a.flags[i] != 0;
+            cnt += __popc(__ballot_sync(full, f));
+            if (!a.hist) continue;
+            uint32_t key = kHistEmpty;
+            long long c = 1;
+            if (f) {
+                const int32_t v = a.list[i];
+                c = (long long)weight_of(v);
+                key = (uint32_t)a.lsrc[i] * kPrioBins + bin_of(a.lgain[i], v);
+            }
+            const unsigned peers = __match_any_sync(full, key);
+            long long tot;
+            group_before<UNIT>(peers, c, &tot);
+            if (f && (peers & lt) == 0) {
+                uint32_t h = (key * 0x9E3779B1u) >> 21;          // 11 bits: kHistSlots
+                bool done = false;
+                for (int probe = 0; probe < 32 && !done; probe++) {
+                    uint32_t cur = *(volatile uint32_t *)&s_key[h];
+                    if (cur == kHistEmpty) {
+                        cur = atomicCAS(&s_key[h], kHistEmpty, key);
+                        if (cur == kHistEmpty) cur = key;
+                    }
+                    if (cur == key) {
+                        atomicAdd(&s_val[h], (unsigned long long)tot);
+                        done = true;
+                    }
+                    h = (h + 1) & (kHistSlots - 1);
+                }
+                if (!done) atomicAdd(&a.hist[key], (unsigned long long)tot);   // crowded: straight to the histogram
+            }
+            __syncwarp();
+        }
+        const long long mine = team::publish<team::Sum>(t, s, 0, cnt);         // (CTA barriers inside)
+        if (a.hist)
+            for (int i = threadIdx.x; i < kHistSlots; i += team::kTT)
+                if (s_key[i] != kHistEmpty) atomicAdd(&a.hist[s_key[i]], s_val[i]);
+        if (blockIdx.x == 0) {
+            for (int i = threadIdx.x; i < kPrioBins; i += team::kTT) a.rep[i] = kNoKey;
+            if (threadIdx.x == 0) *a.exact = 1;
+        }
+        team::sync(t);
+        // ---- compacted in node order, and the cut bin of every source
+        long long np;
+        long long pos = team::collect<team::Sum>(t, 0, &np) + mine;
+        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 32) {
+            const int64_t i = i0 + lane;
+            const bool f = i < g1.e && a.flags[i] != 0;
+            const unsigned m = __ballot_sync(full, f);
+            if (f) {
+                const int64_t p = pos + __popc(m & lt);
+                a.list2[p] = a.list[i];
+                a.lsrc2[p] = a.lsrc[i];
+                a.lgain2[p] = a.lgain[i];
+            }
+            pos += __popc(m);
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_np = (int32_t)np;
     }
-}
-
-// Longest fitting prefix per target; a rejected entry marks its target.
-__global__ void k_mark_admitted(const uint32_t *__restrict__ T, const uint64_t *__restrict__ bkeys,
-                                const int32_t *__restrict__ d_cnt, const int64_t *__restrict__ c_sorted,
-                                const int64_t *__restrict__ c_excl, const int32_t *__restrict__ seg_first,
-                                RebalState st, int32_t *__restrict__ adm, int8_t *__restrict__ reject) {
-    const int64_t cnt = *d_cnt;
-    UPR_FOR(q, cnt) {
-        const int32_t t = (int32_t)bkeys[q];
-        const int64_t incl = c_excl[q] - c_excl[seg_first[t]] + c_sorted[q];
-        const bool ok = st.C[t] + incl <= st.Lb[t];
-        adm[T[q]] = ok ? 1 : 0;
-        if (!ok) reject[t] = 1;
+    long long np;
+    team::collect<team::Sum>(t, 0, &np);
+    if (a.hist) {
+        // a warp per overloaded source, eight bins per lane: the first bin
+        // where the cumulative weight reaches the excess; the row is cleared
+        for (int64_t b = blockIdx.x * team::kTW + (threadIdx.x >> 5); b < K; b += (int64_t)gridDim.x * team::kTW) {
+            if (!a.over[b]) continue;
+            unsigned long long *row = a.hist + b * kPrioBins + lane * 8;
+            unsigned long long w[8], sum = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++) { w[i] = row[i]; row[i] = 0; sum += w[i]; }
+            unsigned long long run = (unsigned long long)team::warp_incl<team::Sum>((long long)sum) - sum;
+            const unsigned long long excess = (unsigned long long)(a.C[b] - a.Lb[b]);
+            int first = kPrioBins - 1;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                run += w[i];
+                if (run >= excess) first = min(first, lane * 8 + i);
+            }
+            for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(full, first, o));
+            if (lane == 0) a.cut[b] = first;
+        }
     }
-}
+    team::sync(t);
 
-__global__ void k_apply_rebal(const int32_t *__restrict__ P, const uint32_t *__restrict__ A,
-                              const int32_t *__restrict__ S, const int32_t *__restrict__ Adm,
-                              const int32_t *__restrict__ d_na, const int32_t *__restrict__ prop_tgt,
-                              const int32_t *__restrict__ vwgt, int32_t *__restrict__ part,
-                              unsigned long long *__restrict__ C, int32_t K, const RebalCtl *__restrict__ ctl,
-                              int32_t *__restrict__ R_node, int32_t *__restrict__ R_from,
-                              int32_t *__restrict__ R_to, int32_t *__restrict__ R_sub, int32_t *__restrict__ r_to,
-                              int32_t *__restrict__ r_at) {
-    extern __shared__ unsigned long long s_delta[];
-    BlockDelta bd = make_block_delta(s_delta, K, C);
+    // ---- the kept proposals in priority order.  First their bins counted for
+    // a one-pass sort, and whether every bin holds one key value
+    auto kept = [&](int64_t i, int32_t *v, int64_t *gain, int *bin) {
+        *v = a.list2[i];
+        *gain = a.lgain2[i];
+        *bin = bin_of(*gain, *v);
+        return !a.hist || *bin <= a.cut[a.lsrc2[i]];
+    };
+    auto key_weight = [&](int32_t v) { return a.gain_only ? 1ull : weight_of(v); };
+    const team::Seg gp = team::warp_seg(np);
+    if (threadIdx.x < kPrioBins) s.rep[threadIdx.x] = kNoKey;
+    __shared__ int s_inexact;
+    if (threadIdx.x == 0) s_inexact = 0;
+    __syncthreads();
+    unsigned long long hi = 0, lo = 0;       // largest key, and largest 2^63 - 1 - key
+    team::sort_count<Item32>(
+        t, s, np,
+        [&](int64_t i, Item32 &it) {
+            int32_t v;
+            int64_t gain;
+            int bin;
+            const bool k = kept(i, &v, &gain, &bin);
+            a.list[i] = v;
+            it.key = (uint32_t)bin;
+            if (!k) return false;
+            if (WIDE) return true;
+            const unsigned long long key = prio_key(gain, key_weight(v), a.gbits, a.cbits);
+            hi = max(hi, key);
+            lo = max(lo, 0x7fffffffffffffffull - key);
+            unsigned long long r = *(volatile unsigned long long *)&s.rep[bin];
+            if (r == kNoKey) {
+                r = atomicCAS(&s.rep[bin], kNoKey, key);
+                if (r == kNoKey) r = key;
+            }
+            if (r != key) s_inexact = 1;
+            return true;
+        },
+        0, 8);
+    team::publish<team::Max>(t, s, 1, team::warp_all<team::Max>((long long)hi));
+    team::publish<team::Max>(t, s, 2, team::warp_all<team::Max>((long long)lo));
+    if (!WIDE) {
+        if (threadIdx.x < kPrioBins && s.rep[threadIdx.x] != kNoKey) {
+            const unsigned long long r = atomicCAS(&a.rep[threadIdx.x], kNoKey, s.rep[threadIdx.x]);
+            if (r != kNoKey && r != s.rep[threadIdx.x]) s_inexact = 1;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && s_inexact) *a.exact = 0;
+    }
+    team::sync(t);
+    int64_t nk;
+    const Item32 *S32 = nullptr;
+    const KeyItem *SK = nullptr;
+    if (!WIDE && *(volatile const int32_t *)a.exact != 0) {
+        nk = team::sort_place<Item32>(
+            t, s, np,
+            [&](int64_t i, Item32 &it) {
+                int32_t v;
+                int64_t gain;
+                int bin;
+                const bool k = kept(i, &v, &gain, &bin);
+                it.key = (uint32_t)bin;
+                it.val = (uint32_t)v;
+                return k;
+            },
+            0, 8, reinterpret_cast<Item32 *>(a.bufA));
+        S32 = reinterpret_cast<const Item32 *>(a.bufA);
+    } else {
+        long long top, low;
+        team::collect<team::Max>(t, 1, &top);
+        team::collect<team::Max>(t, 2, &low);
+        const unsigned long long kmin = WIDE ? 0 : 0x7fffffffffffffffull - (unsigned long long)low;
+        const int bits = WIDE ? 1 + a.gbits + 2 * a.cbits : max(1, 64 - __clzll(top - (long long)kmin));
+        SK = team::sort(
+            t, s, np,
+            [&](int64_t i, KeyItem &it) {
+                int32_t v;
+                int64_t gain;
+                int bin;
+                if (!kept(i, &v, &gain, &bin)) return false;
+                if constexpr (WIDE) it.key = prio_key_wide(gain, key_weight(v), a.gbits, a.cbits);
+                else it.key = prio_key(gain, key_weight(v), a.gbits, a.cbits) - kmin;
+                it.val = (uint32_t)v;
+                return true;
+            },
+            bits, reinterpret_cast<KeyItem *>(a.bufA), reinterpret_cast<KeyItem *>(a.bufB), &nk);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_nk = (int32_t)nk;
+    const team::Seg g = team::warp_seg(nk);
+    for (int64_t j = g.b + lane; j < g.e; j += 32) a.U[j] = S32 ? S32[j].val : SK[j].val;
+    __syncwarp();
+    if (!RANK) team::sync(t);                // (the sorts below read other segments and reuse the buffers)
+
+    // ---- the minimal prefix per source: the weight before a proposal is
+    // below the excess; at[j] = its target, or -1
+    auto weight = [&](int64_t j) { return (long long)weight_of((int32_t)a.U[j]); };
+    auto src_of = [&](int64_t j) { return a.part[a.U[j]]; };
+    auto select = [&](int64_t j, int b, int64_t before) {
+        a.at[j] = before < a.C[b] - a.Lb[b] ? a.prop_tgt[a.U[j]] : -1;
+    };
+    // ---- the longest fitting prefix per target
+    auto tgt_of = [&](int64_t j) { return a.at[j]; };
+    long long adm = 0;
+    auto admit = [&](int64_t j, int b, int64_t before) {
+        if (a.C[b] + before + weight(j) > a.Lb[b]) {
+            a.at[j] = -1;
+            a.reject[b] = 1;
+        }
+    };
+    if constexpr (RANK) {
+        rank_walk<UNIT>(t, s, s_dyn, g, K, t.hist64, src_of, weight, select);
+        rank_walk<UNIT>(t, s, s_dyn, g, K, t.hist64 + (int64_t)gridDim.x * K, tgt_of, weight, admit);
+    } else {
+        sort_walk(a, s, 3, nk, src_of, weight, select);
+        team::sync(t);
+        sort_walk(a, s, 4, nk, tgt_of, weight, admit);
+        team::sync(t);
+    }
+    // ---- the admitted, in priority order, appended to R and applied
+    for (int64_t j = g.b + lane; j < g.e; j += 32) adm += a.at[j] >= 0;
+    const long long mine = team::publish<team::Sum>(t, s, 5, team::warp_all<team::Sum>(adm));
+    team::sync(t);
+    long long na;
+    int64_t pos = a.ctl->nR + team::collect<team::Sum>(t, 5, &na) + mine;
+    const int32_t subround = a.ctl->subrounds;
+    BlockDelta bd = make_block_delta(s.cnt64, K, reinterpret_cast<unsigned long long *>(a.C));
     bd.init();
-    const int64_t cnt = *d_na;
-    const int64_t off = ctl->nR;
-    const int32_t subround = ctl->subrounds;
-    R_node += off; R_from += off; R_to += off; R_sub += off;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < cnt; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = base + threadIdx.x;
-        int32_t a = -1, b = -1;
+    for (int64_t j0 = g.b; j0 < g.e; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const int32_t to = j < g.e ? a.at[j] : -1;
+        const unsigned m = __ballot_sync(full, to >= 0);
+        int32_t from = -1;
         long long c = 0;
-        if (p < cnt) {
-            const int32_t u = P[A[S[Adm[p]]]];
-            a = part[u];
-            b = prop_tgt[u];
-            c = vwgt ? vwgt[u] : 1;
-            R_node[p] = u;
-            R_from[p] = a;
-            R_to[p] = b;
-            R_sub[p] = subround;
-            r_to[u] = b;
-            r_at[u] = (int32_t)(off + p);
-            part[u] = b;
+        if (to >= 0) {
+            const int32_t v = (int32_t)a.U[j];
+            const int64_t p = pos + __popc(m & lt);
+            from = a.part[v];
+            c = (long long)weight_of(v);
+            a.R_node[p] = v;
+            a.R_from[p] = from;
+            a.R_to[p] = to;
+            a.R_sub[p] = subround;
+            a.r_to[v] = to;
+            a.r_at[v] = (int32_t)p;
+            a.part[v] = to;
         }
-        bd.add(a, -c);
-        bd.add(b, c);
+        pos += __popc(m);
+        if (m) {
+            bd.add(from, -c);
+            bd.add(to, c);
+        }
     }
-    bd.flush(C);
+    bd.flush(reinterpret_cast<unsigned long long *>(a.C));
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_na = (int32_t)na;
 }
 
-inline unsigned grid1(int64_t n) { return (unsigned)ceil_div(n > 0 ? n : 1, 256); }
+// ---- the start of a round's rebalancing: the nodes of the overloaded blocks,
+// in node order, are the first list; the overloaded blocks are never targets.
+// One graph (light == nullptr): CTA 0 also begins the first sub-round.
+__global__ void __launch_bounds__(team::kTT, 1) k_reb_start(const RebalStart a) {
+    __shared__ team::Smem s;
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    const team::Seg g = team::warp_seg(a.n);
+    long long cnt = 0;
+    for (int64_t v = g.b + lane; v < g.e; v += 32) {
+        const int32_t b = a.part[v];
+        cnt += a.C[b] > a.Lb[b];
+    }
+    const long long mine = team::publish<team::Sum>(t, s, 0, team::warp_all<team::Sum>(cnt));
+    team::sync(t);
+    long long all;
+    int64_t pos = team::collect<team::Sum>(t, 0, &all) + mine;
+    for (int64_t v0 = g.b; v0 < g.e; v0 += 32) {
+        const int64_t v = v0 + lane;
+        bool f = false;
+        if (v < g.e) {
+            const int32_t b = a.part[v];
+            f = a.C[b] > a.Lb[b];
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (f) a.list[pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
+        pos += __popc(m);
+    }
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x == 0) *a.d_list = (int32_t)all;
+    if (a.batch) return;
+    for (int b = threadIdx.x; b < a.K; b += team::kTT) a.excl[b] = a.C[b] > a.Lb[b] ? 1 : 0;
+    if (threadIdx.x == 0) {
+        a.ctl->stopped = 0;
+        a.ctl->subrounds = 0;
+        a.ctl->nR = 0;
+        a.ctl->flag = 0;
+        a.ctl->ticket = 0;
+    }
+    __syncthreads();
+    begin_subround(a.C, a.Lb, a.K, a.excl, a.over, a.reject, (int32_t)all, a.max_subrounds, a.ctl, a.cond);
+}
 
 }  // namespace
 
@@ -762,12 +970,6 @@ void rebalance_propose_scalar_list(const GraphDev &g, const int32_t *list, const
         default: UPR_PROP(32); break;
     }
 #undef UPR_PROP
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_flag_in_blocks(const int32_t *part, int64_t n, const int8_t *mark, int32_t *flags, cudaStream_t s) {
-    if (n <= 0) return;
-    k_flag_in_blocks<<<grid1(n), 256, 0, s>>>(part, n, mark, flags);
     UPR_LAUNCH_CHECK();
 }
 
@@ -834,92 +1036,35 @@ void rebalance_propose_list(const GraphDev &g, const int32_t *list, const int32_
     rebalance_propose_scalar_list(g, list, d_n1, n1_max, part, W, st, prop_tgt, prop_gain, flags, s);
 }
 
-void rebalance_prefilter(const GraphDev &g, const int32_t *list, const int32_t *d_n1, int64_t n1_max,
-                         const int32_t *flags, const int32_t *prop_gain, const int32_t *part, const int8_t *over,
-                         const int64_t *C, int gbits, int cbits, int gain_only, unsigned long long *hist,
-                         int32_t *cut, int32_t *keep, cudaStream_t s) {
-    if (n1_max <= 0) return;
-    const unsigned hist_grid = (unsigned)std::min<int64_t>(ceil_div(n1_max, 256), (int64_t)device_sm_count() * 4);
-    k_prio_hist<<<hist_grid, 256, 0, s>>>(list, d_n1, flags, prop_gain, g.vwgt, part, gbits, cbits, gain_only,
-                                          hist);
-    UPR_LAUNCH_CHECK();
-    k_prio_cut<<<(unsigned)std::min<int64_t>(g.K(), 4096), kPrioBins, 0, s>>>(g.K(), over, C, g.Lb, hist, cut);
-    UPR_LAUNCH_CHECK();
-    k_prio_keep<<<grid_for(n1_max), 256, 0, s>>>(list, d_n1, flags, prop_gain, g.vwgt, part, cut, gbits, cbits,
-                                                 gain_only, keep);
-    UPR_LAUNCH_CHECK();
+void rebalance_start(const GraphDev &g, RebalStart a, cudaStream_t s) {
+    a.n = g.n;
+    a.K = g.K();
+    a.Lb = g.Lb;
+    a.batch = g.ng > 1;
+    launch_team(k_reb_start, a, a.team.size, s);
 }
 
-void rebalance_prio_cut(const GraphDev &g, const int8_t *over, const int64_t *C, unsigned long long *hist, int32_t *cut,
-                        cudaStream_t s) {
-    k_prio_cut<<<(unsigned)std::min<int64_t>(g.K(), 4096), kPrioBins, 0, s>>>(g.K(), over, C, g.Lb, hist, cut);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_prio_keys(const GraphDev &g, const int32_t *P, const int32_t *d_np, const int32_t *prop_gain,
-                         int gbits, int cbits, int gain_only, uint64_t *keys, uint32_t *vals, int64_t np_max,
-                         cudaStream_t s) {
-    if (np_max <= 0) return;
-    k_prio_keys<<<grid_for(np_max), 256, 0, s>>>(P, d_np, prop_gain, g.vwgt, gbits, cbits, gain_only, keys, vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_prio_sort_wide(const GraphDev &g, const int32_t *P, const int32_t *d_np, const int32_t *prop_gain,
-                              int gbits, int cbits, int gain_only, SortPairs sp, int64_t np_max, Scratch tmp,
-                              cudaStream_t s, uint32_t **order) {
-    if (np_max <= 0) { *order = sp.v; return; }
-    const Count cnt{d_np, np_max};
-    k_prio_keys_lo<<<grid_for(np_max), 256, 0, s>>>(P, d_np, prop_gain, g.vwgt, gbits, cbits, gain_only, sp.k, sp.v);
-    UPR_LAUNCH_CHECK();
-    // 64 bits = 8 passes, an even number: the result is back in (k, v)
-    radix_sort_pairs(sp.k, sp.v, sp.ka, sp.va, cnt, 64, tmp, s);
-    k_prio_keys_hi<<<grid_for(np_max), 256, 0, s>>>(P, sp.v, d_np, prop_gain, g.vwgt, gbits, cbits, gain_only, sp.ka,
-                                                    sp.va);
-    UPR_LAUNCH_CHECK();
-    const bool alt = radix_sort_pairs(sp.ka, sp.va, sp.k, sp.v, cnt, 1 + gbits + 2 * cbits - 64, tmp, s);
-    *order = alt ? sp.v : sp.va;
-}
-
-void rebalance_block_keys(const int32_t *P, const uint32_t *A, const int32_t *S, const int32_t *d_cnt,
-                          const int32_t *blk_of_node, uint64_t *keys, uint32_t *vals, int64_t cnt_max, cudaStream_t s) {
-    if (cnt_max <= 0) return;
-    k_block_keys<<<grid_for(cnt_max), 256, 0, s>>>(P, A, S, d_cnt, blk_of_node, keys, vals);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_seg_weights(const GraphDev &g, const int32_t *P, const uint32_t *A, const int32_t *S,
-                           const uint32_t *B, const uint64_t *bkeys, const int32_t *d_cnt, int64_t *c_sorted,
-                           int32_t *seg_first, int64_t cnt_max, cudaStream_t s) {
-    if (cnt_max <= 0) return;
-    k_seg_weights<<<grid_for(cnt_max), 256, 0, s>>>(P, A, S, B, bkeys, d_cnt, g.vwgt, c_sorted, seg_first);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_mark_selected(const uint32_t *B, const uint64_t *bkeys, const int32_t *d_cnt, const int64_t *c_excl,
-                             const int32_t *seg_first, RebalState st, int32_t *sel, int64_t cnt_max, cudaStream_t s) {
-    if (cnt_max <= 0) return;
-    k_mark_selected<<<grid_for(cnt_max), 256, 0, s>>>(B, bkeys, d_cnt, c_excl, seg_first, st, sel);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_mark_admitted(const uint32_t *T, const uint64_t *bkeys, const int32_t *d_cnt, const int64_t *c_sorted,
-                             const int64_t *c_excl, const int32_t *seg_first, RebalState st, int32_t *adm,
-                             int8_t *reject, int64_t cnt_max, cudaStream_t s) {
-    if (cnt_max <= 0) return;
-    k_mark_admitted<<<grid_for(cnt_max), 256, 0, s>>>(T, bkeys, d_cnt, c_sorted, c_excl, seg_first, st, adm, reject);
-    UPR_LAUNCH_CHECK();
-}
-
-void rebalance_apply(const GraphDev &g, const int32_t *P, const uint32_t *A, const int32_t *S, const int32_t *Adm,
-                     const int32_t *d_na, const int32_t *prop_tgt, int32_t *part, int64_t *C, const RebalCtl *ctl,
-                     int32_t *R_node, int32_t *R_from, int32_t *R_to, int32_t *R_sub, int32_t *r_to, int32_t *r_at,
-                     int64_t na_max, cudaStream_t s) {
-    if (na_max <= 0) return;
-    const int64_t blocks = std::min<int64_t>(ceil_div(na_max, 256), (int64_t)device_sm_count() * 4);
-    k_apply_rebal<<<(unsigned)blocks, 256, block_delta_smem(g.K()), s>>>(
-        P, A, S, Adm, d_na, prop_tgt, g.vwgt, part, (unsigned long long *)C, g.K(), ctl, R_node, R_from, R_to, R_sub,
-        r_to, r_at);
-    UPR_LAUNCH_CHECK();
+void rebalance_order(const GraphDev &g, RebalTeam a, cudaStream_t s) {
+    if (g.n <= 0) return;
+    a.K = g.K();
+    a.kbits = 1;
+    while ((1ll << a.kbits) < a.K) a.kbits++;
+    a.vwgt = g.vwgt;
+    a.Lb = g.Lb;
+    const bool rank = a.K <= kRankK, wide = 1 + a.gbits + 2 * a.cbits > 63;
+    // (weighted: the warps' block sums are 64-bit, 64 KB at K = 256)
+    const size_t shm = rank && g.vwgt ? sizeof(unsigned long long) * team::kTW * (size_t)a.K : 0;
+    auto go = [&](auto kern) { launch_team(kern, a, a.team.size, s, shm); };
+    if (!g.vwgt) {           // (unit weights: keys of at most 34 bits)
+        if (rank) go(k_reb_team<true, true, false>);
+        else go(k_reb_team<true, false, false>);
+    } else if (wide) {
+        if (rank) go(k_reb_team<false, true, true>);
+        else go(k_reb_team<false, false, true>);
+    } else {
+        if (rank) go(k_reb_team<false, true, false>);
+        else go(k_reb_team<false, false, false>);
+    }
 }
 
 // Grid of a batch controller: warp per graph (begin) or thread per block.
@@ -935,26 +1080,17 @@ inline void clear_ticket(RebalCtl *ctl, cudaStream_t s) {
     UPR_CUDA(cudaMemsetAsync(&ctl->flag, 0, sizeof(int32_t) + sizeof(uint32_t), s));
 }
 
-void rebalance_init(const GraphDev &g, const int64_t *C, int8_t *excl, RebalCtl *ctl, cudaStream_t s) {
-    if (g.ng == 1) {
-        k_reb_init<<<1, 256, 0, s>>>(C, g.Lb, g.K(), excl, ctl);
-    } else {
-        clear_ticket(ctl, s);
-        k_reb_init_batch<<<ctl_grid(g.K()), 256, 0, s>>>(C, g.Lb, g.K(), excl, ctl);
-    }
+void rebalance_init_batch(const GraphDev &g, const int64_t *C, int8_t *excl, RebalCtl *ctl, cudaStream_t s) {
+    clear_ticket(ctl, s);
+    k_reb_init_batch<<<ctl_grid(g.K()), 256, 0, s>>>(C, g.Lb, g.K(), excl, ctl);
     UPR_LAUNCH_CHECK();
 }
 
-void rebalance_begin(const GraphDev &g, const int64_t *C, const int8_t *excl, int8_t *over, int8_t *reject,
-                     const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, int32_t *light, cudaStream_t s,
-                     cudaGraphConditionalHandle cond) {
-    if (g.ng == 1) {
-        k_reb_begin<<<1, 256, 0, s>>>(C, g.Lb, g.k, excl, over, reject, d_n1, max_subrounds, ctl, cond);
-    } else {
-        clear_ticket(ctl, s);
-        k_reb_begin_batch<<<ctl_grid((int64_t)g.ng * 32), 256, 0, s>>>(C, g.Lb, g.k, g.ng, excl, over, reject, d_n1,
-                                                                       max_subrounds, ctl, light);
-    }
+void rebalance_begin_batch(const GraphDev &g, const int64_t *C, const int8_t *excl, int8_t *over, int8_t *reject,
+                           const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, int32_t *light, cudaStream_t s) {
+    clear_ticket(ctl, s);
+    k_reb_begin_batch<<<ctl_grid((int64_t)g.ng * 32), 256, 0, s>>>(C, g.Lb, g.k, g.ng, excl, over, reject, d_n1,
+                                                                   max_subrounds, ctl, light);
     UPR_LAUNCH_CHECK();
 }
 
@@ -972,10 +1108,11 @@ void rebalance_continue(const RebalCtl *ctl, int32_t max_subrounds, cudaGraphCon
     UPR_LAUNCH_CHECK();
 }
 
-void rebalance_end(const GraphDev &g, const int64_t *C, int8_t *excl, const int8_t *reject, const int32_t *d_na,
-                   RebalCtl *ctl, cudaStream_t s) {
+void rebalance_end(const GraphDev &g, const int64_t *C, int8_t *excl, int8_t *reject, int8_t *over,
+                   const int32_t *d_na, const int32_t *d_n1, int32_t max_subrounds, RebalCtl *ctl, cudaStream_t s,
+                   cudaGraphConditionalHandle cond) {
     if (g.ng == 1) {
-        k_reb_end<<<1, 256, 0, s>>>(C, g.Lb, g.K(), excl, reject, d_na, ctl);
+        k_reb_end<<<1, 256, 0, s>>>(C, g.Lb, g.K(), excl, reject, over, d_na, d_n1, max_subrounds, ctl, cond);
     } else {
         clear_ticket(ctl, s);
         k_reb_end_batch<<<ctl_grid(g.K()), 256, 0, s>>>(C, g.Lb, g.K(), excl, reject, d_na, ctl);

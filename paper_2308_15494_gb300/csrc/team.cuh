@@ -35,6 +35,7 @@ constexpr int kSortBins = 256;
 struct Smem {
     unsigned long long cnt64[kTW * kSortBins / 2];     // digit counts [kTW][bins], or block-weight changes
     int tot[kSortBins], bef[kSortBins];
+    unsigned long long rep[kSortBins];
     long long w[kTW];
     __device__ __forceinline__ int *cnt() { return reinterpret_cast<int *>(cnt64); }
 };
@@ -121,14 +122,13 @@ struct __align__(16) Item64 {
     uint32_t val, pad;
 };
 
-// One stable pass on the key bits [shift, shift + bits): the items load(i, it)
-// accepts, i < n, to out[0..count); returns count.  Begins with work of its
-// own segment only; ends with a barrier.
+// One stable pass on the key bits [shift, shift + bits) over the items that
+// load(i, it) accepts, i < n, in two halves with a team barrier between them:
+// sort_count counts the digits of the warps' segments, sort_place writes the
+// items to out[0..count), returns count and ends with a barrier.
 template <class Item, class Load>
-__device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits,
-                                             Item *out) {
+__device__ __forceinline__ void sort_count(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
     const int bins = 1 << bits, mask = bins - 1;
     const Seg g = warp_seg(n);
     int *cnt = s.cnt() + warp * bins;
@@ -158,7 +158,17 @@ __device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, 
         }
         t.hist[blockIdx.x * bins + d] = run;
     }
-    sync(t);
+}
+
+template <class Item, class Load>
+__device__ __forceinline__ int64_t sort_place(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits,
+                                              Item *out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int mask = (1 << bits) - 1;
+    const int bins = 1 << bits;
+    const Seg g = warp_seg(n);
+    int *cnt = s.cnt() + warp * bins;
     // first position of every digit: the totals of the smaller digits, and of
     // this digit in the CTAs before
     {
@@ -174,7 +184,6 @@ __device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, 
     }
     __syncthreads();
     const int mine = threadIdx.x < kSortBins ? s.tot[threadIdx.x] : 0;
-    if (lane == 31) s.w[warp] = 0;
     const long long inc = warp_incl<Sum>(mine);
     if (lane == 31) s.w[warp] = inc;
     __syncthreads();
@@ -208,6 +217,14 @@ __device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, 
     }
     sync(t);
     return count;
+}
+
+template <class Item, class Load>
+__device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits,
+                                             Item *out) {
+    sort_count<Item>(t, s, n, load, shift, bits);
+    sync(t);
+    return sort_place<Item>(t, s, n, load, shift, bits, out);
 }
 
 // Stable sort by the low `bits` key bits of the items load accepts; the
@@ -248,10 +265,12 @@ inline int team_size(int64_t n, int beside) {
 }
 
 template <typename Args>
-inline void launch_team(void (*kern)(Args), const Args &a, int size, cudaStream_t s) {
+inline void launch_team(void (*kern)(Args), const Args &a, int size, cudaStream_t s, size_t shm = 0) {
+    if (shm > 0) kernel_setup((const void *)kern, -1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size);
     cfg.blockDim = dim3(team::kTT);
+    cfg.dynamicSmemBytes = shm;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -1,9 +1,10 @@
-"""The ordered-list phases of a round (the selection's ordering, the move
-sequence, the best prefix) as one cooperative launch each: traces equal to the
+"""The ordered-list phases of a round (the selection's ordering, the rebalancing
+sub-rounds, the move sequence, the best prefix) as one cooperative launch each: traces equal to the
 oracle's where the launch changes shape.  Up to 8192 nodes one CTA runs a
 phase; beyond, the lists are cut into warp segments over several CTAs.  Block
-counts beyond 256 need several sort passes, and scores and blocks of more than
-32 bits together a wider sort item."""
+counts beyond 256 need several sort passes (and a rebalancing sub-round sorts
+by block), scores and blocks of more than 32 bits together a wider sort item,
+heavy nodes 128-bit rebalancing keys."""
 from __future__ import annotations
 
 import numpy as np
@@ -32,6 +33,8 @@ CASES = {
     "blocks_two_passes": lambda: synth.random_small(64, 12001, 6.0, 300, weighted=False),
     "wide_items": lambda: synth.random_small(65, 9001, 6.0, 11, max_ew=1 << 26),
     "wide_items_one_cta": lambda: synth.random_small(66, 700, 6.0, 8, max_ew=1 << 26),
+    "blocks_sorted_weighted": lambda: synth.random_small(68, 12001, 6.0, 300),
+    "wide_rebalancing_keys": lambda: synth.random_small(69, 9001, 6.0, 8, max_vw=(1 << 24) - 1, max_ew=1 << 20),
     "heavy_nodes": lambda: synth.random_small(67, 20000, 4.0, 5, max_vw=1000),
 }
 
