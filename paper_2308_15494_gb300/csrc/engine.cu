@@ -97,7 +97,7 @@ __global__ void k_fill_i64(int64_t *a, int64_t n, int64_t v) {
 namespace {
 // Slots of the device counters (upr_ctx::counts).
 enum {
-    CNT_CAND = 0, CNT_M, CNT_P, CNT_A, CNT_I, CNT_BADPART = 7, CNT_L1, CNT_X, CNT_OVER0, CNT_INFEAS, CNT_EXACT, CNT_SLOTS = 32
+    CNT_CAND = 0, CNT_M, CNT_P, CNT_A, CNT_I, CNT_BADPART = 7, CNT_L1, CNT_X, CNT_OVER0, CNT_INFEAS, CNT_EXACT, CNT_NB, CNT_SLOTS = 32
 };
 
 // Per-call sums of the step graph's rounds (upr_ctx::dstats): candidates,
@@ -242,8 +242,7 @@ struct upr_ctx {
     int32_t *part0, *part; int64_t *C0, *C, *cut; int32_t *W;
     int64_t *BW, *PW, *F; int8_t *first_slot;
     // node-indexed
-    int32_t *cand_tgt, *cand_gain, *flags, *flags2, *m_pos, *r_to, *r_at, *prop_tgt, *prop_gain;
-    int64_t *cand_s0;
+    int32_t *cand_tgt, *cand_s0, *cand_gain, *flags, *flags2, *m_pos, *r_to, *r_at, *prop_tgt, *prop_gain;
     // lists
     int32_t *idxA, *L1;
     int32_t *score;
@@ -265,7 +264,7 @@ struct upr_ctx {
     int32_t *counts;          // device counters (CNT_* slots)
     RebalCtl *ctl;            // rebalancing loop control block
     long long *dstats;        // [16] per-call sums of the step graph's rounds
-    uint64_t *vacc; int32_t *vflags; int64_t *scal, *cut_parts;
+    uint64_t *vacc; int32_t *vflags; int64_t *scal, *cut_in;
     int2 *pk;                 // exact gains: position in I and blocks before/after, per node
     Team team;                // the team launches of this binding
     int beside = 1;           // contexts that refine at the same time as this one, with it
@@ -321,7 +320,7 @@ void layout(upr_ctx *c, Arena &A) {
     c->PW = A.take<int64_t>(k * kSlots);
     c->F = A.take<int64_t>(kSlots);
     c->first_slot = A.take<int8_t>(k);
-    for (int32_t **p : {&c->cand_tgt, &c->cand_gain, &c->flags, &c->m_pos, &c->r_to, &c->prop_tgt,
+    for (int32_t **p : {&c->cand_tgt, &c->cand_s0, &c->cand_gain, &c->flags, &c->m_pos, &c->r_to, &c->prop_tgt,
                         &c->prop_gain, &c->idxA, &c->M_node, &c->M_from, &c->M_to, &c->R_node,
                         &c->R_from, &c->R_to, &c->R_sub, &c->I_node, &c->I_from, &c->I_to, &c->emit, &c->qbefore,
                         &c->pos_m, &c->L1, &c->r_at})
@@ -330,7 +329,6 @@ void layout(upr_ctx *c, Arena &A) {
         *p = A.take<int32_t>(n2 + 1);
     c->diff = A.take<int32_t>(n + 2);
     c->diff_excl = A.take<int32_t>(n + 2);
-    c->cand_s0 = A.take<int64_t>(n);
     c->score = A.take<int32_t>(n);
     c->M_score = A.take<int64_t>(n);
     c->I_gain = A.take<int64_t>(n);
@@ -361,7 +359,7 @@ void layout(upr_ctx *c, Arena &A) {
     c->vacc = A.take<uint64_t>(2);
     c->vflags = A.take<int32_t>(2);
     c->scal = A.take<int64_t>(4);    // [0] wmax, [1] degree sum of M, [2] degree sum of undone moves
-    c->cut_parts = A.take<int64_t>(kCutParts + 1);   // twice the input cut: partial sums, total
+    c->cut_in = A.take<int64_t>(ng);                 // the input cut per graph (the first round's node pass)
     c->pk = A.take<int2>(n);
     c->team.size = team_size((int64_t)n, c->beside);
     c->team.hist = A.take<int32_t>((size_t)c->team.size * team::kSortBins);
@@ -815,7 +813,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     RebalCtl *ctl = c->ctl;
 
     UPR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * CNT_SLOTS, s));
-    if (rebalance_only || n == 0) {     // (else the selection's ordering does it)
+    if (rebalance_only) {               // (else the node pass does it)
         UPR_CUDA(cudaMemcpyAsync(c->part, c->part0, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
         UPR_CUDA(cudaMemcpyAsync(c->C, c->C0, sizeof(int64_t) * K, cudaMemcpyDeviceToDevice, s));
     }
@@ -834,11 +832,20 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         UPR_CUDA(cudaEventRecord(c->ev[4], s));
     }
     if (!rebalance_only) {
-        // ---- (b1) availability, slots, bucket weights; F_r
+        // ---- (b1) availability, slots, bucket weights; F_r; the boundary nodes
         // (the first round of a call also sums the input cut here)
-        buckets(G, c->part0, c->W, c->prm.t_num, c->prm.t_den, c->BW, c->PW, c->first_slot,
-                tr ? tr->avail_d : nullptr, tr ? tr->slot_d : nullptr, s, c->cut_pending ? c->cut_parts : nullptr,
-                c->cut);
+        NodePass np{};
+        np.team = c->team;
+        np.part0 = c->part0; np.C0 = c->C0; np.part = c->part; np.C = c->C;
+        np.t_num = c->prm.t_num; np.t_den = c->prm.t_den;
+        np.BW = reinterpret_cast<unsigned long long *>(c->BW); np.PW = c->PW; np.first = c->first_slot;
+        np.avail_out = tr ? tr->avail_d : nullptr;
+        np.slot_out = tr ? tr->slot_d : nullptr;
+        np.own = c->emit;           // (free until the rebalancing)
+        np.list = c->idxA; np.d_list = cnt + CNT_NB;
+        np.cut_pending = c->cut_pending ? 1 : 0;
+        np.cut = c->cut; np.cut_in = c->cut_in;
+        node_pass(G, np, c->W, s);
         c->cut_pending = false;
         // the step graph reads round i's factors from the per-call table F_all
         const int64_t *F = cap ? c->F_all + (int64_t)c->cap_round * kSlots : c->F;
@@ -858,17 +865,19 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         Penalty pen{c->PW, F, c->C0, kind.limit > 0 ? c->Lsel : c->Lb, c->first_slot};
         set_pack(c, pen);
         // ---- (b2) best move per boundary node
+        const NodeList nl{c->idxA, cnt + CNT_NB};
+        const Candidates cand{c->cand_tgt, c->cand_s0, c->cand_gain};
         run_tuned(c, c->sel_tuned, c->sel_cfg, c->sel_cands, &c->sel_pending, c->ev_tune, [&](LaneCfg cfg) {
-            select_moves(G, c->part0, c->W, pen, c->cand_tgt, c->cand_s0, c->cand_gain, c->flags, cfg, s);
+            select_moves(G, nl, c->part0, c->W, pen, cand, cfg, s);
         });
         if (c->prm.lock_rebalanced)        // the oscillation guard (Sec. 2)
-            guard_filter(c->locked, n, c->flags, c->cand_tgt, c->cand_s0, c->cand_gain, s);
+            guard_filter(c->locked, n, nl, cand, s);
         // ---- (b3) inflow penalties, M ordered by (score desc, id), applied
         SelOrder so{};
         so.team = c->team;
-        so.cand_tgt = c->cand_tgt; so.cand_gain = c->cand_gain; so.cand_s0 = c->cand_s0;
+        so.nl = nl; so.cand = cand;
         so.pen = pen;
-        so.part0 = c->part0; so.C0 = c->C0; so.part = c->part; so.C = c->C;
+        so.part0 = c->part0; so.part = c->part; so.C = c->C;
         so.score = c->score;
         so.c_excl = c->c_excl; so.seg_base = c->seg_base;
         so.bufA = c->sb[0].k; so.bufB = c->sb[1].k;
@@ -1021,12 +1030,25 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
             d2h(T->slot, tr->slot_d, sizeof(int32_t) * n, s);
             d2h(T->bucket, c->BW, sizeof(int64_t) * K * kSlots, s);
             if (T->factor) memcpy(T->factor, c->hF, sizeof(int64_t) * kSlots);
-            d2h(T->cand_target, c->cand_tgt, sizeof(int32_t) * n, s);
-            d2h(T->cand_s0, c->cand_s0, sizeof(int64_t) * n, s);
+            // (by boundary-list index on the device)
+            const int32_t nb = hc[CNT_NB];
+            std::vector<int32_t> node(nb), tgt(nb), s0(nb), gain(nb);
+            d2h(node.data(), c->idxA, sizeof(int32_t) * nb, s);
+            d2h(tgt.data(), c->cand_tgt, sizeof(int32_t) * nb, s);
+            d2h(s0.data(), c->cand_s0, sizeof(int32_t) * nb, s);
+            d2h(gain.data(), c->cand_gain, sizeof(int32_t) * nb, s);
+            UPR_CUDA(cudaStreamSynchronize(s));
+            for (int64_t v = 0; v < n; v++) {
+                if (T->cand_target) T->cand_target[v] = -1;
+                if (T->cand_s0) T->cand_s0[v] = 0;
+                if (T->cand_gain) T->cand_gain[v] = 0;
+            }
+            for (int32_t i = 0; i < nb; i++) {
+                if (T->cand_target) T->cand_target[node[i]] = tgt[i];
+                if (T->cand_s0) T->cand_s0[node[i]] = s0[i];
+                if (T->cand_gain) T->cand_gain[node[i]] = gain[i];
+            }
         }
-        std::vector<int32_t> tmp(rebalance_only ? 0 : n);
-        if (T->cand_gain && !rebalance_only)
-            UPR_CUDA(cudaMemcpyAsync(tmp.data(), c->cand_gain, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s));
         d2h(T->M_node, c->M_node, sizeof(int32_t) * nM, s);
         d2h(T->M_to, c->M_to, sizeof(int32_t) * nM, s);
         d2h(T->M_score, c->M_score, sizeof(int64_t) * nM, s);
@@ -1045,8 +1067,6 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         UPR_CUDA(cudaMemcpyAsync(df.data(), c->diff, sizeof(int32_t) * (nI + 1), cudaMemcpyDeviceToHost, s));
         UPR_CUDA(cudaMemcpyAsync(de.data(), c->diff_excl, sizeof(int32_t) * (nI + 1), cudaMemcpyDeviceToHost, s));
         UPR_CUDA(cudaStreamSynchronize(s));
-        if (T->cand_gain && !rebalance_only)
-            for (int64_t v = 0; v < n; v++) T->cand_gain[v] = tmp[v];
         if (T->I_eligible)
             for (int64_t j = 0; j <= nI; j++) T->I_eligible[j] = (hc[CNT_OVER0] + de[j] + df[j]) == 0;
         T->cut_before = *c->hcut;
@@ -1142,8 +1162,8 @@ __global__ void k_part_to_local(const int32_t *part, const int32_t *part_in, con
     }
 }
 
-// need_cut = false: the cut is left to the first round's bucket pass (one
-// graph, a refinement round follows).
+// need_cut = false: the cut is left to the first round's node pass (a
+// refinement round follows).
 upr_status load_part(upr_ctx *c, const int32_t *part, bool need_cut = true) {
     c->table_valid = false;
     copy_in(c->part0, part, sizeof(int32_t) * c->n, c->s);
@@ -1230,9 +1250,13 @@ int lp_round_once(upr_ctx *c, int64_t *cut, int64_t *active_next, RoundInfo &ri)
     UPR_LAUNCH_CHECK();
     Penalty pen{c->PW, c->F, c->C0, c->Lsel, c->first_slot};
     set_pack(c, pen);
-    select_moves(G, c->part0, c->W, pen, c->cand_tgt, c->cand_s0, c->cand_gain, c->flags, c->sel_cfg, s);
-    lp_list(LpList{c->team, c->flags, c->lp_active, n, c->idxA, cnt + CNT_M}, s);
-    lp_apply(G, c->idxA, cnt + CNT_M, c->cand_tgt, c->cand_gain, c->part0, c->part, c->C, c->M_node, c->M_from,
+    // the active nodes' best moves; the movers as indices of that list
+    const NodeList nl{c->idxA, cnt + CNT_NB};
+    const Candidates cand{c->cand_tgt, c->cand_s0, c->cand_gain};
+    lp_list(LpList{c->team, c->lp_active, nullptr, nullptr, n, c->idxA, cnt + CNT_NB}, s);
+    select_moves(G, nl, c->part0, c->W, pen, cand, c->sel_cfg, s);
+    lp_list(LpList{c->team, nullptr, c->cand_tgt, nl.d_n, n, c->qbefore, cnt + CNT_M}, s);
+    lp_apply(G, c->qbefore, cnt + CNT_M, nl, cand, c->part0, c->part, c->C, c->M_node, c->M_from,
              c->M_to, c->M_score, c->m_pos, c->scal + 1, n, s);
     table_move(G, c->W, c->M_node, c->M_from, c->M_to, cnt + CNT_M, nullptr, c->scal + 1, n, c->hub_chunks,
                c->n_chunks, HubMoves{c->m_pos, nullptr, nullptr, nullptr, nullptr, c->M_from, c->M_to}, s);
@@ -1483,10 +1507,10 @@ upr_status refine_impl(upr_ctx *c, int32_t *part, int32_t rounds, upr_stats *sta
     c->lp_attempts = 0;
     UPR_CUDA(cudaEventRecord(c->ev[2], c->s));
     UPR_CUDA(cudaMemsetAsync(c->scal + 3, 0, sizeof(int64_t), c->s));     // degrees of the sequences' nodes
-    // one graph with a balanced input: the first round's bucket pass, which
-    // reads omega(v, V_P(v)) and omega(I(v)) of every node anyway, gives the
-    // cut, instead of a pass over the edges
-    bool defer_cut = ng == 1 && rounds >= 1 && sch == 0 && c->prm.lp_rounds == 0;
+    // a balanced input: the first round's node pass, which reads omega(v,
+    // V_P(v)) and omega(I(v)) of every node anyway, gives the cut (of every
+    // graph), instead of a pass over the edges
+    bool defer_cut = rounds >= 1 && sch == 0 && c->prm.lp_rounds == 0;
     // label propagation on the dense table: its first build gives the cut
     const bool lp_cut = ng == 1 && c->prm.lp_rounds > 0 && !c->G.sp.on();
     upr_status rc = load_part(c, part, !defer_cut && !lp_cut);
@@ -1495,7 +1519,7 @@ upr_status refine_impl(upr_ctx *c, int32_t *part, int32_t rounds, upr_stats *sta
     read_i64(c, c->C0, K, C0h.data());
     bool bal_in = true;
     for (int32_t b = 0; b < K; b++) bal_in = bal_in && C0h[b] <= c->Lmax_g[b / c->k];
-    if (defer_cut && !bal_in) {     // the repair round comes first and has no bucket pass
+    if (defer_cut && !bal_in) {     // the repair round comes first and has no node pass
         edge_cut(c->G, c->part0, c->cut, c->s);
         c->cut_pending = false;
         defer_cut = false;
@@ -1620,9 +1644,8 @@ upr_status refine_impl(upr_ctx *c, int32_t *part, int32_t rounds, upr_stats *sta
     store_part(c, part, keep);
     read_i64(c, c->cut, ng, cout.data());
     if (defer_cut) {
-        read_i64(c, c->cut_parts + kCutParts, 1, cin.data());
-        cin[0] /= 2;
-        st.cut_in = cin[0];
+        read_i64(c, c->cut_in, ng, cin.data());
+        for (int64_t x : cin) st.cut_in += x;
     }
     st.cut_out = 0;
     for (int32_t g = 0; g < ng; g++) {

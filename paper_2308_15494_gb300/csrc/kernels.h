@@ -231,13 +231,36 @@ struct Penalty {
     int pack_bits = 0;
     int gbits = 0;
 };
-// With cut2 (kCutParts + 1 words; one graph): also sums twice the cut of part
-// (Sec. 2: the sum over v of omega(I(v)) - omega(v, V_P(v))) into
-// cut2[kCutParts] and writes the cut to *cut.
-constexpr int kCutParts = 256;
-void buckets(const GraphDev &g, const int32_t *part, const int32_t *W, int32_t t_num, int32_t t_den, int64_t *BW,
-             int64_t *PW, int8_t *first, int8_t *avail_out, int32_t *slot_out, cudaStream_t s,
-             int64_t *cut2 = nullptr, int64_t *cut = nullptr);
+// A list of nodes (device memory) and the selection's results by list index:
+// best target (-1: no candidate), score, gain.
+struct NodeList { const int32_t *node, *d_n; };
+struct Candidates { int32_t *tgt, *s0, *gain; };
+// Buckets and their prefixes, part = part0 and C = C0, the boundary nodes in
+// node order, and with cut_pending the cut of part0 per graph (cut and cut_in).
+struct NodePass {
+    Team team;
+    const int32_t *part0;
+    const int64_t *C0;
+    int32_t *part;
+    int64_t *C;
+    int32_t t_num, t_den;
+    unsigned long long *BW;
+    int64_t *PW;
+    int8_t *first;
+    int8_t *avail_out;                        // nullable
+    int32_t *slot_out;                        // nullable
+    int32_t *own;                             // [n] omega(v, V_P(v))
+    int32_t *list, *d_list;
+    int cut_pending;
+    int64_t *cut, *cut_in;                    // [ng]
+    // set by node_pass
+    int64_t n = 0;
+    int32_t k = 0, kmask = 0, K = 0, ng = 0;
+    int use_shared = 0;
+    const int32_t *W = nullptr, *wI = nullptr, *vwgt = nullptr, *gid = nullptr;
+    SparseRows sp{};
+};
+void node_pass(const GraphDev &g, NodePass a, const int32_t *W, cudaStream_t s);
 // Lanes per node (G) and 16-byte chunks per lane (CH) of the vectorised
 // selection and proposal kernels (k % 4 == 0, k <= 256, 4*G*CH >= k).  A
 // schedule only decides how the work is spread over lanes, never the
@@ -245,20 +268,19 @@ void buckets(const GraphDev &g, const int32_t *part, const int32_t *W, int32_t t
 struct LaneCfg { int32_t G, CH; };
 // The schedules worth timing for k (the default first); returns their number (0..3).
 int lane_candidates(int32_t k, LaneCfg *out);
-void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Penalty pen, int32_t *cand_tgt,
-                  int64_t *cand_s0, int32_t *cand_gain, int32_t *flags, LaneCfg cfg, cudaStream_t s);
+void select_moves(const GraphDev &g, NodeList nl, const int32_t *part, const int32_t *W, Penalty pen, Candidates out,
+                  LaneCfg cfg, cudaStream_t s);
 // Step (b3): the candidates' inflow penalties, M in its order and applied
 // (team.cuh).  bufA / bufB: 16 n bytes each.
 struct SelOrder {
     Team team;
-    const int32_t *cand_tgt, *cand_gain;      // [n] best target (-1: no candidate) and its gain
-    const int64_t *cand_s0;                   // [n] score without inflow
+    NodeList nl;
+    Candidates cand;
     Penalty pen;
     const int32_t *part0;
-    const int64_t *C0;
-    int32_t *part;                            // [n] becomes part0 with M applied
-    int64_t *C;                               // [K] becomes C0 with M applied
-    int32_t *score;                           // [n] kept score of a candidate, else 0
+    int32_t *part;                            // [n] part0; becomes part0 with M applied
+    int64_t *C;                               // [K] likewise
+    int32_t *score;                           // [n] kept score by list index, else 0
     int64_t *c_excl, *seg_base;               // [n], [K] scratch
     void *bufA, *bufB;
     int32_t *M_node, *M_from, *M_to;
@@ -267,7 +289,6 @@ struct SelOrder {
     int64_t *deg_sum;                         // degree sum of M
     int32_t *d_cand, *d_moves;                // candidates, |M|
     // set by select_order
-    int64_t n = 0;
     int K = 0, kbits = 0;
     const int32_t *vwgt = nullptr;
     const int64_t *xadj = nullptr;
@@ -474,8 +495,7 @@ struct Rollback {
 // r_to >= 0); and no candidate among the locked nodes.
 void guard_locks(const struct Rollback &rb, int64_t max, int64_t n, const int32_t *m_pos, const int32_t *r_to,
                  int8_t *locked, cudaStream_t s);
-void guard_filter(const int8_t *locked, int64_t n, int32_t *flags, int32_t *cand_tgt, int64_t *cand_s0,
-                  int32_t *cand_gain, cudaStream_t s);
+void guard_filter(const int8_t *locked, int64_t n_max, NodeList nl, Candidates cand, cudaStream_t s);
 // W(P o I) -> W(P o I^{j*}): delta updates of the undone moves (pk: positions
 // in I), or nothing when 4 * (their degree sum *deg_sum; a batch's is summed
 // here, onto the 0 that seq_best left) >= m, in which case the caller rebuilds
@@ -495,19 +515,21 @@ void seq_apply_prefix_seg(const GraphDev &g, const int32_t *I_node, const int32_
 // ---- lp.cu: unconstrained label propagation (Sec. 5)
 // active[v] = 1 for the boundary nodes of part (table W of part)
 void lp_boundary(const GraphDev &g, const int32_t *part, const int32_t *W, int8_t *active, cudaStream_t s);
-// list[0..*d_cnt) = the active nodes with a set flag, in node order
+// list[0..*d_cnt) = the active nodes (active given, i < n), or the indices of
+// the candidates (tgt given, i < *d_n), ascending
 struct LpList {
     Team team;
-    const int32_t *flags;
     const int8_t *active;
+    const int32_t *tgt, *d_n;
     int64_t n;
     int32_t *list, *d_cnt;
 };
 void lp_list(const LpList &a, cudaStream_t s);
-// the listed movers (d_cnt of them, node order) to cand_tgt: part (a copy of
-// part0), C, the move list, m_pos markers and the movers' degree sum
-void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, const int32_t *cand_tgt,
-              const int32_t *cand_gain, const int32_t *part0, int32_t *part, int64_t *C, int32_t *M_node,
+// the listed candidates (indices into nl, d_cnt of them, ascending) to their
+// targets: part (a copy of part0), C, the move list, m_pos markers and the
+// movers' degree sum
+void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, NodeList nl, Candidates cand,
+              const int32_t *part0, int32_t *part, int64_t *C, int32_t *M_node,
               int32_t *M_from, int32_t *M_to, int64_t *M_score, int32_t *m_pos, int64_t *deg_sum, int64_t max_count,
               cudaStream_t s);
 // next[u] = 1 for the unmoved neighbours u of the nodes whose block changed

@@ -17,20 +17,21 @@ __global__ void k_lp_boundary(const GraphDev g, const int32_t *__restrict__ part
     }
 }
 
-// The movers, in node order: candidates in V_a.
+// The nodes of V_a, or the indices of the candidates among them, ascending.
 __global__ void __launch_bounds__(team::kTT, 1) k_lp_list(const LpList a) {
     __shared__ team::Smem s;
     const int lane = threadIdx.x & 31;
-    const team::Seg g = team::warp_seg(a.n);
+    const team::Seg g = team::warp_seg(a.active ? a.n : (int64_t)*a.d_n);
+    auto in = [&](int64_t v) { return a.active ? a.active[v] != 0 : a.tgt[v] >= 0; };
     long long cnt = 0;
-    for (int64_t v = g.b + lane; v < g.e; v += 32) cnt += a.flags[v] && a.active[v];
+    for (int64_t v = g.b + lane; v < g.e; v += 32) cnt += in(v);
     const long long mine = team::publish<team::Sum>(a.team, s, 0, team::warp_all<team::Sum>(cnt));
     team::sync(a.team);
     long long all;
     int64_t pos = team::collect<team::Sum>(a.team, 0, &all) + mine;
     for (int64_t v0 = g.b; v0 < g.e; v0 += 32) {
         const int64_t v = v0 + lane;
-        const bool f = v < g.e && a.flags[v] && a.active[v];
+        const bool f = v < g.e && in(v);
         const unsigned m = __ballot_sync(0xffffffffu, f);
         if (f) a.list[pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
         pos += __popc(m);
@@ -41,8 +42,8 @@ __global__ void __launch_bounds__(team::kTT, 1) k_lp_list(const LpList a) {
 // All moves at once: the listed nodes (node order) to their targets; the move
 // list M (for the table update and the markers), block weights, and the
 // degree sum of the moved nodes (delta update or rebuild).
-__global__ void k_lp_apply(const int32_t *__restrict__ movers, const int32_t *__restrict__ d_cnt,
-                           const int32_t *__restrict__ cand_tgt, const int32_t *__restrict__ cand_gain,
+__global__ void k_lp_apply(const int32_t *__restrict__ movers, const int32_t *__restrict__ d_cnt, NodeList nl,
+                           Candidates cand,
                            const int32_t *__restrict__ vwgt, const int64_t *__restrict__ xadj,
                            const int32_t *__restrict__ part0, int32_t *__restrict__ part,
                            unsigned long long *__restrict__ C, int32_t K, int32_t *__restrict__ M_node,
@@ -58,14 +59,14 @@ __global__ void k_lp_apply(const int32_t *__restrict__ movers, const int32_t *__
         int32_t a = -1, b = -1;
         long long c = 0;
         if (p < cnt) {
-            const int32_t v = movers[p];
+            const int32_t i = movers[p], v = nl.node[i];
             a = part0[v];
-            b = cand_tgt[v];
+            b = cand.tgt[i];
             c = vwgt ? vwgt[v] : 1;
             M_node[p] = v;
             M_from[p] = a;
             M_to[p] = b;
-            M_score[p] = cand_gain[v];
+            M_score[p] = cand.gain[i];
             m_pos[v] = (int32_t)p;
             part[v] = b;
             degs += xadj[v + 1] - xadj[v];
@@ -215,8 +216,8 @@ void lp_boundary(const GraphDev &g, const int32_t *part, const int32_t *W, int8_
 
 void lp_list(const LpList &a, cudaStream_t s) { launch_team(k_lp_list, a, a.team.size, s); }
 
-void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, const int32_t *cand_tgt,
-              const int32_t *cand_gain, const int32_t *part0, int32_t *part, int64_t *C, int32_t *M_node,
+void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, NodeList nl, Candidates cand,
+              const int32_t *part0, int32_t *part, int64_t *C, int32_t *M_node,
               int32_t *M_from, int32_t *M_to, int64_t *M_score, int32_t *m_pos, int64_t *deg_sum, int64_t max_count,
               cudaStream_t s) {
     UPR_CUDA(cudaMemsetAsync(deg_sum, 0, sizeof(int64_t), s));
@@ -224,7 +225,7 @@ void lp_apply(const GraphDev &g, const int32_t *movers, const int32_t *d_cnt, co
     const int32_t K = g.K();
     const size_t shm = block_delta_smem(K);
     const int64_t blocks = std::min<int64_t>(ceil_div(max_count, 256), (int64_t)device_sm_count() * 4);
-    k_lp_apply<<<(unsigned)blocks, 256, shm, s>>>(movers, d_cnt, cand_tgt, cand_gain, g.vwgt, g.xadj, part0, part,
+    k_lp_apply<<<(unsigned)blocks, 256, shm, s>>>(movers, d_cnt, nl, cand, g.vwgt, g.xadj, part0, part,
                                                   (unsigned long long *)C, K, M_node, M_from, M_to, M_score, m_pos,
                                                   (unsigned long long *)deg_sum);
     UPR_LAUNCH_CHECK();

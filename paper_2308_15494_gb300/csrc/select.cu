@@ -73,114 +73,158 @@ __device__ __forceinline__ int64_t penalty(const Penalty &p, int32_t b, int64_t 
     return (int64_t)(((u128)(uint64_t)cu * (uint64_t)p.F[lo]) >> kQ);
 }
 
-__global__ void k_buckets(const int32_t *__restrict__ part, const int32_t *__restrict__ W,
-                          const int32_t *__restrict__ wI, const int32_t *__restrict__ vwgt, int64_t n, int32_t k,
-                          int32_t kmask, int32_t K, int32_t t_num, int32_t t_den, unsigned long long *__restrict__ BW,
-                          int use_shared, int8_t *__restrict__ avail_out, int32_t *__restrict__ slot_out,
-                          SparseRows sp, unsigned long long *__restrict__ cut2) {
-    extern __shared__ unsigned long long s_bw[];
+// (b1) in one team launch: availability, slots and bucket weights of every
+// node, the bucket prefixes, the round-start cut when it is still unknown (the
+// sum over the nodes of omega(I(v)) - omega(v, V_P(v)) is twice the cut, Sec.
+// 2), and the list of the boundary nodes in node order, which the selection
+// and the ordering work on (a node with all its neighbours in its own block
+// has no block to move to).  The working partition and block weights start
+// from the round's.  Bound by the gather of one table sector per node, four
+// in flight per thread; 1024 threads share one histogram, where 256-thread
+// CTAs fitted the weighted one of K = 256 (149 KB) only once per SM and took
+// 298 us for 2^22 nodes with hashed rows.
+__global__ void __launch_bounds__(team::kTT, 1) k_node_pass(const NodePass a) {
+    __shared__ team::Smem s;
     __shared__ uint64_t s_p3[41];
-    for (int i = threadIdx.x; i < 41; i += blockDim.x) s_p3[i] = c_pow3[i];
-    const int bins = K * kSlots;
+    extern __shared__ unsigned long long s_bw[];
+    const Team &t = a.team;
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const int64_t n = a.n;
+    const int bins = a.K * kSlots;
+    unsigned int *s_bw32 = reinterpret_cast<unsigned int *>(s_bw);
+    for (int i = threadIdx.x; i < 41; i += team::kTT) s_p3[i] = c_pow3[i];
+    if (a.use_shared)
+        for (int i = threadIdx.x; i < (a.vwgt ? 2 : 1) * bins; i += team::kTT) s_bw32[i] = 0;
+    UPR_TEAM_FOR(b, a.K) a.C[b] = a.C0[b];
     __syncthreads();
-    if (use_shared) {
-        // (unit weights: 32-bit counts, half the words)
-        unsigned int *s_w32 = reinterpret_cast<unsigned int *>(s_bw);
-        for (int i = threadIdx.x; i < (vwgt ? 2 : 1) * bins; i += blockDim.x) s_w32[i] = 0;
-        __syncthreads();
-    }
-    long long out_w = 0;      // weight of the edges leaving v's block, summed over this thread's nodes
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t a = part[v];
-        const int32_t wIv = wI[v];
-        // an isolated node's row is zero: no gather
-        const int64_t own = wIv == 0 ? 0
-                            : sp.on() ? sp_get(sp, v, blk_local(a, k, kmask))
-                                      : W[v * (int64_t)k + blk_local(a, k, kmask)];
-        const int64_t c = vwgt ? vwgt[v] : 1;
-        const bool av = (int64_t)t_den * own >= (int64_t)t_num * (int64_t)wIv;
-        out_w += (long long)wIv - own;
-        const int s = slot_of((uint64_t)own, (uint64_t)c, s_p3);
-        if (av) {
-            if (use_shared && !vwgt)      // unit weights: a CTA's counts fit 32-bit shared-memory atomics
-                atomicAdd(reinterpret_cast<unsigned int *>(s_bw) + a * kSlots + (s - kSlotLo), 1u);
-            else
-                atomicAdd(&(use_shared ? s_bw : BW)[a * kSlots + (s - kSlotLo)], (unsigned long long)c);
-        }
-        if (avail_out) avail_out[v] = av ? 1 : 0;
-        if (slot_out) slot_out[v] = s;
-    }
-    if (use_shared) {
-        __syncthreads();
-        if (!vwgt) {
-            const unsigned int *s_bw32 = reinterpret_cast<const unsigned int *>(s_bw);
-            for (int i = threadIdx.x; i < bins; i += blockDim.x)
-                if (s_bw32[i]) atomicAdd(&BW[i], (unsigned long long)s_bw32[i]);
-        } else {
-            for (int i = threadIdx.x; i < bins; i += blockDim.x)
-                if (s_bw[i]) atomicAdd(&BW[i], s_bw[i]);
-        }
-    }
-    if (cut2) {
-        __shared__ long long s_cw[8];
+    const team::Seg g = team::warp_seg(n);
+    long long cnt = 0, out_w = 0;      // boundary nodes; weight of the edges that leave the nodes' blocks
+    int32_t cur = -1;                  // a batch: the graph out_w belongs to
+    auto flush_cut = [&]() {
         out_w = warp_sum(out_w);
-        if ((threadIdx.x & 31) == 0) s_cw[threadIdx.x >> 5] = out_w;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long t = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += s_cw[w];
-            if (t) atomicAdd(&cut2[blockIdx.x % kCutParts], (unsigned long long)t);
+        if (lane == 0 && cur >= 0 && out_w) atomicAdd(reinterpret_cast<unsigned long long *>(&a.cut[cur]),
+                                                      (unsigned long long)out_w);
+        out_w = 0;
+    };
+    for (int64_t b0 = g.b; b0 < g.e; b0 += 128) {
+        int32_t p[4], wi[4];
+        int64_t own[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int64_t v = b0 + 32 * j + lane;
+            p[j] = v < g.e ? a.part0[v] : 0;
+            wi[j] = v < g.e ? a.wI[v] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int64_t v = b0 + 32 * j + lane;
+            // an isolated node's row is zero: no gather
+            own[j] = wi[j] == 0 ? 0
+                     : a.sp.on() ? sp_get(a.sp, v, blk_local(p[j], a.k, a.kmask))
+                                 : a.W[v * (int64_t)a.k + blk_local(p[j], a.k, a.kmask)];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int64_t v = b0 + 32 * j + lane;
+            const bool in = v < g.e;
+            if (in) {
+                const int64_t c = a.vwgt ? a.vwgt[v] : 1;
+                const bool av = (int64_t)a.t_den * own[j] >= (int64_t)a.t_num * (int64_t)wi[j];
+                const int sl = slot_of((uint64_t)own[j], (uint64_t)c, s_p3);
+                if (av) {
+                    const int at = p[j] * kSlots + (sl - kSlotLo);
+                    if (!a.use_shared) atomicAdd(&a.BW[at], (unsigned long long)c);
+                    else if (!a.vwgt) atomicAdd(&s_bw32[at], 1u);      // (a CTA's counts fit 32 bits)
+                    else atomicAdd(&s_bw[at], (unsigned long long)c);
+                }
+                a.part[v] = p[j];
+                a.own[v] = (int32_t)own[j];
+                if (a.avail_out) a.avail_out[v] = av ? 1 : 0;
+                if (a.slot_out) a.slot_out[v] = sl;
+            }
+            cnt += __popc(__ballot_sync(full, in && own[j] < wi[j]));
+            const long long w = in ? (long long)wi[j] - own[j] : 0;
+            if (!a.cut_pending || !a.gid) {
+                out_w += w;
+            } else {
+                // nodes of one graph are contiguous: the warp keeps a running
+                // sum until its graph changes
+                const int32_t gi = in ? a.gid[v] : -1;
+                const int32_t g0 = __shfl_sync(full, gi, 0);
+                if (!__all_sync(full, gi == cur || gi < 0)) {
+                    flush_cut();
+                    cur = g0;
+                    if (!__all_sync(full, gi == cur || gi < 0)) {       // several graphs in these 32 nodes
+                        if (gi >= 0 && w) atomicAdd(reinterpret_cast<unsigned long long *>(&a.cut[gi]),
+                                                    (unsigned long long)w);
+                        continue;
+                    }
+                }
+                out_w += w;
+            }
         }
     }
-}
-
-// cut2[0 .. kCutParts): partial sums of twice the cut (spread over many words
-// so that the CTAs' atomics do not queue on one address); cut2[kCutParts] =
-// their total; cut = half of it.
-__global__ void __launch_bounds__(kCutParts) k_half_cut(unsigned long long *__restrict__ cut2,
-                                                        int64_t *__restrict__ cut) {
-    __shared__ unsigned long long s_w[kCutParts / 32];
-    unsigned long long v = cut2[threadIdx.x];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < kCutParts / 32; w++) t += s_w[w];
-        cut2[kCutParts] = t;
-        cut[0] = (int64_t)(t / 2);
+    if (a.cut_pending && a.gid) flush_cut();
+    const long long mine = team::publish<team::Sum>(t, s, 0, cnt);
+    team::publish<team::Sum>(t, s, 1, team::warp_all<team::Sum>(out_w));     // (CTA barriers: the histogram is complete)
+    if (a.use_shared)
+        for (int i = threadIdx.x; i < bins; i += team::kTT) {
+            const unsigned long long w = a.vwgt ? s_bw[i] : s_bw32[i];
+            if (w) atomicAdd(&a.BW[i], w);
+        }
+    team::sync(t);
+    long long all;
+    int64_t pos = team::collect<team::Sum>(t, 0, &all) + mine;
+    for (int64_t v0 = g.b; v0 < g.e; v0 += 32) {
+        const int64_t v = v0 + lane;
+        const bool f = v < g.e && a.own[v] < a.wI[v];
+        const unsigned m = __ballot_sync(full, f);
+        if (f) a.list[pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
+        pos += __popc(m);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_list = (int32_t)all;
+    if (a.cut_pending) {
+        if (!a.gid) {
+            long long twice;
+            team::collect<team::Sum>(t, 1, &twice);
+            if (blockIdx.x == 0 && threadIdx.x == 0) a.cut[0] = a.cut_in[0] = twice / 2;
+        } else {
+            UPR_TEAM_FOR(i, a.ng) a.cut[i] = a.cut_in[i] = a.cut[i] / 2;
+        }
+    }
+    // the buckets' prefixes, a warp per block
+    for (int64_t b = blockIdx.x * team::kTW + (threadIdx.x >> 5); b < a.K; b += (int64_t)gridDim.x * team::kTW) {
+        long long run = 0;
+        int first = -1;
+        for (int l0 = 0; l0 < kSlots; l0 += 32) {
+            const int l = l0 + lane;
+            const long long inc = run + team::warp_incl<team::Sum>(l < kSlots ? (long long)a.BW[b * kSlots + l] : 0);
+            if (l < kSlots) a.PW[b * kSlots + l] = inc;
+            const unsigned some = __ballot_sync(full, l < kSlots && inc >= 1);
+            if (first < 0 && some) first = l0 + __ffs(some) - 1;
+            run = __shfl_sync(full, inc, 31);
+        }
+        if (lane == 0) a.first[b] = (int8_t)first;
     }
 }
 
-__global__ void k_bucket_prefix(const int64_t *__restrict__ BW, int64_t *__restrict__ PW, int8_t *__restrict__ first,
-                                int32_t K) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= K) return;
-    int64_t acc = 0;
-    int f = -1;
-    for (int l = 0; l < kSlots; l++) {
-        acc += BW[b * kSlots + l];
-        PW[b * kSlots + l] = acc;
-        if (f < 0 && acc >= 1) f = l;
-    }
-    first[b] = (int8_t)f;
-}
-
+// The selection kernels work on a list of nodes (the boundary nodes in a
+// round, the active nodes in label propagation) and write by list index.
 // G lanes per node: best target by (gain - penalty) among adjacent blocks,
 // ties to the smaller block id; candidate iff the score is positive and v is
 // a boundary node.
 template <int G>
-__global__ void __launch_bounds__(256) k_select(const GraphDev g, const int32_t *__restrict__ part,
-                                                const int32_t *__restrict__ W, Penalty pen,
-                                                int32_t *__restrict__ cand_tgt, int64_t *__restrict__ cand_s0,
-                                                int32_t *__restrict__ cand_gain, int32_t *__restrict__ flags) {
+__global__ void __launch_bounds__(256) k_select(const GraphDev g, NodeList nl, const int32_t *__restrict__ part,
+                                                const int32_t *__restrict__ W, Penalty pen, Candidates out) {
     constexpr int kGroups = 256 / G;
     const int gid = threadIdx.x / G, gl = threadIdx.x % G;
-    const int64_t n = g.n;
+    const int64_t n = *nl.d_n;
     const int32_t k = g.k;
     for (int64_t base = (int64_t)blockIdx.x * kGroups; base < n; base += (int64_t)gridDim.x * kGroups) {
-        const int64_t v = base + gid;
-        const bool active = v < n;
+        const int64_t i = base + gid;
+        const bool active = i < n;
+        const int64_t v = active ? nl.node[i] : 0;
         int64_t best = 0;
         int32_t bt = -1, bg = 0, b0 = 0;
         if (active) {
@@ -210,10 +254,9 @@ __global__ void __launch_bounds__(256) k_select(const GraphDev g, const int32_t 
         const int32_t gsel = group_sum<G>((id >= 0 && bt == id) ? bg : 0);
         if (active && gl == 0) {
             const bool cand = id >= 0 && s > 0;
-            cand_tgt[v] = cand ? b0 + id : -1;
-            cand_s0[v] = cand ? s : 0;
-            cand_gain[v] = cand ? gsel : 0;
-            flags[v] = cand ? 1 : 0;
+            out.tgt[i] = cand ? b0 + id : -1;
+            out.s0[i] = cand ? (int32_t)s : 0;
+            out.gain[i] = cand ? gsel : 0;
         }
     }
 }
@@ -230,15 +273,14 @@ __device__ __forceinline__ int32_t int4_get(const int4 &x, int c) {
 // memory.  A move into a block with room for it costs no penalty and needs no
 // search.
 template <int G, int CH, bool EXACT, bool BATCH, bool PACK = false>
-__global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, const int32_t *__restrict__ part,
+__global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, NodeList nl, const int32_t *__restrict__ part,
                                                     const int32_t *__restrict__ W, Penalty pen, int smem_pw,
-                                                    int32_t *__restrict__ cand_tgt, int64_t *__restrict__ cand_s0,
-                                                    int32_t *__restrict__ cand_gain, int32_t *__restrict__ flags) {
+                                                    Candidates out) {
     // s_slack[b] = L_max - C[b] clamped to 2^31 - 1 (blocks start balanced, so
     // it is >= 0): a node of weight c < 2^31 overfills b iff c > s_slack[b],
     // and then x = c - s_slack[b] is exact.
     extern __shared__ int64_t s_mem[];
-    const int64_t n = g.n;
+    const int64_t n = *nl.d_n;
     const int32_t k = g.k;
     int64_t *s_F = s_mem;
     int64_t *s_PW = s_mem + kSlots;
@@ -310,14 +352,19 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, const int3
                 cst[j][cc] = (kmask - b) - (p >= 0 ? (p << kb) : 0);
             }
     }
-    for (int64_t base = (int64_t)blockIdx.x * kGroups; base < n; base += (int64_t)gridDim.x * kGroups) {
-        const int64_t v = base + gid;
-        const bool active = v < n;
+    // (the next node's id is loaded one iteration ahead, so that a row's load
+    // does not wait for it)
+    const int64_t step = (int64_t)gridDim.x * kGroups;
+    const int64_t i0 = (int64_t)blockIdx.x * kGroups + gid;
+    int32_t vnext = i0 < n ? nl.node[i0] : 0;
+    for (int64_t base = (int64_t)blockIdx.x * kGroups; base < n; base += step) {
+        const int64_t i = base + gid;
+        const bool active = i < n;
+        const int64_t v = vnext;
+        if (i + step < n) vnext = nl.node[i + step];
         int4 r[CH];
         int32_t a = 0, b0 = 0;
         const int4 zero = make_int4(0, 0, 0, 0);
-        // (rows are loaded without waiting for omega(I(v)): skipping the zero
-        // rows of isolated nodes behind that load measured slower)
         const int32_t wIv = active ? g.wI[v] : 0;
         if (active) {
             const int32_t ag = part[v];
@@ -357,10 +404,9 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, const int3
                 const bool cand = pbest >= (1 << kb);
                 const int32_t b = kmask - (pbest & kmask);
                 const int32_t sc = pbest >> kb;
-                cand_tgt[v] = cand ? b0 + b : -1;
-                cand_s0[v] = cand ? sc : 0;
-                cand_gain[v] = cand ? sc + s_pen[b] : 0;
-                flags[v] = cand ? 1 : 0;
+                out.tgt[i] = cand ? b0 + b : -1;
+                out.s0[i] = cand ? sc : 0;
+                out.gain[i] = cand ? sc + s_pen[b] : 0;
             }
             continue;
         }
@@ -417,10 +463,9 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, const int3
         const int32_t gsel = group_sum<G>((id >= 0 && bt == id) ? bg : 0);
         if (active && gl == 0) {
             const bool cand = id >= 0 && sbest > 0;
-            cand_tgt[v] = cand ? b0 + id : -1;
-            cand_s0[v] = cand ? sbest : 0;
-            cand_gain[v] = cand ? gsel : 0;
-            flags[v] = cand ? 1 : 0;
+            out.tgt[i] = cand ? b0 + id : -1;
+            out.s0[i] = cand ? sbest : 0;
+            out.gain[i] = cand ? gsel : 0;
         }
     }
 }
@@ -429,17 +474,17 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, const int3
 // (hash order, so ties compare block ids explicitly); penalties as in
 // k_select_vec with the per-block values read from global memory.
 template <int G>
-__global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, const int32_t *__restrict__ part,
-                                                       Penalty pen, int32_t *__restrict__ cand_tgt,
-                                                       int64_t *__restrict__ cand_s0, int32_t *__restrict__ cand_gain,
-                                                       int32_t *__restrict__ flags) {
+__global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, NodeList nl,
+                                                       const int32_t *__restrict__ part, Penalty pen,
+                                                       Candidates out) {
     constexpr int kGroups = 256 / G;
     const int gid = threadIdx.x / G, gl = threadIdx.x % G;
-    const int64_t n = g.n;
+    const int64_t n = *nl.d_n;
     const SparseRows &sp = g.sp;
     for (int64_t base = (int64_t)blockIdx.x * kGroups; base < n; base += (int64_t)gridDim.x * kGroups) {
-        const int64_t v = base + gid;
-        const bool active = v < n;
+        const int64_t i = base + gid;
+        const bool active = i < n;
+        const int64_t v = active ? nl.node[i] : 0;
         int32_t best = 0, bt = -1, bg = 0, b0 = 0;
         if (active) {
             const int32_t ag = part[v];
@@ -448,8 +493,8 @@ __global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, const i
             const int32_t own = sp_get(sp, v, a);
             if (own < g.wI[v]) {
                 const int32_t c = g.vwgt ? g.vwgt[v] : 1;
-                for (int64_t i = sp.off[v] + gl; i < sp.off[v + 1]; i += G) {
-                    const int2 e = sp.slot[i];
+                for (int64_t q = sp.off[v] + gl; q < sp.off[v + 1]; q += G) {
+                    const int2 e = sp.slot[q];
                     if (e.x == kEmpty || e.y <= own) continue;      // gain <= 0 (the own block among them)
                     const int32_t b = e.x, gain = e.y - own;
                     const int64_t sl = pen.Lb[b0 + b] - pen.C[b0 + b];
@@ -484,10 +529,9 @@ __global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, const i
         const int32_t gsel = group_sum<G>((id >= 0 && bt == id) ? bg : 0);
         if (active && gl == 0) {
             const bool cand = id >= 0 && sbest > 0;
-            cand_tgt[v] = cand ? b0 + id : -1;
-            cand_s0[v] = cand ? sbest : 0;
-            cand_gain[v] = cand ? gsel : 0;
-            flags[v] = cand ? 1 : 0;
+            out.tgt[i] = cand ? b0 + id : -1;
+            out.s0[i] = cand ? sbest : 0;
+            out.gain[i] = cand ? gsel : 0;
         }
     }
 }
@@ -499,23 +543,22 @@ __global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, const i
 // 10 us for lists of 10^4 to 10^6 nodes, nearly all of it latency.
 // Keys hold (largest - score), so their width follows the largest score that
 // occurs, not the largest omega(I(v)): power-law graphs sort in two 8-bit
-// passes where the bound asks for three.  The node itself is the sort's value
-// and the kept scores go to a node-indexed array, so nothing is compacted.
+// passes where the bound asks for three.  The node's index in the boundary
+// list is the sort's value and the kept scores go to an array by that index,
+// so nothing is compacted.
 template <class Item>
 __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     __shared__ team::Smem s;
     const Team &t = a.team;
     const int lane = threadIdx.x & 31;
-    const int64_t n = a.n;
-    // the working partition and block weights start from the round's; the
-    // candidates' largest score
+    const int64_t n = *a.nl.d_n;
+    const Candidates &cd = a.cand;
+    // the candidates' largest score
     uint32_t mx = 0;
-    UPR_TEAM_FOR(v, n) {
-        a.part[v] = a.part0[v];
-        a.score[v] = 0;
-        if (a.cand_tgt[v] >= 0) mx = max(mx, (uint32_t)a.cand_s0[v]);
+    UPR_TEAM_FOR(i, n) {
+        a.score[i] = 0;
+        mx = max(mx, (uint32_t)cd.s0[i]);
     }
-    UPR_TEAM_FOR(b, a.K) a.C[b] = a.C0[b];
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.deg_sum = 0;
     team::publish<team::Max>(t, s, 0, team::warp_all<team::Max>(mx));
     team::sync(t);
@@ -527,12 +570,11 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     Item *bufA = reinterpret_cast<Item *>(a.bufA), *bufB = reinterpret_cast<Item *>(a.bufB);
     const Item *S = team::sort(
         t, s, n,
-        [&](int64_t v, Item &it) {
-            const int32_t tgt = a.cand_tgt[v];
-            if (tgt < 0) return false;
-            it.key = ((Key)tgt << sbits) | (Key)((uint32_t)top - (uint32_t)a.cand_s0[v]);
-            it.val = (uint32_t)v;
-            return true;
+        [&](int64_t i, Item &it) {
+            const int32_t tgt = cd.tgt[i], s0 = cd.s0[i];
+            it.key = ((Key)tgt << sbits) | (Key)((uint32_t)top - (uint32_t)s0);
+            it.val = (uint32_t)i;
+            return tgt >= 0;
         },
         sbits + a.kbits, bufA, bufB, &cand);
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_cand = (int32_t)cand;
@@ -543,7 +585,7 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     long long base = 0;
     if (a.vwgt) {
         long long x = 0;
-        for (int64_t j = g.b + lane; j < g.e; j += 32) x += a.vwgt[S[j].val];
+        for (int64_t j = g.b + lane; j < g.e; j += 32) x += a.vwgt[a.nl.node[S[j].val]];
         const long long mine = team::publish<team::Sum>(t, s, 1, team::warp_all<team::Sum>(x));
         team::sync(t);
         long long all;
@@ -553,7 +595,7 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
         const int64_t j = j0 + lane;
         long long pre = j;
         if (a.vwgt) {
-            const long long c = j < g.e ? a.vwgt[S[j].val] : 0;
+            const long long c = j < g.e ? a.vwgt[a.nl.node[S[j].val]] : 0;
             const long long inc = team::warp_incl<team::Sum>(c);
             pre = base + inc - c;
             base += __shfl_sync(0xffffffffu, inc, 31);
@@ -569,13 +611,12 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     for (int64_t j = g.b + lane; j < g.e; j += 32) {
         const Item it = S[j];
         const int32_t tg = (int32_t)(it.key >> sbits);
-        const int32_t v = (int32_t)it.val;
-        const int64_t c = a.vwgt ? a.vwgt[v] : 1;
+        const int64_t c = a.vwgt ? a.vwgt[a.nl.node[it.val]] : 1;
         const int64_t inflow = (a.vwgt ? a.c_excl[j] : j) - a.seg_base[tg];
         const int64_t p = penalty(a.pen, tg, a.pen.C[tg] + inflow + c - a.pen.Lb[tg], c);
-        const int64_t sc = (int64_t)a.cand_gain[v] - p;
+        const int64_t sc = (int64_t)cd.gain[it.val] - p;
         if (p >= 0 && sc > 0) {
-            a.score[v] = (int32_t)sc;
+            a.score[it.val] = (int32_t)sc;
             kept_top = max(kept_top, (uint32_t)sc);
         }
     }
@@ -589,10 +630,10 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     using team::Item32;
     const Item32 *M = team::sort(
         t, s, n,
-        [&](int64_t v, Item32 &it) {
-            const int32_t sc = a.score[v];
+        [&](int64_t i, Item32 &it) {
+            const int32_t sc = a.score[i];
             it.key = (uint32_t)ktop - (uint32_t)sc;
-            it.val = (uint32_t)v;
+            it.val = (uint32_t)i;
             return sc > 0;
         },
         ktop > 0 ? team::bits_of((uint32_t)ktop - 1) : 0, reinterpret_cast<Item32 *>(a.bufA),
@@ -608,9 +649,9 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
         long long c = 0;
         if (p < gm.e) {
             const Item32 it = M[p];
-            const int32_t v = (int32_t)it.val;
+            const int32_t v = a.nl.node[it.val];
             from = a.part0[v];
-            to = a.cand_tgt[v];
+            to = cd.tgt[it.val];
             c = a.vwgt ? a.vwgt[v] : 1;
             a.M_node[p] = v;
             a.M_from[p] = from;
@@ -632,7 +673,6 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
 
 void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s) {
     if (g.n <= 0) return;
-    a.n = g.n;
     a.K = g.K();
     a.vwgt = g.vwgt;
     a.xadj = g.xadj;
@@ -643,35 +683,23 @@ void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s) {
     else launch_team(k_sel_order<team::Item64>, a, a.team.size, s);
 }
 
-void buckets(const GraphDev &g, const int32_t *part, const int32_t *W, int32_t t_num, int32_t t_den, int64_t *BW,
-             int64_t *PW, int8_t *first, int8_t *avail_out, int32_t *slot_out, cudaStream_t s, int64_t *cut2,
-             int64_t *cut) {
+void node_pass(const GraphDev &g, NodePass a, const int32_t *W, cudaStream_t s) {
     ensure_pow3();
-    const int32_t K = g.K();
-    UPR_CUDA(cudaMemsetAsync(BW, 0, sizeof(int64_t) * K * kSlots, s));
-    unsigned long long *c2 = nullptr;
-    if (cut2) {
-        if (g.ng != 1) throw CudaError{cudaErrorInvalidValue, "buckets: the cut is summed for one graph"};
-        UPR_CUDA(cudaMemsetAsync(cut2, 0, sizeof(int64_t) * (kCutParts + 1), s));
-        c2 = reinterpret_cast<unsigned long long *>(cut2);
-    }
-    if (g.n > 0) {
-        const size_t shm = (g.vwgt ? sizeof(unsigned long long) : sizeof(unsigned int)) * (size_t)K * kSlots;
-        const int use_shared = shm <= 200 * 1024;
-        if (use_shared && shm > 48 * 1024)
-            kernel_setup((const void *)k_buckets, -1);
-        const unsigned blocks = wave_grid((const void *)k_buckets, 256, use_shared ? shm : 0, ceil_div(g.n, 256));
-        k_buckets<<<blocks, 256, use_shared ? shm : 0, s>>>(part, W, g.wI, g.vwgt, g.n, g.k, g.kmask, K,
-                                                                      t_num, t_den, (unsigned long long *)BW,
-                                                                      use_shared, avail_out, slot_out, g.sp, c2);
-        UPR_LAUNCH_CHECK();
-    }
-    if (c2) {
-        k_half_cut<<<1, kCutParts, 0, s>>>(c2, cut);
-        UPR_LAUNCH_CHECK();
-    }
-    k_bucket_prefix<<<(unsigned)ceil_div(K, 128), 128, 0, s>>>(BW, PW, first, K);
-    UPR_LAUNCH_CHECK();
+    a.n = g.n;
+    a.k = g.k;
+    a.kmask = g.kmask;
+    a.K = g.K();
+    a.ng = g.ng;
+    a.W = W;
+    a.sp = g.sp;
+    a.wI = g.wI;
+    a.vwgt = g.vwgt;
+    a.gid = g.gid;
+    UPR_CUDA(cudaMemsetAsync(a.BW, 0, sizeof(int64_t) * a.K * kSlots, s));
+    if (a.cut_pending && g.ng > 1) UPR_CUDA(cudaMemsetAsync(a.cut, 0, sizeof(int64_t) * g.ng, s));
+    const size_t shm = (g.vwgt ? sizeof(unsigned long long) : sizeof(unsigned int)) * (size_t)a.K * kSlots;
+    a.use_shared = shm <= 184 * 1024;            // (the team's own shared memory is static, 37 KB)
+    launch_team(k_node_pass, a, a.team.size, s, a.use_shared ? shm : 0);
 }
 
 int select_group(int k) {
@@ -699,12 +727,11 @@ namespace {
 
 template <int G, int CH>
 void launch_select_vec(bool exact, bool batch, unsigned blocks, size_t shm, cudaStream_t s, const GraphDev &g,
-                       const int32_t *part, const int32_t *W, const Penalty &pen, int smem_pw, int32_t *cand_tgt,
-                       int64_t *cand_s0, int32_t *cand_gain, int32_t *flags) {
+                       NodeList nl, const int32_t *part, const int32_t *W, const Penalty &pen, int smem_pw,
+                       Candidates out) {
     // one full wave of CTAs at most (the kernel loops over the nodes)
     auto go = [&](auto kern) {
-        kern<<<wave_grid((const void *)kern, 256, shm, blocks), 256, shm, s>>>(g, part, W, pen, smem_pw, cand_tgt,
-                                                                             cand_s0, cand_gain, flags);
+        kern<<<wave_grid((const void *)kern, 256, shm, blocks), 256, shm, s>>>(g, nl, part, W, pen, smem_pw, out);
     };
     const bool pack = !batch && pen.pack_bits > 0 && g.vwgt == nullptr;
     if constexpr (CH == 1 || (G == 32 && CH == 2)) {
@@ -722,14 +749,14 @@ void launch_select_vec(bool exact, bool batch, unsigned blocks, size_t shm, cuda
 
 }  // namespace
 
-void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Penalty pen, int32_t *cand_tgt,
-                  int64_t *cand_s0, int32_t *cand_gain, int32_t *flags, LaneCfg cfg, cudaStream_t s) {
+void select_moves(const GraphDev &g, NodeList nl, const int32_t *part, const int32_t *W, Penalty pen, Candidates out,
+                  LaneCfg cfg, cudaStream_t s) {
     if (g.n == 0) return;
     const int k = g.k;
     const bool batch = g.ng > 1;
     if (g.sp.on()) {
         const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(g.n, 256 / 8), (int64_t)sm_count_sel() * 8);
-        k_select_sparse<8><<<blocks, 256, 0, s>>>(g, part, pen, cand_tgt, cand_s0, cand_gain, flags);
+        k_select_sparse<8><<<blocks, 256, 0, s>>>(g, nl, part, pen, out);
         UPR_LAUNCH_CHECK();
         return;
     }
@@ -748,8 +775,7 @@ void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Pena
         const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(g.n, groups), (int64_t)sm_count_sel() * 8);
 #define UPR_SELC(GG, CC)                                                                                       \
     if (G == GG && CH == CC) {                                                                                 \
-        launch_select_vec<GG, CC>(exact, batch, blocks, shm, s, g, part, W, pen, smem_pw, cand_tgt, cand_s0,   \
-                                  cand_gain, flags);                                                           \
+        launch_select_vec<GG, CC>(exact, batch, blocks, shm, s, g, nl, part, W, pen, smem_pw, out);            \
         UPR_LAUNCH_CHECK();                                                                                    \
         return;                                                                                                \
     }
@@ -762,7 +788,7 @@ void select_moves(const GraphDev &g, const int32_t *part, const int32_t *W, Pena
     const int G = select_group(k);
     const int64_t groups = 256 / G;
     const int64_t blocks = std::min<int64_t>(ceil_div(g.n, groups), (int64_t)sm_count_sel() * 16);
-#define UPR_SEL(GG) k_select<GG><<<(unsigned)blocks, 256, 0, s>>>(g, part, W, pen, cand_tgt, cand_s0, cand_gain, flags)
+#define UPR_SEL(GG) k_select<GG><<<(unsigned)blocks, 256, 0, s>>>(g, nl, part, W, pen, out)
     switch (G) {
         case 2: UPR_SEL(2); break;
         case 4: UPR_SEL(4); break;

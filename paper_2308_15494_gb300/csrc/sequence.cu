@@ -788,15 +788,13 @@ __global__ void k_guard_locks(Rollback rb, const int32_t *__restrict__ m_pos, co
 }
 
 // no candidate among the locked nodes
-__global__ void k_guard_filter(const int8_t *__restrict__ locked, int64_t n, int32_t *__restrict__ flags,
-                               int32_t *__restrict__ cand_tgt, int64_t *__restrict__ cand_s0,
-                               int32_t *__restrict__ cand_gain) {
-    UPR_FOR(v, n) {
-        if (!locked[v]) continue;
-        flags[v] = 0;
-        cand_tgt[v] = -1;
-        cand_s0[v] = 0;
-        cand_gain[v] = 0;
+__global__ void k_guard_filter(const int8_t *__restrict__ locked, NodeList nl, Candidates cand) {
+    const int64_t n = *nl.d_n;
+    UPR_FOR(i, n) {
+        if (!locked[nl.node[i]]) continue;
+        cand.tgt[i] = -1;
+        cand.s0[i] = 0;
+        cand.gain[i] = 0;
     }
 }
 
@@ -898,10 +896,9 @@ void guard_locks(const Rollback &rb, int64_t max, int64_t n, const int32_t *m_po
     UPR_LAUNCH_CHECK();
 }
 
-void guard_filter(const int8_t *locked, int64_t n, int32_t *flags, int32_t *cand_tgt, int64_t *cand_s0,
-                  int32_t *cand_gain, cudaStream_t s) {
-    if (n <= 0) return;
-    k_guard_filter<<<grid_for(n), 256, 0, s>>>(locked, n, flags, cand_tgt, cand_s0, cand_gain);
+void guard_filter(const int8_t *locked, int64_t n_max, NodeList nl, Candidates cand, cudaStream_t s) {
+    if (n_max <= 0) return;
+    k_guard_filter<<<grid_for(n_max), 256, 0, s>>>(locked, nl, cand);
     UPR_LAUNCH_CHECK();
 }
 
