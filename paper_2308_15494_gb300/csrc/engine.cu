@@ -180,7 +180,6 @@ struct upr_ctx {
     // with sparse rows there is no dense table in the arena: one is allocated
     // here only if a round falls back to it (or for the debug entry point)
     int32_t *W_own = nullptr; size_t W_own_bytes = 0;
-    int32_t sp_buf_cap = 1;
     // the rebalancing loop as one CUDA graph (a while node over one sub-round),
     // built for the binding and the proposal schedule it was captured with
     cudaStream_t s_cap = nullptr;     // capture stream (non-blocking)
@@ -865,7 +864,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         Penalty pen{c->PW, F, c->C0, kind.limit > 0 ? c->Lsel : c->Lb, c->first_slot};
         set_pack(c, pen);
         // ---- (b2) best move per boundary node
-        const NodeList nl{c->idxA, cnt + CNT_NB};
+        const NodeList nl{c->idxA, cnt + CNT_NB, c->emit};
         const Candidates cand{c->cand_tgt, c->cand_s0, c->cand_gain};
         run_tuned(c, c->sel_tuned, c->sel_cfg, c->sel_cands, &c->sel_pending, c->ev_tune, [&](LaneCfg cfg) {
             select_moves(G, nl, c->part0, c->W, pen, cand, cfg, s);
@@ -1771,7 +1770,7 @@ void parallel_segments(int64_t n, int parts, F fn) {
 std::vector<int64_t> bind_key(const upr_ctx *c) {
     static_assert(sizeof(upr_params) % sizeof(int64_t) == 0, "parameters as whole words");
     std::vector<int64_t> key = {c->n, c->m, c->k, c->ng, c->team.size, c->G.kmask, c->G.adjw != nullptr, c->G.vwgt != nullptr,
-                                c->sp_slots, c->sp_buf_cap, c->sparse_on, c->n_chunks, c->n_tiles, c->tile_nodes,
+                                c->sp_slots, c->sparse_on, c->n_chunks, c->n_tiles, c->tile_nodes,
                                 c->gbits, c->cbits, c->wmax, c->Lmax, c->total_w, c->eps_ppm,
                                 (int64_t)(uintptr_t)c->mem, (int64_t)c->mem_bytes, (int64_t)(uintptr_t)c->W};
     const size_t words = sizeof(upr_params) / sizeof(int64_t);
@@ -1896,7 +1895,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
         }
     }
     // staging layout: packed offsets [n + 1], schedule counts [4 nseg], 8
-    // words (totals, largest row, check flag); a batch adds each graph's own
+    // words (totals, check flag); a batch adds each graph's own
     // offsets [n + ng] and the graphs' node and entry offsets [ng + 1] x 2
     const int64_t nseg = sched_segments(n);
     const int64_t xs_need = n + 1 + 4 * nseg + 8 + (ng > 1 ? n + ng + 2 * (ng + 1) : 0);
@@ -1910,7 +1909,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
         }
         c->xs_cap = xs_need;
     }
-    int64_t *sx = c->xs, *scnt = c->xs + n + 1, *stot = scnt + 4 * nseg;   // stot: 4 totals, cap, check flag
+    int64_t *sx = c->xs, *scnt = c->xs + n + 1, *stot = scnt + 4 * nseg;   // stot: 4 totals, -, check flag
     UPR_CUDA(cudaMemsetAsync(stot, 0, 8 * sizeof(int64_t), s));
     if (ng == 1) {
         if (n > 0) copy_in(sx, gs[0].xadj, sizeof(int64_t) * (n + 1), s);
@@ -1939,26 +1938,29 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
         UPR_CUDA(cudaMemcpyAsync(d_eoff, eoff.data(), sizeof(int64_t) * (ng + 1), cudaMemcpyHostToDevice, s));
         xadj_pack(raw, d_noff, d_eoff, ng, n, sx, reinterpret_cast<int32_t *>(stot + 5), s);
     }
-    const int32_t tile_nodes = (int32_t)std::max<int64_t>(4, std::min<int64_t>(512, 8192 / k));
     // sparse rows: a power of two >= min(k, 2 deg(v)) + 1 slots per row (mode 3:
     // min(k, deg(v)) + 1); chosen by size (mode 0) when k >= 128 and the rows
-    // take at most half the bytes of the dense table
+    // take at most half the bytes of the dense table (else the schedules are
+    // counted again for dense tiles)
+    const int32_t dense_nodes = (int32_t)std::max<int64_t>(4, std::min<int64_t>(512, 8192 / k));
     const int mode = prm.table;
-    const int sp_mode = (k % 4 == 0 && k <= kSparseRowMax / 2 && (mode >= 2 || (mode == 0 && k >= 128)))
-                            ? (mode == 3 ? 3 : 1) : 0;
-    sched_count(sx, n, m, tile_nodes, sp_mode, k, scnt, stot, reinterpret_cast<unsigned long long *>(stot + 4), s);
+    int sp_mode = (k % 4 == 0 && k <= kSparseRowMax / 2 && (mode >= 2 || (mode == 0 && k >= 128)))
+                      ? (mode == 3 ? 3 : 1) : 0;
     int64_t *ht = c->h;                      // (the pinned block's first words: free outside a call)
-    UPR_CUDA(cudaMemcpyAsync(ht, stot, 6 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    UPR_CUDA(cudaStreamSynchronize(s));
+    auto count = [&] {
+        sched_count(sx, n, m, sp_mode ? kSparseTileNodes : dense_nodes, sp_mode, k, scnt, stot, s);
+        UPR_CUDA(cudaMemcpyAsync(ht, stot, 6 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        UPR_CUDA(cudaStreamSynchronize(s));
+    };
+    count();
     if ((int32_t)ht[5] != 0) return UPR_ERR_INVALID;
-    const int64_t n_hubs = ht[3];
-    {
-        int64_t total = sp_mode ? ht[2] : 0, buf_cap = sp_mode ? std::max<int64_t>(1, ht[4]) : 1;
-        if (sp_mode && mode == 0 && total * (int64_t)sizeof(int2) * 2 > n * (int64_t)k * (int64_t)sizeof(int32_t))
-            total = 0, buf_cap = 1;
-        c->sp_slots = total;
-        c->sp_buf_cap = (int32_t)buf_cap;
+    if (sp_mode && mode == 0 && ht[2] * (int64_t)sizeof(int2) * 2 > n * (int64_t)k * (int64_t)sizeof(int32_t)) {
+        sp_mode = 0;
+        count();
     }
+    const int32_t tile_nodes = sp_mode ? kSparseTileNodes : dense_nodes;
+    const int64_t n_hubs = ht[3];
+    c->sp_slots = sp_mode ? ht[2] : 0;
     const int sp_write = c->sp_slots > 0 ? sp_mode : 0;
     const auto t_sched = std::chrono::steady_clock::now();
     c->m = m; c->k = k;
@@ -2033,7 +2035,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     UPR_CUDA(cudaMemsetAsync(c->sp_over, 0, sizeof(int32_t), s));
     c->G = GraphDev{n,      m,        k,       ng,   kmask, c->xadj, c->adj, any_adjw ? c->adjw : nullptr,
                     any_vwgt ? c->vwgt : nullptr, c->wI, c->Lb, c->gid,
-                    SparseRows{c->sp_off, c->sparse_on ? c->sp_slot : nullptr, c->sp_over, c->sp_buf_cap}};
+                    SparseRows{c->sp_off, c->sparse_on ? c->sp_slot : nullptr, c->sp_over}};
     if (prm.autotune) recall_tuning(c);
     if (ng > 1) {
         // node -> graph, and graph-local neighbour ids made global

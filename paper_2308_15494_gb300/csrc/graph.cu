@@ -112,9 +112,10 @@ __device__ __forceinline__ uint64_t entry_hash(uint64_t a, uint64_t b, uint64_t 
 // another graph), 4 self loop, 8 edge weight, 16 node weight, 32 duplicate
 // neighbour in a row, 128 a row not strictly increasing (no error: rows with
 // strictly increasing ids have no duplicates, others get the exact duplicate
-// check); asymmetry shows as differing sums of hash(v,u,w) and
-// hash(u,v,w) over the entries (an asymmetric graph whose sums agree passes:
-// probability about 2^-64 for a graph not built against the hash).
+// check); asymmetry shows as differing sums of hash(min, max, w) over the
+// entries (v, u) with v < u and over those with v > u (an asymmetric graph
+// whose sums agree passes: probability about 2^-64 for a graph not built
+// against the hash).
 __global__ void k_validate_entries(const int64_t *__restrict__ xadj, const int32_t *__restrict__ adj,
                                    const int32_t *__restrict__ adjw, const int32_t *__restrict__ gid, int64_t n,
                                    int64_t m, unsigned long long *__restrict__ acc, int32_t *__restrict__ flags) {
@@ -136,8 +137,9 @@ __global__ void k_validate_entries(const int64_t *__restrict__ xadj, const int32
             if (u < 0 || u >= n || (gid && gid[u] != gid[v])) { f |= 2; continue; }
             if (u == v) f |= 4;
             if (w <= 0) f |= 8;
-            h1 += entry_hash((uint64_t)v, (uint64_t)u, (uint64_t)(uint32_t)w);
-            h2 += entry_hash((uint64_t)u, (uint64_t)v, (uint64_t)(uint32_t)w);
+            const uint64_t h = entry_hash((uint64_t)min(v, (int64_t)u), (uint64_t)max(v, (int64_t)u),
+                                          (uint64_t)(uint32_t)w);
+            if (v < u) h1 += h; else h2 += h;
         }
     }
     h1 = warp_sum(h1);
@@ -352,18 +354,12 @@ template <bool WEIGHTED, int LOCAL, int UNROLL>
 __device__ __forceinline__ void table_tile(const TableTile t, const int64_t *__restrict__ xadj,
                                            const int32_t *__restrict__ adj, const int32_t *__restrict__ adjw,
                                            const int32_t *__restrict__ part, int32_t k, int32_t kmask,
-                                           int32_t *__restrict__ W, const SparseRows &sp, bool bulk) {
+                                           int32_t *__restrict__ W, bool bulk) {
     extern __shared__ int4 s_raw[];
     const int nn = t.v1 - t.v0;
     int64_t *s_x = reinterpret_cast<int64_t *>(s_raw);           // nn + 1 row starts
     int *rows = reinterpret_cast<int *>(s_x + ((nn + 2) & ~1));    // nn * k
     for (int i = threadIdx.x; i <= nn; i += blockDim.x) s_x[i] = xadj[t.v0 + i];
-    // hashed rows: the tile's row offsets, fetched now so that the write-out
-    // does not wait for them row by row
-    int64_t *s_off = sp.on() ? reinterpret_cast<int64_t *>(reinterpret_cast<int2 *>(rows + nn * k) + 8 * sp.buf_cap)
-                             : nullptr;
-    if (sp.on())
-        for (int i = threadIdx.x; i <= nn; i += blockDim.x) s_off[i] = sp.off[t.v0 + i];
     // (k % 4 != 0: the rows' block is not a whole number of 16-byte words)
     const bool quads = k % 4 == 0;
     const int words4 = nn * k / 4;
@@ -419,37 +415,6 @@ __device__ __forceinline__ void table_tile(const TableTile t, const int64_t *__r
         }
     }
     __syncthreads();
-    if (sp.on()) {
-        // sparse table: a warp per row fills the row's slots in its own shared
-        // buffer (each non-zero column is claimed once, by the lane that holds
-        // it), then stores them with coalesced 8-byte stores
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        int2 *buf = reinterpret_cast<int2 *>(rows + nn * k) + warp * sp.buf_cap;
-        for (int r = warp; r < nn; r += (int)(blockDim.x >> 5)) {
-            const int64_t o = s_off[r];
-            const uint32_t cap = (uint32_t)(s_off[r + 1] - o);
-            if (cap > (uint32_t)sp.buf_cap) {
-                // a hub: its row is empty here, the chunk pass fills it
-                for (uint32_t i = lane; i < cap; i += 32) sp.slot[o + i] = make_int2(kEmpty, 0);
-                continue;
-            }
-            for (uint32_t i = lane; i < cap; i += 32) buf[i] = make_int2(kEmpty, 0);
-            __syncwarp();
-            for (int c = lane; c < k; c += 32) {
-                const int w = rows[r * k + c];
-                if (!w) continue;
-                uint32_t h = sp_home(c, cap);
-                for (uint32_t i = 0; i < cap; i++) {
-                    if (atomicCAS(&buf[h].x, kEmpty, c) == kEmpty) { buf[h].y = w; break; }
-                    h = (h + 1) & (cap - 1);
-                }
-            }
-            __syncwarp();
-            for (uint32_t i = lane; i < cap; i += 32) sp.slot[o + i] = buf[i];
-            __syncwarp();
-        }
-        return;
-    }
     if (!quads) {
         int32_t *dst1 = W + (int64_t)t.v0 * k;
         for (int i = threadIdx.x; i < nn * k; i += blockDim.x) __stcs(dst1 + i, rows[i]);
@@ -486,10 +451,95 @@ __global__ void __launch_bounds__(256) k_table_tiles(const TableTile *__restrict
                                                         const int32_t *__restrict__ adjw,
                                                         const int32_t *__restrict__ part, int32_t k, int32_t kmask,
                                                         int32_t *__restrict__ W, const int64_t *__restrict__ deg_sum,
-                                                        int64_t m, SparseRows sp, bool bulk) {
+                                                        int64_t m, bool bulk) {
     if (deg_sum && *deg_sum * 4 < m) return;      // the delta update handles this case
     for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-        table_tile<WEIGHTED, LOCAL, UNROLL>(tiles[ti], xadj, adj, adjw, part, k, kmask, W, sp, bulk);
+        table_tile<WEIGHTED, LOCAL, UNROLL>(tiles[ti], xadj, adj, adjw, part, k, kmask, W, bulk);
+        __syncthreads();                          // the next tile reuses the shared memory
+    }
+}
+
+// Hashed rows, tiled: the tile's rows (contiguous in the slot array) are
+// hashed directly in shared memory, one insert per adjacency entry, and stored
+// as one block.  (Summing dense rows first and hashing their non-zero columns
+// reads and zeroes k columns per row for the few blocks a row has: 2.34 ms for
+// 2^22 nodes of average degree 12 at k = 256, against 0.68 ms here.)  The
+// table's rows are min(k, 2 deg) + 1 slots rounded up, so an insert always
+// finds a slot.  Hub rows are left empty for their chunks.
+template <bool WEIGHTED, int LOCAL>
+__global__ void __launch_bounds__(256) k_table_tiles_hashed(const TableTile *__restrict__ tiles, int64_t n_tiles,
+                                                            const int64_t *__restrict__ xadj,
+                                                            const int32_t *__restrict__ adj,
+                                                            const int32_t *__restrict__ adjw,
+                                                            const int32_t *__restrict__ part, int32_t k,
+                                                            int32_t kmask, const int64_t *__restrict__ deg_sum,
+                                                            int64_t m, SparseRows sp) {
+    if (deg_sum && *deg_sum * 4 < m) return;      // the delta update handles this case
+    __shared__ __align__(16) int2 s_slot[kTileSlots];
+    __shared__ int s_x[kSparseTileNodes + 1], s_o[kSparseTileNodes + 1];      // first entry and slot of each row
+    constexpr int kU = 8;                         // entries in flight per thread
+    for (int64_t ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
+        const TableTile t = tiles[ti];
+        const int nn = t.v1 - t.v0;
+        const int64_t o0 = sp.off[t.v0];
+        for (int i = threadIdx.x; i <= nn; i += blockDim.x) {
+            s_x[i] = (int)min(xadj[t.v0 + i] - t.e0, t.e1 - t.e0);
+            s_o[i] = (int)(sp.off[t.v0 + i] - o0);
+        }
+        __syncthreads();
+        // a hub closes its tile: its row starts where the entries end
+        const bool hub = xadj[t.v1] - t.e0 > t.e1 - t.e0;
+        const int rows = hub ? nn - 1 : nn, slots = s_o[rows];
+        for (int i = threadIdx.x; i < slots; i += blockDim.x) s_slot[i] = make_int2(kEmpty, 0);
+        __syncthreads();
+        const int cnt = (int)(t.e1 - t.e0);
+        for (int c0 = threadIdx.x; c0 < cnt; c0 += blockDim.x * kU) {
+            int u[kU], w[kU], p[kU];
+#pragma unroll
+            for (int r = 0; r < kU; r++) {
+                const int e = c0 + r * blockDim.x;
+                u[r] = e < cnt ? __ldcs(adj + t.e0 + e) : 0;
+                w[r] = WEIGHTED ? (e < cnt ? __ldcs(adjw + t.e0 + e) : 0) : 1;
+            }
+#pragma unroll
+            for (int r = 0; r < kU; r++)
+                p[r] = c0 + r * (int)blockDim.x < cnt ? tile_col<LOCAL>(part[u[r]], k, kmask) : 0;
+#pragma unroll
+            for (int r = 0; r < kU; r++) {
+                const int e = c0 + r * blockDim.x;
+                if (e >= cnt) continue;
+                int lo = 0, hi = rows - 1;        // the entry's row: the last one that starts at or before it
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (s_x[mid] <= e) lo = mid; else hi = mid - 1;
+                }
+                const uint32_t cap = (uint32_t)(s_o[lo + 1] - s_o[lo]);
+                int2 *row = s_slot + s_o[lo];
+                uint32_t h = sp_home(p[r], cap);
+                for (uint32_t i = 0; i < cap; i++) {
+                    int key = *(volatile int *)&row[h].x;
+                    if (key == kEmpty) {
+                        key = atomicCAS(&row[h].x, kEmpty, p[r]);
+                        if (key == kEmpty) key = p[r];
+                    }
+                    if (key == p[r]) {
+                        atomicAdd(&row[h].y, w[r]);
+                        break;
+                    }
+                    h = (h + 1) & (cap - 1);
+                }
+            }
+        }
+        __syncthreads();
+        int2 *dst = sp.slot + o0;
+        if (((uintptr_t)dst & 15) == 0) {
+            for (int i = threadIdx.x; i < slots / 2; i += blockDim.x)
+                reinterpret_cast<int4 *>(dst)[i] = reinterpret_cast<const int4 *>(s_slot)[i];
+            if ((slots & 1) && threadIdx.x == 0) dst[slots - 1] = s_slot[slots - 1];
+        } else {
+            for (int i = threadIdx.x; i < slots; i += blockDim.x) dst[i] = s_slot[i];
+        }
+        for (int i = slots + threadIdx.x; i < s_o[nn]; i += blockDim.x) dst[i] = make_int2(kEmpty, 0);
         __syncthreads();                          // the next tile reuses the shared memory
     }
 }
@@ -662,14 +712,6 @@ void validate_duplicates(const GraphDev &g, int32_t *d_flags, const int32_t *hub
     }
 }
 
-size_t table_tile_smem(int32_t k, int32_t nodes, int32_t sparse_buf_cap) {
-    const size_t rows = sizeof(int64_t) * (size_t)((nodes + 2) & ~1) + sizeof(int) * (size_t)nodes * k;
-    // hashed rows: 8 warps' staging buffers and the tile's nodes + 1 row offsets
-    return sparse_buf_cap > 0 ? ((rows + 15) & ~(size_t)15) + 8 * sizeof(int2) * (size_t)sparse_buf_cap +
-                                    sizeof(int64_t) * (size_t)(nodes + 1)
-                              : rows;
-}
-
 // The tiles' dense row blocks are written by one bulk copy each (about 1.5 %
 // faster on the R-MAT build than the threads' streaming stores);
 // UPR_TILE_BULK=0 selects the stores (an A/B switch between equivalent forms)
@@ -679,19 +721,47 @@ bool bulk_rows() {
     return env == 1;
 }
 
+static void gain_table_hubs(const GraphDev &g, const int32_t *part, int32_t *W, const HubChunk *hub_chunks,
+                            int64_t n_chunks, const int64_t *deg_sum, cudaStream_t s) {
+    if (n_chunks <= 0) return;
+    k_table_hub_chunks<<<(unsigned)n_chunks, 512, sizeof(int) * g.k, s>>>(hub_chunks, g.adj, g.adjw, part, g.k, g.kmask,
+                                                                         W, deg_sum, g.m, g.sp);
+    UPR_LAUNCH_CHECK();
+}
+
 void gain_table(const GraphDev &g, const int32_t *part, int32_t *W, const HubChunk *hub_chunks, int64_t n_chunks,
                 const TableTile *tiles, int64_t n_tiles, int32_t tile_nodes, const int64_t *deg_sum, cudaStream_t s) {
     if (g.n == 0) return;
     if (tiles && n_tiles > 0) {
-        const size_t shm = table_tile_smem(g.k, tile_nodes, g.sp.on() ? g.sp.buf_cap : 0);
         const int local = g.ng == 1 ? 0 : g.kmask ? 1 : 2;
+        if (g.sp.on()) {
+            auto launch = [&](auto kern) {
+                const unsigned grid = deg_sum ? wave_grid((const void *)kern, 256, 0, n_tiles) : (unsigned)n_tiles;
+                kern<<<grid, 256, 0, s>>>(tiles, n_tiles, g.xadj, g.adj, g.adjw, part, g.k, g.kmask, deg_sum, g.m,
+                                          g.sp);
+            };
+            if (g.adjw) {
+                if (local == 0) launch(k_table_tiles_hashed<true, 0>);
+                else if (local == 1) launch(k_table_tiles_hashed<true, 1>);
+                else launch(k_table_tiles_hashed<true, 2>);
+            } else {
+                if (local == 0) launch(k_table_tiles_hashed<false, 0>);
+                else if (local == 1) launch(k_table_tiles_hashed<false, 1>);
+                else launch(k_table_tiles_hashed<false, 2>);
+            }
+            UPR_LAUNCH_CHECK();
+            gain_table_hubs(g, part, W, hub_chunks, n_chunks, deg_sum, s);
+            return;
+        }
+        // the tile's row starts and its rows
+        const size_t shm = sizeof(int64_t) * (size_t)((tile_nodes + 2) & ~1) + sizeof(int) * (size_t)tile_nodes * g.k;
         auto launch = [&](auto kern) {
             // about four tiles per SM and the rest of the unified memory as L1:
             // the gathers of part[] need the L1 more than extra CTAs
             kernel_setup((const void *)kern, 64);
             const unsigned grid = deg_sum ? wave_grid((const void *)kern, 256, shm, n_tiles) : (unsigned)n_tiles;
             kern<<<grid, 256, shm, s>>>(tiles, n_tiles, g.xadj, g.adj, g.adjw, part, g.k, g.kmask, W, deg_sum, g.m,
-                                        g.sp, bulk_rows());
+                                        bulk_rows());
         };
         // 16 entries in flight per thread (8 with weights); the default
         // shared/L1 split: a smaller L1 slows the gathers of part[] down
@@ -708,11 +778,7 @@ void gain_table(const GraphDev &g, const int32_t *part, int32_t *W, const HubChu
     } else {
         throw CudaError{cudaErrorInvalidValue, "gain_table: a binding without table tiles"};
     }
-    if (n_chunks > 0) {
-        k_table_hub_chunks<<<(unsigned)n_chunks, 512, sizeof(int) * g.k, s>>>(hub_chunks, g.adj, g.adjw, part, g.k,
-                                                                             g.kmask, W, deg_sum, g.m, g.sp);
-        UPR_LAUNCH_CHECK();
-    }
+    gain_table_hubs(g, part, W, hub_chunks, n_chunks, deg_sum, s);
 }
 
 }  // namespace upr

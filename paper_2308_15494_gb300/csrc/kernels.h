@@ -22,7 +22,6 @@ struct SparseRows {
     const int64_t *off;   // [n+1] first slot of each row
     int2 *slot;           // (local block or kEmpty, weight); null: the table is dense
     int32_t *overflow;
-    int32_t buf_cap;      // largest row of a node of degree <= kHubDegree (the build's staging buffer)
     __host__ __device__ bool on() const { return slot != nullptr; }
 };
 
@@ -145,18 +144,21 @@ void incident_weights(const GraphDev &g, int32_t *wI, int64_t *wmax, cudaStream_
 // *cut = the cut of part (one graph) from the gain table W = W(part) (dense or hashed rows) and omega(I(v)).
 void cut_from_table(const GraphDev &g, const int32_t *part, const int32_t *W, int64_t *cut, cudaStream_t s);
 // A tile of the table build: nodes [v0, v1) and the adjacency entries [e0, e1)
-// of its non-hub nodes (a hub, if any, is the tile's last node).
+// of its non-hub nodes (a hub, if any, is the tile's last node).  With hashed
+// rows its non-hub rows have at most kTileSlots slots.
+constexpr int kTileSlots = 4096;
+constexpr int kSparseTileNodes = 128;         // rows of a tile with hashed rows
 struct TableTile { int64_t e0, e1; int32_t v0, v1; };
 // Static schedules from the packed offsets (bind.cu), over segments of
 // kSchedSegment nodes.  sched_count: cnt[4 s + 0..3] = exclusive offsets of
 // segment s's hub chunks, tiles, hashed-row slots and hubs; tot[0..3] = the
-// totals; *cap_max = the largest hashed row of a non-hub node.  sp_mode 0:
+// totals.  sp_mode 0:
 // no hashed rows, 1: min(k, 2 deg) + 1 slots rounded up to a power of two,
 // 3: min(k, deg) + 1.  sched_write fills the arrays (nullptr: not written).
 constexpr int64_t kSchedSegment = 1024;
 int64_t sched_segments(int64_t n);
 void sched_count(const int64_t *xadj, int64_t n, int64_t m, int tile_nodes, int sp_mode, int32_t k, int64_t *cnt,
-                 int64_t *tot, unsigned long long *cap_max, cudaStream_t s);
+                 int64_t *tot, cudaStream_t s);
 void sched_write(const int64_t *xadj, int64_t n, int64_t m, int tile_nodes, int sp_mode, int32_t k,
                  const int64_t *off, HubChunk *chunks, TableTile *tiles, int64_t *sp_off, int32_t *hubs,
                  cudaStream_t s);
@@ -176,8 +178,6 @@ constexpr int64_t kGatherChunk = 1 << 16;
 void gather_host(const HostSeg *d_segs, int64_t nseg, size_t elem, void *dst, cudaStream_t s);
 void xadj_pack(const int64_t *raw, const int64_t *noff, const int64_t *eoff, int32_t ng, int64_t n, int64_t *out,
                int32_t *bad, cudaStream_t s);
-// Shared memory of one tile of `nodes` rows (plus per-warp row buffers for the sparse table).
-size_t table_tile_smem(int32_t k, int32_t nodes, int32_t sparse_buf_cap);
 // W must hold n*k ints.  Rows of hubs (degree > kHubDegree) are completed by the chunk pass.
 // By the binding's tiles (every binding with nodes has them).
 // With deg_sum: runs only when 4 * (*deg_sum) >= m (the rebuild alternative to table_move).
@@ -231,9 +231,10 @@ struct Penalty {
     int pack_bits = 0;
     int gbits = 0;
 };
-// A list of nodes (device memory) and the selection's results by list index:
+// A list of nodes (device memory; own: given when they are boundary nodes, all
+// nodes' omega(v, V_P(v)) by node) and the selection's results by list index:
 // best target (-1: no candidate), score, gain.
-struct NodeList { const int32_t *node, *d_n; };
+struct NodeList { const int32_t *node, *d_n, *own = nullptr; };
 struct Candidates { int32_t *tgt, *s0, *gain; };
 // Buckets and their prefixes, part = part0 and C = C0, the boundary nodes in
 // node order, and with cut_pending the cut of part0 per graph (cut and cut_in).
