@@ -1,6 +1,4 @@
-// Block-wide scan of 256-thread CTAs, and the grid barrier of cooperative
-// launches (every wait bounded; one that gives up sets the error word, and the
-// launch runs to its end).
+// Block-wide scan of 256-thread CTAs.
 #pragma once
 
 #include "kernels.h"
@@ -43,31 +41,6 @@ __device__ __forceinline__ T block_exclusive(T v, T *s_warp, T *total) {
     if (lane == 0) excl = Op::template identity<T>();
     __syncthreads();
     return Op::template apply<T>(warp_prefix, excl);
-}
-
-// ---- the grid barrier of cooperative launches
-constexpr int kMaxSpin = 1 << 22;            // polls before a wait gives up (error word set)
-
-__device__ __forceinline__ bool gave_up(const int32_t *err) { return *(volatile const int32_t *)err != 0; }
-
-// Grid barrier on a 64-bit arrival counter that only grows: the barrier that
-// a CTA reaches with arrival number `old` ends when the count reaches the
-// next multiple of the grid size.
-__device__ __forceinline__ void grid_sync(unsigned long long *count, int32_t *err) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned long long old = atomicAdd(count, 1ull);
-        const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
-        for (int it = 0;; it++) {
-            unsigned long long v;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
-            if (v >= target) break;
-            if (it >= kMaxSpin || ((it & 1023) == 1023 && gave_up(err))) { atomicOr(err, 2); break; }
-            if (it >= 16) __nanosleep(32);
-        }
-    }
-    __syncthreads();
 }
 
 }  // namespace prim

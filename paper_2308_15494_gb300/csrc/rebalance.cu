@@ -663,39 +663,51 @@ __global__ void __launch_bounds__(team::kTT, 1) k_reb_team(const RebalTeam a) {
             __syncthreads();
         }
         long long cnt = 0;
-        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 32) {
-            const int64_t i = i0 + lane;
-            const bool f = i < g1.e && a.flags[i] != 0;
-            cnt += __popc(__ballot_sync(full, f));
-            if (!a.hist) continue;
-            uint32_t key = kHistEmpty;
-            long long c = 1;
-            if (f) {
-                const int32_t v = a.list[i];
-                c = (long long)weight_of(v);
-                key = (uint32_t)a.lsrc[i] * kPrioBins + bin_of(a.lgain[i], v);
-            }
-            const unsigned peers = __match_any_sync(full, key);
-            long long tot;
-            group_before<UNIT>(peers, c, &tot);
-            if (f && (peers & lt) == 0) {
-                uint32_t h = (key * 0x9E3779B1u) >> 21;          // 11 bits: kHistSlots
-                bool done = false;
-                for (int probe = 0; probe < 32 && !done; probe++) {
-                    uint32_t cur = *(volatile uint32_t *)&s_key[h];
-                    if (cur == kHistEmpty) {
-                        cur = atomicCAS(&s_key[h], kHistEmpty, key);
-                        if (cur == kHistEmpty) cur = key;
-                    }
-                    if (cur == key) {
-                        atomicAdd(&s_val[h], (unsigned long long)tot);
-                        done = true;
-                    }
-                    h = (h + 1) & (kHistSlots - 1);
+        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 128) {
+            bool f[4];
+            uint32_t key[4];
+            long long c[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int64_t i = i0 + 32 * q + lane;
+                f[q] = false;
+                if (i0 + 32 * q >= g1.e) break;
+                f[q] = i < g1.e && a.flags[i] != 0;
+                key[q] = kHistEmpty;
+                c[q] = 1;
+                if (a.hist && f[q]) {
+                    const int32_t v = UNIT ? 0 : a.list[i];
+                    c[q] = (long long)weight_of(v);
+                    key[q] = (uint32_t)a.lsrc[i] * kPrioBins + bin_of(a.lgain[i], v);
                 }
-                if (!done) atomicAdd(&a.hist[key], (unsigned long long)tot);   // crowded: straight to the histogram
             }
-            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (i0 + 32 * q >= g1.e) break;
+                cnt += __popc(__ballot_sync(full, f[q]));
+                if (!a.hist) continue;
+                const unsigned peers = __match_any_sync(full, key[q]);
+                long long tot;
+                group_before<UNIT>(peers, c[q], &tot);
+                if (f[q] && (peers & lt) == 0) {
+                    uint32_t h = (key[q] * 0x9E3779B1u) >> 21;          // 11 bits: kHistSlots
+                    bool done = false;
+                    for (int probe = 0; probe < 32 && !done; probe++) {
+                        uint32_t at = *(volatile uint32_t *)&s_key[h];
+                        if (at == kHistEmpty) {
+                            at = atomicCAS(&s_key[h], kHistEmpty, key[q]);
+                            if (at == kHistEmpty) at = key[q];
+                        }
+                        if (at == key[q]) {
+                            atomicAdd(&s_val[h], (unsigned long long)tot);
+                            done = true;
+                        }
+                        h = (h + 1) & (kHistSlots - 1);
+                    }
+                    if (!done) atomicAdd(&a.hist[key[q]], (unsigned long long)tot);   // crowded: straight there
+                }
+                __syncwarp();
+            }
         }
         const long long mine = team::publish<team::Sum>(t, s, 0, cnt);         // (CTA barriers inside)
         if (a.hist)
@@ -709,17 +721,27 @@ __global__ void __launch_bounds__(team::kTT, 1) k_reb_team(const RebalTeam a) {
         // ---- compacted in node order, and the cut bin of every source
         long long np;
         long long pos = team::collect<team::Sum>(t, 0, &np) + mine;
-        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 32) {
-            const int64_t i = i0 + lane;
-            const bool f = i < g1.e && a.flags[i] != 0;
-            const unsigned m = __ballot_sync(full, f);
-            if (f) {
-                const int64_t p = pos + __popc(m & lt);
-                a.list2[p] = a.list[i];
-                a.lsrc2[p] = a.lsrc[i];
-                a.lgain2[p] = a.lgain[i];
+        for (int64_t i0 = g1.b; i0 < g1.e; i0 += 128) {
+            bool f[4];
+            int32_t v[4], src[4], gain[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int64_t i = i0 + 32 * q + lane;
+                f[q] = i < g1.e && a.flags[i] != 0;
+                if (i < g1.e) { v[q] = a.list[i]; src[q] = a.lsrc[i]; gain[q] = a.lgain[i]; }
             }
-            pos += __popc(m);
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (i0 + 32 * q >= g1.e) break;
+                const unsigned m = __ballot_sync(full, f[q]);
+                if (f[q]) {
+                    const int64_t p = pos + __popc(m & lt);
+                    a.list2[p] = v[q];
+                    a.lsrc2[p] = src[q];
+                    a.lgain2[p] = gain[q];
+                }
+                pos += __popc(m);
+            }
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_np = (int32_t)np;
     }

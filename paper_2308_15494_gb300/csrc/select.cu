@@ -83,6 +83,8 @@ __device__ __forceinline__ int64_t penalty(const Penalty &p, int32_t b, int64_t 
 // in flight per thread; 1024 threads share one histogram, where 256-thread
 // CTAs fitted the weighted one of K = 256 (149 KB) only once per SM and took
 // 298 us for 2^22 nodes with hashed rows.
+constexpr int kSlotTable = 1024;
+
 __global__ void __launch_bounds__(team::kTT, 1) k_node_pass(const NodePass a) {
     __shared__ team::Smem s;
     __shared__ uint64_t s_p3[41];
@@ -94,6 +96,12 @@ __global__ void __launch_bounds__(team::kTT, 1) k_node_pass(const NodePass a) {
     const int bins = a.K * kSlots;
     unsigned int *s_bw32 = reinterpret_cast<unsigned int *>(s_bw);
     for (int i = threadIdx.x; i < 41; i += team::kTT) s_p3[i] = c_pow3[i];
+    // unit weights: the slots of the small omegas, computed once a CTA
+    __shared__ int8_t s_slot[kSlotTable];
+    if (!a.vwgt) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < kSlotTable; i += team::kTT) s_slot[i] = (int8_t)slot_of((uint64_t)i, 1, s_p3);
+    }
     if (a.use_shared)
         for (int i = threadIdx.x; i < (a.vwgt ? 2 : 1) * bins; i += team::kTT) s_bw32[i] = 0;
     UPR_TEAM_FOR(b, a.K) a.C[b] = a.C0[b];
@@ -126,17 +134,22 @@ __global__ void __launch_bounds__(team::kTT, 1) k_node_pass(const NodePass a) {
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
+            if (b0 + 32 * j >= g.e) break;
             const int64_t v = b0 + 32 * j + lane;
             const bool in = v < g.e;
             if (in) {
                 const int64_t c = a.vwgt ? a.vwgt[v] : 1;
                 const bool av = (int64_t)a.t_den * own[j] >= (int64_t)a.t_num * (int64_t)wi[j];
-                const int sl = slot_of((uint64_t)own[j], (uint64_t)c, s_p3);
+                const int sl = !a.vwgt && own[j] < kSlotTable ? s_slot[own[j]]
+                                                              : slot_of((uint64_t)own[j], (uint64_t)c, s_p3);
                 if (av) {
                     const int at = p[j] * kSlots + (sl - kSlotLo);
                     if (!a.use_shared) atomicAdd(&a.BW[at], (unsigned long long)c);
                     else if (!a.vwgt) atomicAdd(&s_bw32[at], 1u);      // (a CTA's counts fit 32 bits)
-                    else atomicAdd(&s_bw[at], (unsigned long long)c);
+                    else {       // 32-bit words with a carry: shared memory has no native 64-bit add
+                        const unsigned int w = (unsigned int)c, old = atomicAdd(&s_bw32[2 * at], w);
+                        if (old + w < old) atomicAdd(&s_bw32[2 * at + 1], 1u);
+                    }
                 }
                 a.part[v] = p[j];
                 a.own[v] = (int32_t)own[j];
@@ -490,8 +503,8 @@ __global__ void __launch_bounds__(256) k_select_sparse(const GraphDev g, NodeLis
             const int32_t ag = part[v];
             const int32_t a = blk_local(g, ag);
             b0 = ag - a;
-            const int32_t own = sp_get(sp, v, a);
-            if (own < g.wI[v]) {
+            const int32_t own = nl.own ? nl.own[v] : sp_get(sp, v, a);
+            if (nl.own || own < g.wI[v]) {
                 const int32_t c = g.vwgt ? g.vwgt[v] : 1;
                 for (int64_t q = sp.off[v] + gl; q < sp.off[v + 1]; q += G) {
                     const int2 e = sp.slot[q];
@@ -608,16 +621,32 @@ __global__ void __launch_bounds__(team::kTT, 1) k_sel_order(const SelOrder a) {
     }
     team::sync(t);
     uint32_t kept_top = 0;
-    for (int64_t j = g.b + lane; j < g.e; j += 32) {
-        const Item it = S[j];
-        const int32_t tg = (int32_t)(it.key >> sbits);
-        const int64_t c = a.vwgt ? a.vwgt[a.nl.node[it.val]] : 1;
-        const int64_t inflow = (a.vwgt ? a.c_excl[j] : j) - a.seg_base[tg];
-        const int64_t p = penalty(a.pen, tg, a.pen.C[tg] + inflow + c - a.pen.Lb[tg], c);
-        const int64_t sc = (int64_t)cd.gain[it.val] - p;
-        if (p >= 0 && sc > 0) {
-            a.score[it.val] = (int32_t)sc;
-            kept_top = max(kept_top, (uint32_t)sc);
+    for (int64_t j0 = g.b + lane; j0 < g.e; j0 += 128) {
+        Item it[4];
+        int32_t gain[4];
+        int64_t c[4], room[4], inflow[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+            if (j0 + 32 * r < g.e) it[r] = S[j0 + 32 * r];
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const int64_t j = j0 + 32 * r;
+            if (j >= g.e) continue;
+            const int32_t tg = (int32_t)(it[r].key >> sbits);
+            gain[r] = cd.gain[it[r].val];
+            c[r] = a.vwgt ? a.vwgt[a.nl.node[it[r].val]] : 1;
+            inflow[r] = (a.vwgt ? a.c_excl[j] : j) - a.seg_base[tg];
+            room[r] = a.pen.Lb[tg] - a.pen.C[tg];
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            if (j0 + 32 * r >= g.e) continue;
+            const int64_t p = penalty(a.pen, (int32_t)(it[r].key >> sbits), inflow[r] + c[r] - room[r], c[r]);
+            const int64_t sc = (int64_t)gain[r] - p;
+            if (p >= 0 && sc > 0) {
+                a.score[it[r].val] = (int32_t)sc;
+                kept_top = max(kept_top, (uint32_t)sc);
+            }
         }
     }
     team::publish<team::Max>(t, s, 2, team::warp_all<team::Max>(kept_top));

@@ -230,12 +230,14 @@ __global__ void __launch_bounds__(team::kTT, 1) k_seq_build(const SeqBuild a) {
                     const int64_t D = a.C0[b] + a.ex[j] + cw(a.vwgt, a.M_node[it.val >> 1]) - a.ex[a.ebeg[b]];
                     if (D > Lmax) {
                         // smallest x in [1, |R_b|] with D - (weight of R_b[0..x)) <= L_max, else |R_b|
-                        const int64_t base = a.ex[r0];
+                        const int64_t base = a.ex[r0], over = D - Lmax;
                         int lo = 1, hi = r1 - r0;
-                        while (lo < hi) {
-                            const int mid = lo + ((hi - lo) >> 1);
-                            if (D - (a.ex[r0 + mid] - base) <= Lmax) hi = mid; else lo = mid + 1;
-                        }
+                        if (!a.vwgt) lo = (int)min((int64_t)hi, over);      // (unit weights: x = the excess)
+                        else
+                            while (lo < hi) {
+                                const int mid = lo + ((hi - lo) >> 1);
+                                if (over <= a.ex[r0 + mid] - base) hi = mid; else lo = mid + 1;
+                            }
                         need = (uint32_t)lo;
                     }
                 }
@@ -300,8 +302,10 @@ __global__ void __launch_bounds__(team::kTT, 1) k_seq_build(const SeqBuild a) {
             sl += __shfl_sync(full, inc, 31);
         }
         team::sync(t);
-        // R's entries: after the event that emits them, or behind M in block order
-        for (int64_t j = g.b + lane; j < g.e; j += 32) {
+        // R's entries: after the event that emits them, or behind M in block
+        // order (strided over the team: they lie in runs, a few segments hold
+        // them all)
+        UPR_TEAM_FOR(j, L) {
             const Item32 it = S[j];
             if (!(it.key & kIsR)) continue;
             const uint32_t b = blk_of(it.key), i = it.val;

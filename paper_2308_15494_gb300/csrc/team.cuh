@@ -31,6 +31,7 @@ constexpr int kTW = kTT / 32;
 constexpr int kTeamMax = 160;            // CTAs at most
 constexpr int kTotSlots = 24;            // published per-CTA totals (one slot per scan of a kernel)
 constexpr int kSortBins = 256;
+constexpr int kMaxSpin = 1 << 22;        // polls before a barrier's wait gives up (error word set)
 
 struct Smem {
     unsigned long long cnt64[kTW * kSortBins / 2];     // digit counts [kTW][bins], or block-weight changes
@@ -40,9 +41,42 @@ struct Smem {
     __device__ __forceinline__ int *cnt() { return reinterpret_cast<int *>(cnt64); }
 };
 
+constexpr int kClusterMax = 16;          // teams up to this size run as one cluster
+
+// The team's barrier: a CTA barrier for one CTA, a cluster barrier for a
+// cluster, else a grid barrier on an arrival counter that only grows: the
+// barrier a CTA reaches with arrival number `old` ends when the count reaches
+// the next multiple of the grid size.  Every wait is bounded: one that gives
+// up sets the error word, and the launch runs to its end.  (About 1.2 us with
+// 152 CTAs.  Arriving without the old value, by a release reduction, took 0.15
+// us longer; an epoch word per CTA polled by a warp of every CTA 1 us longer.)
 __device__ __forceinline__ void sync(const Team &t) {
-    if (gridDim.x == 1) __syncthreads();     // (one CTA: its own writes are visible to it)
-    else prim::grid_sync(t.bar, t.err);
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return;
+    }
+    if (gridDim.x <= kClusterMax) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        return;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned long long old = atomicAdd(t.bar, 1ull);
+        const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
+        for (int it = 0;; it++) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(t.bar) : "memory");
+            if (v >= target) break;
+            if (it >= kMaxSpin || ((it & 1023) == 1023 && *(volatile const int32_t *)t.err != 0)) {
+                atomicOr(t.err, 2);
+                break;
+            }
+            if (it >= 16) __nanosleep(32);
+        }
+    }
+    __syncthreads();
 }
 
 struct Seg { int64_t b, e; };
@@ -202,6 +236,7 @@ __device__ __forceinline__ int64_t sort_place(const Team &t, Smem &s, int64_t n,
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
+            if (b + 32 * j >= g.e) break;             // (uniform over the warp: short segments skip the rest)
             const int d = ok[j] ? (int)(it[j].key >> shift) & mask : -1;
             const unsigned peers = __match_any_sync(0xffffffffu, d);
             const int rank = __popc(peers & lt);
@@ -238,7 +273,7 @@ __device__ __forceinline__ const Item *sort(const Team &t, Smem &s, int64_t n, L
     Item *src = A, *dst = B;
     for (int p = 1; p < passes; p++) {
         const Item *from = src;
-        sort_pass(
+        sort_pass<Item>(
             t, s, cnt, [from](int64_t i, Item &it) { it = from[i]; return true; }, p * per, min(per, bits - p * per),
             dst);
         Item *x = src; src = dst; dst = x;
@@ -251,17 +286,21 @@ __device__ __forceinline__ int bits_of(uint32_t x) { return 32 - __clz((int)x); 
 
 }  // namespace team
 
-// CTAs of the team kernels of a binding of n nodes: one CTA up to 8192 nodes
-// (its barriers are __syncthreads), else one per 1024 nodes, at most one per
-// SM.  A cooperative launch starts only when all its CTAs fit at once, so
+// CTAs of the team kernels of a binding of n nodes: one up to 2048 nodes (its
+// barriers are __syncthreads), else one per 1024 nodes; up to kClusterMax of
+// them as one cluster (its hardware barrier takes a fraction of the 1.2 us of a
+// grid barrier), for graphs of up to 65536 nodes; beyond, at most one per SM.
+// A cooperative launch starts only when all its CTAs fit at once, so
 // contexts that refine side by side (the batches of a mixed context) share
 // the SMs between them; with the whole GPU each, they would wait for one
 // another at every launch (1024 Chung-Lu graphs in five batches: 18.0 ms at
 // 30 CTAs each, 20.5 ms at 152; one batch alone: 18.0 ms at 152, 29.5 ms at 30).
 inline int team_size(int64_t n, int beside) {
-    if (n <= 8192) return 1;
+    if (n <= 2048) return 1;
+    const int64_t want = ceil_div(n, (int64_t)1024);
+    if (n <= 65536) return (int)std::min<int64_t>(want, team::kClusterMax);
     const int sms = std::min(device_sm_count(), team::kTeamMax);
-    return (int)std::min<int64_t>(std::max(8, sms / std::max(1, beside)), ceil_div(n, (int64_t)1024));
+    return (int)std::min<int64_t>(std::max(team::kClusterMax + 1, sms / std::max(1, beside)), want);
 }
 
 template <typename Args>
@@ -273,8 +312,15 @@ inline void launch_team(void (*kern)(Args), const Args &a, int size, cudaStream_
     cfg.dynamicSmemBytes = shm;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    if (size > team::kClusterMax) {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        if (size > 8) UPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    }
     cfg.attrs = attr;
     cfg.numAttrs = size > 1 ? 1 : 0;
     UPR_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
