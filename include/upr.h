@@ -251,7 +251,7 @@ void upr_destroy(upr_ctx *ctx);
  * default) and returns after synchronising it.  Before any kernel indexes
  * with them it checks, on the device, that part is in [0, k), that xadj[0] =
  * 0, xadj[n] = m and xadj is non-decreasing, and that every neighbour id is
- * in [0, n).  Errors: UPR_ERR_INVALID (sizes, k, pointers that are not
+ * in [0, n) (each id by the kernel that reads through it).  Errors: UPR_ERR_INVALID (sizes, k, pointers that are not
  * device memory of the current device, a failed check above), UPR_ERR_CUDA.
  * Symmetry, self loops and weights are not checked (see upr_create's
  * validate). */

@@ -138,8 +138,9 @@ inline unsigned grid_for(int64_t max) {
 struct HubChunk { int32_t v; int32_t pad; int64_t begin, end; };
 // C[0..K) = block weights of part.
 void block_weights(const GraphDev &g, const int32_t *part, int64_t *C, cudaStream_t s);
-// cut[0..ng) = edge cut of each graph.
-void edge_cut(const GraphDev &g, const int32_t *part, int64_t *cut, cudaStream_t s);
+// cut[0..ng) = edge cut of each graph.  bad (given: neighbour ids unchecked so
+// far): set non-zero when one lies outside [0, n); none is read through.
+void edge_cut(const GraphDev &g, const int32_t *part, int64_t *cut, cudaStream_t s, int64_t *bad = nullptr);
 void incident_weights(const GraphDev &g, int32_t *wI, int64_t *wmax, cudaStream_t s);
 // *cut = the cut of part (one graph) from the gain table W = W(part) (dense or hashed rows) and omega(I(v)).
 void cut_from_table(const GraphDev &g, const int32_t *part, const int32_t *W, int64_t *cut, cudaStream_t s);

@@ -34,25 +34,16 @@ __device__ __forceinline__ void set_flag(int32_t flag_slot) {
     atomicOr(reinterpret_cast<unsigned long long *>(&g_noalloc_scratch[flag_slot]), 1ull);
 }
 
-__global__ void k_part_in_range(const int32_t *__restrict__ part, int64_t n, int32_t k, int32_t flag_slot) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n && (part[v] < 0 || part[v] >= k)) set_flag(flag_slot);
-}
-
-// The CSR offsets: xadj[0] = 0, xadj[n] = m, non-decreasing.  The cut kernels
-// find an entry's node by walking xadj, so they run only after this holds.
-__global__ void k_xadj_valid(const int64_t *__restrict__ xadj, int64_t n, int64_t m, int32_t flag_slot) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v > n) return;
-    const bool bad = (v == 0 && xadj[0] != 0) || (v == n && xadj[n] != m) || (v < n && xadj[v + 1] < xadj[v]);
-    if (bad) set_flag(flag_slot);
-}
-
-// Neighbour ids in [0, n): the cut kernels read part[] at every neighbour.
-__global__ void k_adj_in_range(const int32_t *__restrict__ adj, int64_t m, int64_t n, int32_t flag_slot) {
+// The partition in [0, k), and the CSR offsets: xadj[0] = 0, xadj[n] = m,
+// non-decreasing.  The block weights index by part and the cut kernel finds an
+// entry's node from xadj, so both run only after this holds; the cut kernel
+// checks every neighbour id itself before it reads through it.
+__global__ void k_input_valid(const int32_t *__restrict__ part, const int64_t *__restrict__ xadj, int64_t n,
+                              int64_t m, int32_t k, int32_t flag_slot) {
     bool bad = false;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
-        bad |= adj[e] < 0 || adj[e] >= n;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        bad |= part[v] < 0 || part[v] >= k || xadj[v + 1] < xadj[v] || (v == 0 && xadj[0] != 0) ||
+               (v == n - 1 && xadj[n] != m);
     if (__syncthreads_or(bad) && threadIdx.x == 0) set_flag(flag_slot);
 }
 
@@ -81,30 +72,26 @@ extern "C" upr_status upr_cut_noalloc(const upr_graph *g, int32_t k, const int32
     try {
         upr::GraphDev G{g->n, g->m, k, 1, -1, g->xadj, g->adjncy, g->adjwgt, g->vwgt, nullptr, nullptr, nullptr};
         // the flag keeps the previous call's value: clear it first; then the
-        // partition's range and the CSR's offsets and neighbour ids, all
-        // before any kernel that indexes with them
+        // partition's range and the CSR's offsets, before any kernel that
+        // indexes with them
         UPR_CUDA(cudaMemsetAsync(scratch + k + 1, 0, sizeof(int64_t), s));
         if (g->n > 0) {
-            k_part_in_range<<<(unsigned)upr::ceil_div(g->n, 256), 256, 0, s>>>(part, g->n, k, k + 1);
-            UPR_LAUNCH_CHECK();
-            k_xadj_valid<<<(unsigned)upr::ceil_div(g->n + 1, 256), 256, 0, s>>>(g->xadj, g->n, g->m, k + 1);
+            k_input_valid<<<upr::grid_for(g->n), 256, 0, s>>>(part, g->xadj, g->n, g->m, k, k + 1);
             UPR_LAUNCH_CHECK();
         }
-        if (g->m > 0) {
-            const int64_t blocks = std::min<int64_t>(upr::ceil_div(g->m, 256), 4096);
-            k_adj_in_range<<<(unsigned)blocks, 256, 0, s>>>(g->adjncy, g->m, g->n, k + 1);
-            UPR_LAUNCH_CHECK();
-        }
-        int64_t bad = 0;
-        UPR_CUDA(cudaMemcpyAsync(&bad, scratch + k + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        int64_t out[kNoAllocMaxK + 2];          // block weights, cut, flag (the layout of the scratch)
+        UPR_CUDA(cudaMemcpyAsync(out, scratch + k + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         UPR_CUDA(cudaStreamSynchronize(s));
-        if (bad) return UPR_ERR_INVALID;
+        if (out[0] || (g->n == 0 && g->m > 0)) return UPR_ERR_INVALID;     // (no node: no valid neighbour)
         // both wrappers zero their accumulators before accumulating
         upr::block_weights(G, part, scratch, s);
-        upr::edge_cut(G, part, scratch + k, s);
-        UPR_CUDA(cudaMemcpyAsync(cut, scratch + k, sizeof(int64_t), cudaMemcpyDefault, s));
-        if (block_weights)
-            UPR_CUDA(cudaMemcpyAsync(block_weights, scratch, sizeof(int64_t) * k, cudaMemcpyDefault, s));
+        upr::edge_cut(G, part, scratch + k, s, scratch + k + 1);
+        UPR_CUDA(cudaMemcpyAsync(out, scratch, sizeof(int64_t) * (k + 2), cudaMemcpyDeviceToHost, s));
+        UPR_CUDA(cudaStreamSynchronize(s));
+        if (out[k + 1]) return UPR_ERR_INVALID;
+        // (cut and block_weights may be host or device memory)
+        UPR_CUDA(cudaMemcpyAsync(cut, out + k, sizeof(int64_t), cudaMemcpyDefault, s));
+        if (block_weights) UPR_CUDA(cudaMemcpyAsync(block_weights, out, sizeof(int64_t) * k, cudaMemcpyDefault, s));
         UPR_CUDA(cudaStreamSynchronize(s));
     } catch (const upr::CudaError &) {
         return UPR_ERR_CUDA;

@@ -88,3 +88,22 @@ def test_batch_over_several_ctas(upr, count, k):
             assert status[i] == 0 and np.array_equal(part[a:b], p0) and cut[i] == c0, i
         else:
             assert status[i] == upr.UPR_ERR_INFEASIBLE and np.array_equal(part[a:b], w.part), i
+
+
+@pytest.mark.parametrize("n,deg,k", [(2000, 9.0, 3), (40000, 1.2, 5), (9000, 40.0, 64)])
+def test_cut_and_block_weights_over_chunks(upr, n, deg, k):
+    """Chunks of 8192 entries: several rows each, more rows than are staged
+    (many short and empty ones), and rows that span chunks; block weights of
+    nodes in block order and not."""
+    import torch
+    w = synth.random_small(90 + k, n, deg, k, hubs=1 if deg > 9 else 0, isolated=n // 3 if deg < 2 else 0)
+    ctx = upr.create_from_workload(w)
+    dev = [None if a is None else torch.from_numpy(np.ascontiguousarray(a)).cuda()
+           for a in (w.xadj, w.adj, w.vwgt, w.adjw)]
+    for part in (w.part, np.sort(w.part), np.zeros(n, np.int32)):
+        part = np.ascontiguousarray(part, np.int32)
+        c0, bw0 = oracle.cut(w, part)
+        c, bw = upr.upr_cut(ctx, part)
+        assert c == c0 and np.array_equal(bw, bw0)
+        c, bw = upr.upr_cut_noalloc(dev[0], dev[1], torch.from_numpy(part).cuda(), k, vwgt=dev[2], adjw=dev[3])
+        assert c == c0 and np.array_equal(bw, bw0)
