@@ -109,8 +109,10 @@ typedef struct {
                                     dense table; after label propagation too; round 1's
                                     table build precedes the graph; the per-phase times of
                                     the stats are then 0); 0: the host launches every
-                                    sub-round and reads its stop flag.  Results never
-                                    depend on it. 1                                          */
+                                    sub-round and reads its stop flag.  With 1 and 2, a
+                                    small graph (m + n k at most 2^19, schedule 0, at most
+                                    256 rounds) is refined by one launch from the first
+                                    call on.  Results never depend on it. 1                  */
     int32_t schedule;            /* round driver (Sec. 4.4, Sec. 6.2): 0 every round
                                     unconstrained with the tau schedule.  6 the paper's
                                     final configuration: the first U rounds unconstrained
@@ -178,7 +180,8 @@ typedef struct {
     int32_t select_lanes;        /* lanes per node of the selection kernel (0: scalar)  */
     int32_t propose_lanes;       /* lanes per node of the proposal kernel (0: scalar)   */
     int32_t sparse_table;        /* 1: the rounds ran on the sparse gain table            */
-    int32_t rebalance_graphs;    /* rounds whose rebalancing loop ran as one graph launch */
+    int32_t rebalance_graphs;    /* rounds whose rebalancing loop ran as one graph launch
+                                    (or in the one launch of a small graph's rounds)     */
     int32_t constrained_rounds;  /* constrained rounds (schedules 1-6)                   */
     int32_t lp_rounds;           /* label propagation rounds kept (Sec. 5)               */
     int32_t lp_table_builds;     /* full gain-table builds of label propagation (also in

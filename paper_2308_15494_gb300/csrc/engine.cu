@@ -361,8 +361,9 @@ void layout(upr_ctx *c, Arena &A) {
     c->cut_in = A.take<int64_t>(ng);                 // the input cut per graph (the first round's node pass)
     c->pk = A.take<int2>(n);
     c->team.size = team_size((int64_t)n, c->beside);
-    c->team.hist = A.take<int32_t>((size_t)c->team.size * team::kSortBins);
-    c->team.hist64 = A.take<unsigned long long>(2 * (size_t)c->team.size * team::kSortBins);
+    const size_t ctas = (size_t)std::max(c->team.size, n <= kSmallNodes ? team::kClusterMax : 1);
+    c->team.hist = A.take<int32_t>(ctas * team::kSortBins);
+    c->team.hist64 = A.take<unsigned long long>(2 * ctas * team::kSortBins);
     c->team.tot = A.take<long long>((size_t)team::kTotSlots * team::kTeamMax);
     c->team.bar = A.take<unsigned long long>(1);
     c->team.err = A.take<int32_t>(1);
@@ -548,6 +549,138 @@ void set_pack(const upr_ctx *c, Penalty &pen) {
     }
 }
 
+// ---- the arguments of the team launches, fixed for a binding
+NodeList boundary_list(const upr_ctx *c) { return NodeList{c->idxA, c->counts + CNT_NB, c->emit}; }
+
+NodePass node_pass_of(upr_ctx *c) {
+    NodePass np{};
+    np.team = c->team;
+    np.part0 = c->part0; np.C0 = c->C0; np.part = c->part; np.C = c->C;
+    np.t_num = c->prm.t_num; np.t_den = c->prm.t_den;
+    np.BW = reinterpret_cast<unsigned long long *>(c->BW); np.PW = c->PW; np.first = c->first_slot;
+    np.own = c->emit;           // (free until the rebalancing)
+    np.list = c->idxA; np.d_list = c->counts + CNT_NB;
+    np.cut_pending = c->cut_pending ? 1 : 0;
+    np.cut = c->cut; np.cut_in = c->cut_in;
+    return np;
+}
+
+SelOrder sel_order_of(upr_ctx *c, const Penalty &pen) {
+    SelOrder so{};
+    so.team = c->team;
+    so.nl = boundary_list(c); so.cand = Candidates{c->cand_tgt, c->cand_s0, c->cand_gain};
+    so.pen = pen;
+    so.part0 = c->part0; so.part = c->part; so.C = c->C;
+    so.score = c->score;
+    so.c_excl = c->c_excl; so.seg_base = c->seg_base;
+    so.bufA = c->sb[0].k; so.bufB = c->sb[1].k;
+    so.M_node = c->M_node; so.M_from = c->M_from; so.M_to = c->M_to; so.M_score = c->M_score; so.m_pos = c->m_pos;
+    so.deg_sum = c->scal + 1;
+    so.d_cand = c->counts + CNT_CAND; so.d_moves = c->counts + CNT_M;
+    return so;
+}
+
+RebalStart reb_start_of(upr_ctx *c, cudaGraphConditionalHandle cond) {
+    RebalStart a{};
+    a.team = c->team;
+    a.part = c->part;
+    a.C = c->C;
+    a.list = c->L1;
+    a.d_list = c->counts + CNT_L1;
+    a.excl = c->excl_d; a.over = c->over_d; a.reject = c->reject_d;
+    a.max_subrounds = c->prm.max_subrounds;
+    a.ctl = c->ctl;
+    a.cond = cond;
+    return a;
+}
+
+RebalState reb_state_of(upr_ctx *c) {
+    const bool batch = c->ng > 1;
+    RebalState st{c->C, c->over_d, c->excl_d, batch ? c->light_g : &c->ctl->light, c->Lb};
+    const int kb = std::max(1, bit_length((uint64_t)(c->G.k - 1)));
+    if (!batch && !c->G.vwgt && c->gbits + kb <= 31) st.pack_bits = kb;
+    st.lsrc = c->emit;          // list-indexed proposal blocks and gains (sequence-phase arrays, free here)
+    st.lgain = c->qbefore;
+    return st;
+}
+
+RebalTeam reb_team_of(upr_ctx *c, const RebalState &st) {
+    RebalTeam m{};
+    m.team = c->team;
+    m.flags = c->flags;
+    m.list = c->L1;
+    m.lsrc = st.lsrc;
+    m.lgain = st.lgain;
+    m.d_n1 = &c->ctl->n1_active;
+    m.list2 = reinterpret_cast<int32_t *>(c->sb[2].k);
+    m.lsrc2 = m.list2 + c->n;
+    m.lgain2 = m.lsrc2 + c->n;
+    m.gbits = c->gbits;
+    m.cbits = c->cbits;
+    m.gain_only = c->prm.gain_priority;
+    m.hist = c->prio_hist;
+    m.rep = c->prio_rep;
+    m.cut = c->prio_cut;
+    m.exact = c->counts + CNT_EXACT;
+    m.over = c->over_d;
+    m.C = c->C;
+    m.bufA = c->sb[0].k;            // (two neighbouring 16 n arrays each)
+    m.bufB = c->sb[1].k;
+    m.U = c->sb[2].v;
+    m.at = reinterpret_cast<int32_t *>(c->sb[2].va);
+    m.c_excl = c->c_excl;
+    m.seg_base = c->seg_base;
+    m.part = c->part;
+    m.prop_tgt = c->prop_tgt;
+    m.reject = c->reject_d;
+    m.ctl = c->ctl;
+    m.R_node = c->R_node; m.R_from = c->R_from; m.R_to = c->R_to; m.R_sub = c->R_sub;
+    m.r_to = c->r_to; m.r_at = c->r_at;
+    m.d_np = c->counts + CNT_L1;
+    m.d_nk = c->counts + CNT_P;
+    m.d_na = c->counts + CNT_A;
+    return m;
+}
+
+// (a batch: I sorted by graph, into X_*, free once I is built)
+SeqBuild seq_build_of(upr_ctx *c) {
+    SeqBuild sq{};
+    sq.team = c->team;
+    sq.M_node = c->M_node; sq.M_from = c->M_from; sq.M_to = c->M_to; sq.dM = c->counts + CNT_M;
+    sq.R_node = c->R_node; sq.R_from = c->R_from; sq.R_to = c->R_to; sq.dR = &c->ctl->nR;
+    sq.part0 = c->part0; sq.m_pos = c->m_pos; sq.r_to = c->r_to; sq.C0 = c->C0;
+    sq.append = c->prm.append;
+    // (24 n bytes each: two neighbouring 16 n arrays)
+    sq.bufA = c->sb[0].k; sq.bufB = c->sb[1].k; sq.ex = c->c_sorted;
+    sq.qmax = reinterpret_cast<uint32_t *>(c->packed);
+    sq.rbeg = c->rbeg; sq.rend = c->rend; sq.ebeg = c->ebeg; sq.eend = c->eend; sq.qfin = c->qfin;
+    sq.left_excl = c->left_excl;
+    sq.emit = c->emit; sq.pos_m = c->pos_m;
+    sq.X_node = c->X_node; sq.X_from = c->X_from; sq.X_to = c->X_to; sq.fin = c->flags2;
+    sq.I_node = c->I_node; sq.I_from = c->I_from; sq.I_to = c->I_to;
+    sq.pk = c->pk; sq.diff = c->diff; sq.deg_sum = c->scal + 3;
+    sq.dX = c->counts + CNT_X; sq.dI = c->counts + CNT_I;
+    sq.O_node = c->X_node; sq.O_from = c->X_from; sq.O_to = c->X_to; sq.seg_beg = c->seg_beg; sq.seg_end = c->seg_end;
+    return sq;
+}
+
+SeqBest seq_best_of(upr_ctx *c) {
+    SeqBest sb{};
+    sb.team = c->team;
+    const bool batch = c->ng > 1;
+    sb.I_node = batch ? c->X_node : c->I_node; sb.I_from = batch ? c->X_from : c->I_from;
+    sb.I_to = batch ? c->X_to : c->I_to; sb.dI = c->counts + CNT_I;
+    sb.gain = c->I_gain; sb.Gsum = c->Gsum;
+    sb.bufA = c->sb[0].k; sb.bufB = c->sb[1].k;
+    sb.diff = c->diff; sb.diff_excl = c->diff_excl;
+    sb.part0 = c->part0; sb.C0 = c->C0; sb.cut = c->cut;
+    sb.best = c->best; sb.undone = c->scal + 2;
+    sb.d_over0 = c->counts + CNT_OVER0; sb.d_infeasible = c->counts + CNT_INFEAS;
+    sb.reset = 1;
+    sb.M_node = c->M_node; sb.dM = c->counts + CNT_M; sb.R_node = c->R_node; sb.dR = &c->ctl->nR; sb.m_pos = c->m_pos; sb.r_to = c->r_to;
+    return sb;
+}
+
 // One rebalancing sub-round (Sec. 6), enqueued on s.  Every argument is fixed
 // for the binding (the sub-round number and every list length live in device
 // memory), so the same launches can be captured once and replayed.  first:
@@ -578,41 +711,7 @@ bool enqueue_subround(upr_ctx *c, const RebalState &st, int32_t *light, bool fir
     // node without a proposal has no block with room for it (the lightest
     // allowed block has the most room, and rooms only shrink), so it never
     // proposes again
-    RebalTeam m{};
-    m.team = c->team;
-    m.flags = c->flags;
-    m.list = c->L1;
-    m.lsrc = st.lsrc;
-    m.lgain = st.lgain;
-    m.d_n1 = &ctl->n1_active;
-    m.list2 = reinterpret_cast<int32_t *>(c->sb[2].k);
-    m.lsrc2 = m.list2 + n;
-    m.lgain2 = m.lsrc2 + n;
-    m.gbits = c->gbits;
-    m.cbits = c->cbits;
-    m.gain_only = c->prm.gain_priority;
-    m.hist = c->prio_hist;
-    m.rep = c->prio_rep;
-    m.cut = c->prio_cut;
-    m.exact = cnt + CNT_EXACT;
-    m.over = c->over_d;
-    m.C = c->C;
-    m.bufA = c->sb[0].k;            // (two neighbouring 16 n arrays each)
-    m.bufB = c->sb[1].k;
-    m.U = c->sb[2].v;
-    m.at = reinterpret_cast<int32_t *>(c->sb[2].va);
-    m.c_excl = c->c_excl;
-    m.seg_base = c->seg_base;
-    m.part = c->part;
-    m.prop_tgt = c->prop_tgt;
-    m.reject = c->reject_d;
-    m.ctl = ctl;
-    m.R_node = c->R_node; m.R_from = c->R_from; m.R_to = c->R_to; m.R_sub = c->R_sub;
-    m.r_to = c->r_to; m.r_at = c->r_at;
-    m.d_np = cnt + CNT_L1;
-    m.d_nk = cnt + CNT_P;
-    m.d_na = cnt + CNT_A;
-    rebalance_order(G, m, s);
+    rebalance_order(G, reb_team_of(c, st), s);
     table_move(G, c->W, c->R_node, c->R_from, c->R_to, cnt + CNT_A, &ctl->nR, nullptr, n, c->hub_chunks, c->n_chunks,
                HubMoves{nullptr, c->r_to, c->r_at, &ctl->nR, cnt + CNT_A, c->R_from, c->R_to}, s);
     rebalance_end(G, c->C, c->excl_d, c->reject_d, c->over_d, cnt + CNT_A, cnt + CNT_L1, c->prm.max_subrounds, ctl, s,
@@ -624,16 +723,7 @@ bool enqueue_subround(upr_ctx *c, const RebalState &st, int32_t *light, bool fir
 // loop's condition, since its body begins each sub-round itself); one graph's
 // first list and the first sub-round's begin, with the condition.
 void loop_head(upr_ctx *c, cudaGraphConditionalHandle cond, cudaStream_t s) {
-    RebalStart a{};
-    a.team = c->team;
-    a.part = c->part;
-    a.C = c->C;
-    a.list = c->L1;
-    a.d_list = c->counts + CNT_L1;
-    a.excl = c->excl_d; a.over = c->over_d; a.reject = c->reject_d;
-    a.max_subrounds = c->prm.max_subrounds;
-    a.ctl = c->ctl;
-    a.cond = cond;
+    const RebalStart a = reb_start_of(c, cond);
     if (c->ng > 1) rebalance_init_batch(c->G, c->C, c->excl_d, c->ctl, s);
     rebalance_start(c->G, a, s);
     if (c->ng > 1 && cond) rebalance_continue(c->ctl, c->prm.max_subrounds, cond, s);
@@ -716,13 +806,7 @@ void rebalance_phase(upr_ctx *c, int32_t r, RoundInfo &ri, TraceSink *tr) {
     int32_t *cnt = c->counts;
     RebalCtl *ctl = c->ctl;
     int32_t *light = batch ? c->light_g : &ctl->light;
-    RebalState st{c->C, c->over_d, c->excl_d, light, c->Lb};
-    {
-        const int kb = std::max(1, bit_length((uint64_t)(G.k - 1)));
-        if (!batch && !G.vwgt && c->gbits + kb <= 31) st.pack_bits = kb;
-    }
-    st.lsrc = c->emit;          // list-indexed proposal blocks and gains (sequence-phase arrays, free here)
-    st.lgain = c->qbefore;
+    const RebalState st = reb_state_of(c);
     if (c->capturing) {
         // inside the step graph: the loop as a while node whose body is one
         // sub-round followed by the condition kernel (captured on a side
@@ -833,17 +917,9 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     if (!rebalance_only) {
         // ---- (b1) availability, slots, bucket weights; F_r; the boundary nodes
         // (the first round of a call also sums the input cut here)
-        NodePass np{};
-        np.team = c->team;
-        np.part0 = c->part0; np.C0 = c->C0; np.part = c->part; np.C = c->C;
-        np.t_num = c->prm.t_num; np.t_den = c->prm.t_den;
-        np.BW = reinterpret_cast<unsigned long long *>(c->BW); np.PW = c->PW; np.first = c->first_slot;
+        NodePass np = node_pass_of(c);
         np.avail_out = tr ? tr->avail_d : nullptr;
         np.slot_out = tr ? tr->slot_d : nullptr;
-        np.own = c->emit;           // (free until the rebalancing)
-        np.list = c->idxA; np.d_list = cnt + CNT_NB;
-        np.cut_pending = c->cut_pending ? 1 : 0;
-        np.cut = c->cut; np.cut_in = c->cut_in;
         node_pass(G, np, c->W, s);
         c->cut_pending = false;
         // the step graph reads round i's factors from the per-call table F_all
@@ -864,7 +940,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         Penalty pen{c->PW, F, c->C0, kind.limit > 0 ? c->Lsel : c->Lb, c->first_slot};
         set_pack(c, pen);
         // ---- (b2) best move per boundary node
-        const NodeList nl{c->idxA, cnt + CNT_NB, c->emit};
+        const NodeList nl = boundary_list(c);
         const Candidates cand{c->cand_tgt, c->cand_s0, c->cand_gain};
         run_tuned(c, c->sel_tuned, c->sel_cfg, c->sel_cands, &c->sel_pending, c->ev_tune, [&](LaneCfg cfg) {
             select_moves(G, nl, c->part0, c->W, pen, cand, cfg, s);
@@ -872,18 +948,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
         if (c->prm.lock_rebalanced)        // the oscillation guard (Sec. 2)
             guard_filter(c->locked, n, nl, cand, s);
         // ---- (b3) inflow penalties, M ordered by (score desc, id), applied
-        SelOrder so{};
-        so.team = c->team;
-        so.nl = nl; so.cand = cand;
-        so.pen = pen;
-        so.part0 = c->part0; so.part = c->part; so.C = c->C;
-        so.score = c->score;
-        so.c_excl = c->c_excl; so.seg_base = c->seg_base;
-        so.bufA = c->sb[0].k; so.bufB = c->sb[1].k;
-        so.M_node = c->M_node; so.M_from = c->M_from; so.M_to = c->M_to; so.M_score = c->M_score; so.m_pos = c->m_pos;
-        so.deg_sum = c->scal + 1;
-        so.d_cand = cnt + CNT_CAND; so.d_moves = cnt + CNT_M;
-        select_order(G, so, c->gbits, s);
+        select_order(G, sel_order_of(c, pen), c->gbits, s);
         // W' for P o M: the delta update costs two atomics per adjacency entry of a
         // moved node, a rebuild streams the graph and the table once; each kernel
         // checks on the device which of the two applies
@@ -901,25 +966,7 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     // ---- (c1) interleave M and R_1..R_k (or append R after M: a variant of Sec. 7.2)
     const int32_t *dM = cnt + CNT_M, *dR = &ctl->nR;
     const int32_t *dI = cnt + CNT_I;
-    // (a batch: I sorted by graph, into X_*, free once I is built)
-    SeqBuild sq{};
-    sq.team = c->team;
-    sq.M_node = c->M_node; sq.M_from = c->M_from; sq.M_to = c->M_to; sq.dM = dM;
-    sq.R_node = c->R_node; sq.R_from = c->R_from; sq.R_to = c->R_to; sq.dR = dR;
-    sq.part0 = c->part0; sq.m_pos = c->m_pos; sq.r_to = c->r_to; sq.C0 = c->C0;
-    sq.append = c->prm.append;
-    // (24 n bytes each: two neighbouring 16 n arrays)
-    sq.bufA = c->sb[0].k; sq.bufB = c->sb[1].k; sq.ex = c->c_sorted;
-    sq.qmax = reinterpret_cast<uint32_t *>(c->packed);
-    sq.rbeg = c->rbeg; sq.rend = c->rend; sq.ebeg = c->ebeg; sq.eend = c->eend; sq.qfin = c->qfin;
-    sq.left_excl = c->left_excl;
-    sq.emit = c->emit; sq.pos_m = c->pos_m;
-    sq.X_node = c->X_node; sq.X_from = c->X_from; sq.X_to = c->X_to; sq.fin = c->flags2;
-    sq.I_node = c->I_node; sq.I_from = c->I_from; sq.I_to = c->I_to;
-    sq.pk = c->pk; sq.diff = c->diff; sq.deg_sum = c->scal + 3;
-    sq.dX = cnt + CNT_X; sq.dI = cnt + CNT_I;
-    sq.O_node = c->X_node; sq.O_from = c->X_from; sq.O_to = c->X_to; sq.seg_beg = c->seg_beg; sq.seg_end = c->seg_end;
-    seq_build(G, sq, s);
+    seq_build(G, seq_build_of(c), s);
     const int32_t *Iv = c->I_node, *If = c->I_from, *It = c->I_to;
     if (batch) { Iv = c->X_node; If = c->X_from; It = c->X_to; }
 
@@ -942,17 +989,8 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     }
     if (tr) UPR_CUDA(cudaMemcpyAsync(c->hcut, c->cut, sizeof(int64_t), cudaMemcpyDeviceToHost, s));   // cut before the round
     const bool guard = c->prm.lock_rebalanced && !rebalance_only;
-    SeqBest sb{};
-    sb.team = c->team;
-    sb.I_node = Iv; sb.I_from = If; sb.I_to = It; sb.dI = dI;
-    sb.gain = c->I_gain; sb.Gsum = c->Gsum;
-    sb.bufA = c->sb[0].k; sb.bufB = c->sb[1].k;
-    sb.diff = c->diff; sb.diff_excl = c->diff_excl;
-    sb.part0 = c->part0; sb.C0 = c->C0; sb.cut = c->cut;
-    sb.best = c->best; sb.undone = c->scal + 2;
-    sb.d_over0 = cnt + CNT_OVER0; sb.d_infeasible = cnt + CNT_INFEAS;
+    SeqBest sb = seq_best_of(c);
     sb.reset = guard ? 0 : 1;
-    sb.M_node = c->M_node; sb.dM = dM; sb.R_node = c->R_node; sb.dR = dR; sb.m_pos = c->m_pos; sb.r_to = c->r_to;
     seq_best(G, sb, s);
     if (batch) {
         count_over(G, c->C0, c->over0_g, s);
@@ -1433,6 +1471,25 @@ bool build_step_graph(upr_ctx *c, int32_t rounds, int32_t total) {
     return c->step_exec != nullptr;
 }
 
+// The penalty factors of rounds 1..rounds, copied in one piece.
+void upload_factors(upr_ctx *c, int32_t rounds, int32_t total) {
+    if (c->F_all_cap < rounds) {
+        if (c->F_all) cudaFree(c->F_all);
+        if (c->hF_all) cudaFreeHost(c->hF_all);
+        c->F_all = nullptr;
+        c->hF_all = nullptr;
+        c->F_all_cap = 0;
+        UPR_CUDA(cudaMalloc(&c->F_all, sizeof(int64_t) * kSlots * (size_t)rounds));
+        UPR_CUDA(cudaMallocHost(&c->hF_all, sizeof(int64_t) * kSlots * (size_t)rounds));
+        c->F_all_cap = rounds;
+    }
+    // (a call ends by synchronising its stream, so no earlier copy still reads hF_all)
+    for (int32_t i = 1; i <= rounds; i++)
+        penalty_factors(c->prm.round_offset + i, total, c->prm.tau1_num, c->prm.tau1_den,
+                        c->hF_all + (size_t)(i - 1) * kSlots);
+    UPR_CUDA(cudaMemcpyAsync(c->F_all, c->hF_all, sizeof(int64_t) * kSlots * rounds, cudaMemcpyHostToDevice, c->s));
+}
+
 // Rounds 1..rounds of a call as one graph launch (params.graphs == 2, the
 // plain tau schedule, dense table, lane schedules settled): round 1's table
 // build runs (timed) before the graph, the rounds' penalty factors are copied
@@ -1459,22 +1516,8 @@ bool run_step_graph(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
         st.gain_table_builds++;
         c->table_valid = true;
     }
-    if (c->F_all_cap < rounds) {
-        if (c->F_all) cudaFree(c->F_all);
-        if (c->hF_all) cudaFreeHost(c->hF_all);
-        c->F_all = nullptr;
-        c->hF_all = nullptr;
-        c->F_all_cap = 0;
-        UPR_CUDA(cudaMalloc(&c->F_all, sizeof(int64_t) * kSlots * (size_t)rounds));
-        UPR_CUDA(cudaMallocHost(&c->hF_all, sizeof(int64_t) * kSlots * (size_t)rounds));
-        c->F_all_cap = rounds;
-    }
-    UPR_CUDA(cudaStreamSynchronize(s));          // hF_all may still be read by the previous call's copy
-    for (int32_t i = 1; i <= rounds; i++)
-        penalty_factors(c->prm.round_offset + i, total, c->prm.tau1_num, c->prm.tau1_den,
-                        c->hF_all + (size_t)(i - 1) * kSlots);
+    upload_factors(c, rounds, total);
     if (!same && !build_step_graph(c, rounds, total)) return false;
-    UPR_CUDA(cudaMemcpyAsync(c->F_all, c->hF_all, sizeof(int64_t) * kSlots * rounds, cudaMemcpyHostToDevice, s));
     UPR_CUDA(cudaMemsetAsync(c->dstats, 0, sizeof(long long) * 16, s));
     UPR_CUDA(cudaGraphLaunch(c->step_exec, s));
     long long d[16];
@@ -1492,6 +1535,92 @@ bool run_step_graph(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
     st.rebalance_graphs += rounds;
     g_upr_launches += (c->step_kernels + (long long)c->reb_body_kernels * d[3]);
     return true;
+}
+
+// All rounds in one launch (small.cu): one small graph, the plain tau schedule,
+// the dense table.  The line is on what a round reads at most, adjacency
+// entries and table cells: one cluster has a tenth of the chip's SMs, and the
+// launches and waits it saves are worth some 40 us a round.  Four rounds, step
+// by step -> one launch: 8192 nodes, degree 32, 32 blocks (2^19 of them)
+// 0.85 -> 0.82 ms; 16384 nodes, degree 16, 8 blocks 1.10 -> 0.98; 32768,
+// degree 8, 2 blocks 1.22 -> 1.16; beyond the line: 8192, degree 16, 64 blocks,
+// weighted 1.16 -> 1.23, 16384, degree 128 0.99 -> 1.13, 65536, degree 8
+// 1.31 -> 1.47.  More rounds than kSmallRounds go step by step, so that one
+// launch stays within some tens of milliseconds.
+constexpr int64_t kSmallWork = 1 << 19;
+constexpr int32_t kSmallRounds = 256;
+
+int64_t small_work(const upr_ctx *c) { return c->G.m + c->G.n * c->G.k; }
+
+// CTAs: one for the smallest graphs, whose steps are shorter than the barriers
+// of a cluster (1024 nodes, degree 8: 0.50 ms by one, 0.55 by eight; 2048,
+// degree 16: 0.52 and 0.51), then eight (2048, degree 32, 32 blocks: 0.77 by
+// one, 0.67 by eight; 4096: 0.66 by four, 0.61 by eight), then a cluster of 16
+// (16384: 0.98, by eight 1.01).
+int small_size(const upr_ctx *c) {
+    if (c->n <= 2048 && small_work(c) <= 1 << 16) return 1;
+    return c->n <= 8192 ? 8 : team::kClusterMax;
+}
+
+bool small_applies(const upr_ctx *c, int32_t rounds) {
+    return c->prm.graphs >= 1 && c->prm.schedule == 0 && !c->prm.lock_rebalanced && rounds >= 1 &&
+           rounds <= kSmallRounds && !log_enabled() && small_work(c) <= kSmallWork &&
+           small_refine_ok(c->G, c->gbits, c->cbits);
+}
+
+void run_small(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
+    cudaStream_t s = c->s;
+    upload_factors(c, rounds, total);
+    UPR_CUDA(cudaMemsetAsync(c->counts, 0, sizeof(int32_t) * CNT_SLOTS, s));
+    SmallRefine a{};
+    a.team = c->team;
+    a.team.size = small_size(c);
+    a.g = c->G;
+    a.W = c->W;
+    a.build = c->table_valid ? 0 : 1;
+    a.chunks = c->hub_chunks;
+    a.n_chunks = c->n_chunks;
+    a.rounds = rounds;
+    a.F = c->F_all;
+    a.np = node_pass_of(c);
+    a.so = sel_order_of(c, Penalty{c->PW, c->F_all, c->C0, c->Lb, c->first_slot});
+    a.rs = reb_start_of(c, 0);
+    a.st = reb_state_of(c);
+    a.rt = reb_team_of(c, a.st);
+    a.prop_gain = c->prop_gain;
+    a.flags = c->flags;
+    a.sq = seq_build_of(c);
+    a.sb = seq_best_of(c);
+    a.ctl = c->ctl;
+    a.d = c->dstats;
+    c->cut_pending = false;
+    c->table_valid = false;
+    small_refine(a, s);
+    long long *d = reinterpret_cast<long long *>(c->h);      // (the pinned block's first words)
+    UPR_CUDA(cudaMemcpyAsync(d, c->dstats, sizeof(long long) * 16, cudaMemcpyDeviceToHost, s));
+    UPR_CUDA(cudaMemcpyAsync(c->hcnt + 40, c->team.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    UPR_CUDA(cudaStreamSynchronize(s));
+    if (c->hcnt[40] != 0) throw CudaError{cudaErrorLaunchTimeout, "barrier wait"};
+    if (d[7] != 0) throw CudaError{cudaErrorInvalidValue, "small refinement: infeasible round"};
+    c->table_valid = true;
+    st.rounds_run += rounds;
+    st.n_candidates += d[0];
+    st.n_moves += d[1];
+    st.n_rebalance_moves += d[2];
+    st.subrounds += (int32_t)d[3];
+    st.n_sequence += d[4];
+    st.n_applied += d[5];
+    st.rebalance_graphs += rounds;
+    if (a.build) {
+        st.gain_table_builds++;
+        st.ms_gain_table += d[10] * 1e-6;
+    }
+    // (graphs = 2: as when the rounds run as one graph, from the second call on)
+    if (c->prm.graphs == 1 || c->calls_bound < 2) {
+        st.ms_select += d[11] * 1e-6;
+        st.ms_rebalance += d[12] * 1e-6;
+        st.ms_sequence += d[13] * 1e-6;
+    }
 }
 
 upr_status refine_impl(upr_ctx *c, int32_t *part, int32_t rounds, upr_stats *stats, upr_status *status,
@@ -1602,7 +1731,13 @@ upr_status refine_impl(upr_ctx *c, int32_t *part, int32_t rounds, upr_stats *sta
     const bool settled = no_choice || !worth_tuning(c) || (c->sel_tuned && c->prop_tuned);
     const bool step = c->prm.graphs == 2 && sch == 0 && !c->G.sp.on() && rounds >= 1 && !log_enabled() && settled &&
                       c->calls_bound >= 2;
-    const int32_t first_round = step && run_step_graph(c, rounds, total, st) ? rounds + 1 : 1;
+    int32_t first_round = 1;
+    if (small_applies(c, rounds)) {
+        run_small(c, rounds, total, st);
+        first_round = rounds + 1;
+    } else if (step && run_step_graph(c, rounds, total, st)) {
+        first_round = rounds + 1;
+    }
     for (int32_t i = first_round; i <= rounds; i++) {
         RoundInfo ri;
         RoundKind kind;

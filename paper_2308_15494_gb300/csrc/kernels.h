@@ -262,6 +262,7 @@ struct NodePass {
     const int32_t *W = nullptr, *wI = nullptr, *vwgt = nullptr, *gid = nullptr;
     SparseRows sp{};
 };
+size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W);
 void node_pass(const GraphDev &g, NodePass a, const int32_t *W, cudaStream_t s);
 // Lanes per node (G) and 16-byte chunks per lane (CH) of the vectorised
 // selection and proposal kernels (k % 4 == 0, k <= 256, 4*G*CH >= k).  A
@@ -295,6 +296,9 @@ struct SelOrder {
     const int32_t *vwgt = nullptr;
     const int64_t *xadj = nullptr;
 };
+// (the *_args functions fill the fields a wrapper sets; they return the dynamic
+// shared memory of the launch)
+void select_order_args(const GraphDev &g, SelOrder &a);
 void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s);
 
 // ---- rebalance.cu: step (d)
@@ -348,6 +352,7 @@ struct RebalStart {
     int K = 0, batch = 0;
     const int64_t *Lb = nullptr;
 };
+void rebalance_start_args(const GraphDev &g, RebalStart &a);
 void rebalance_start(const GraphDev &g, RebalStart a, cudaStream_t s);
 // A sub-round after its proposals: the proposers (flags by list index, their
 // blocks and gains in lsrc / lgain) become the list, the minimal prefix per
@@ -383,6 +388,8 @@ struct RebalTeam {
     const int32_t *vwgt = nullptr;
     const int64_t *Lb = nullptr;
 };
+constexpr int kRebRankK = 256;       // blocks up to which a sub-round ranks by per-warp block sums
+size_t rebalance_order_args(const GraphDev &g, RebalTeam &a);
 void rebalance_order(const GraphDev &g, RebalTeam a, cudaStream_t s);
 // Loop control of a batch: the excluded set and the control block; a
 // sub-round's begin (light: each graph's lightest non-excluded block).
@@ -453,6 +460,7 @@ struct SeqBuild {
     const int32_t *vwgt = nullptr, *gid = nullptr;
     const int64_t *xadj = nullptr, *Lb = nullptr;
 };
+void seq_build_args(const GraphDev &g, SeqBuild &a);
 void seq_build(const GraphDev &g, SeqBuild a, cudaStream_t s);
 void seq_gains(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
                const int32_t *d_nI, int64_t max, const int2 *pk, int64_t *gain, const HubChunk *hub_chunks,
@@ -482,6 +490,7 @@ struct SeqBest {
     const int32_t *vwgt = nullptr, *gid = nullptr;
     const int64_t *xadj = nullptr, *Lb = nullptr;
 };
+void seq_best_args(const GraphDev &g, SeqBest &a);
 void seq_best(const GraphDev &g, SeqBest a, cudaStream_t s);
 // The moves of I undone after the best prefix: positions i >= j* (one graph,
 // best[1] = j*, -1 = none kept) or i - seg_beg[g] >= best_j[g] (a batch, gid set).
@@ -513,6 +522,36 @@ void seq_best_seg(const GraphDev &g, const int32_t *I_node, const int32_t *d_nI,
 void seq_apply_prefix_seg(const GraphDev &g, const int32_t *I_node, const int32_t *I_from, const int32_t *I_to,
                           const int32_t *d_nI, int64_t max, const int32_t *seg_beg, const long long *best_j,
                           int32_t *part0, int64_t *C0, cudaStream_t s);
+
+// ---- small.cu: all rounds of a call on a small graph in one launch
+// The team is one CTA or one cluster (n <= kSmallNodes), the table dense, keys
+// within 63 bits and scores and blocks within 32.
+constexpr int64_t kSmallNodes = 65536;
+struct SmallRefine {
+    Team team;
+    GraphDev g;
+    int32_t *W;
+    int build;                               // the table is built first (else it is valid)
+    const HubChunk *chunks;
+    int64_t n_chunks;
+    int32_t rounds;
+    const int64_t *F;                        // [rounds][kSlots] penalty factors
+    NodePass np;                             // cut_pending: of the first round
+    SelOrder so;
+    RebalStart rs;
+    RebalTeam rt;
+    RebalState st;
+    int32_t *prop_gain, *flags;
+    SeqBuild sq;
+    SeqBest sb;
+    RebalCtl *ctl;
+    // sums over the rounds: candidates, moves, rebalancing moves, sub-rounds,
+    // |I|, applied, -, infeasible rounds; [10..13]: ns in the table build,
+    // selection, rebalancing, sequence
+    long long *d;
+};
+bool small_refine_ok(const GraphDev &g, int gbits, int cbits);
+void small_refine(SmallRefine a, cudaStream_t s);
 
 // ---- lp.cu: unconstrained label propagation (Sec. 5)
 // active[v] = 1 for the boundary nodes of part (table W of part)

@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(team::kTT, 1) k_lp_list(const LpList a) {
     const long long mine = team::publish<team::Sum>(a.team, s, 0, team::warp_all<team::Sum>(cnt));
     team::sync(a.team);
     long long all;
-    int64_t pos = team::collect<team::Sum>(a.team, 0, &all) + mine;
+    int64_t pos = team::collect<team::Sum>(a.team, s, 0, &all) + mine;
     for (int64_t v0 = g.b; v0 < g.e; v0 += 32) {
         const int64_t v = v0 + lane;
         const bool f = v < g.e && in(v);

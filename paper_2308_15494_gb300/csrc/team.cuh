@@ -38,7 +38,19 @@ struct Smem {
     int tot[kSortBins], bef[kSortBins];
     unsigned long long rep[kSortBins];
     long long w[kTW];
+    static constexpr bool kCluster = false;            // the team's totals are in global memory
     __device__ __forceinline__ int *cnt() { return reinterpret_cast<int *>(cnt64); }
+};
+// Of a kernel whose teams are one CTA or one cluster: a CTA's totals for the
+// team stay in its shared memory (a write and a read through the L2 cost about
+// 1.2 us per step).  The kernels of larger teams are compiled without it: with
+// both forms in one kernel and a test at each use, 2^18 nodes, 8 blocks took
+// 2.88 ms instead of 2.77.
+struct ClusterSmem : Smem {
+    static constexpr bool kCluster = true;
+    unsigned long long row64[2][kSortBins];            // block weights,
+    int row[kSortBins];                                // digits,
+    long long sums[kTotSlots];                         // and scans
 };
 
 constexpr int kClusterMax = 16;          // teams up to this size run as one cluster
@@ -77,6 +89,36 @@ __device__ __forceinline__ void sync(const Team &t) {
         }
     }
     __syncthreads();
+}
+
+// A value of CTA c's shared memory (c in this team, a cluster).
+template <typename T>
+__device__ __forceinline__ T remote(const T *mine, int c) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "one word");
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(mine)), "r"(c));
+    if constexpr (sizeof(T) == 4) {
+        uint32_t v;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+        return (T)v;
+    } else {
+        unsigned long long v;
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+        return (T)v;
+    }
+}
+
+// A per-CTA value published in a slot, and CTA c's after a barrier.
+template <class Sm>
+__device__ __forceinline__ void put(const Team &t, Sm &s, int slot, long long v) {
+    if constexpr (Sm::kCluster) s.sums[slot] = v;
+    else t.tot[slot * kTeamMax + blockIdx.x] = v;
+}
+template <class Sm>
+__device__ __forceinline__ long long get(const Team &t, const Sm &s, int slot, int c) {
+    if constexpr (Sm::kCluster) return remote(&s.sums[slot], c);
+    else return t.tot[slot * kTeamMax + c];
 }
 
 struct Seg { int64_t b, e; };
@@ -119,25 +161,30 @@ __device__ __forceinline__ long long warp_incl(long long v) {
 
 // Publishes the CTA's total of the warps' values x (equal in a warp's lanes)
 // in the slot; returns the total of the warps before this one in the CTA.
-template <class Op>
-__device__ __forceinline__ long long publish(const Team &t, Smem &s, int slot, long long x) {
+template <class Op, class Sm>
+__device__ __forceinline__ long long publish(const Team &t, Sm &s, int slot, long long x) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) s.w[warp] = x;
     __syncthreads();
     const long long inc = warp_incl<Op>(s.w[lane]);
     const long long before = __shfl_sync(0xffffffffu, inc, warp > 0 ? warp - 1 : 0);
-    if (threadIdx.x == kTT - 1) t.tot[slot * kTeamMax + blockIdx.x] = inc;
+    if (threadIdx.x == kTT - 1) put(t, s, slot, inc);
     __syncthreads();
     return warp > 0 ? before : Op::id();
 }
 
 // After a barrier: the published totals of the CTAs before this one, and of all.
-template <class Op>
-__device__ __forceinline__ long long collect(const Team &t, int slot, long long *all) {
+template <class Op, class Sm>
+__device__ __forceinline__ long long collect(const Team &t, const Sm &s, int slot, long long *all) {
     const int lane = threadIdx.x & 31;
+    if constexpr (Sm::kCluster)
+        if (gridDim.x == 1) {
+            *all = s.sums[slot];
+            return Op::id();
+        }
     long long b = Op::id(), a = Op::id();
     for (int c = lane; c < (int)gridDim.x; c += 32) {
-        const long long v = t.tot[slot * kTeamMax + c];
+        const long long v = get(t, s, slot, c);
         a = Op::op(a, v);
         if (c < (int)blockIdx.x) b = Op::op(b, v);
     }
@@ -160,8 +207,8 @@ struct __align__(16) Item64 {
 // load(i, it) accepts, i < n, in two halves with a team barrier between them:
 // sort_count counts the digits of the warps' segments, sort_place writes the
 // items to out[0..count), returns count and ends with a barrier.
-template <class Item, class Load>
-__device__ __forceinline__ void sort_count(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits) {
+template <class Item, class Load, class Sm>
+__device__ __forceinline__ void sort_count(const Team &t, Sm &s, int64_t n, Load load, int shift, int bits) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int bins = 1 << bits, mask = bins - 1;
     const Seg g = warp_seg(n);
@@ -190,12 +237,13 @@ __device__ __forceinline__ void sort_count(const Team &t, Smem &s, int64_t n, Lo
             s.cnt()[w * bins + d] = run;
             run += c;
         }
-        t.hist[blockIdx.x * bins + d] = run;
+        if constexpr (Sm::kCluster) s.row[d] = run;
+        else t.hist[blockIdx.x * bins + d] = run;
     }
 }
 
-template <class Item, class Load>
-__device__ __forceinline__ int64_t sort_place(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits,
+template <class Item, class Load, class Sm>
+__device__ __forceinline__ int64_t sort_place(const Team &t, Sm &s, int64_t n, Load load, int shift, int bits,
                                               Item *out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -209,7 +257,9 @@ __device__ __forceinline__ int64_t sort_place(const Team &t, Smem &s, int64_t n,
         const int d = threadIdx.x & mask;
         int tot = 0, bef = 0;
         for (int c = threadIdx.x >> bits; c < (int)gridDim.x; c += kTT >> bits) {
-            const int v = t.hist[c * bins + d];
+            int v;
+            if constexpr (Sm::kCluster) v = remote(&s.row[d], c);
+            else v = t.hist[c * bins + d];
             tot += v;
             if (c < (int)blockIdx.x) bef += v;
         }
@@ -254,8 +304,8 @@ __device__ __forceinline__ int64_t sort_place(const Team &t, Smem &s, int64_t n,
     return count;
 }
 
-template <class Item, class Load>
-__device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, Load load, int shift, int bits,
+template <class Item, class Load, class Sm>
+__device__ __forceinline__ int64_t sort_pass(const Team &t, Sm &s, int64_t n, Load load, int shift, int bits,
                                              Item *out) {
     sort_count<Item>(t, s, n, load, shift, bits);
     sync(t);
@@ -264,8 +314,8 @@ __device__ __forceinline__ int64_t sort_pass(const Team &t, Smem &s, int64_t n, 
 
 // Stable sort by the low `bits` key bits of the items load accepts; the
 // result is returned (A or B), its length in *count.
-template <class Item, class Load>
-__device__ __forceinline__ const Item *sort(const Team &t, Smem &s, int64_t n, Load load, int bits, Item *A, Item *B,
+template <class Item, class Load, class Sm>
+__device__ __forceinline__ const Item *sort(const Team &t, Sm &s, int64_t n, Load load, int bits, Item *A, Item *B,
                                             int64_t *count) {
     const int passes = bits <= 8 ? 1 : (bits + 7) / 8;
     const int per = max(1, (bits + passes - 1) / passes);
