@@ -80,11 +80,14 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, NodeList n
     // PACK (unit weights, one graph): a node of weight 1 pays the same
     // penalty p(b) into block b wherever it comes from, so p(b) (-1:
     // forbidden) is fixed for the launch; the lane keeps, per column it
-    // scores, a bit "allowed" and the constant (2^kb - 1 - b) - (p(b) << kb)
+    // scores, the constant (2^kb - 1 - b) - (p(b) << kb), or one so low that no
+    // omega (omega << kb < 2^30) lifts it above another score.  The node's own
+    // omega comes off the maximum instead of every column: two instructions a
+    // column where a mask of the allowed ones took five (with the same change to
+    // the proposals, 2^22 nodes, 64 blocks: 17.74 -> 17.52 ms)
     const int kb = PACK ? pen.pack_bits : 0;
     const int32_t kmask = (1 << kb) - 1;
     int32_t *s_pen = reinterpret_cast<int32_t *>(s_first + ((k + 3) & ~3));
-    uint32_t okm = 0;
     int32_t cst[CH][4];
     if (PACK) {
         for (int b = threadIdx.x; b < k; b += blockDim.x) {
@@ -125,8 +128,7 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, NodeList n
             for (int cc = 0; cc < 4; cc++) {
                 const int b = 4 * (gl + G * j) + cc;
                 const int32_t p = (EXACT || b < k) ? s_pen[b] : -1;
-                if (p >= 0) okm |= 1u << (4 * j + cc);
-                cst[j][cc] = (kmask - b) - (p >= 0 ? (p << kb) : 0);
+                cst[j][cc] = p >= 0 ? (kmask - b) - (p << kb) : INT32_MIN;
             }
     }
     // (the next node's id is loaded one iteration ahead, so that a row's load
@@ -167,13 +169,12 @@ __global__ void __launch_bounds__(256) k_select_vec(const GraphDev g, NodeList n
             int32_t pbest = 0;
             if (active && own < wIv) {
                 const int32_t ownk = own << kb;
+                int32_t top = ownk;
 #pragma unroll
                 for (int j = 0; j < CH; j++)
 #pragma unroll
-                    for (int cc = 0; cc < 4; cc++) {
-                        const int32_t key = (int4_get(r[j], cc) << kb) - ownk + cst[j][cc];
-                        pbest = max(pbest, ((okm >> (4 * j + cc)) & 1u) ? key : 0);
-                    }
+                    for (int cc = 0; cc < 4; cc++) top = max(top, (int4_get(r[j], cc) << kb) + cst[j][cc]);
+                pbest = top - ownk;
             }
             for (int o = G / 2; o > 0; o >>= 1) pbest = max(pbest, __shfl_xor_sync(0xffffffffu, pbest, o));
             if (active && gl == 0) {
