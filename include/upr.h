@@ -112,7 +112,8 @@ typedef struct {
                                     sub-round and reads its stop flag.  With 1 and 2, a
                                     small graph (m + n k at most 2^19, schedule 0, at most
                                     256 rounds) is refined by one launch from the first
-                                    call on.  Results never depend on it. 1                  */
+                                    call on (with 2, where one graph launch can run instead,
+                                    only up to 2^15).  Results never depend on it. 1         */
     int32_t schedule;            /* round driver (Sec. 4.4, Sec. 6.2): 0 every round
                                     unconstrained with the tau schedule.  6 the paper's
                                     final configuration: the first U rounds unconstrained

