@@ -61,7 +61,7 @@ def build(verbose: bool = False) -> str:
             print(r.stdout, r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(cus))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(os.cpu_count() or 1, len(cus))) as ex:
         objs = list(ex.map(compile_one, cus))
     tmp = LIB + f".tmp{os.getpid()}"
     r = subprocess.run([nvcc] + ARCH + ["-shared", "-o", tmp] + objs + ["-lpthread"], capture_output=True, text=True)

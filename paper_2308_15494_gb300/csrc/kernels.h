@@ -551,7 +551,10 @@ struct SmallRefine {
     long long *d;
 };
 bool small_refine_ok(const GraphDev &g, int gbits, int cbits);
-void small_refine(SmallRefine a, cudaStream_t s);
+void small_refine(const SmallRefine &a, cudaStream_t s);
+// (unit node weights; sub-rounds that rank by block sums, K <= kRebRankK)
+template <bool UNIT, bool RANK>
+void small_form(SmallRefine a, cudaStream_t s);
 
 // ---- lp.cu: unconstrained label propagation (Sec. 5)
 // active[v] = 1 for the boundary nodes of part (table W of part)
