@@ -117,10 +117,12 @@ __device__ __forceinline__ BlockDelta make_block_delta(unsigned long long *smem,
     return K <= kMaxK ? BlockDelta{reinterpret_cast<unsigned int *>(smem), K, nullptr} : BlockDelta{nullptr, K, C};
 }
 
+// The dynamic shared memory a launch of this kernel can have: the device's
+// opt-in maximum less the kernel's static shared memory (engine.cu).
+size_t dynamic_smem(const void *func);
 // Kernel attributes are per process and device, shared by every host thread:
-// a kernel's dynamic shared-memory limit is raised once to the device's
-// opt-in maximum less its static shared memory (a ceiling only: occupancy
-// follows the launch's actual size)
+// a kernel's dynamic shared-memory limit is raised once to dynamic_smem (a
+// ceiling only: occupancy follows the launch's actual size)
 // and its shared/L1 split set, never changed afterwards, so no thread can
 // lower a limit another thread's launch relies on.
 void kernel_setup(const void *func, int carveout_percent);   // engine.cu; -1 = no carveout preference

@@ -141,6 +141,21 @@ int upr::resident_ctas(const void *func, int threads, size_t shm) {
     return n;
 }
 
+size_t upr::dynamic_smem(const void *func) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> cache;
+    int dev = 0;
+    UPR_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find({dev, func});
+    if (it != cache.end()) return it->second;
+    int optin = 0;
+    UPR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    cudaFuncAttributes fa;
+    UPR_CUDA(cudaFuncGetAttributes(&fa, func));     // static shared memory counts against the same limit
+    return cache[{dev, func}] = (size_t)optin - fa.sharedSizeBytes;
+}
+
 void upr::kernel_setup(const void *func, int carveout_percent) {
     static std::mutex mu;
     static std::set<std::pair<int, const void *>> done;
@@ -148,12 +163,7 @@ void upr::kernel_setup(const void *func, int carveout_percent) {
     UPR_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(mu);
     if (done.count({dev, func})) return;
-    int optin = 0;
-    UPR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    cudaFuncAttributes fa;
-    UPR_CUDA(cudaFuncGetAttributes(&fa, func));     // static shared memory counts against the same limit
-    UPR_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  optin - (int)fa.sharedSizeBytes));
+    UPR_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_smem(func)));
     if (carveout_percent >= 0)
         UPR_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent));
     done.insert({dev, func});

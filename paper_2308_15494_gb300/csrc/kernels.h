@@ -262,7 +262,12 @@ struct NodePass {
     const int32_t *W = nullptr, *wI = nullptr, *vwgt = nullptr, *gid = nullptr;
     SparseRows sp{};
 };
-size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W);
+// room: the dynamic shared memory the kernel that runs the pass can have; a
+// histogram beyond it stays in global memory.  (A kernel's static part counts
+// against the same 227 KB of a CTA: 38 KB in k_node_pass, 45 KB in the small
+// graphs' kernel.)
+constexpr size_t kNodePassSmem = 184 * 1024;
+size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W, size_t room);
 void node_pass(const GraphDev &g, NodePass a, const int32_t *W, cudaStream_t s);
 // Lanes per node (G) and 16-byte chunks per lane (CH) of the vectorised
 // selection and proposal kernels (k % 4 == 0, k <= 256, 4*G*CH >= k).  A

@@ -332,7 +332,7 @@ void select_order(const GraphDev &g, SelOrder a, int gbits, cudaStream_t s) {
     else launch_team(k_sel_order<team::Item64>, a, a.team.size, s);
 }
 
-size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W) {
+size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W, size_t room) {
     a.n = g.n;
     a.k = g.k;
     a.kmask = g.kmask;
@@ -344,12 +344,12 @@ size_t node_pass_args(const GraphDev &g, NodePass &a, const int32_t *W) {
     a.vwgt = g.vwgt;
     a.gid = g.gid;
     const size_t shm = (g.vwgt ? sizeof(unsigned long long) : sizeof(unsigned int)) * (size_t)a.K * kSlots;
-    a.use_shared = shm <= 184 * 1024;            // (the team's own shared memory is static, 38 KB)
+    a.use_shared = shm <= room;
     return a.use_shared ? shm : 0;
 }
 
 void node_pass(const GraphDev &g, NodePass a, const int32_t *W, cudaStream_t s) {
-    const size_t shm = node_pass_args(g, a, W);
+    const size_t shm = node_pass_args(g, a, W, std::min(kNodePassSmem, dynamic_smem((const void *)k_node_pass)));
     UPR_CUDA(cudaMemsetAsync(a.BW, 0, sizeof(int64_t) * a.K * kSlots, s));
     if (a.cut_pending && g.ng > 1) UPR_CUDA(cudaMemsetAsync(a.cut, 0, sizeof(int64_t) * g.ng, s));
     launch_team(k_node_pass, a, a.team.size, s, shm);

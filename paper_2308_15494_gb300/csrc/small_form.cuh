@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(team::kTT, 1) k_small_refine(const __grid_cons
 
 template <bool UNIT, bool RANK>
 void small_form(SmallRefine a, cudaStream_t s) {
-    size_t shm = node_pass_args(a.g, a.np, a.W);
+    size_t shm = node_pass_args(a.g, a.np, a.W, dynamic_smem((const void *)k_small_refine<UNIT, RANK>));
     select_order_args(a.g, a.so);
     rebalance_start_args(a.g, a.rs);
     shm = std::max(shm, rebalance_order_args(a.g, a.rt));
