@@ -22,8 +22,17 @@ constexpr int kQ = 20;                       // fixed-point bits of the penalty 
 constexpr int kMaxK = 4096;
 constexpr int kHubDegree = 4096;             // nodes above this degree get CTA-wide treatment
 
-// A failing CUDA call is turned into UPR_ERR_CUDA by the entry points.
+// A failing CUDA call is turned into UPR_ERR_CUDA (a failed allocation into
+// UPR_ERR_OOM) by the entry points.
 struct CudaError { cudaError_t e; const char *what; };
+
+// The status of a failed call.  The runtime keeps a host thread's last error
+// until it is read, and every launch is followed by a read: left there, it
+// would fail the thread's next call, on any context, at its first launch.
+inline upr_status failed_status(const CudaError &e) {
+    cudaGetLastError();
+    return e.e == cudaErrorMemoryAllocation ? UPR_ERR_OOM : UPR_ERR_CUDA;
+}
 
 #define UPR_CUDA(call)                                                     \
     do {                                                                   \

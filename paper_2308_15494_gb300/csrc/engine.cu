@@ -37,7 +37,7 @@ bool log_enabled() {
 // UPR_LOG: name the failing CUDA call and its error.
 upr_status cuda_failure(const CudaError &e) {
     if (log_enabled()) fprintf(stderr, "upr: %s failed: %s\n", e.what, cudaGetErrorString(e.e));
-    return e.e == cudaErrorMemoryAllocation ? UPR_ERR_OOM : UPR_ERR_CUDA;
+    return failed_status(e);
 }
 
 // Bump allocator over one cudaMalloc; a first pass with base == nullptr sizes it.

@@ -243,7 +243,7 @@ upr_status mixed_create(const upr_graph *graphs, int32_t n_graphs, const int32_t
         UPR_CUDA(cudaEventCreate(&mb->ev_t1));
         rc = mixed_bind(mb, graphs, n_graphs, k, eps, mb->prm);
     } catch (const CudaError &e) {
-        rc = e.e == cudaErrorMemoryAllocation ? UPR_ERR_OOM : UPR_ERR_CUDA;
+        rc = failed_status(e);
     } catch (const std::bad_alloc &) {
         rc = UPR_ERR_OOM;
     }
@@ -259,7 +259,7 @@ upr_status mixed_rebind(MixedBatch *mb, const upr_graph *graphs, int32_t n_graph
         UPR_CUDA(cudaSetDevice(mb->device));
         return mixed_bind(mb, graphs, n_graphs, k, eps, mb->prm);
     } catch (const CudaError &e) {
-        return e.e == cudaErrorMemoryAllocation ? UPR_ERR_OOM : UPR_ERR_CUDA;
+        return failed_status(e);
     } catch (const std::bad_alloc &) {
         return UPR_ERR_OOM;
     }
@@ -336,7 +336,7 @@ upr_status mixed_refine(MixedBatch *mb, int32_t *part, int32_t rounds, uint64_t 
         st.ms_device = ms;
         if (stats) *stats = st;
     } catch (const CudaError &e) {
-        return e.e == cudaErrorMemoryAllocation ? UPR_ERR_OOM : UPR_ERR_CUDA;
+        return failed_status(e);
     }
     return UPR_OK;
 }
@@ -360,7 +360,7 @@ upr_status mixed_cut(MixedBatch *mb, const int32_t *part, int64_t *cut, int64_t 
             }
         }
     } catch (const CudaError &e) {
-        return UPR_ERR_CUDA;
+        return failed_status(e);
     }
     return UPR_OK;
 }

@@ -93,8 +93,8 @@ extern "C" upr_status upr_cut_noalloc(const upr_graph *g, int32_t k, const int32
         UPR_CUDA(cudaMemcpyAsync(cut, out + k, sizeof(int64_t), cudaMemcpyDefault, s));
         if (block_weights) UPR_CUDA(cudaMemcpyAsync(block_weights, out, sizeof(int64_t) * k, cudaMemcpyDefault, s));
         UPR_CUDA(cudaStreamSynchronize(s));
-    } catch (const upr::CudaError &) {
-        return UPR_ERR_CUDA;
+    } catch (const upr::CudaError &e) {
+        return upr::failed_status(e);
     }
     return UPR_OK;
 }

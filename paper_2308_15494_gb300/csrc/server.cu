@@ -315,9 +315,9 @@ upr_status upr_server_create(const upr_server_params *p, upr_server **out) {
     upr_server *s = new (std::nothrow) upr_server();
     if (!s) return UPR_ERR_OOM;
     s->p = prm;
-    if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return UPR_ERR_CUDA; }
+    if (cudaGetDevice(&s->device) != cudaSuccess) { cudaGetLastError(); delete s; return UPR_ERR_CUDA; }
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { delete s; return UPR_ERR_CUDA; }
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); delete s; return UPR_ERR_CUDA; }
     s->budget = prm.memory_budget > 0 ? (size_t)prm.memory_budget : free_b / 10 * 8;
     s->held.assign(prm.max_jobs, 0);
     try {

@@ -47,3 +47,54 @@ def test_small_graph_where_the_buckets_stop_fitting(upr, n, k, weighted, graphs)
     assert w.m + n * k <= 1 << 19
     ctx = upr.create_from_workload(w, params=_params(upr, graphs=graphs))
     _refined_as_the_oracle(upr, ctx, w, calls=2)
+
+
+AFTER_A_FAILED_CALL = r"""
+import sys
+sys.path.insert(0, {root!r})
+import numpy as np, torch
+import oracle, synth
+import paper_2308_15494_gb300 as upr
+
+def valid(k):
+    w = synth.random_small(9, 900, 6.0, k)
+    ctx = upr.create_from_workload(w)
+    p = w.part.copy()
+    st = upr.upr_refine(ctx, p, 3)
+    rc, p0, c0, _ = oracle.refine(w, w.part, rounds=3)
+    assert rc == oracle.OK and np.array_equal(p, p0) and st.cut_out == c0
+    return ctx, w
+
+kept, w = valid(5)                         # (everything is loaded and warm)
+graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+x = torch.zeros(8, device="cuda")
+status = None
+try:
+    with torch.cuda.stream(side):
+        graph.capture_begin(capture_error_mode="global")
+        x.add_(1)
+        try:                               # allocates: refused while the thread captures
+            upr.create_from_workload(w)
+        except upr.UprError as e:
+            status = e.status
+        graph.capture_end()
+except RuntimeError:                       # (the refused call has ended the capture)
+    pass
+assert status in (upr.UPR_ERR_CUDA, upr.UPR_ERR_OOM), status
+p = w.part.copy()
+upr.upr_refine(kept, p, 3)                 # a kept context, then a new one
+valid(7)
+print("ok")
+"""
+
+
+def test_a_failed_call_leaves_the_next_one_alone(upr):
+    """A call that a CUDA error ends (here: an allocation that the runtime
+    refuses during a stream capture) does not fail the calls after it."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", AFTER_A_FAILED_CALL.format(root=root)], cwd=root, capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
