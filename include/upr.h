@@ -391,6 +391,14 @@ void upr_server_destroy(upr_server *s);
  * omega(I(v)).  W (n*k int32) and wI (n int64) are host buffers (NULL to skip). */
 upr_status upr_debug_gain_table(upr_ctx *ctx, const int32_t *part, int32_t *W, int64_t *wI);
 
+/* One grid barrier of the context's launches (those of more than 65536 nodes
+ * have them: UPR_ERR_INVALID otherwise) in which the last `absent` CTAs never
+ * arrive (absent < *ctas).  *ctas = the CTAs of such a launch, *passed = those
+ * that went past the barrier: all with absent = 0, none otherwise.  A barrier
+ * that gave up stays closed: the context's calls return UPR_ERR_CUDA until it
+ * is bound anew (upr_batch_rebind). */
+upr_status upr_debug_barrier(upr_ctx *ctx, int32_t absent, int32_t *ctas, int32_t *passed);
+
 /* Trace of one round (host buffers; any pointer may be NULL).  Capacities:
  * node-indexed arrays n, the pre-merge sequence 2n, I_eligible n+1, bucket
  * k*73 (slot s in column s+32), factor 73. */

@@ -85,6 +85,7 @@ SIGNATURES = {
     "upr_wait": (I32, [P, U64, I64, P, ctypes.POINTER(I64), ctypes.POINTER(Stats)]),
     "upr_server_destroy": (None, [P]),
     "upr_debug_gain_table": (I32, [P, P, P, P]),
+    "upr_debug_barrier": (I32, [P, I32, ctypes.POINTER(I32), ctypes.POINTER(I32)]),
     "upr_debug_round": (I32, [P, P, I32, I32, I32, ctypes.POINTER(Trace)]),
     "upr_batch_create": (I32, [ctypes.POINTER(Graph), I32, I32, P, ctypes.POINTER(Params), ctypes.POINTER(P)]),
     "upr_batch_create_mixed": (I32, [ctypes.POINTER(Graph), I32, P, P, ctypes.POINTER(Params), ctypes.POINTER(P)]),
@@ -246,6 +247,15 @@ def upr_debug_gain_table(ctx: Context, part) -> tuple[np.ndarray, np.ndarray]:
     if rc != UPR_OK:
         raise UprError(rc, "upr_debug_gain_table")
     return W, wI
+
+
+def upr_debug_barrier(ctx, absent: int = 0) -> tuple[int, int]:
+    """One grid barrier of ctx's launches without its last `absent` CTAs; returns (CTAs, CTAs that passed)."""
+    ctas, passed = I32(), I32()
+    rc = load().upr_debug_barrier(ctx.handle, absent, ctypes.byref(ctas), ctypes.byref(passed))
+    if rc != UPR_OK:
+        raise UprError(rc, "upr_debug_barrier")
+    return ctas.value, passed.value
 
 
 def upr_debug_round(ctx: Context, part: np.ndarray, r: int, R: int, rebalance_only: bool = False):

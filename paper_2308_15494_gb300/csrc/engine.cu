@@ -2446,6 +2446,20 @@ upr_status upr_debug_gain_table(upr_ctx *c, const int32_t *part, int32_t *W, int
     return UPR_OK;
 }
 
+upr_status upr_debug_barrier(upr_ctx *c, int32_t absent, int32_t *ctas, int32_t *passed) {
+    if (!c || c->mix || c->n < 0 || !ctas || !passed) return UPR_ERR_INVALID;
+    try {
+        int32_t got = 0;
+        if (!barrier_probe(c->team, absent, c->counts + CNT_SLOTS, c->s)) return UPR_ERR_INVALID;
+        read_i32(c, c->counts + CNT_SLOTS, 1, &got);
+        *ctas = c->team.size;
+        *passed = got;
+    } catch (const CudaError &e) {
+        return cuda_failure(e);
+    }
+    return UPR_OK;
+}
+
 upr_status upr_debug_round(upr_ctx *c, int32_t *part, int32_t r, int32_t R, int32_t rebalance_only, upr_trace *trace) {
     if (!c || c->mix || c->n < 0 || c->ng != 1 || !part || !trace || R < 1 || R > 65536 ||
         (!rebalance_only && (r < 1 || r > R)))

@@ -124,6 +124,10 @@ struct Team {
     int size = 1;
 };
 
+// team.cu: one grid barrier of the team, which its last `absent` CTAs never
+// reach; *passed = the CTAs that went past it.  False: the team has no grid barrier.
+bool barrier_probe(const Team &t, int absent, int32_t *passed, cudaStream_t s);
+
 // Grid-stride loop over a device-held count (all threads of the grid).
 #define UPR_FOR(i, cnt) \
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (cnt); i += (int64_t)gridDim.x * blockDim.x)

@@ -345,6 +345,7 @@ __device__ __forceinline__ Appended reb_team_body(const RebalTeam &a, Sm &s, uns
     const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
     const int K = a.K;
     const int64_t n1 = *a.d_n1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_na = 0;      // (until R is appended to)
     if (n1 == 0) {                           // (no sub-round runs, or nothing is listed)
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_np = *a.d_nk = *a.d_na = 0;
         return Appended{a.ctl->nR, 0};
@@ -634,6 +635,7 @@ template <class Sm>
 __device__ __forceinline__ void reb_start_body(const RebalStart &a, Sm &s) {
     const Team &t = a.team;
     const int lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.cond) cudaGraphSetConditional(a.cond, 0);    // (until it is known)
     const team::Seg g = team::warp_seg(a.n);
     long long cnt = 0;
     for (int64_t v = g.b + lane; v < g.e; v += 32) {

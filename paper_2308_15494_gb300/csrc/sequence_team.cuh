@@ -278,11 +278,16 @@ __device__ __forceinline__ void seq_build_body(const SeqBuild &a, Sm &s) {
     deg = warp_sum(deg);
     if (lane == 0 && deg) atomicAdd(reinterpret_cast<unsigned long long *>(a.deg_sum), (unsigned long long)deg);
     UPR_TEAM_FOR(j, nI + 1) a.diff[j] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *a.dX = (int32_t)nX;
-        *a.dI = (int32_t)nI;
+    auto lengths = [&] {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            *a.dX = (int32_t)nX;
+            *a.dI = (int32_t)nI;
+        }
+    };
+    if (!a.gid) {
+        lengths();
+        return;
     }
-    if (!a.gid) return;
     // a batch: each graph's moves contiguous, in their own order
     UPR_TEAM_FOR(g, a.ng) a.seg_beg[g] = a.seg_end[g] = 0;
     team::sync(t);
@@ -306,6 +311,7 @@ __device__ __forceinline__ void seq_build_body(const SeqBuild &a, Sm &s) {
         if (q == 0 || S[q - 1].key != it.key) a.seg_beg[it.key] = (int32_t)q;
         if (q == nI - 1 || S[q + 1].key != it.key) a.seg_end[it.key] = (int32_t)(q + 1);
     }
+    lengths();
 }
 
 // ---- (c2) after the exact gains, in one team launch: prefix gains, the

@@ -31,7 +31,8 @@ constexpr int kTW = kTT / 32;
 constexpr int kTeamMax = 160;            // CTAs at most
 constexpr int kTotSlots = 24;            // published per-CTA totals (one slot per scan of a kernel)
 constexpr int kSortBins = 256;
-constexpr int kMaxSpin = 1 << 22;        // polls before a barrier's wait gives up (error word set)
+constexpr int kMaxSpin = 1 << 22;        // polls before a barrier's wait gives up (some seconds)
+constexpr unsigned long long kBroken = 1ull << 63;     // in the arrival counter: a wait gave up
 
 struct Smem {
     unsigned long long cnt64[kTW * kSortBins / 2];     // digit counts [kTW][bins], or block-weight changes
@@ -58,10 +59,19 @@ constexpr int kClusterMax = 16;          // teams up to this size run as one clu
 // The team's barrier: a CTA barrier for one CTA, a cluster barrier for a
 // cluster, else a grid barrier on an arrival counter that only grows: the
 // barrier a CTA reaches with arrival number `old` ends when the count reaches
-// the next multiple of the grid size.  Every wait is bounded: one that gives
-// up sets the error word, and the launch runs to its end.  (About 1.2 us with
-// 152 CTAs.  Arriving without the old value, by a release reduction, took 0.15
-// us longer; an epoch word per CTA polled by a warp of every CTA 1 us longer.)
+// the next multiple of the grid size.  (About 1.2 us with 152 CTAs.  Arriving
+// without the old value, by a release reduction, took 0.15 us longer; an epoch
+// word per CTA polled by a warp of every CTA 1 us longer.)
+//
+// Every wait on the counter is bounded.  One that gives up sets the counter's
+// top bit, by an exchange that succeeds only while the barrier is incomplete:
+// so every CTA passes a barrier or none does, and a CTA that meets the bit sets
+// the error word and leaves the kernel, at this barrier and at the first one of
+// every later launch (until the next binding clears the counter).  No step then
+// runs on what another CTA has not published, and what a kernel writes behind
+// its last barrier is there in full or not at all: the lengths that other
+// kernels read are written there, and are 0 before.  (A sub-round's next list
+// has its length earlier; it holds nodes either way.)
 __device__ __forceinline__ void sync(const Team &t) {
     if (gridDim.x == 1) {
         __syncthreads();
@@ -73,22 +83,26 @@ __device__ __forceinline__ void sync(const Team &t) {
         return;
     }
     __syncthreads();
+    int broken = 0;
     if (threadIdx.x == 0) {
-        __threadfence();
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
         const unsigned long long old = atomicAdd(t.bar, 1ull);
         const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
         for (int it = 0;; it++) {
             unsigned long long v;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(t.bar) : "memory");
-            if (v >= target) break;
-            if (it >= kMaxSpin || ((it & 1023) == 1023 && *(volatile const int32_t *)t.err != 0)) {
-                atomicOr(t.err, 2);
+            broken = (v & kBroken) != 0;
+            if (broken || v >= target) break;
+            // (the exchange fails only when another CTA has just arrived or given up)
+            if (it >= kMaxSpin && atomicCAS(t.bar, v, v | kBroken) == v) {
+                broken = 1;
                 break;
             }
             if (it >= 16) __nanosleep(32);
         }
+        if (broken) atomicOr(t.err, 2);
     }
-    __syncthreads();
+    if (__syncthreads_or(broken)) asm volatile("exit;");
 }
 
 // A value of CTA c's shared memory (c in this team, a cluster).

@@ -98,3 +98,54 @@ def test_a_failed_call_leaves_the_next_one_alone(upr):
     r = subprocess.run([sys.executable, "-c", AFTER_A_FAILED_CALL.format(root=root)], cwd=root, capture_output=True,
                        text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("graphs", [0, 1, 2])
+def test_a_barrier_that_gives_up_stops_every_step(upr, graphs):
+    """A grid barrier that one CTA never reaches: the wait runs out and no CTA
+    goes past it.  The context's next calls then end with an error status, the
+    partition as it was, in every form of the rounds (launched one by one, the
+    rebalancing loops or the whole call as captured graphs), and a binding
+    brings the context back."""
+    w = synth.random_small(73, 70000, 5.0, 6, hubs=1)
+    ctx = upr.create_from_workload(w, params=_params(upr, graphs=graphs))
+    _refined_as_the_oracle(upr, ctx, w, calls=4)
+    ctas, passed = upr.upr_debug_barrier(ctx, 0)
+    assert ctas > 16 and passed == ctas
+    ctas, passed = upr.upr_debug_barrier(ctx, 1)
+    assert passed == 0
+    for _ in range(2):
+        p = w.part.copy()
+        with pytest.raises(upr.UprError) as e:
+            upr.upr_refine(ctx, p, 3)
+        assert e.value.status == upr.UPR_ERR_CUDA and np.array_equal(p, w.part)
+    upr.upr_rebind(ctx, w.xadj, w.adj, w.k, w.eps, vwgt=w.vwgt, adjw=w.adjw)
+    _refined_as_the_oracle(upr, ctx, w, calls=3)
+
+
+def test_a_batch_whose_barrier_gave_up(upr):
+    ws = [synth.random_small(74 + i, 18000, 5.0, 6) for i in range(4)]
+    ctx = upr.create_batch_from_workloads(ws)
+    part0 = np.concatenate([w.part for w in ws]).astype(np.int32)
+    p = part0.copy()
+    status, _, cut, _ = upr.upr_batch_refine(ctx, p, 3)
+    assert upr.upr_debug_barrier(ctx, 2)[1] == 0
+    q = part0.copy()
+    with pytest.raises(upr.UprError) as e:
+        upr.upr_batch_refine(ctx, q, 3)
+    assert e.value.status == upr.UPR_ERR_CUDA and np.array_equal(q, part0)
+    upr.upr_batch_rebind(ctx, [(w.xadj, w.adj, w.vwgt, w.adjw) for w in ws], [w.k for w in ws], [w.eps for w in ws])
+    q = part0.copy()
+    upr.upr_batch_refine(ctx, q, 3)
+    assert np.array_equal(q, p)
+    for i, w in enumerate(ws):
+        rc, p0, c0, _ = oracle.refine(w, w.part, rounds=3)
+        a, b = ctx.offsets[i], ctx.offsets[i + 1]
+        assert rc == status[i] == 0 and np.array_equal(p[a:b], p0) and cut[i] == c0
+
+
+def test_a_small_team_has_no_grid_barrier(upr):
+    ctx = upr.create_from_workload(synth.random_small(75, 5000, 5.0, 6))
+    with pytest.raises(upr.UprError) as e:
+        upr.upr_debug_barrier(ctx, 0)
+    assert e.value.status == upr.UPR_ERR_INVALID
