@@ -290,6 +290,8 @@ struct upr_ctx {
 
 namespace {
 
+// The workspace of a context whose sizes and team are set.  (Arithmetic alone:
+// the server sizes queued jobs with it, on threads that may have no device.)
 void layout(upr_ctx *c, Arena &A) {
     const size_t n = (size_t)std::max<int64_t>(c->n, 1), m = (size_t)std::max<int64_t>(c->m, 1);
     const size_t kr = (size_t)c->k;                   // table row width
@@ -370,7 +372,6 @@ void layout(upr_ctx *c, Arena &A) {
     c->scal = A.take<int64_t>(4);    // [0] wmax, [1] degree sum of M, [2] degree sum of undone moves
     c->cut_in = A.take<int64_t>(ng);                 // the input cut per graph (the first round's node pass)
     c->pk = A.take<int2>(n);
-    c->team.size = team_size((int64_t)n, c->beside);
     const size_t ctas = (size_t)std::max(c->team.size, n <= kSmallNodes ? team::kClusterMax : 1);
     c->team.hist = A.take<int32_t>(ctas * team::kSortBins);
     c->team.hist64 = A.take<unsigned long long>(2 * ctas * team::kSortBins);
@@ -2038,7 +2039,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     } up_guard{c};
     if (ng == 1 && m > 0 && c->mem) {
         upr_ctx dry;
-        dry.n = n; dry.m = m; dry.k = k; dry.ng = ng; dry.beside = c->beside;
+        dry.n = n; dry.m = m; dry.k = k; dry.ng = ng;
         Arena D;
         D.base = reinterpret_cast<char *>((uintptr_t)1 << 20);
         layout(&dry, D);
@@ -2121,6 +2122,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     const auto t_sched = std::chrono::steady_clock::now();
     c->m = m; c->k = k;
     c->n = n;                       // layout needs the sizes
+    c->team.size = team_size(n, c->beside, std::min(device_sm_count(), team::kTeamMax));
     c->n_chunks = ht[0];
     c->n_tiles = tile_nodes ? ht[1] : 0;
     c->tile_nodes = tile_nodes;
@@ -2495,6 +2497,7 @@ size_t upr_ctx_footprint(int64_t n, int64_t m, int32_t k, int32_t ng) {
     c.n_chunks = m / 4096 + 1;
     c.n_tiles = n + 1;
     c.sp_slots = 0;     // the dense layout bounds the sparse one (rows chosen by size take half as many bytes)
+    c.team.size = team_size(n, 1, team::kTeamMax);
     Arena A;
     layout(&c, A);
     // plus the staging buffer of the offsets and schedule counts

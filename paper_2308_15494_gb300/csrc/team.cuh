@@ -359,11 +359,11 @@ __device__ __forceinline__ int bits_of(uint32_t x) { return 32 - __clz((int)x); 
 // the SMs between them; with the whole GPU each, they would wait for one
 // another at every launch (1024 Chung-Lu graphs in five batches: 18.0 ms at
 // 30 CTAs each, 20.5 ms at 152; one batch alone: 18.0 ms at 152, 29.5 ms at 30).
-inline int team_size(int64_t n, int beside) {
+// sms: the device's SMs, at most kTeamMax.
+inline int team_size(int64_t n, int beside, int sms) {
     if (n <= 2048) return 1;
     const int64_t want = ceil_div(n, (int64_t)1024);
     if (n <= 65536) return (int)std::min<int64_t>(want, team::kClusterMax);
-    const int sms = std::min(device_sm_count(), team::kTeamMax);
     return (int)std::min<int64_t>(std::max(team::kClusterMax + 1, sms / std::max(1, beside)), want);
 }
 
