@@ -190,6 +190,7 @@ struct upr_ctx {
     // with sparse rows there is no dense table in the arena: one is allocated
     // here only if a round falls back to it (or for the debug entry point)
     int32_t *W_own = nullptr; size_t W_own_bytes = 0;
+    TableTile *tiles_own = nullptr;   // and the tiles of its builds
     // the rebalancing loop as one CUDA graph (a while node over one sub-round),
     // built for the binding and the proposal schedule it was captured with
     cudaStream_t s_cap = nullptr;     // capture stream (non-blocking)
@@ -1129,6 +1130,9 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     return infeasible ? UPR_ERR_INFEASIBLE : UPR_OK;
 }
 
+// Rows of a tile of the dense table's build (at most 32 KB of shared memory up to 2048 columns).
+int32_t dense_tile_nodes(int32_t k) { return (int32_t)std::max<int64_t>(4, std::min<int64_t>(512, 8192 / k)); }
+
 // The dense table of a context bound with sparse rows (allocated on first use).
 void ensure_dense(upr_ctx *c) {
     if (c->W) return;
@@ -1146,6 +1150,33 @@ void ensure_dense(upr_ctx *c) {
     c->W = c->W_own;
 }
 
+// From hashed rows to the dense table for the rest of the binding, with tiles
+// for dense rows: those of hashed rows hold kSparseTileNodes rows, 128 KB of
+// shared memory at 256 columns, one CTA per SM (2^19 nodes, 256 blocks: 0.24 ms
+// a build on them, 0.16 on dense tiles; 2^17 nodes 0.070 and 0.050).
+void use_dense(upr_ctx *c) {
+    ensure_dense(c);
+    // (the binding's staging and hub list, in place again: the tiles alone differ)
+    const int32_t nodes = dense_tile_nodes(c->k);
+    int64_t *cnt = c->xs + c->n + 1, *tot = cnt + 4 * sched_segments(c->n), n_tiles = 0;
+    sched_count(c->xadj, c->n, c->m, nodes, 0, c->k, cnt, tot, c->s);
+    read_i64(c, tot + 1, 1, &n_tiles);
+    if (c->tiles_own) { cudaFree(c->tiles_own); c->tiles_own = nullptr; }
+    if (cudaMalloc(&c->tiles_own, sizeof(TableTile) * (size_t)std::max<int64_t>(n_tiles, 1)) != cudaSuccess) {
+        cudaGetLastError();
+        throw CudaError{cudaErrorMemoryAllocation, "dense table tiles"};
+    }
+    sched_write(c->xadj, c->n, c->m, nodes, 0, c->k, cnt, c->hub_chunks, c->tiles_own, nullptr,
+                reinterpret_cast<int32_t *>(c->sb[0].v), c->s);
+    c->tiles = c->tiles_own;
+    c->n_tiles = n_tiles;
+    c->tile_nodes = nodes;
+    c->sparse_on = false;
+    c->G.sp.slot = nullptr;
+    c->table_valid = false;
+    c->gen++;
+}
+
 // A round; when a sparse row overflows, the round runs again from the same
 // state on rows built afresh, and when fresh rows overflow, on the dense table.
 upr_status run_round(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only, RoundInfo &ri, TraceSink *tr,
@@ -1158,11 +1189,7 @@ upr_status run_round(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only, Roun
             continue;
         }
         if (rc != kRedoDense) return rc;
-        ensure_dense(c);
-        c->sparse_on = false;
-        c->G.sp.slot = nullptr;
-        c->table_valid = false;
-        c->gen++;
+        use_dense(c);
     }
 }
 
@@ -1171,6 +1198,7 @@ void free_ctx(upr_ctx *c) {
     if (c->mix) mixed_destroy(c->mix);
     if (c->mem) cudaFree(c->mem);
     if (c->W_own) cudaFree(c->W_own);
+    if (c->tiles_own) cudaFree(c->tiles_own);
     if (c->reb_exec) cudaGraphExecDestroy(c->reb_exec);
     if (c->step_exec) cudaGraphExecDestroy(c->step_exec);
     if (c->s_cap) cudaStreamDestroy(c->s_cap);
@@ -1376,12 +1404,7 @@ bool lp_round(upr_ctx *c, int64_t *cut, int64_t *active_next, RoundInfo &ri) {
         const int rc = lp_round_once(c, cut, active_next, ri);
         if (rc != kLpRedo) return rc == 1;
         c->table_valid = false;
-        if (attempt >= 1) {
-            ensure_dense(c);
-            c->sparse_on = false;
-            c->G.sp.slot = nullptr;
-            c->gen++;
-        }
+        if (attempt >= 1) use_dense(c);
     }
 }
 
@@ -2099,7 +2122,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     // min(k, deg(v)) + 1); chosen by size (mode 0) when k >= 128 and the rows
     // take at most half the bytes of the dense table (else the schedules are
     // counted again for dense tiles)
-    const int32_t dense_nodes = (int32_t)std::max<int64_t>(4, std::min<int64_t>(512, 8192 / k));
+    const int32_t dense_nodes = dense_tile_nodes(k);
     const int mode = prm.table;
     int sp_mode = (k % 4 == 0 && k <= kSparseRowMax / 2 && (mode >= 2 || (mode == 0 && k >= 128)))
                       ? (mode == 3 ? 3 : 1) : 0;
@@ -2128,6 +2151,7 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     c->tile_nodes = tile_nodes;
     Arena A;
     if (c->W_own) { cudaFree(c->W_own); c->W_own = nullptr; c->W_own_bytes = 0; }
+    if (c->tiles_own) { cudaFree(c->tiles_own); c->tiles_own = nullptr; }
     c->gen++;                       // kernels captured for the previous binding are stale
     c->rounds_bound = 0;
     c->calls_bound = 0;

@@ -159,7 +159,7 @@ struct TableTile { int64_t e0, e1; int32_t v0, v1; };
 // segment s's hub chunks, tiles, hashed-row slots and hubs; tot[0..3] = the
 // totals.  sp_mode 0:
 // no hashed rows, 1: min(k, 2 deg) + 1 slots rounded up to a power of two,
-// 3: min(k, deg) + 1.  sched_write fills the arrays (nullptr: not written).
+// 3: min(k, deg) + 1.  sched_write fills the arrays (sp_off with hashed rows).
 constexpr int64_t kSchedSegment = 1024;
 int64_t sched_segments(int64_t n);
 void sched_count(const int64_t *xadj, int64_t n, int64_t m, int tile_nodes, int sp_mode, int32_t k, int64_t *cnt,

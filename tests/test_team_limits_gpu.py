@@ -149,3 +149,32 @@ def test_a_small_team_has_no_grid_barrier(upr):
     with pytest.raises(upr.UprError) as e:
         upr.upr_debug_barrier(ctx, 0)
     assert e.value.status == upr.UPR_ERR_INVALID
+
+
+@pytest.mark.parametrize("k,deg", [(8, 3.0), (128, 9.0), (256, 9.0)])
+def test_dense_rounds_after_hashed_rows_ran_out(upr, k, deg):
+    """Rows of min(k, deg) + 1 slots run out and the binding goes on with the
+    dense table, on tiles of its own (512 rows at k = 8, 32 at k = 256): results,
+    a later call's and the table itself as the oracle's; a binding after it
+    starts on hashed rows again."""
+    w = synth.random_small(76 + k, 9000, deg, k, hubs=1)
+    ctx = upr.create_from_workload(w, params=_params(upr, table=3))
+    for _ in range(2):
+        st = _refined_as_the_oracle(upr, ctx, w, calls=2)
+        assert st.sparse_table == 0
+        W, _ = upr.upr_debug_gain_table(ctx, w.part)
+        assert np.array_equal(W, oracle.gain_table(w, w.part)[0])
+        upr.upr_rebind(ctx, w.xadj, w.adj, w.k, w.eps, vwgt=w.vwgt, adjw=w.adjw)
+        W, _ = upr.upr_debug_gain_table(ctx, w.part)          # (from the hashed rows)
+        assert np.array_equal(W, oracle.gain_table(w, w.part)[0])
+
+
+def test_label_propagation_falls_back_from_hashed_rows(upr):
+    w = synth.random_small(77, 9000, 9.0, 128)
+    ctx = upr.create_from_workload(w, params=_params(upr, table=3, lp_rounds=4))
+    rc, p0, c0, _ = oracle.refine(w, w.part, rounds=3, p=oracle.params(lp_rounds=4))
+    for _ in range(2):
+        p = w.part.copy()
+        st = upr.upr_refine(ctx, p, 3)
+        assert np.array_equal(p, p0) and st.cut_out == c0
+    assert st.sparse_table == 0
