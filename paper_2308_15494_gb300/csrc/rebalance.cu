@@ -70,9 +70,10 @@ __global__ void __launch_bounds__(256) k_propose_vec(const GraphDev g, const int
     const int gbase = (threadIdx.x & 31) & ~(G - 1);
     // PACK (unit weights, one graph): a column's score is one integer,
     // (omega << kb) + (2^kb - 1 - b), whose maximum is the largest omega, ties
-    // to the smaller block.  The second part is fixed for the launch, and so
-    // low for a block without room for a node of weight 1 that the score is
-    // negative (omega << kb < 2^30); a score below 2^kb has omega = 0.  The
+    // to the smaller block.  The second part is fixed for the launch, and -2^31
+    // for a block without room for a node of weight 1: omega << kb is at most
+    // 2^31 - 2^kb (gb + kb <= 31), so that such a score is negative and every
+    // other one stays below 2^31; a score below 2^kb has omega = 0.  The
     // loop issues instructions rather than waits for rows (2.2 million rows of
     // 64 blocks, 0.6 of every issue slot at 3.7 TB/s), and this takes two per
     // column, where a mask of the allowed columns took six (with the same change to

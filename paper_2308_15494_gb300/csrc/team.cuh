@@ -31,7 +31,7 @@ constexpr int kTW = kTT / 32;
 constexpr int kTeamMax = 160;            // CTAs at most
 constexpr int kTotSlots = 24;            // published per-CTA totals (one slot per scan of a kernel)
 constexpr int kSortBins = 256;
-constexpr int kMaxSpin = 1 << 22;        // polls before a barrier's wait gives up (some seconds)
+constexpr int kMaxSpin = 1 << 22;        // polls before a barrier's wait gives up (about a second)
 constexpr unsigned long long kBroken = 1ull << 63;     // in the arrival counter: a wait gave up
 
 struct Smem {

@@ -7,6 +7,7 @@ import pytest
 
 import oracle
 import synth
+from tests.test_parity_gpu import _compare_traces
 
 pytestmark = pytest.mark.gpu
 
@@ -178,3 +179,30 @@ def test_label_propagation_falls_back_from_hashed_rows(upr):
         st = upr.upr_refine(ctx, p, 3)
         assert np.array_equal(p, p0) and st.cut_out == c0
     assert st.sparse_table == 0
+
+
+@pytest.mark.parametrize("bits", [30, 31, 32])
+@pytest.mark.parametrize("k", [4, 24, 64])
+def test_packed_scores_at_their_width(upr, k, bits):
+    """Unit node weights and edge weights so heavy that the largest omega(I(v))
+    and a column index take `bits` bits together: the selection packs a score
+    and its column into one integer up to 30, the proposals up to 31."""
+    w = synth.random_small(78 + k, 3000, 8.0, k, weighted=False, hubs=1, balanced=False)
+    gb = bits - max(1, (k - 1).bit_length())
+    adjw = synth.edge_weights_uniform(w.xadj, w.adj, 1, 16, 5).astype(np.int64)
+    heaviest = max(int(adjw[w.xadj[v]:w.xadj[v + 1]].sum()) for v in range(w.n))
+    adjw *= ((1 << gb) - 1) // heaviest
+    heaviest = max(int(adjw[w.xadj[v]:w.xadj[v + 1]].sum()) for v in range(w.n))
+    assert heaviest.bit_length() == gb
+    w.adjw = adjw.astype(np.int32)
+    ctx = upr.create_from_workload(w, params=_params(upr, graphs=0))       # (the rounds launched step by step)
+    st = _refined_as_the_oracle(upr, ctx, w)
+    assert st.repaired_input == 1 and st.n_rebalance_moves > 0 and st.n_moves > 0
+    rc, p, t = upr.upr_debug_round(ctx, w.part, 0, 2, rebalance_only=True)
+    rc0, p0, _, o = oracle.run_round(w, w.part, 0, 2, rebalance_only=True)
+    assert rc == rc0 == 0 and np.array_equal(p, p0)
+    _compare_traces(t, o)
+    rc, p, t = upr.upr_debug_round(ctx, p0, 1, 2)
+    rc0, p1, _, o = oracle.run_round(w, p0, 1, 2)
+    assert rc == rc0 == 0 and np.array_equal(p, p1)
+    _compare_traces(t, o)
