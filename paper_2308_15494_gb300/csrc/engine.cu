@@ -1130,6 +1130,19 @@ upr_status run_round_once(upr_ctx *c, int32_t r, int32_t R, bool rebalance_only,
     return infeasible ? UPR_ERR_INFEASIBLE : UPR_OK;
 }
 
+// Room for the penalty factors of a call's rounds, on the device and page-locked.
+void reserve_factors(upr_ctx *c, int32_t rounds) {
+    if (c->F_all_cap >= rounds) return;
+    if (c->F_all) cudaFree(c->F_all);
+    if (c->hF_all) cudaFreeHost(c->hF_all);
+    c->F_all = nullptr;
+    c->hF_all = nullptr;
+    c->F_all_cap = 0;
+    UPR_CUDA(cudaMalloc(&c->F_all, sizeof(int64_t) * kSlots * (size_t)rounds));
+    UPR_CUDA(cudaMallocHost(&c->hF_all, sizeof(int64_t) * kSlots * (size_t)rounds));
+    c->F_all_cap = rounds;
+}
+
 // Rows of a tile of the dense table's build (at most 32 KB of shared memory up to 2048 columns).
 int32_t dense_tile_nodes(int32_t k) { return (int32_t)std::max<int64_t>(4, std::min<int64_t>(512, 8192 / k)); }
 
@@ -1507,16 +1520,7 @@ bool build_step_graph(upr_ctx *c, int32_t rounds, int32_t total) {
 
 // The penalty factors of rounds 1..rounds, copied in one piece.
 void upload_factors(upr_ctx *c, int32_t rounds, int32_t total) {
-    if (c->F_all_cap < rounds) {
-        if (c->F_all) cudaFree(c->F_all);
-        if (c->hF_all) cudaFreeHost(c->hF_all);
-        c->F_all = nullptr;
-        c->hF_all = nullptr;
-        c->F_all_cap = 0;
-        UPR_CUDA(cudaMalloc(&c->F_all, sizeof(int64_t) * kSlots * (size_t)rounds));
-        UPR_CUDA(cudaMallocHost(&c->hF_all, sizeof(int64_t) * kSlots * (size_t)rounds));
-        c->F_all_cap = rounds;
-    }
+    reserve_factors(c, rounds);
     // (a call ends by synchronising its stream, so no earlier copy still reads hF_all)
     for (int32_t i = 1; i <= rounds; i++)
         penalty_factors(c->prm.round_offset + i, total, c->prm.tau1_num, c->prm.tau1_den,
@@ -1603,10 +1607,13 @@ int small_size(const upr_ctx *c) {
     return c->n <= 8192 ? 8 : team::kClusterMax;
 }
 
-bool small_applies(const upr_ctx *c, int32_t rounds) {
-    return c->prm.graphs >= 1 && c->prm.schedule == 0 && !c->prm.lock_rebalanced && rounds >= 1 &&
-           rounds <= kSmallRounds && !log_enabled() && small_work(c) <= kSmallWork &&
+bool small_binding(const upr_ctx *c) {
+    return c->prm.graphs >= 1 && c->prm.schedule == 0 && !c->prm.lock_rebalanced && small_work(c) <= kSmallWork &&
            small_refine_ok(c->G, c->gbits, c->cbits);
+}
+
+bool small_applies(const upr_ctx *c, int32_t rounds) {
+    return rounds >= 1 && rounds <= kSmallRounds && !log_enabled() && small_binding(c);
 }
 
 void run_small(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
@@ -2260,6 +2267,8 @@ upr_status bind_graphs(upr_ctx *c, const upr_graph *gs, int32_t ng, int32_t k, c
     UPR_CUDA(cudaMemsetAsync(c->counts, 0, 64 * sizeof(int32_t), s));
     fill_i32(c->m_pos, n, -1, s);
     fill_i32(c->r_to, n, -1, s);
+    // (refinement allocates nothing: the one launch of a small graph has its factors' room from here)
+    if (small_binding(c)) reserve_factors(c, kSmallRounds);
     UPR_CUDA(cudaStreamSynchronize(s));
     c->bkey = bind_key(c);
     if (kept_ok && c->bkey == key0) {
