@@ -1575,7 +1575,7 @@ bool run_step_graph(upr_ctx *c, int32_t rounds, int32_t total, upr_stats &st) {
     return true;
 }
 
-// All rounds in one launch (small.cu): one small graph, the plain tau schedule,
+// All rounds in one launch (small_form.cuh): one small graph, the plain tau schedule,
 // the dense table.  The line is on what a round reads at most, adjacency
 // entries and table cells: one cluster has a tenth of the chip's SMs, and the
 // launches and waits it saves are worth some 40 us a round.  Four rounds, step

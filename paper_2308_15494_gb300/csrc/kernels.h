@@ -532,7 +532,7 @@ void seq_apply_prefix_seg(const GraphDev &g, const int32_t *I_node, const int32_
                           const int32_t *d_nI, int64_t max, const int32_t *seg_beg, const long long *best_j,
                           int32_t *part0, int64_t *C0, cudaStream_t s);
 
-// ---- small.cu: all rounds of a call on a small graph in one launch
+// ---- small.cu, small_form.cuh: all rounds of a call on a small graph in one launch
 // The team is one CTA or one cluster (n <= kSmallNodes), the table dense, keys
 // within 63 bits and scores and blocks within 32.
 constexpr int64_t kSmallNodes = 65536;
